@@ -48,7 +48,7 @@ typedef enum {
     LRD_ERR_BAD_RANK = 2,     /* r < 1 or r > min(K, N); no multiple fits in lrd_rank_quantize */
     LRD_ERR_ALIGNMENT = 3,    /* a base pointer is not aligned to its element size / workspace not 256-B aligned */
     LRD_ERR_WORKSPACE = 4,    /* workspace NULL or too small */
-    LRD_ERR_UNSUPPORTED = 5,  /* convolution geometry other than k = 3, stride 1, pad 1 */
+    LRD_ERR_UNSUPPORTED = 5,  /* convolution geometry outside the set in lrd_tucker2_desc_t */
     LRD_ERR_ARCH = 6,         /* current device is not sm_100 */
     LRD_ERR_CUDA = 7,         /* a CUDA runtime / driver call failed */
     LRD_ERR_TIMEOUT = 8,      /* a bounded device-side wait ran out (see lrd_check_device_status) */
@@ -89,8 +89,8 @@ typedef struct {
     int64_t B, H, W, C, S, r1, r2;  /* NHWC activations [B][H][W][C] -> [B][H][W][S] */
     int64_t k, stride, pad;         /* k x k core: k odd, 1..7; stride 1 or 2 (on the core); pad = (k - 1) / 2.
                                      * The output is [B][Ho][Wo][S] with Ho = (H - 1) / stride + 1, Wo likewise.
-                                     * k = 3, stride = 1 runs the core on the tensor-core kernels (bf16, shapes
-                                     * permitting); every other geometry runs it on the general fp32-FMA kernels.
+                                     * bf16 runs the core on the tensor-core kernels whatever its k and stride (ranks off a
+                                     * multiple of 8 are repacked), fp32 on the general FMA kernels.
                                      * Anything else: LRD_ERR_UNSUPPORTED. */
     int32_t dtype;
 } lrd_tucker2_desc_t;

@@ -1,6 +1,6 @@
 // Tucker-2 decomposed k x k convolution (NHWC): 1x1 product, k x k core (which carries the layer's stride), 1x1
-// product, and the backward pass through them under a freeze mask.  The 3 x 3, stride-1 core runs on the
-// tensor-core kernels where the shape allows; every other geometry runs the core on the general kernels.
+// product, and the backward pass through them under a freeze mask.  The core runs on the tensor-core kernels
+// where the data type and the channel counts allow, whatever its k and stride, else on the general kernels.
 #include "conv.cuh"
 
 #include "streams.cuh"
@@ -15,7 +15,7 @@ struct Tk {
     int64_t Po;             // output pixels B Ho Wo (rows of Z2, Y, dY, dZ2)
     int64_t taps;           // k * k
     ConvGeom g;
-    bool plain;             // 3 x 3, stride 1: the geometry the tensor-core core kernels take
+    bool plain;             // 3 x 3, stride 1: the geometry the one-launch data passes take
     lrd_dtype_t dt;
 };
 
@@ -33,26 +33,25 @@ Tk parse(const lrd_tucker2_desc_t* d) {
 
 size_t act_bytes(const Tk& t, int64_t pixels, int64_t ch) { return align_up((size_t)(pixels > 0 ? pixels : 1) * ch * elem_size(t.dt), 256); }
 
-// Scratch of the three weight-gradient launches of the backward pass, one region each: they may run side by side.
-struct Scratch { size_t dB, dA, filter; };
+// Scratch of the dB and dA launches of the backward pass, one region each: they may run side by side.
+struct Scratch { size_t dB, dA; };
 
 Scratch split_regions(const Tk& t) {
-    Scratch r{0, 0, 0};
+    Scratch r{0, 0};
     if (t.P < 1) return r;
     r.dB = colsum_scratch_bytes(t.Po, t.S);
     if (t.dt == LRD_BF16) {
         const size_t a = tc_split_workspace_bytes(t.S, t.r2, t.Po);
         r.dB = r.dB > a ? r.dB : a;
         r.dA = tc_split_workspace_bytes(t.C, t.r1, t.P);
-        if (t.plain) r.filter = tc_conv_filter_scratch_bytes(t.B, t.H, t.W, t.r1, t.r2);
     }
-    r.dB = align_up(r.dB, 256); r.dA = align_up(r.dA, 256); r.filter = align_up(r.filter, 256);
+    r.dB = align_up(r.dB, 256); r.dA = align_up(r.dA, 256);
     return r;
 }
 
 size_t split_bytes(const Tk& t) {
     const Scratch r = split_regions(t);
-    return r.dB + r.dA + r.filter;
+    return r.dB + r.dA;
 }
 
 bool g_tucker_overlap = true;
@@ -61,7 +60,7 @@ bool g_tucker_overlap = true;
 // layer, the factors -- small -- are copied into the workspace with the ranks rounded up to multiples of 16 and
 // zeros in the padding, the layer runs on the tensor-core kernels at the padded ranks, and Z1 / Z2 / dA / dG / dB
 // are copied between the caller's packed layout and padded buffers.
-bool needs_repack(const Tk& t) { return t.plain && t.dt == LRD_BF16 && (t.r1 % 8 || t.r2 % 8) && t.C % 8 == 0 && t.S % 8 == 0; }
+bool needs_repack(const Tk& t) { return t.dt == LRD_BF16 && (t.r1 % 8 || t.r2 % 8) && t.C % 8 == 0 && t.S % 8 == 0; }
 int64_t pad16(int64_t r) { return (r + 15) / 16 * 16; }
 lrd_tucker2_desc_t padded_desc(const lrd_tucker2_desc_t& d) {
     lrd_tucker2_desc_t q = d;
@@ -70,13 +69,14 @@ lrd_tucker2_desc_t padded_desc(const lrd_tucker2_desc_t& d) {
 }
 struct Repack { size_t A, G, Bm, Z1, Z2, dA, dG, dB, total; };
 Repack repack_layout(const Tk& t, size_t inner) {
-    const size_t r1 = (size_t)pad16(t.r1), r2 = (size_t)pad16(t.r2), P = (size_t)(t.P > 0 ? t.P : 1), e = 2;
+    const size_t r1 = (size_t)pad16(t.r1), r2 = (size_t)pad16(t.r2), P = (size_t)(t.P > 0 ? t.P : 1), Po = (size_t)(t.Po > 0 ? t.Po : 1), e = 2;
+    const size_t taps = (size_t)t.taps;
     Repack o;
     size_t at = align_up(inner, 256);
     auto take = [&at](size_t bytes) { const size_t here = at; at += align_up(bytes, 256); return here; };
-    o.A = take((size_t)t.C * r1 * e); o.G = take(r2 * 9 * r1 * e); o.Bm = take((size_t)t.S * r2 * e);
-    o.Z1 = take(P * r1 * e); o.Z2 = take(P * r2 * e);
-    o.dA = take((size_t)t.C * r1 * e); o.dG = take(r2 * 9 * r1 * e); o.dB = take((size_t)t.S * r2 * e);
+    o.A = take((size_t)t.C * r1 * e); o.G = take(r2 * taps * r1 * e); o.Bm = take((size_t)t.S * r2 * e);
+    o.Z1 = take(P * r1 * e); o.Z2 = take(Po * r2 * e);
+    o.dA = take((size_t)t.C * r1 * e); o.dG = take(r2 * taps * r1 * e); o.dB = take((size_t)t.S * r2 * e);
     o.total = at;
     return o;
 }
@@ -124,8 +124,8 @@ lrd_status_t tucker2_fwd(const lrd_tucker2_desc_t* d, const void* X, const void*
         const Repack o = repack_layout(t, inner);
         uint8_t* w = (uint8_t*)ws;
         LRD_TRY(copy2d_bf16(w + o.A, q.r1, A, t.r1, t.C, t.r1, q.r1, s));
-        LRD_TRY(copy2d_bf16(w + o.G, q.r1, G, t.r1, t.r2 * 9, t.r1, q.r1, s));
-        LRD_TRY(zero_fill(w + o.G + (size_t)t.r2 * 9 * q.r1 * 2, (q.r2 - t.r2) * 9, q.r1, q.r1, LRD_BF16, s));
+        LRD_TRY(copy2d_bf16(w + o.G, q.r1, G, t.r1, t.r2 * t.taps, t.r1, q.r1, s));
+        LRD_TRY(zero_fill(w + o.G + (size_t)t.r2 * t.taps * q.r1 * 2, (q.r2 - t.r2) * t.taps, q.r1, q.r1, LRD_BF16, s));
         LRD_TRY(copy2d_bf16(w + o.Bm, q.r2, Bm, t.r2, t.S, t.r2, q.r2, s));
         LRD_TRY(tucker2_fwd(&q, X, w + o.A, w + o.G, w + o.Bm, bias, Y, Z1_save ? w + o.Z1 : nullptr, Z2_save ? w + o.Z2 : nullptr, freeze,
                             w, inner, path, s));
@@ -141,12 +141,10 @@ lrd_status_t tucker2_fwd(const lrd_tucker2_desc_t* d, const void* X, const void*
     void* Z2 = Z2_save ? Z2_save : (void*)((uint8_t*)ws + act_bytes(t, t.P, t.r1));
     LRD_TRY(run_gemm(make_gemm(t.P, t.r1, t.C, X, t.C, false, A, t.r1, true, Z1, t.r1, nullptr, t.dt), path, false, nullptr, 0, s));
     // core + last 1x1 in one launch where the shape allows: Z2 then stays on chip unless the caller saves it
-    if (t.plain && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
-        tc_conv_chain_eligible(false, t.B, t.H, t.W, t.r1, t.r2, t.S, t.dt, Z1, G, Bm, Y, Z2_save) &&
-        (!bias || ((uintptr_t)bias % 2) == 0))
-        return tc_conv3x3_chain(false, Z1, G, Bm, bias, Y, Z2_save, t.B, t.H, t.W, t.r1, t.r2, t.S, s);
-    if (t.plain) LRD_TRY(conv3x3_fwd(Z1, G, Z2, t.B, t.H, t.W, t.r1, t.r2, t.dt, path, s));
-    else LRD_TRY(simt_conv_fwd(Z1, G, Z2, t.B, t.g, t.r1, t.r2, t.dt, s));
+    if ((path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
+        tc_conv_chain_eligible(false, t.B, t.g, t.r1, t.r2, t.S, t.dt, Z1, G, Bm, Y, Z2_save) && (!bias || ((uintptr_t)bias % 2) == 0))
+        return tc_conv_chain(false, Z1, G, Bm, bias, Y, Z2_save, t.B, t.g, t.r1, t.r2, t.S, s);
+    LRD_TRY(conv_fwd(Z1, G, Z2, t.B, t.g, t.r1, t.r2, t.dt, path, s));
     return run_gemm(make_gemm(t.Po, t.S, t.r2, Z2, t.r2, false, Bm, t.r2, false, Y, t.S, bias, t.dt), path, false, nullptr, 0, s);
 }
 
@@ -170,8 +168,8 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
         const Repack o = repack_layout(t, inner);
         uint8_t* w = (uint8_t*)ws;
         LRD_TRY(copy2d_bf16(w + o.A, q.r1, A, t.r1, t.C, t.r1, q.r1, s));
-        LRD_TRY(copy2d_bf16(w + o.G, q.r1, G, t.r1, t.r2 * 9, t.r1, q.r1, s));
-        LRD_TRY(zero_fill(w + o.G + (size_t)t.r2 * 9 * q.r1 * 2, (q.r2 - t.r2) * 9, q.r1, q.r1, LRD_BF16, s));
+        LRD_TRY(copy2d_bf16(w + o.G, q.r1, G, t.r1, t.r2 * t.taps, t.r1, q.r1, s));
+        LRD_TRY(zero_fill(w + o.G + (size_t)t.r2 * t.taps * q.r1 * 2, (q.r2 - t.r2) * t.taps, q.r1, q.r1, LRD_BF16, s));
         LRD_TRY(copy2d_bf16(w + o.Bm, q.r2, Bm, t.r2, t.S, t.r2, q.r2, s));
         if (core) LRD_TRY(copy2d_bf16(w + o.Z1, q.r1, Z1_save, t.r1, t.P, t.r1, q.r1, s));
         if (factors) LRD_TRY(copy2d_bf16(w + o.Z2, q.r2, Z2_save, t.r2, t.Po, t.r2, q.r2, s));
@@ -183,7 +181,7 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
             LRD_TRY(copy2d_bf16(dA, t.r1, w + o.dA, q.r1, t.C, q.r1, t.r1, s));
             LRD_TRY(copy2d_bf16(dB, t.r2, w + o.dB, q.r2, t.S, q.r2, t.r2, s));
         }
-        if (core) LRD_TRY(copy2d_bf16(dG, t.r1, w + o.dG, q.r1, t.r2 * 9, q.r1, t.r1, s));
+        if (core) LRD_TRY(copy2d_bf16(dG, t.r1, w + o.dG, q.r1, t.r2 * t.taps, q.r1, t.r1, s));
         return LRD_OK;
     }
 
@@ -193,7 +191,6 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     uint8_t* scratch0 = (uint8_t*)ws + act_bytes(t, t.P, t.r1) + act_bytes(t, t.Po, t.r2);
     float* pB = (float*)scratch0;
     float* pA = (float*)(scratch0 + reg.dB);
-    float* pF = (float*)(scratch0 + reg.dB + reg.dA);
     (void)ws_bytes;
 
     // What depends on what: dZ2 = dY Bm first; the transposed core (+ dX) and the filter gradient both need dZ2 and
@@ -221,8 +218,7 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     if (factors && sB != s) launch_dB();
 
     auto launch_filter = [&](cudaStream_t st_f) {
-        if (t.plain) keep(conv3x3_bwd_filter(dZ2, Z1_save, dG, t.B, t.H, t.W, t.r1, t.r2, t.dt, path, pF, reg.filter, st_f));
-        else keep(simt_conv_bwd_filter(dZ2, Z1_save, dG, t.B, t.g, t.r1, t.r2, t.dt, st_f));
+        keep(conv_bwd_filter(dZ2, Z1_save, dG, t.B, t.g, t.r1, t.r2, t.dt, path, st_f));
     };
     // the whole data path (dZ2 = dY Bm, transposed core, dX = dZ1 A^T) in one launch where the shape allows; dZ2 is
     // written only for the filter gradient, dZ1 only for dA.  (Giving the filter gradient a dZ2 product of its own
@@ -241,12 +237,11 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
         else launch_filter(sF);
     }
     // transposed core + first 1x1 (dX = dZ1 A^T) in one launch where the shape allows; dZ1 is written only for dA
-    const bool fuse_dx = !one_launch && dX && t.plain && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
-                         tc_conv_chain_eligible(true, t.B, t.H, t.W, t.r1, t.r2, t.C, t.dt, dZ2, G, A, dX, factors ? dZ1 : nullptr);
+    const bool fuse_dx = !one_launch && dX && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
+                         tc_conv_chain_eligible(true, t.B, t.g, t.r1, t.r2, t.C, t.dt, dZ2, G, A, dX, factors ? dZ1 : nullptr);
     if (one_launch) {
-    } else if (fuse_dx) keep(tc_conv3x3_chain(true, dZ2, G, A, nullptr, dX, factors ? dZ1 : nullptr, t.B, t.H, t.W, t.r1, t.r2, t.C, s));
-    else if ((dX || factors) && t.plain) keep(conv3x3_bwd_data(dZ2, G, dZ1, t.B, t.H, t.W, t.r1, t.r2, t.dt, path, s));
-    else if (dX || factors) keep(simt_conv_bwd_data(dZ2, G, dZ1, t.B, t.g, t.r1, t.r2, t.dt, s));
+    } else if (fuse_dx) keep(tc_conv_chain(true, dZ2, G, A, nullptr, dX, factors ? dZ1 : nullptr, t.B, t.g, t.r1, t.r2, t.C, s));
+    else if (dX || factors) keep(conv_bwd_data(dZ2, G, dZ1, t.B, t.g, t.r1, t.r2, t.dt, path, s));
     if (dX && !fuse_dx && !one_launch) keep(run_gemm(make_gemm(t.P, t.C, t.r1, dZ1, t.r1, false, A, t.r1, false, dX, t.C, nullptr, t.dt), path, false, nullptr, 0, s));
     if (factors) {
         if (sB == s) launch_dB();
@@ -261,26 +256,21 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
 
 void tucker2_overlap(bool on) { g_tucker_overlap = on; }
 
-// Core convolution dispatch: tensor-core implicit GEMM where the geometry qualifies, else the general kernels.
-lrd_status_t conv3x3_fwd(const void* in, const void* G, void* out, int64_t B, int64_t H, int64_t W, int64_t ci,
-                         int64_t co, lrd_dtype_t dt, int path, cudaStream_t s) {
-    if (path != LRD_PATH_GENERAL && tc_conv_eligible(B, H, W, ci, co, dt, in, G, out))
-        return tc_conv3x3(false, in, G, out, B, H, W, ci, co, s);
-    return simt_conv_fwd(in, G, out, B, conv_geom(H, W, 3, 1), ci, co, dt, s);
+// Core convolution dispatch: tensor-core implicit GEMM where data type and channel counts qualify, else the general kernels.
+lrd_status_t conv_fwd(const void* in, const void* G, void* out, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt, int path,
+                      cudaStream_t s) {
+    if (path != LRD_PATH_GENERAL && tc_conv_eligible(B, g, ci, co, dt, in, G, out)) return tc_conv(false, in, G, out, B, g, ci, co, s);
+    return simt_conv_fwd(in, G, out, B, g, ci, co, dt, s);
 }
-lrd_status_t conv3x3_bwd_data(const void* dout, const void* G, void* din, int64_t B, int64_t H, int64_t W, int64_t ci,
-                              int64_t co, lrd_dtype_t dt, int path, cudaStream_t s) {
-    if (path != LRD_PATH_GENERAL && tc_conv_eligible(B, H, W, ci, co, dt, dout, G, din))
-        return tc_conv3x3(true, dout, G, din, B, H, W, ci, co, s);
-    return simt_conv_bwd_data(dout, G, din, B, conv_geom(H, W, 3, 1), ci, co, dt, s);
+lrd_status_t conv_bwd_data(const void* dout, const void* G, void* din, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt,
+                           int path, cudaStream_t s) {
+    if (path != LRD_PATH_GENERAL && tc_conv_eligible(B, g, ci, co, dt, dout, G, din)) return tc_conv(true, dout, G, din, B, g, ci, co, s);
+    return simt_conv_bwd_data(dout, G, din, B, g, ci, co, dt, s);
 }
-lrd_status_t conv3x3_bwd_filter(const void* dout, const void* in, void* dG, int64_t B, int64_t H, int64_t W,
-                                int64_t ci, int64_t co, lrd_dtype_t dt, int path, float* scratch, size_t scratch_bytes,
-                                cudaStream_t s) {
-    if (path != LRD_PATH_GENERAL && tc_conv_eligible(B, H, W, ci, co, dt, dout, in, dG) &&
-        scratch_bytes >= tc_conv_filter_scratch_bytes(B, H, W, ci, co))
-        return tc_conv3x3_filter(dout, in, dG, B, H, W, ci, co, scratch, scratch_bytes, s);
-    return simt_conv_bwd_filter(dout, in, dG, B, conv_geom(H, W, 3, 1), ci, co, dt, s);
+lrd_status_t conv_bwd_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt,
+                             int path, cudaStream_t s) {
+    if (path != LRD_PATH_GENERAL && tc_conv_eligible(B, g, ci, co, dt, dout, in, dG)) return tc_conv_filter(dout, in, dG, B, g, ci, co, s);
+    return simt_conv_bwd_filter(dout, in, dG, B, g, ci, co, dt, s);
 }
 
 }  // namespace lrd

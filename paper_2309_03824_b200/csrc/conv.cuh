@@ -39,22 +39,18 @@ lrd_status_t simt_conv_bwd_data(const void* dout, const void* G, void* din, int6
 lrd_status_t simt_conv_bwd_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci,
                                   int64_t co, lrd_dtype_t dt, cudaStream_t s);
 
-// Tensor-core 3x3 core (bf16, W <= 128, channel counts multiples of 8, 16-byte aligned bases).
-bool tc_conv_eligible(int64_t B, int64_t H, int64_t W, int64_t ci, int64_t co, lrd_dtype_t dt, const void* p0,
-                      const void* p1, const void* p2);
-size_t tc_conv_filter_scratch_bytes(int64_t B, int64_t H, int64_t W, int64_t ci, int64_t co);
-lrd_status_t tc_conv3x3(bool dgrad, const void* img, const void* G, void* out, int64_t B, int64_t H, int64_t W, int64_t ci,
-                        int64_t co, cudaStream_t s);
+// Tensor-core k x k core (bf16, channel counts multiples of 8, 16-byte aligned bases; any geometry above).
+bool tc_conv_eligible(int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt, const void* p0, const void* p1, const void* p2);
+lrd_status_t tc_conv(bool dgrad, const void* img, const void* G, void* out, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, cudaStream_t s);
 // The core followed by the 1x1 product that consumes it, in one launch (the core's result stays on chip unless
 // core_out asks for it): forward (dgrad = false) out2 = conv(img, G) Q^T + bias2 with Q = Bm [S x r2]; backward
 // (dgrad = true) out2 = conv^T(img, G) Q^T with Q = A [C x r1].  n2 = rows of Q = columns of out2 (<= 256).
-bool tc_conv_chain_eligible(bool dgrad, int64_t B, int64_t H, int64_t W, int64_t ci, int64_t co, int64_t n2, lrd_dtype_t dt,
+bool tc_conv_chain_eligible(bool dgrad, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, int64_t n2, lrd_dtype_t dt,
                             const void* img, const void* G, const void* Q, const void* out2, const void* core_out);
-lrd_status_t tc_conv3x3_chain(bool dgrad, const void* img, const void* G, const void* Q, const void* bias2, void* out2,
-                              void* core_out, int64_t B, int64_t H, int64_t W, int64_t ci, int64_t co, int64_t n2,
-                              cudaStream_t s);
-lrd_status_t tc_conv3x3_filter(const void* dout, const void* in, void* dG, int64_t B, int64_t H, int64_t W, int64_t ci,
-                               int64_t co, float* scratch, size_t scratch_bytes, cudaStream_t s);
+lrd_status_t tc_conv_chain(bool dgrad, const void* img, const void* G, const void* Q, const void* bias2, void* out2, void* core_out,
+                           int64_t B, const ConvGeom& g, int64_t ci, int64_t co, int64_t n2, cudaStream_t s);
+// Filter gradient, one launch, no scratch.
+lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, cudaStream_t s);
 
 // A whole data pass of the layer in one launch (3 x 3 core, stride 1; ranks <= 128 and multiples of 16, at most 256 output
 // channels, images at most 40 pixels wide): forward (dgrad = false) out3 = conv(in P1, G) P3^T + bias3 with P1 = A [C x r1],
@@ -68,13 +64,12 @@ lrd_status_t tucker_fused(bool dgrad, const void* in, const void* P1, const void
                           void* save1, void* save2, int64_t B, int64_t H, int64_t W, int64_t c_in, int64_t nA, int64_t nB,
                           int64_t n3, cudaStream_t s);
 
-// Path dispatch for the 3x3, stride-1 core (tensor-core kernel where the shape qualifies, else general).
-lrd_status_t conv3x3_fwd(const void* in, const void* G, void* out, int64_t B, int64_t H, int64_t W, int64_t ci,
-                         int64_t co, lrd_dtype_t dt, int path, cudaStream_t s);
-lrd_status_t conv3x3_bwd_data(const void* dout, const void* G, void* din, int64_t B, int64_t H, int64_t W, int64_t ci,
-                              int64_t co, lrd_dtype_t dt, int path, cudaStream_t s);
-lrd_status_t conv3x3_bwd_filter(const void* dout, const void* in, void* dG, int64_t B, int64_t H, int64_t W,
-                                int64_t ci, int64_t co, lrd_dtype_t dt, int path, float* scratch, size_t scratch_bytes,
-                                cudaStream_t s);
+// Path dispatch for the core (tensor-core kernels where the shape qualifies, else general).
+lrd_status_t conv_fwd(const void* in, const void* G, void* out, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt, int path,
+                      cudaStream_t s);
+lrd_status_t conv_bwd_data(const void* dout, const void* G, void* din, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt,
+                           int path, cudaStream_t s);
+lrd_status_t conv_bwd_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt,
+                             int path, cudaStream_t s);
 
 }  // namespace lrd

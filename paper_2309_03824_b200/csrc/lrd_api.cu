@@ -795,7 +795,7 @@ static lrd_status_t conv3x3_check(int64_t B, int64_t H, int64_t W, int64_t C, in
 
 size_t lrd_conv3x3_workspace_bytes(int64_t B, int64_t H, int64_t W, int64_t C, int64_t S, int dtype) {
     if (conv3x3_check(B, H, W, C, S, dtype) != LRD_OK) return 0;
-    return align_up(dtype == LRD_BF16 ? tc_conv_filter_scratch_bytes(B, H, W, C, S) : 0, 256) + 256;
+    return 256;                          // (every step of the layer writes its result directly)
 }
 
 static lrd_status_t lrd_conv3x3_fwd_impl(int64_t B, int64_t H, int64_t W, int64_t C, int64_t S, int dtype, const void* X, const void* Wk,
@@ -806,7 +806,7 @@ static lrd_status_t lrd_conv3x3_fwd_impl(int64_t B, int64_t H, int64_t W, int64_
         if (!elem_aligned(p, dtype)) return LRD_ERR_ALIGNMENT;
     LRD_TRY(check_arch());
     if (B == 0) return LRD_OK;
-    return conv3x3_fwd(X, Wk, Y, B, H, W, C, S, (lrd_dtype_t)dtype, g_path.load(), (cudaStream_t)cuda_stream);
+    return conv_fwd(X, Wk, Y, B, conv_geom(H, W, 3, 1), C, S, (lrd_dtype_t)dtype, g_path.load(), (cudaStream_t)cuda_stream);
 }
 
 static lrd_status_t lrd_conv3x3_bwd_impl(int64_t B, int64_t H, int64_t W, int64_t C, int64_t S, int dtype, const void* dY, const void* X,
@@ -819,8 +819,9 @@ static lrd_status_t lrd_conv3x3_bwd_impl(int64_t B, int64_t H, int64_t W, int64_
     LRD_TRY(check_arch());
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (B == 0) return zero_fill(dW, S, 9 * C, 9 * C, (lrd_dtype_t)dtype, s);
-    if (dX) LRD_TRY(conv3x3_bwd_data(dY, Wk, dX, B, H, W, C, S, (lrd_dtype_t)dtype, g_path.load(), s));
-    return conv3x3_bwd_filter(dY, X, dW, B, H, W, C, S, (lrd_dtype_t)dtype, g_path.load(), (float*)workspace, workspace_bytes - 256, s);
+    const ConvGeom g = conv_geom(H, W, 3, 1);
+    if (dX) LRD_TRY(conv_bwd_data(dY, Wk, dX, B, g, C, S, (lrd_dtype_t)dtype, g_path.load(), s));
+    return conv_bwd_filter(dY, X, dW, B, g, C, S, (lrd_dtype_t)dtype, g_path.load(), s);
 }
 
 size_t lrd_tucker2_workspace_bytes(const lrd_tucker2_desc_t* desc, lrd_tucker_freeze_t freeze, int is_bwd) {

@@ -18,9 +18,15 @@
 // 128 lanes) and store.  The single-thread instructions are issued under elect.sync by a converged warp.  Both
 // operands may be K-major (reduction index contiguous) or MN-major (row / column index contiguous),
 // which covers every product of the forward and backward pass without a transposed copy.
+//
+// CONV: the filter gradient of a k x k convolution, dG[o][tap][i] = sum_p dout[p][o] in[p stride + tap - pad][i], is
+// the same product with the taps side by side as columns (a tap takes whole 64-column blocks): A = dout[pixels x co],
+// and a block of B is 64 consecutive output pixels' input channels at one tap, fetched by TMA in im2col mode.  The
+// reduction runs over all pixels whatever the image size.
 #include <algorithm>
 
 #include "common.cuh"
+#include "conv.cuh"
 #include "ptx.cuh"
 #include "tc.cuh"
 #include "tma.cuh"
@@ -59,15 +65,24 @@ struct TcParams {
     const __nv_bfloat16* bias;
     int partial;        // 1: write fp32 partials
     int cluster_splits; // > 1: the gridDim.z blocks of a tile are one cluster and reduce through shared memory
+    // CONV: input channels, 64-column blocks of a tap and of all taps, k of the k x k taps, output grid, stride, pad
+    int cv_ci, cv_nkc, cv_nblk, cv_k, cv_Ho, cv_Wo, cv_stride, cv_pad;
     float* colsum_partial;        // ONES, split: [splits][M] partial sums over k of A
     __nv_bfloat16* colsum_out;    // ONES, not split: [M]
     unsigned int* timeout_flag;
 };
 
-template <int BN, bool A_MN, bool B_MN, bool ONES = false>
+// CONV: column of dG (= tap * ci + channel) that column `col` of the product belongs to; -1: padding
+__device__ __forceinline__ int conv_col(const TcParams& p, int col) {
+    const int blk = col / 64, c = (blk % p.cv_nkc) * 64 + col % 64;
+    return blk < p.cv_nblk && c < p.cv_ci ? (blk / p.cv_nkc) * p.cv_ci + c : -1;
+}
+
+template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcParams p) {
     static_assert(!ONES || (A_MN && B_MN && BN <= 192), "the ones block rides on an MN-major B of at most 192 columns");
+    static_assert(!CONV || (A_MN && B_MN && !ONES && BN <= 192), "the filter gradient: both operands MN-major, split over a cluster or not at all");
     using C = Cfg<BN, ONES>;
     constexpr int STAGES = C::STAGES;
     extern __shared__ uint8_t smem_raw[];
@@ -154,7 +169,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t fb = smem_u32(&full_bar[s]);
             const uint32_t b_dst = smem_base + s * C::STAGE_BYTES + A_STAGE_BYTES;
             const int k0 = kb * BK;
-            if (elect_one()) {
+            if (CONV) {
+                // 64 output pixels from pixel k0 on; a column block = 64 channels at one tap (blocks past the last tap load
+                // the last one again, their columns are never stored)
+                const int w = (k0 % p.cv_Wo) * p.cv_stride - p.cv_pad, hh = (k0 / p.cv_Wo) % p.cv_Ho, im = k0 / (p.cv_Wo * p.cv_Ho);
+                if (elect_one()) {
+#pragma unroll
+                    for (int j = 0; j < BN / 64; ++j) {
+                        const int blk = min(n0 / 64 + j, p.cv_nblk - 1), tap = blk / p.cv_nkc;
+                        tma_load_im2col(b_dst + j * 8192, &tmB, fb, (blk % p.cv_nkc) * 64, w, hh * p.cv_stride - p.cv_pad, im,
+                                        (uint32_t)(tap % p.cv_k), (uint32_t)(tap / p.cv_k));
+                    }
+                }
+            } else if (elect_one()) {
                 if (B_MN) {
 #pragma unroll
                     for (int j = 0; j < BN / 64; ++j) tma_load_2d(b_dst + j * 8192, &tmB, fb, n0 + 64 * j, k0);
@@ -298,8 +325,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             auto store8 = [&](uint32_t c4, const uint32_t (&w)[4], const float (&acc)[8]) {
                 const int64_t col = gcol0 + c4;
                 if (grow >= p.M || col >= p.N) return;
-                __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + col;
-                if (col + 8 <= p.N) {
+                const int64_t at = CONV ? conv_col(p, (int)col) : col;        // (CONV: 8 columns are inside or outside together)
+                if (CONV && at < 0) return;
+                __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + at;
+                if (CONV || col + 8 <= p.N) {
                     *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
                 } else {
                     for (int e = 0; e < 8; ++e)
@@ -307,7 +336,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
             };
             // 16 columns (one whole 32-byte sector) per store instruction where the layout allows, else two 16-byte stores
-            const bool sectors = (p.ldc % 16 == 0) && (((uintptr_t)p.C & 31u) == 0) && (gcol0 % 16 == 0);
+            const bool sectors = (p.ldc % 16 == 0) && (((uintptr_t)p.C & 31u) == 0) && (gcol0 % 16 == 0) && (!CONV || p.cv_ci % 16 == 0);
             for (uint32_t c4 = 0; c4 < cs; c4 += 16) {
                 uint32_t w0[4], w1[4];
                 float a0[8], a1[8];
@@ -316,7 +345,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (second) sum8(c4 + 8, w1, a1);
                 const int64_t col = gcol0 + c4;
                 if (sectors && second && grow < p.M && col + 16 <= p.N) {
-                    __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + col;
+                    const int64_t at = CONV ? conv_col(p, (int)col) : col;
+                    if (CONV && at < 0) continue;
+                    __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + at;
                     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                                  ::"l"(dst), "r"(w0[0]), "r"(w0[1]), "r"(w0[2]), "r"(w0[3]), "r"(w1[0]), "r"(w1[1]), "r"(w1[2]), "r"(w1[3]) : "memory");
                 } else {
@@ -374,6 +405,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     __nv_bfloat16* dst = (__nv_bfloat16*)p.C + row * p.ldc + col0;
 #pragma unroll
                     for (int g = 0; g < 4; ++g) {
+                        if (CONV) {                        // 8 columns of one tap, inside or outside together
+                            const int at = conv_col(p, (int)col0 + g * 8);
+                            if (at >= 0)
+                                *reinterpret_cast<uint4*>((__nv_bfloat16*)p.C + row * p.ldc + at) =
+                                    make_uint4(pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1])), pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3])),
+                                               pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5])), pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7])));
+                            continue;
+                        }
                         float f[8];
 #pragma unroll
                         for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * g + e]);
@@ -457,9 +496,9 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
         }
 }
 
-template <int BN, bool A_MN, bool B_MN, bool ONES = false>
+template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false>
 lrd_status_t launch(const CUtensorMap& tA, const CUtensorMap& tB, const TcParams& p, dim3 grid, cudaStream_t stream) {
-    auto kern = tc_gemm_kernel<BN, A_MN, B_MN, ONES>;
+    auto kern = tc_gemm_kernel<BN, A_MN, B_MN, ONES, CONV>;
     static bool configured_on[kMaxDevices] = {};     // per instantiation; the attribute is sticky per function
     bool& configured = configured_on[device_slot()];
     if (!configured) {
@@ -653,7 +692,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
                              : make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb, (uint32_t)bn, BK));
     if (!ok) return LRD_ERR_CUDA;
 
-    TcParams p;
+    TcParams p{};
     p.M = g.M; p.N = g.N; p.ldp = ldp; p.kb_total = kb_total; p.kb_per_split = kb_per;
     p.partial = splits > 1 ? 1 : 0;
     p.cluster_splits = cluster;
@@ -685,6 +724,34 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
         ones ? (__nv_bfloat16*)g.a_colsum : nullptr);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
+}
+
+// Filter gradient (see CONV above): M = co, N = taps x 64-column blocks, K = output pixels.
+lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co,
+                            cudaStream_t stream) {
+    if (!tc_conv_eligible(B, g, ci, co, LRD_BF16, dout, in, dG)) return LRD_ERR_UNSUPPORTED;
+    const int64_t P = B * g.Ho * g.Wo, taps = (int64_t)g.k * g.k, nkc = (ci + 63) / 64, N = taps * nkc * 64;
+    SplitPlan sp = pick_split(co, N, P, true);             // (tiles of at most 192 columns)
+    if (sp.cluster < 2) sp.cluster = 1;                    // tiles enough to fill the GPU: each reduces over all pixels
+    CUtensorMap tA, tB;
+    bool ok = make_tmap_2d_bf16(&tA, dout, (uint64_t)P, (uint64_t)co, (uint64_t)co, BK, 64);
+    ok = ok && make_tmap_im2col_bf16(&tB, in, (uint64_t)B, (uint64_t)g.H, (uint64_t)g.W, (uint64_t)ci, -g.pad, -g.pad, g.Ho, g.Wo, g.stride, BK);
+    if (!ok) return LRD_ERR_CUDA;
+    TcParams p{};
+    p.M = co; p.N = N; p.ldp = N;
+    p.kb_total = (int)((P + BK - 1) / BK);
+    p.kb_per_split = (p.kb_total + sp.cluster - 1) / sp.cluster;
+    p.cluster_splits = sp.cluster;
+    p.timeout_flag = device_timeout_flag();
+    p.C = dG; p.ldc = taps * ci;
+    p.cv_ci = (int)ci; p.cv_nkc = (int)nkc; p.cv_nblk = (int)(taps * nkc); p.cv_k = g.k;
+    p.cv_Ho = g.Ho; p.cv_Wo = g.Wo; p.cv_stride = g.stride; p.cv_pad = g.pad;
+    dim3 grid((unsigned)((N + sp.bn - 1) / sp.bn), (unsigned)((co + BM - 1) / BM), (unsigned)sp.cluster);
+    switch (sp.bn) {
+        case 192: return launch<192, true, true, false, true>(tA, tB, p, grid, stream);
+        case 128: return launch<128, true, true, false, true>(tA, tB, p, grid, stream);
+        default:  return launch<64, true, true, false, true>(tA, tB, p, grid, stream);
+    }
 }
 
 }  // namespace lrd

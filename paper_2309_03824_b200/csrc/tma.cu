@@ -24,6 +24,23 @@ EncodeTiledFn encoder() {
     return fn;
 }
 
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                   const int*, const int*, cuuint32_t, cuuint32_t, const cuuint32_t*, CUtensorMapInterleave,
+                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeIm2colFn im2col_encoder() {
+    static EncodeIm2colFn fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &p, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = (EncodeIm2colFn)p;
+    });
+    return fn;
+}
+
 }  // namespace
 
 bool make_tmap_2d_bf16(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld_elems,
@@ -63,6 +80,34 @@ bool make_tmap_nhwc_bf16(CUtensorMap* out, const void* base, uint64_t B, uint64_
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool make_tmap_im2col_bf16(CUtensorMap* out, const void* base, uint64_t B, uint64_t H, uint64_t W, uint64_t C, int low_h, int low_w,
+                           int n_h, int n_w, int step, uint32_t pixels) {
+    EncodeIm2colFn fn = im2col_encoder();
+    if (!fn) return false;
+    cuuint64_t dims[4] = {C, W, H, B};
+    cuuint64_t strides[3] = {C * 2, W * C * 2, H * W * C * 2};
+    // the window positions run from the lower corner to the tensor's last element plus the upper corner: (n - 1) step
+    // beyond the lower corner is the last one
+    int lower[2] = {low_w, low_h};
+    int upper[2] = {low_w + (n_w - 1) * step - ((int)W - 1), low_h + (n_h - 1) * step - ((int)H - 1)};
+    cuuint32_t estr[4] = {1, (cuuint32_t)step, (cuuint32_t)step, 1};
+    auto encode = [&] {
+        return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, lower, upper, 64, pixels, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    CUresult rc = encode();
+    if (rc == CUDA_ERROR_INVALID_CONTEXT) {          // a host thread without a context yet, as above
+        cudaFree(nullptr);
+        rc = encode();
+    }
+    if (rc != CUDA_SUCCESS && getenv("LRD_LOG_ERRORS"))
+        fprintf(stderr, "lrd: cuTensorMapEncodeIm2col failed (%d): %llu x %llu x %llu x %llu corners %d %d / %d %d step %d pixels %u\n", (int)rc,
+                (unsigned long long)B, (unsigned long long)H, (unsigned long long)W, (unsigned long long)C, lower[0], lower[1], upper[0], upper[1],
+                step, pixels);
+    return rc == CUDA_SUCCESS;
 }
 
 }  // namespace lrd
