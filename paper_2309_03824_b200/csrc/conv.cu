@@ -57,19 +57,20 @@ size_t split_bytes(const Tk& t) {
 bool g_tucker_overlap = true;
 
 // Ranks that are not multiples of 8 (rows of A, Bm, G, Z1, Z2 then start off 16-byte boundaries): as for the linear
-// layer, the factors -- small -- are copied into the workspace with the ranks rounded up to multiples of 16 and
+// layer, the factors -- small -- are copied into the workspace with the ranks rounded up to multiples of 16 (or 8) and
 // zeros in the padding, the layer runs on the tensor-core kernels at the padded ranks, and Z1 / Z2 / dA / dG / dB
 // are copied between the caller's packed layout and padded buffers.
 bool needs_repack(const Tk& t) { return t.dt == LRD_BF16 && (t.r1 % 8 || t.r2 % 8) && t.C % 8 == 0 && t.S % 8 == 0; }
-int64_t pad16(int64_t r) { return (r + 15) / 16 * 16; }
+// (8 where 16 would pass the layer's channels, which are multiples of 8 here: a rank is at most that)
+int64_t padded(int64_t r, int64_t channels) { return (r + 15) / 16 * 16 <= channels ? (r + 15) / 16 * 16 : (r + 7) / 8 * 8; }
 lrd_tucker2_desc_t padded_desc(const lrd_tucker2_desc_t& d) {
     lrd_tucker2_desc_t q = d;
-    q.r1 = pad16(d.r1); q.r2 = pad16(d.r2);
+    q.r1 = padded(d.r1, d.C); q.r2 = padded(d.r2, d.S);
     return q;
 }
 struct Repack { size_t A, G, Bm, Z1, Z2, dA, dG, dB, total; };
 Repack repack_layout(const Tk& t, size_t inner) {
-    const size_t r1 = (size_t)pad16(t.r1), r2 = (size_t)pad16(t.r2), P = (size_t)(t.P > 0 ? t.P : 1), Po = (size_t)(t.Po > 0 ? t.Po : 1), e = 2;
+    const size_t r1 = (size_t)padded(t.r1, t.C), r2 = (size_t)padded(t.r2, t.S), P = (size_t)(t.P > 0 ? t.P : 1), Po = (size_t)(t.Po > 0 ? t.Po : 1), e = 2;
     const size_t taps = (size_t)t.taps;
     Repack o;
     size_t at = align_up(inner, 256);

@@ -115,8 +115,10 @@ ChainArgs bwd_chain_args(const Linear& L, const void* dY, const void* V, const v
 // the rank rounded up to a multiple of 16 and zero columns, the layer runs on the tensor-core kernels at the padded
 // rank (the zero columns add nothing), and Z / dU / dV are copied between the caller's packed layout and padded
 // buffers.  The rank itself is unchanged: this is what an odd rank costs on this hardware beside a rounded one.
-bool needs_repack(const Linear& L) { return L.dt == LRD_BF16 && L.r > 0 && (L.ldv % 8 || L.ldu % 8 || L.ldz % 8); }
 int64_t padded_rank(const Linear& L) { return (L.r + 15) / 16 * 16; }
+bool needs_repack(const Linear& L) {      // (a padded rank that passes K or N is no layer: such small ones run on the general path)
+    return L.dt == LRD_BF16 && L.r > 0 && (L.ldv % 8 || L.ldu % 8 || L.ldz % 8) && padded_rank(L) <= (L.K < L.N ? L.K : L.N);
+}
 lrd_linear_desc_t padded_desc(const lrd_linear_desc_t& d, const Linear& L) {
     lrd_linear_desc_t q = d;
     q.r = padded_rank(L);

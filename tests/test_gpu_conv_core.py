@@ -13,7 +13,7 @@ GEOMS = [  # B, H, W, C, S, r1, r2, k, stride
     (1, 3, 140, 16, 16, 16, 16, 3, 1), (1, 139, 5, 16, 24, 16, 8, 3, 2), (3, 7, 7, 64, 80, 40, 72, 3, 2), (5, 1, 1, 16, 16, 8, 16, 3, 2),
     (2, 1, 6, 16, 16, 16, 8, 5, 1), (3, 8, 9, 16, 16, 8, 8, 7, 2), (5, 7, 7, 64, 72, 33, 41, 3, 2), (2, 14, 14, 512, 512, 320, 264, 3, 2),
     (2, 9, 9, 64, 256, 64, 192, 5, 2), (6, 16, 15, 32, 32, 16, 16, 1, 2), (4, 12, 12, 40, 24, 24, 16, 1, 1), (9, 28, 28, 64, 64, 32, 48, 3, 2),
-    (2, 12, 12, 256, 200, 192, 192, 3, 2)]
+    (2, 12, 12, 256, 200, 192, 192, 3, 2), (1, 8, 9, 8, 24, 4, 20, 3, 1)]
 
 
 @pytest.mark.parametrize("geom", GEOMS, ids=["x".join(map(str, g)) for g in GEOMS])

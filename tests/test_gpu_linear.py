@@ -368,3 +368,10 @@ def test_backward_accumulates_over_micro_batches(dtype, shape, freeze):
         assert np.array_equal(host(dU), start["dU"].astype(np.float64)) and np.array_equal(host(db), start["db"].astype(np.float64))
     if freeze == b.LRD_FREEZE_V:
         assert np.array_equal(host(dV), start["dV"].astype(np.float64))
+
+
+@pytest.mark.parametrize("shape", [(100, 24, 24, 20), (65, 20, 40, 20), (33, 8, 16, 5), (70, 40, 32, 31)])
+@pytest.mark.parametrize("freeze", [b.LRD_FREEZE_NONE, b.LRD_FREEZE_U, b.LRD_FREEZE_V])
+def test_packed_ranks_close_to_the_layer_width(shape, freeze):
+    """Packed odd ranks whose padded rank (a multiple of 16) would pass K or N, and one that just fits."""
+    check_linear(wl.random_factor_case(*shape, "bf16", 640 + shape[3]), freeze)
