@@ -1,8 +1,9 @@
 """Thin ctypes binding of liblrd_b200.so: same names as include/lrd.h, argument marshalling only.
 
 Tensors are torch CUDA tensors (or None); the binding passes their device pointers and the
-current CUDA stream.  There is no fallback: if the library is not built or cannot be loaded,
-importing this module raises.
+current CUDA stream.  The calls of a training step are marshalled in C (csrc/binding_native.c), the others
+through ctypes.  There is no fallback: if the library is not built or cannot be loaded, importing this
+module raises.
 """
 from __future__ import annotations
 
@@ -14,6 +15,7 @@ LIB_PATH = os.path.join(_HERE, "liblrd_b200.so")
 if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2309_03824_b200.build`")
 _lib = C.CDLL(LIB_PATH)
+from . import _native  # noqa: E402  (linked to the library loaded above)
 
 # enums -------------------------------------------------------------------------------------------
 (LRD_OK, LRD_ERR_INVALID_ARG, LRD_ERR_BAD_RANK, LRD_ERR_ALIGNMENT, LRD_ERR_WORKSPACE, LRD_ERR_UNSUPPORTED,
@@ -133,6 +135,16 @@ def _stream(stream):
         return C.c_void_p(int(stream))
     import torch
     return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+
+def _stream_source():
+    """(current device, device -> its current stream as an integer): asked for once, on the first call without a stream."""
+    import torch
+    torch.cuda.current_stream()          # brings the CUDA state of the process up
+    return torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+
+
+_native.set_stream_source(_stream_source)
 
 
 def _ws(workspace):
@@ -272,120 +284,79 @@ def lrd_tucker2_workspace_bytes(desc, freeze, is_bwd):
 
 # device entry points ---------------------------------------------------------------------------------
 def lrd_linear_fwd(desc, X, V, U, bias, Y, Z_save, freeze, workspace, stream=None, check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_linear_fwd(C.byref(desc), _ptr(X), _ptr(V), _ptr(U), _ptr(bias), _ptr(Y), _ptr(Z_save), freeze, w, n,
-                             _stream(stream))
-    if check:
+    st = _native.linear_fwd(desc, X, V, U, bias, Y, Z_save, freeze, workspace, stream)
+    if check and st:
         _check(st)
     return st
 
 
 def lrd_linear_bwd(desc, dY, X, V, U, Z_save, dX, dU, dV, dbias, freeze, workspace, stream=None, check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_linear_bwd(C.byref(desc), _ptr(dY), _ptr(X), _ptr(V), _ptr(U), _ptr(Z_save), _ptr(dX), _ptr(dU),
-                             _ptr(dV), _ptr(dbias), freeze, w, n, _stream(stream))
-    if check:
+    st = _native.linear_bwd(desc, dY, X, V, U, Z_save, dX, dU, dV, dbias, freeze, workspace, stream)
+    if check and st:
         _check(st)
     return st
 
 
 def lrd_linear_bwd_data(desc, dY, V, U, dX, freeze, workspace, stream=None, check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_linear_bwd_data(C.byref(desc), _ptr(dY), _ptr(V), _ptr(U), _ptr(dX), freeze, w, n, _stream(stream))
-    if check:
+    st = _native.linear_bwd_data(desc, dY, V, U, dX, freeze, workspace, stream)
+    if check and st:
         _check(st)
     return st
 
 
 def lrd_linear_bwd_weights(desc, dY, X, Z_save, dU, dV, dbias, freeze, workspace, stream=None, check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_linear_bwd_weights(C.byref(desc), _ptr(dY), _ptr(X), _ptr(Z_save), _ptr(dU), _ptr(dV), _ptr(dbias), freeze, w, n,
-                                     _stream(stream))
-    if check:
+    st = _native.linear_bwd_weights(desc, dY, X, Z_save, dU, dV, dbias, freeze, workspace, stream)
+    if check and st:
         _check(st)
     return st
 
 
-def _ptr_array(ts, n):
-    """Host array of n device pointers (NULL entries for None); None for a list that is None as a whole."""
-    if ts is None:
-        return None
-    if len(ts) != n:
-        raise ValueError("every per-layer list of a group has one entry per layer")
-    return (C.c_void_p * n)(*[None if t is None else t.data_ptr() for t in ts])
-
-
-def _group_common(descs, workspaces):
-    n = len(descs)
-    darr = (lrd_linear_desc_t * n)(*descs)
-    ws = [_ws(w) for w in workspaces]
-    warr = (C.c_void_p * n)(*[w[0] for w in ws])
-    wbytes = (C.c_size_t * n)(*[w[1] for w in ws])
-    return n, darr, warr, wbytes
-
-
 def lrd_linear_group_fwd(descs, X, V, U, bias, Y, Z_save, freeze, workspaces, stream=None, check=True):
     """n independent layers side by side: every argument but freeze/stream is a list with one entry per layer."""
-    n, darr, warr, wbytes = _group_common(descs, workspaces)
-    st = _lib.lrd_linear_group_fwd(n, darr, _ptr_array(X, n), _ptr_array(V, n), _ptr_array(U, n), _ptr_array(bias, n),
-                                   _ptr_array(Y, n), _ptr_array(Z_save, n), freeze, warr, wbytes, _stream(stream))
-    if check:
+    st = _native.linear_group_fwd(descs, X, V, U, bias, Y, Z_save, freeze, workspaces, stream)
+    if check and st:
         _check(st)
     return st
 
 
 def lrd_linear_group_bwd(descs, dY, X, V, U, Z_save, dX, dU, dV, dbias, freeze, workspaces, stream=None, check=True):
-    n, darr, warr, wbytes = _group_common(descs, workspaces)
-    st = _lib.lrd_linear_group_bwd(n, darr, _ptr_array(dY, n), _ptr_array(X, n), _ptr_array(V, n), _ptr_array(U, n),
-                                   _ptr_array(Z_save, n), _ptr_array(dX, n), _ptr_array(dU, n), _ptr_array(dV, n),
-                                   _ptr_array(dbias, n), freeze, warr, wbytes, _stream(stream))
-    if check:
+    st = _native.linear_group_bwd(descs, dY, X, V, U, Z_save, dX, dU, dV, dbias, freeze, workspaces, stream)
+    if check and st:
         _check(st)
     return st
 
 
 def lrd_linear_bwd_accumulate(desc, dY, X, V, U, Z_save, dX, dU, dV, dbias, freeze, workspace, stream=None, check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_linear_bwd_accumulate(C.byref(desc), _ptr(dY), _ptr(X), _ptr(V), _ptr(U), _ptr(Z_save), _ptr(dX), _ptr(dU),
-                                        _ptr(dV), _ptr(dbias), freeze, w, n, _stream(stream))
-    if check:
+    st = _native.linear_bwd_accumulate(desc, dY, X, V, U, Z_save, dX, dU, dV, dbias, freeze, workspace, stream)
+    if check and st:
         _check(st)
     return st
 
 
 def lrd_dense_fwd(desc, X, W, bias, Y, workspace, stream=None, check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_dense_fwd(C.byref(desc), _ptr(X), _ptr(W), _ptr(bias), _ptr(Y), w, n, _stream(stream))
-    if check:
+    st = _native.dense_fwd(desc, X, W, bias, Y, workspace, stream)
+    if check and st:
         _check(st)
     return st
 
 
 def lrd_dense_bwd(desc, dY, X, W, dX, dW, dbias, workspace, stream=None, check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_dense_bwd(C.byref(desc), _ptr(dY), _ptr(X), _ptr(W), _ptr(dX), _ptr(dW), _ptr(dbias), w, n,
-                            _stream(stream))
-    if check:
+    st = _native.dense_bwd(desc, dY, X, W, dX, dW, dbias, workspace, stream)
+    if check and st:
         _check(st)
     return st
 
 
 def lrd_tucker2_fwd(desc, X, A, G, Bm, bias, Y, Z1_save, Z2_save, freeze, workspace, stream=None, check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_tucker2_fwd(C.byref(desc), _ptr(X), _ptr(A), _ptr(G), _ptr(Bm), _ptr(bias), _ptr(Y), _ptr(Z1_save),
-                              _ptr(Z2_save), freeze, w, n, _stream(stream))
-    if check:
+    st = _native.tucker2_fwd(desc, X, A, G, Bm, bias, Y, Z1_save, Z2_save, freeze, workspace, stream)
+    if check and st:
         _check(st)
     return st
 
 
-def lrd_tucker2_bwd(desc, dY, X, A, G, Bm, Z1_save, Z2_save, dX, dA, dG, dB, dbias, freeze, workspace, stream=None,
-                    check=True):
-    w, n = _ws(workspace)
-    st = _lib.lrd_tucker2_bwd(C.byref(desc), _ptr(dY), _ptr(X), _ptr(A), _ptr(G), _ptr(Bm), _ptr(Z1_save),
-                              _ptr(Z2_save), _ptr(dX), _ptr(dA), _ptr(dG), _ptr(dB), _ptr(dbias), freeze, w, n,
-                              _stream(stream))
-    if check:
+def lrd_tucker2_bwd(desc, dY, X, A, G, Bm, Z1_save, Z2_save, dX, dA, dG, dB, dbias, freeze, workspace, stream=None, check=True):
+    st = _native.tucker2_bwd(desc, dY, X, A, G, Bm, Z1_save, Z2_save, dX, dA, dG, dB, dbias, freeze, workspace, stream)
+    if check and st:
         _check(st)
     return st
 

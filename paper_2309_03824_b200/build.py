@@ -4,25 +4,27 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblrd_b200.so")
+NATIVE = os.path.join(HERE, "_native.so")         # the binding's call marshalling (a CPython extension linked to LIB)
 SOURCES = ["lrd_api.cu", "simt.cu", "tma.cu", "tc_gemm.cu", "tc_gemm_persistent.cu", "chain.cu", "chain_pair.cu", "conv.cu", "conv_tc.cu", "tucker_fused.cu", "streams.cu", "selftest.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "-cudart", "static"]
 
 
 def _stale():
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "lrd.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
 def build(force=False, verbose=False):
-    """Compile every .cu of the library into liblrd_b200.so next to this file."""
+    """Compile every .cu of the library into liblrd_b200.so next to this file, and the binding's native part beside it."""
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -45,6 +47,8 @@ def build(force=False, verbose=False):
     if failed:
         raise RuntimeError("nvcc failed")
     subprocess.check_call([nvcc, "-shared", "-cudart", "static", "-o", LIB, *objs])
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                           os.path.join(CSRC, "binding_native.c"), "-o", NATIVE, "-L", HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
     return LIB
 
 
