@@ -1,6 +1,6 @@
 // Fused chain  Out[M x N2] = (In[M x K1] P[K1 x r]) Q[N2 x r]^T (+ bias)  on sm_100a.
 //
-// A cluster of C blocks owns one 128-row tile.
+// A cluster of C blocks (1 to 16) owns one 128-row tile.
 //   Phase 1  block c forms its r/C-column slice of T = In P in tensor memory (TMA-fed tcgen05.mma:
 //            In K-major, the slice of P MN-major), one or two 64-deep k-blocks per stage, as many
 //            stages as the shared memory beside the T buffer holds.
@@ -32,7 +32,7 @@ using namespace ptx;
 
 constexpr int kThreads = 192;
 constexpr int kMaxStages = 12;
-constexpr int kMaxCluster = 4;       // blocks per row tile
+constexpr int kMaxCluster = 16;      // blocks per row tile (more than 8: a non-portable cluster size, allowed per function)
 constexpr int kMaxKb2 = 8;           // 64-column k-blocks of T (r <= 512)
 constexpr uint32_t kSmemLimit = 224 * 1024;         // dynamic shared memory; the rest is left for the barriers and the bias
 constexpr uint32_t kInTileBytes = 128 * 64 * 2;     // In tile of one k-block: 128 rows x 64 k
@@ -48,9 +48,9 @@ struct ChainParams {
     const __nv_bfloat16* bias;
     int has_tsave;
     unsigned int* timeout_flag;
-    // Phase 2 of block c walks over the 64-column k-blocks of T in the order kb_order[c] (4 bits per position)
-    // and needs the slices in kb_slices[c] (a 4-bit mask per position) for the k-block at that position.
-    uint32_t kb_order[kMaxCluster], kb_slices[kMaxCluster];
+    // Phase 2 of block c walks over the 64-column k-blocks of T in the order kb_order[c] (4 bits per position); k-block
+    // kb needs the slices kb_lo .. kb_hi (4 bits per k-block each).
+    uint32_t kb_order[kMaxCluster], kb_lo, kb_hi;
 };
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -81,8 +81,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0);
     const int lane = threadIdx.x % 32;
     const int c = (int)cluster_ctarank();
-    const uint32_t my_order = c == 0 ? p.kb_order[0] : (c == 1 ? p.kb_order[1] : (c == 2 ? p.kb_order[2] : p.kb_order[3]));
-    const uint32_t my_slices = c == 0 ? p.kb_slices[0] : (c == 1 ? p.kb_slices[1] : (c == 2 ? p.kb_slices[2] : p.kb_slices[3]));
+    const uint32_t my_order = p.kb_order[c];
     const int m0 = blockIdx.y * 128;
     const int ng1 = (p.kb1 + p.G1 - 1) / p.G1;                                 // stage turns of phase 1
     // phase-1 stage: G1 In tiles, then the P boxes (one per column atom, 64 G1 rows tall)
@@ -103,15 +102,17 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
         prefetch_tmap(&tmQ);
         prefetch_tmap(&tmOut);
         mbar_init(smem_u32(&tacc_bar), 1);
-        // one barrier per slice of T: this block's own slice is ready after one arrival (written by its gather
-        // warps), a peer's slice once its bytes have landed
-        for (int j = 0; j < p.C; ++j) mbar_init(smem_u32(&tready_bar[j]), 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&out_full[i]), 1);
             mbar_init(smem_u32(&out_empty[i]), 4);
         }
-        for (int j = 0; j < p.C; ++j)
-            if (j != c) mbar_expect_tx(smem_u32(&tready_bar[j]), 256u * (uint32_t)p.RS);
+        fence_mbar_init();
+    }
+    // one barrier per slice of T (one slice per lane): this block's own slice is ready after one arrival (written by its
+    // gather warps), a peer's slice once its bytes have landed
+    if (warp == 2 && lane < p.C) {
+        mbar_init(smem_u32(&tready_bar[lane]), 1);
+        if (lane != c) mbar_expect_tx(smem_u32(&tready_bar[lane]), 256u * (uint32_t)p.RS);
         fence_mbar_init();
     }
     if (warp == 1) {
@@ -231,7 +232,8 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
                 const int kb = (int)((my_order >> (4 * i)) & 15u);
                 const int nks = min(4, p.ks2 - kb * 4);
                 if (i2 == 0) {
-                    uint32_t need = ((my_slices >> (4 * i)) & 15u) & ~slices_ready;
+                    const uint32_t lo = (p.kb_lo >> (4 * kb)) & 15u, hi = (p.kb_hi >> (4 * kb)) & 15u;
+                    uint32_t need = ((2u << hi) - (1u << lo)) & ~slices_ready;
                     while (need && ok) {
                         const int j = __ffs(need) - 1;
                         ok = mbar_wait_cluster_uniform(smem_u32(&tready_bar[j]), 0, ab);
@@ -417,26 +419,31 @@ int g_tune_C = 0, g_tune_G1 = 0, g_tune_BN2 = 0;    // 0 = automatic
 
 inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-// Column chunk width of phase 2: the block with the most chunks sets the pace, so minimise
-// (chunks of the busiest block) x width; wider chunks on ties (fewer, larger copies).
+// Column chunk width of phase 2: the block with the most chunks sets the pace, so minimise (chunks of the busiest
+// block) x (width + 64): a stage of the issue loop costs some 500 clocks whatever its width, as much as 64 columns more.
 int pick_bn2(int64_t N2, int C) {
     if (g_tune_BN2) return g_tune_BN2;
-    const int cands[3] = {256, 192, 128};
+    const int cands[4] = {256, 192, 128, 64};
     int best = 128;
     int64_t best_cost = -1;
     for (int bn : cands) {
         const int64_t chunks = (N2 + bn - 1) / bn;
-        const int64_t cost = ((chunks + C - 1) / C) * bn;
+        const int64_t cost = ((chunks + C - 1) / C) * (bn + 64);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = bn; }
     }
     return best;
 }
 
+bool set_attributes() {
+    return cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
+           cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+}
+
 // Clusters of C blocks that can be resident at once (a cluster needs C free SMs inside one GPC).
 int max_active_clusters(int C) {
-    static int cache_on[kMaxDevices][5] = {};
+    static int cache_on[kMaxDevices][kMaxCluster + 1] = {};
     int* cache = cache_on[device_slot()];
-    if (C < 2 || C > 4) return kNumSms;
+    if (C < 2 || C > kMaxCluster) return kNumSms;
     if (cache[C] == 0) {
         int n = 0;
         cudaLaunchConfig_t cfg = {};
@@ -450,14 +457,13 @@ int max_active_clusters(int C) {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, chain_kernel, &cfg) != cudaSuccess || n < 1) {
+        if (!set_attributes() || cudaOccupancyMaxActiveClusters(&n, chain_kernel, &cfg) != cudaSuccess || n < 1) {
             cudaGetLastError();
-            n = (kNumSms - 20) / C;                     // no answer (no device yet): a cautious guess
+            n = C > 8 ? 0 : (kNumSms - 20) / C;         // no answer (no device yet): a cautious guess
         }
-        cache[C] = n;
+        cache[C] = n + 1;                               // (0: not asked yet)
     }
-    return cache[C];
+    return cache[C] - 1;
 }
 
 bool make_plan(const ChainArgs& a, Plan* out) {
@@ -473,8 +479,7 @@ bool make_plan(const ChainArgs& a, Plan* out) {
     const int kb1 = (int)((a.K1 + 63) / 64);
     Plan best{};
     bool found = false;
-    const int cands[4] = {4, 3, 2, 1};
-    for (int C : cands) {
+    for (int C = kMaxCluster; C >= 1; --C) {
         if (g_tune_C && C != g_tune_C) continue;
         if (a.r % (16 * C)) continue;
         const int RS = (int)a.r / C;
@@ -501,11 +506,14 @@ bool make_plan(const ChainArgs& a, Plan* out) {
         const uint32_t after1 = (uint32_t)t_bytes + used2;
         Plan pl{C, RS, swb, BN2, G1, S1, S2, s1b, kb2_bytes, (uint32_t)t_bytes, 1024u + (used1 > after1 ? used1 : after1)};
         // prefer the largest cluster whose blocks are all resident at once (within this launch's share of the
-        // SMs, when it runs beside other launches); else the smallest feasible
-        if (!found) { best = pl; found = true; }
-        const int64_t room = a.sm_share > 0 && !g_tune_C ? (int64_t)a.sm_share / C : (int64_t)max_active_clusters(C);
-        if (tiles <= room && tiles <= max_active_clusters(C)) { best = pl; break; }
+        // SMs, when it runs beside other launches); else the smallest feasible.  With few row tiles the kernel is one
+        // block's latency -- its share of P and Q through one SM -- so more blocks per tile shorten it: 768 -> 3072 at
+        // r = 384 and 128 tokens 26.1 / 16.5 / 13.6 / 12.1 / 10.9 us with 2 / 4 / 6 / 8 / 12 blocks
         best = pl;
+        found = true;
+        if (g_tune_C) break;
+        const int64_t room = a.sm_share > 0 ? (int64_t)a.sm_share / C : (int64_t)max_active_clusters(C);
+        if (tiles <= room && tiles <= max_active_clusters(C)) break;
     }
     if (!found) return false;
     *out = best;
@@ -565,33 +573,30 @@ lrd_status_t chain_launch(const ChainArgs& a, cudaStream_t stream) {
     // A block sends its slice of T to the peers c + 1, c + 2, ... in turn, so slice j reaches block c as the
     // ((c - j) mod C)-th arrival (0 = its own); phase 2 takes the k-blocks in the order in which the last slice
     // they touch arrives.  The order depends on the launch shape only, so results stay reproducible.
+    p.kb_lo = p.kb_hi = 0;
+    for (int kb = 0; kb < p.kb2; ++kb) {
+        p.kb_lo |= (uint32_t)(kb * 64 / p.RS) << (4 * kb);
+        p.kb_hi |= (uint32_t)((kb * 64 + std::min(4, p.ks2 - kb * 4) * 16 - 1) / p.RS) << (4 * kb);
+    }
     for (int c = 0; c < kMaxCluster; ++c) {
-        p.kb_order[c] = 0; p.kb_slices[c] = 0;
+        p.kb_order[c] = 0;
         if (c >= p.C) continue;
-        int n = 0;
-        for (int rank = 0; rank < p.C; ++rank)
-            for (int kb = 0; kb < p.kb2; ++kb) {
-                const int nks = std::min(4, p.ks2 - kb * 4);
-                const int j_lo = kb * 64 / p.RS, j_hi = (kb * 64 + nks * 16 - 1) / p.RS;
-                int worst = 0;
-                uint32_t mask = 0;
-                for (int j = j_lo; j <= j_hi; ++j) {
-                    worst = std::max(worst, (c - j + p.C) % p.C);
-                    mask |= 1u << j;
-                }
-                if (worst != rank) continue;
-                p.kb_order[c] |= (uint32_t)kb << (4 * n);
-                p.kb_slices[c] |= mask << (4 * n);
-                ++n;
-            }
+        int n = 0, last[kMaxKb2];            // arrival of the last slice a k-block needs
+        for (int kb = 0; kb < p.kb2; ++kb) {
+            last[kb] = 0;
+            for (int j = (int)((p.kb_lo >> (4 * kb)) & 15u); j <= (int)((p.kb_hi >> (4 * kb)) & 15u); ++j)
+                last[kb] = std::max(last[kb], (c - j + p.C) % p.C);
+        }
+        for (int rank = 0; rank < p.C && n < p.kb2; ++rank)
+            for (int kb = 0; kb < p.kb2; ++kb)
+                if (last[kb] == rank) p.kb_order[c] |= (uint32_t)kb << (4 * n++);
     }
     p.timeout_flag = device_timeout_flag();
 
     static bool configured_on[kMaxDevices] = {};
     bool& configured = configured_on[device_slot()];
     if (!configured) {
-        if (cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess)
-            return LRD_ERR_CUDA;
+        if (!set_attributes()) return LRD_ERR_CUDA;
         configured = true;
     }
     cudaLaunchConfig_t cfg = {};

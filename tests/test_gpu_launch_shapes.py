@@ -49,6 +49,16 @@ def test_chain_kernel_clusters_of_three(shape):
         b.lrd_chain_pair_tuning(0, 0, 0, 0)
 
 
+@pytest.mark.parametrize("shape", [(100, 776, 520, 192), (64, 768, 3072, 384), (128, 264, 1000, 256), (300, 520, 520, 512), (1, 136, 136, 112),
+                                   (700, 256, 264, 160)])
+def test_chain_kernel_clusters_of_up_to_sixteen(shape):
+    """Few row tiles: clusters of 7, 8, 10, 12 and 16 blocks per tile, some blocks without a chunk of their own."""
+    b.lrd_chain_pair_tuning(1, 0, 0, 0)
+    case = wl.random_factor_case(*shape, "bf16", 960 + shape[0])
+    for freeze in (b.LRD_FREEZE_NONE, b.LRD_FREEZE_U):
+        check_linear(case, freeze, path=b.LRD_PATH_FUSED)
+
+
 @pytest.mark.parametrize("mode", [(2, 1, 0, 0), (2, 2, 0, 0), (2, 3, 0, 0), (2, 4, 0, 0), (2, 0, 1, 0), (2, 0, 2, 0), (2, 2, 1, 128), (2, 1, 3, 64),
                                   (2, 0, 0, 192)])
 @pytest.mark.parametrize("shape", [(400, 776, 520, 192), (300, 520, 1000, 384), (1100, 3072, 136, 128)])
