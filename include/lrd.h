@@ -318,8 +318,8 @@ lrd_status_t lrd_dense_bwd(const lrd_linear_desc_t* desc, const void* dY, const 
 
 /* The paper has no counterpart for this entry point; it exists for the sake of its callers.
  *
- * dbias[N] = column sums of dY[M x N] (leading dimension ldy, 0 = packed), the same quantity and the
- * same kernels as the dbias output of lrd_linear_bwd, but WITHOUT a workspace argument: the partial
+ * dbias[N] = column sums of dY[M x N] (leading dimension ldy, 0 = packed), the same quantity as the
+ * dbias output of lrd_linear_bwd, but WITHOUT a workspace argument: the partial
  * sums go to a fixed 2 MiB array that lives inside the library's device image.  It is meant for code
  * that has no way to obtain scratch memory when it needs the result - for instance a plug-in that is
  * handed ready-made tensors by a framework whose allocator it must not call, a callback running where

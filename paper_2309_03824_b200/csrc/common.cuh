@@ -33,8 +33,7 @@ struct GemmArgs {
     const void* B; int64_t ldb; bool b_mn_major;
     void* C; int64_t ldc;
     const void* bias;          // [N] or nullptr, same dtype as C
-    void* a_colsum = nullptr;  // optional [M]: sum over k of A(m, k) (the bias gradient when A is dY); only on the
-                               // tensor-core path with both operands MN-major, see tc_gemm_colsum_ok()
+    void* a_colsum = nullptr;  // optional [M]: sum over k of A(m, k) (the bias gradient when A is dY); both operands MN-major
     lrd_dtype_t dtype;         // storage type of A, B, C, bias
     int max_cluster_split = 0; // split weight gradients: largest cluster to split the reduction over (0 = automatic).  A
                                // launch meant to run BESIDE others asks for 2: clusters of 4 or 8 need that many free
@@ -53,14 +52,6 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // General fp32-FMA path (any shape, any alignment).
 lrd_status_t simt_gemm(const GemmArgs& g, cudaStream_t stream);
-lrd_status_t simt_colsum(const void* A, int64_t lda, int64_t M, int64_t N, void* out, lrd_dtype_t dtype,
-                         cudaStream_t stream);
-
-// Column sums of A[M x N] (bias gradient), rows added in a fixed order.  With `scratch` of at least
-// colsum_scratch_bytes(M, N) the sum runs in two stages over many blocks; without, in one kernel.
-size_t colsum_scratch_bytes(int64_t M, int64_t N);
-lrd_status_t colsum(const void* A, int64_t lda, int64_t M, int64_t N, void* out, lrd_dtype_t dtype, float* scratch,
-                    size_t scratch_bytes, cudaStream_t stream);
 
 // One product on the path chosen by `path` (an lrd_path_t): the tensor-core kernel when the
 // operands qualify, else the general kernel.

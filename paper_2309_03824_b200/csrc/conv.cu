@@ -39,10 +39,8 @@ struct Scratch { size_t dB, dA; };
 Scratch split_regions(const Tk& t) {
     Scratch r{0, 0};
     if (t.P < 1) return r;
-    r.dB = colsum_scratch_bytes(t.Po, t.S);
     if (t.dt == LRD_BF16) {
-        const size_t a = tc_split_workspace_bytes(t.S, t.r2, t.Po);
-        r.dB = r.dB > a ? r.dB : a;
+        r.dB = tc_split_workspace_bytes(t.S, t.r2, t.Po);
         r.dA = tc_split_workspace_bytes(t.C, t.r1, t.P);
     }
     r.dB = align_up(r.dB, 256); r.dA = align_up(r.dA, 256);
@@ -208,13 +206,8 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     }
     auto launch_dB = [&]() {
         GemmArgs gb = make_gemm(t.S, t.r2, t.Po, dY, t.S, true, Z2_save, t.r2, true, dB, t.r2, nullptr, t.dt);
-        bool db_done = false;
-        if (dbias && path != LRD_PATH_GENERAL) {          // the bias gradient rides on the dB product (A = dY)
-            gb.a_colsum = dbias;
-            if (tc_gemm_colsum_ok(gb)) db_done = true; else gb.a_colsum = nullptr;
-        }
+        gb.a_colsum = dbias;                              // the bias gradient rides on the dB product (A = dY)
         keep(run_gemm(gb, path, true, pB, reg.dB, sB));
-        if (dbias && !db_done) keep(colsum(dY, t.S, t.Po, t.S, dbias, t.dt, pB, reg.dB, sB));
     };
     if (factors && sB != s) launch_dB();
 

@@ -149,9 +149,9 @@ size_t linear_grad_scratch_bytes(const Linear& L) {     // dU, dV and dbias of o
     return align_up((size_t)L.N * L.ldu * e, 256) + align_up((size_t)L.K * L.ldv * e, 256) + align_up((size_t)L.N * e, 256);
 }
 
-size_t linear_split_bytes(const Linear& L) {     // scratch after dZ: split partials of dU / dV, partial column sums
+size_t linear_split_bytes(const Linear& L) {     // scratch after dZ: split partials of dU / dV
     if (L.M < 1) return 0;
-    size_t need = colsum_scratch_bytes(L.M, L.N);
+    size_t need = 0;
     if (L.dt == LRD_BF16) {
         const size_t a = tc_split_workspace_bytes(L.N, L.r, L.M), b = tc_split_workspace_bytes(L.K, L.r, L.M);
         need = need > a ? need : a;
@@ -434,7 +434,7 @@ size_t lrd_dense_workspace_bytes(const lrd_linear_desc_t* desc, int is_bwd) {
     Linear L;
     if (parse_linear(desc, &L, true) != LRD_OK) return 0;
     if (!is_bwd || L.M < 1) return 256;
-    size_t need = colsum_scratch_bytes(L.M, L.N);
+    size_t need = 0;
     if (L.dt == LRD_BF16) {
         const size_t a = tc_split_workspace_bytes(L.N, L.K, L.M);
         need = need > a ? need : a;
@@ -576,14 +576,9 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
     if (do_w && (plan & LRD_PLAN_DU)) {
         GemmArgs gu = gemm(L.N, L.r, L.M, dY, L.ldy, true, Z_save, L.ldz, true, dU, L.ldu, nullptr, L.dt);
         gu.max_cluster_split = wsplit;
-        bool db_done = false;
-        if (dbias && g_path.load() != LRD_PATH_GENERAL) {      // db rides on the dU product (A = dY): no second pass over dY
-            gu.a_colsum = dbias;
-            if (tc_gemm_colsum_ok(gu)) db_done = true; else gu.a_colsum = nullptr;
-        }
+        gu.a_colsum = dbias;               // db rides on the dU product (A = dY): no second pass over dY
         cudaStream_t su = side ? side : s;
         LRD_TRY(run_gemm(gu, true, partials, partial_bytes, su));
-        if (dbias && !db_done) LRD_TRY(colsum(dY, L.ldy, L.M, L.N, dbias, L.dt, partials, partial_bytes, su));
         if (side && (plan & LRD_PLAN_DV)) {
             if (cudaEventRecord(side_done, side) != cudaSuccess || cudaStreamWaitEvent(s, side_done, 0) != cudaSuccess) return LRD_ERR_CUDA;
         }
@@ -777,14 +772,8 @@ static lrd_status_t lrd_dense_bwd_impl(const lrd_linear_desc_t* desc, const void
     float* partials = (float*)((uint8_t*)workspace + 256);
     if (dX) LRD_TRY(run_gemm(gemm(L.M, L.K, L.N, dY, L.ldy, false, W, L.ldv, true, dX, L.ldx, nullptr, L.dt), false, nullptr, 0, s));
     GemmArgs gw = gemm(L.N, L.K, L.M, dY, L.ldy, true, X, L.ldx, true, dW, L.ldv, nullptr, L.dt);
-    bool db_done = false;
-    if (dbias && g_path.load() != LRD_PATH_GENERAL) {
-        gw.a_colsum = dbias;
-        if (tc_gemm_colsum_ok(gw)) db_done = true; else gw.a_colsum = nullptr;
-    }
-    LRD_TRY(run_gemm(gw, true, partials, workspace_bytes - 256, s));
-    if (dbias && !db_done) LRD_TRY(colsum(dY, L.ldy, L.M, L.N, dbias, L.dt, partials, workspace_bytes - 256, s));
-    return LRD_OK;
+    gw.a_colsum = dbias;
+    return run_gemm(gw, true, partials, workspace_bytes - 256, s);
 }
 
 // ---- the undecomposed 3x3 convolution (the layer a Tucker-2 layer replaces) ---------------------------------------

@@ -1,9 +1,15 @@
 // General path: shared-memory tiled fp32-FMA matrix product for any shape, leading dimension and
-// operand orientation, and a deterministic column sum.  Used for fp32 layers (which must not use
+// operand orientation (the column sums of its A operand a by-product where asked for).  Used for fp32 layers (which must not use
 // reduced-precision tensor math) and for bf16 layers whose ranks or strides do not meet the
 // 16-byte alignment the tensor-core path needs.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "conv.cuh"
+#include "ptx.cuh"
+#include "tc.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace lrd {
 
@@ -33,166 +39,265 @@ lrd_status_t read_and_clear_device_timeout(bool* raised) {
 
 namespace {
 
-// 64 x 64 output tile, 64-deep k-tile: the layers that land here are small or oddly shaped, their grids a handful of
-// blocks, and what a block waits for is the latency of a tile's loads -- a deep tile has fewer of those waits
-// (16-deep tiles: 41 us for 256 x 512 -> 40 on 4 blocks).
-constexpr int TM = 64, TN = 64, TK = 64, NT = 256;
-constexpr int kFetch = TM * TK / NT;        // elements of each operand a thread brings in per tile
-
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 template <typename T> __device__ __forceinline__ T from_f32(float x);
 template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
 
-// Operand loaders: element (m, k) of A and (k, n) of B as fp32, zero outside the problem.
-template <typename T> struct PlainA {          // [M x K] (k contiguous) or [K x M] (m contiguous)
-    const T* p; int64_t ld; int mn;
-    __device__ bool k_fastest() const { return !mn; }
-    __device__ float operator()(int64_t m, int64_t k) const { return to_f32(mn ? p[k * ld + m] : p[m * ld + k]); }
+// Operand loaders: element (m, k) of A and (k, n) of B as fp32, asked for inside the problem only.  What depends on the
+// row of A or the column of B alone (divisions by image sizes, mostly) is worked out once per thread and row: `row(m)` /
+// `col(n)`, then `at(row, k)` / `at(k, col)`.
+template <typename T, bool MN> struct PlainA {          // [M x K] (k contiguous) or [K x M] (m contiguous)
+    static constexpr bool kFastest = !MN;
+    const T* p; int64_t ld;
+    using Row = const T*;
+    __device__ Row row(int64_t m) const { return MN ? p + m : p + m * ld; }
+    __device__ float at(Row r, int64_t k) const { return to_f32(MN ? r[k * ld] : r[k]); }
 };
-template <typename T> struct PlainB {          // [N x K] (k contiguous) or [K x N] (n contiguous)
-    const T* p; int64_t ld; int mn;
-    __device__ bool k_fastest() const { return !mn; }
-    __device__ float operator()(int64_t k, int64_t n) const { return to_f32(mn ? p[k * ld + n] : p[n * ld + k]); }
+template <typename T, bool MN> struct PlainB {          // [N x K] (k contiguous) or [K x N] (n contiguous)
+    static constexpr bool kFastest = !MN;
+    const T* p; int64_t ld;
+    using Col = const T*;
+    __device__ Col col(int64_t n) const { return MN ? p + n : p + n * ld; }
+    __device__ float at(int64_t k, Col c) const { return to_f32(MN ? c[k * ld] : c[k]); }
 };
+struct Pixel { int64_t b; int h, w; };
+__device__ __forceinline__ Pixel pixel_of(int64_t m, int H, int W) {
+    if (m >> 31) {                                           // (a 64-bit division costs some ten times a 32-bit one)
+        const int64_t q = m / W;
+        return Pixel{q / H, (int)(q % H), (int)(m % W)};
+    }
+    const unsigned u = (unsigned)m, q = u / (unsigned)W;
+    return Pixel{(int64_t)(q / (unsigned)H), (int)(q % (unsigned)H), (int)(u % (unsigned)W)};
+}
 // k x k taps of an NHWC image as the A operand of the core's forward product: m = output pixel (b, ho, wo),
 // kidx = tap * C + channel; the tap (kh, kw) of output pixel (ho, wo) is input pixel (ho * stride + kh - pad,
 // wo * stride + kw - pad); pixels outside the image read as zero.
 template <typename T> struct ConvFwdA {
+    static constexpr bool kFastest = true;
     const T* p; ConvGeom g; int C;
-    __device__ bool k_fastest() const { return true; }
-    __device__ float operator()(int64_t m, int64_t kidx) const {
-        const int t = (int)(kidx / C), c = (int)(kidx % C);
-        const int wo = (int)(m % g.Wo), ho = (int)((m / g.Wo) % g.Ho);
-        const int64_t b = m / ((int64_t)g.Wo * g.Ho);
-        const int h = ho * g.stride + t / g.k - g.pad, w = wo * g.stride + t % g.k - g.pad;
+    using Row = Pixel;
+    __device__ Row row(int64_t m) const {
+        const Pixel o = pixel_of(m, g.Ho, g.Wo);
+        return Pixel{o.b, o.h * g.stride - g.pad, o.w * g.stride - g.pad};
+    }
+    __device__ float at(Row r, int64_t kidx) const {
+        const int t = (int)kidx / C, c = (int)kidx % C, h = r.h + t / g.k, w = r.w + t % g.k;
         if (h < 0 || h >= g.H || w < 0 || w >= g.W) return 0.f;
-        return to_f32(p[((b * g.H + h) * g.W + w) * C + c]);
+        return to_f32(p[((r.b * g.H + h) * g.W + w) * C + c]);
     }
 };
 // The same taps seen from the input side, as the A operand of the data gradient: m = input pixel (b, h, w),
 // kidx = tap * C + o; input pixel (h, w) met tap (kh, kw) of output pixel ((h + pad - kh) / stride,
 // (w + pad - kw) / stride) where both divisions are exact and the result lies inside the output.
 template <typename T> struct ConvBwdA {
+    static constexpr bool kFastest = true;
     const T* p; ConvGeom g; int C;
-    __device__ bool k_fastest() const { return true; }
-    __device__ float operator()(int64_t m, int64_t kidx) const {
-        const int t = (int)(kidx / C), c = (int)(kidx % C);
-        const int w = (int)(m % g.W), h = (int)((m / g.W) % g.H);
-        const int64_t b = m / ((int64_t)g.W * g.H);
-        const int hs = h + g.pad - t / g.k, ws = w + g.pad - t % g.k;
+    using Row = Pixel;
+    __device__ Row row(int64_t m) const {
+        const Pixel q = pixel_of(m, g.H, g.W);
+        return Pixel{q.b, q.h + g.pad, q.w + g.pad};
+    }
+    __device__ float at(Row r, int64_t kidx) const {
+        const int t = (int)kidx / C, c = (int)kidx % C;
+        const int hs = r.h - t / g.k, ws = r.w - t % g.k;
         if (hs < 0 || ws < 0 || hs % g.stride || ws % g.stride) return 0.f;
         const int ho = hs / g.stride, wo = ws / g.stride;
         if (ho >= g.Ho || wo >= g.Wo) return 0.f;
-        return to_f32(p[((b * g.Ho + ho) * g.Wo + wo) * C + c]);
+        return to_f32(p[((r.b * g.Ho + ho) * g.Wo + wo) * C + c]);
     }
 };
-// One tap of an NHWC image as the B operand of the filter gradient: kidx = output pixel, n = channel.
-template <typename T> struct ConvTapB {
-    const T* p; ConvGeom g; int C, kh, kw;
-    __device__ bool k_fastest() const { return false; }
-    __device__ float operator()(int64_t kidx, int64_t n) const {
-        const int wo = (int)(kidx % g.Wo), ho = (int)((kidx / g.Wo) % g.Ho);
-        const int64_t b = kidx / ((int64_t)g.Wo * g.Ho);
-        const int h = ho * g.stride + kh - g.pad, w = wo * g.stride + kw - g.pad;
+// All taps of an NHWC image as the B operand of the filter gradient: kidx = output pixel, n = tap * C + channel.
+template <typename T> struct ConvTapsB {
+    static constexpr bool kFastest = false;
+    const T* p; ConvGeom g; int C;
+    struct Col { int h, w, c; };
+    __device__ Col col(int64_t n) const {
+        const int t = (int)n / C;
+        return Col{t / g.k - g.pad, t % g.k - g.pad, (int)n % C};
+    }
+    __device__ float at(int64_t kidx, Col x) const {
+        const Pixel o = pixel_of(kidx, g.Ho, g.Wo);
+        const int h = o.h * g.stride + x.h, w = o.w * g.stride + x.w;
         if (h < 0 || h >= g.H || w < 0 || w >= g.W) return 0.f;
-        return to_f32(p[((b * g.H + h) * g.W + w) * C + n]);
+        return to_f32(p[((o.b * g.H + h) * g.W + w) * C + x.c]);
     }
 };
 // The core G[o][tap][i] as the B operand of the data gradient: kidx = tap * Co + o, n = i.
 template <typename T> struct CoreTransposedB {
+    static constexpr bool kFastest = false;
     const T* p; int Ci, Co, taps;
-    __device__ bool k_fastest() const { return false; }
-    __device__ float operator()(int64_t kidx, int64_t n) const {
-        const int64_t t = kidx / Co, o = kidx % Co;
-        return to_f32(p[(o * taps + t) * Ci + n]);
+    using Col = const T*;
+    __device__ Col col(int64_t n) const { return p + n; }
+    __device__ float at(int64_t kidx, Col c) const {
+        const int t = (int)kidx / Co, o = (int)kidx % Co;
+        return to_f32(c[((int64_t)o * taps + t) * Ci]);
     }
 };
 
-template <typename T, typename LA, typename LB>
-__global__ void __launch_bounds__(NT) simt_gemm_kernel(int64_t M, int64_t N, int64_t K, const LA la, const LB lb,
-                                                       T* __restrict__ C, int64_t ldc, const T* __restrict__ bias) {
-    __shared__ float As[TK][TM + 4];
-    __shared__ float Bs[TK][TN + 4];
+// One output tile per cluster.  A block's 256 threads form groups of GM x GN threads, each thread with RM x RN
+// accumulators; the groups take every KS-th k of a tile (KS = 256 / (GM GN)) and their sums are added through shared
+// memory.  The reduction is further split over the blocks of the cluster (gridDim.z), whose partial tiles are added
+// through distributed shared memory: group by group and rank by rank, a fixed order.  What the small layers that land
+// here wait for is latency -- a serial reduction on a handful of blocks -- so small tiles and many blocks come first,
+// and the large tile, which reads shared memory least, where it fills the GPU by itself.
+// 256 x 512 -> 40 in fp32: 37 us on 4 blocks of 64 x 64 without a split, 7.1 us on 16 tiles x 8 splits; forward +
+// backward of the 256-token layer 139 -> 31 us.
+constexpr int NT = 256, TK = 32, kMaxSplit = 8;
+template <int RM_, int RN_, int GM_, int GN_> struct SimtCfg {
+    static constexpr int RM = RM_, RN = RN_, GM = GM_, GN = GN_;
+    static constexpr int TM = RM * GM, TN = RN * GN, KS = NT / (GM * GN);
+    static constexpr int LDA = TM + 4, LDB = TN + 4;
+    static constexpr int kTiles = TK * (LDA + LDB), kRed = KS * TM * TN;              // floats
+    static constexpr int kSmem = (kTiles > kRed ? kTiles : kRed) + TM;                // + one column sum per row
+};
+using Small = SimtCfg<4, 4, 8, 8>;       // 32 x 32, four groups
+using Medium = SimtCfg<4, 4, 16, 16>;    // 64 x 64
+using Large = SimtCfg<8, 4, 16, 16>;     // 128 x 64
+
+// grid: (row tiles x column tiles, 1, splits)
+template <typename T, typename C_, typename LA, typename LB>
+__global__ void __launch_bounds__(NT, 2) simt_gemm_kernel(int64_t M, int64_t N, int64_t K, int64_t k_per_split, const LA la, const LB lb,
+                                                          T* __restrict__ C, int64_t ldc, const T* __restrict__ bias, T* __restrict__ a_colsum) {
+    constexpr int TM = C_::TM, TN = C_::TN, KS = C_::KS, RM = C_::RM, RN = C_::RN, LDA = C_::LDA, LDB = C_::LDB;
+    constexpr int FA = TM * TK / NT, FB = TN * TK / NT;      // elements of each operand a thread brings in per tile
+    __shared__ __align__(16) float smem[C_::kSmem];
+    float* As = smem;
+    float* Bs = smem + TK * LDA;
+    ptx::griddep_launch_dependents();
+    ptx::griddep_wait();
     const int t = threadIdx.x;
-    const int64_t m0 = (int64_t)blockIdx.y * TM, n0 = (int64_t)blockIdx.x * TN;
-    const int tx = t % 16, ty = t / 16;  // thread computes rows ty*4.., cols tx*4..
-    float acc[4][4] = {};
+    const int64_t n_tiles = (N + TN - 1) / TN;
+    const int64_t m0 = (int64_t)(blockIdx.x / n_tiles) * TM, n0 = (int64_t)(blockIdx.x % n_tiles) * TN;
+    const int64_t k_begin = (int64_t)blockIdx.z * k_per_split, k_end = k_begin + k_per_split < K ? k_begin + k_per_split : K;
+    const int grp = t / (C_::GM * C_::GN), gt = t % (C_::GM * C_::GN);
+    const int tx = gt % C_::GN, ty = gt / C_::GN;            // thread computes rows ty * RM .., columns tx * RN .. of its group
+    constexpr bool ak = LA::kFastest, bk = LB::kFastest;
+    const bool sums = a_colsum && n0 == 0;                   // this tile column also adds up A over k
+    float acc[RM][RN] = {};
+    float csum = 0.f;                                        // of row t % TM, the k of this thread's share
+    // Where a thread's elements of a tile lie: 16 k x 16 rows per pass where k is the contiguous index, else TM (TN)
+    // rows x NT / TM k per pass.
+    constexpr int AR = ak ? TM / 16 : 1, BR = bk ? TN / 16 : 1;
+    typename LA::Row arow[AR];
+    typename LB::Col bcol[BR];
+    const int64_t m_last = M - 1, n_last = N - 1;
+#pragma unroll
+    for (int i = 0; i < AR; ++i) { const int64_t m = m0 + (ak ? t / 16 + 16 * i : t % TM); arow[i] = la.row(m < M ? m : m_last); }
+#pragma unroll
+    for (int i = 0; i < BR; ++i) { const int64_t n = n0 + (bk ? t / 16 + 16 * i : t % TN); bcol[i] = lb.col(n < N ? n : n_last); }
     // The next tile's elements are fetched into registers before the current tile is multiplied: their global-memory
     // latency then runs beside the arithmetic instead of in front of it (the order of the additions is unchanged).
-    float ra[kFetch], rb[kFetch];
+    float ra[FA], rb[FB];
     auto fetch = [&](int64_t k0) {
 #pragma unroll
-        for (int i = 0; i < kFetch; ++i) {
-            int mm, kk;
-            if (la.k_fastest()) { mm = t / 16 + 16 * (i % 4); kk = t % 16 + 16 * (i / 4); } else { kk = t / 64 + 4 * i; mm = t % 64; }
-            const int64_t m = m0 + mm, k = k0 + kk;
-            ra[i] = (m < M && k < K) ? la(m, k) : 0.f;
-            int nn;
-            if (lb.k_fastest()) { nn = t / 16 + 16 * (i % 4); kk = t % 16 + 16 * (i / 4); } else { kk = t / 64 + 4 * i; nn = t % 64; }
-            const int64_t n = n0 + nn, kb = k0 + kk;
-            rb[i] = (n < N && kb < K) ? lb(kb, n) : 0.f;
+        for (int i = 0; i < FA; ++i) {
+            const int mm = ak ? t / 16 + 16 * (i % AR) : t % TM, kk = ak ? t % 16 + 16 * (i / AR) : t / TM + NT / TM * i;
+            ra[i] = (m0 + mm < M && k0 + kk < k_end) ? la.at(arow[i % AR], k0 + kk) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < FB; ++i) {
+            const int nn = bk ? t / 16 + 16 * (i % BR) : t % TN, kk = bk ? t % 16 + 16 * (i / BR) : t / TN + NT / TN * i;
+            rb[i] = (n0 + nn < N && k0 + kk < k_end) ? lb.at(k0 + kk, bcol[i % BR]) : 0.f;
         }
     };
-    fetch(0);
-    for (int64_t k0 = 0; k0 < K; k0 += TK) {
+    if (k_begin < k_end) fetch(k_begin);
+    for (int64_t k0 = k_begin; k0 < k_end; k0 += TK) {
 #pragma unroll
-        for (int i = 0; i < kFetch; ++i) {
-            int mm, kk;
-            if (la.k_fastest()) { mm = t / 16 + 16 * (i % 4); kk = t % 16 + 16 * (i / 4); } else { kk = t / 64 + 4 * i; mm = t % 64; }
-            As[kk][mm] = ra[i];
-            int nn;
-            if (lb.k_fastest()) { nn = t / 16 + 16 * (i % 4); kk = t % 16 + 16 * (i / 4); } else { kk = t / 64 + 4 * i; nn = t % 64; }
-            Bs[kk][nn] = rb[i];
+        for (int i = 0; i < FA; ++i) {
+            const int mm = ak ? t / 16 + 16 * (i % AR) : t % TM, kk = ak ? t % 16 + 16 * (i / AR) : t / TM + NT / TM * i;
+            As[kk * LDA + mm] = ra[i];
+        }
+#pragma unroll
+        for (int i = 0; i < FB; ++i) {
+            const int nn = bk ? t / 16 + 16 * (i % BR) : t % TN, kk = bk ? t % 16 + 16 * (i / BR) : t / TN + NT / TN * i;
+            Bs[kk * LDB + nn] = rb[i];
         }
         __syncthreads();
-        if (k0 + TK < K) fetch(k0 + TK);
+        if (k0 + TK < k_end) fetch(k0 + TK);
+        if (sums) {
+            constexpr int per = TK / (NT / TM);
+            const int m = t % TM, kk0 = t / TM * per;
 #pragma unroll
-        for (int kk = 0; kk < TK; ++kk) {
-            float a[4], b[4];
+            for (int i = 0; i < per; ++i) csum += As[(kk0 + i) * LDA + m];
+        }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty * 4 + i]; b[i] = Bs[kk][tx * 4 + i]; }
+        for (int kq = 0; kq < TK / KS; ++kq) {
+            const int kk = kq * KS + grp;
+            float a[RM], b[RN];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < RM; i += 4) {
+                const float4 x = *reinterpret_cast<const float4*>(&As[kk * LDA + ty * RM + i]);
+                a[i] = x.x; a[i + 1] = x.y; a[i + 2] = x.z; a[i + 3] = x.w;
+            }
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            for (int j = 0; j < RN; j += 4) {
+                const float4 x = *reinterpret_cast<const float4*>(&Bs[kk * LDB + tx * RN + j]);
+                b[j] = x.x; b[j + 1] = x.y; b[j + 2] = x.z; b[j + 3] = x.w;
+            }
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+                for (int j = 0; j < RN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
+    auto put = [&](int64_t m, int64_t n, float v) {
+        if (bias) v += to_f32(bias[n]);
+        C[m * ldc + n] = from_f32<T>(v);
+    };
+    const int S = (int)gridDim.z;
+    if (KS == 1 && S == 1) {                                 // nothing to add up: straight from the registers
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int64_t m = m0 + ty * 4 + i;
-        if (m >= M) continue;
+        for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t n = n0 + tx * 4 + j;
-            if (n >= N) continue;
-            float v = acc[i][j];
-            if (bias) v += to_f32(bias[n]);
-            C[m * ldc + n] = from_f32<T>(v);
-        }
+            for (int j = 0; j < RN; ++j) {
+                const int64_t m = m0 + ty * RM + i, n = n0 + tx * RN + j;
+                if (m < M && n < N) put(m, n, acc[i][j]);
+            }
     }
-}
-
-// out[n] = sum_m A[m][n], rows added in a fixed order (thread-strided partials, then a tree in
-// shared memory whose shape does not depend on timing).
-template <typename T>
-__global__ void __launch_bounds__(256) simt_colsum_kernel(const T* __restrict__ A, int64_t lda, int64_t M, int64_t N,
-                                                          T* __restrict__ out) {
-    __shared__ float part[8][33];
-    const int c = threadIdx.x % 32, g = threadIdx.x / 32;
-    const int64_t n = (int64_t)blockIdx.x * 32 + c;
-    float s = 0.f;
-    if (n < N)
-        for (int64_t m = g; m < M; m += 8) s += to_f32(A[m * lda + n]);
-    part[g][c] = s;
-    __syncthreads();
-    if (g == 0 && n < N) {
-        float tot = 0.f;
+    float* csums = smem + C_::kSmem - TM;
+    if (sums) {                                              // the shares of a row, added in ascending order
+        smem[t] = csum;                                      // (the tiles are dead)
+        __syncthreads();
+        if (t < TM) {
+            float x = 0.f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) tot += part[i][c];
-        out[n] = from_f32<T>(tot);
+            for (int i = 0; i < NT / TM; ++i) x += smem[i * TM + t];
+            csums[t] = x;
+        }
+        __syncthreads();
+    }
+    if (KS > 1 || S > 1) {
+        float* red = smem;                                   // [KS][TM][TN]
+#pragma unroll
+        for (int i = 0; i < RM; ++i)
+#pragma unroll
+            for (int j = 0; j < RN; j += 4)
+                *reinterpret_cast<float4*>(&red[(grp * TM + ty * RM + i) * TN + tx * RN + j]) = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+        cg::cluster_group cluster = cg::this_cluster();
+        if (S > 1) cluster.sync(); else __syncthreads();
+        const int rank = S > 1 ? (int)cluster.block_rank() : 0;
+        for (int e = rank * NT + t; e < TM * TN; e += S * NT) {
+            const int64_t m = m0 + e / TN, n = n0 + e % TN;
+            if (m >= M || n >= N) continue;
+            float v = 0.f;
+            for (int z = 0; z < S; ++z) {
+                const float* src = S > 1 ? cluster.map_shared_rank(red, z) : red;
+#pragma unroll
+                for (int q = 0; q < KS; ++q) v += src[q * TM * TN + e];
+            }
+            put(m, n, v);
+        }
+        if (sums && rank == 0 && t < TM && m0 + t < M) {
+            float v = 0.f;
+            for (int z = 0; z < S; ++z) v += (S > 1 ? cluster.map_shared_rank(csums, z) : csums)[t];
+            a_colsum[m0 + t] = from_f32<T>(v);
+        }
+        if (S > 1) cluster.sync();                           // no block leaves while a peer still reads its partial tile
+    } else if (sums && t < TM && m0 + t < M) {
+        a_colsum[m0 + t] = from_f32<T>(csums[t]);
     }
 }
 
@@ -243,26 +348,78 @@ lrd_status_t colsum_two_stage_t(const void* A, int64_t lda, int64_t M, int64_t N
     return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
 }
 
+// Tile and split.  A block's time is its fused multiply-adds (per thread and k: RM RN of them, and the shared-memory reads
+// around them: the small tile runs at about half the rate of the large one) plus some 3000 clocks of loads, sums and
+// stores; two blocks share an SM.  The reduction is split while the grid has fewer than two blocks per SM and a share
+// still has 32 k.
+struct SimtPlan { int cfg, splits; };
+SimtPlan simt_plan(int64_t M, int64_t N, int64_t K) {
+    const int tm[3] = {128, 64, 32}, tn[3] = {64, 64, 32};
+    const double per_k[3] = {90.0, 48.0, 18.0};              // clocks of a block per k
+    SimtPlan best{2, 1};
+    double best_cost = 1e300;
+    for (int c = 0; c < 3; ++c) {
+        const int64_t tiles = ((M + tm[c] - 1) / tm[c]) * ((N + tn[c] - 1) / tn[c]);
+        for (int S = 1; S <= kMaxSplit; ++S) {
+            if (S > 1 && (tiles * S > 2 * kNumSms || (K + S - 1) / S < TK)) break;
+            const double waves = (double)((tiles * S + 2 * kNumSms - 1) / (2 * kNumSms));
+            const double share = (double)((K + S - 1) / S);
+            const double crowd = tiles * S > kNumSms ? 1.6 : 1.0;                       // two blocks on an SM share its units
+            const double cost = waves * (share * per_k[c] * crowd + 3000.0 + (S > 1 ? 1200.0 : 0.0));
+            if (cost < best_cost) { best_cost = cost; best = {c, S}; }
+        }
+    }
+    return best;
+}
+
+template <typename T, typename Cfg, typename LA, typename LB>
+lrd_status_t simt_launch(int splits, int64_t M, int64_t N, int64_t K, const LA& la, const LB& lb, T* C, int64_t ldc, const T* bias, T* a_colsum,
+                         cudaStream_t stream) {
+    const int64_t per = ((K + splits - 1) / splits + TK - 1) / TK * TK;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((N + Cfg::TN - 1) / Cfg::TN) * ((M + Cfg::TM - 1) / Cfg::TM)), 1, (unsigned)splits);
+    cfg.blockDim = dim3(NT, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) before it touches global memory
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = (unsigned)splits;
+    cfg.attrs = attr;
+    cfg.numAttrs = splits > 1 ? 2 : 1;
+    if (!cuda_ok(cudaLaunchKernelEx(&cfg, simt_gemm_kernel<T, Cfg, LA, LB>, M, N, K, per, la, lb, C, ldc, bias, a_colsum), "cudaLaunchKernelEx(general product)"))
+        return LRD_ERR_CUDA;
+    count_launch();
+    return LRD_OK;
+}
+
+template <typename T, typename LA, typename LB>
+lrd_status_t simt_product(int64_t M, int64_t N, int64_t K, const LA& la, const LB& lb, void* C, int64_t ldc, const void* bias, void* a_colsum,
+                          cudaStream_t s) {
+    const SimtPlan pl = simt_plan(M, N, K);
+    switch (pl.cfg) {
+        case 0:  return simt_launch<T, Large>(pl.splits, M, N, K, la, lb, (T*)C, ldc, (const T*)bias, (T*)a_colsum, s);
+        case 1:  return simt_launch<T, Medium>(pl.splits, M, N, K, la, lb, (T*)C, ldc, (const T*)bias, (T*)a_colsum, s);
+        default: return simt_launch<T, Small>(pl.splits, M, N, K, la, lb, (T*)C, ldc, (const T*)bias, (T*)a_colsum, s);
+    }
+}
+
 template <typename T>
 lrd_status_t simt_gemm_t(const GemmArgs& g, cudaStream_t stream) {
-    dim3 grid((unsigned)((g.N + TN - 1) / TN), (unsigned)((g.M + TM - 1) / TM));
-    PlainA<T> la{(const T*)g.A, g.lda, g.a_mn_major};
-    PlainB<T> lb{(const T*)g.B, g.ldb, g.b_mn_major};
-    simt_gemm_kernel<T><<<grid, NT, 0, stream>>>(g.M, g.N, g.K, la, lb, (T*)g.C, g.ldc, (const T*)g.bias);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
+    const T *A = (const T*)g.A, *B = (const T*)g.B;
+    auto run = [&](const auto& la, const auto& lb) { return simt_product<T>(g.M, g.N, g.K, la, lb, g.C, g.ldc, g.bias, g.a_colsum, stream); };
+    if (g.a_mn_major)
+        return g.b_mn_major ? run(PlainA<T, true>{A, g.lda}, PlainB<T, true>{B, g.ldb}) : run(PlainA<T, true>{A, g.lda}, PlainB<T, false>{B, g.ldb});
+    return g.b_mn_major ? run(PlainA<T, false>{A, g.lda}, PlainB<T, true>{B, g.ldb}) : run(PlainA<T, false>{A, g.lda}, PlainB<T, false>{B, g.ldb});
 }
 
 template <typename T>
 lrd_status_t conv_fwd_t(const void* in, const void* G, void* out, int64_t B, const ConvGeom& g, int ci, int co, cudaStream_t stream) {
     // M = output pixels, N = co, K = taps * ci, B = G as [co x taps * ci] (k contiguous)
     const int64_t P = B * g.Ho * g.Wo, K = (int64_t)g.k * g.k * ci;
-    dim3 grid((unsigned)((co + TN - 1) / TN), (unsigned)((P + TM - 1) / TM));
-    ConvFwdA<T> la{(const T*)in, g, ci};
-    PlainB<T> lb{(const T*)G, K, 0};
-    simt_gemm_kernel<T><<<grid, NT, 0, stream>>>(P, co, K, la, lb, (T*)out, co, (const T*)nullptr);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
+    return simt_product<T>(P, co, K, ConvFwdA<T>{(const T*)in, g, ci}, PlainB<T, false>{(const T*)G, K}, out, co, nullptr, nullptr, stream);
 }
 
 template <typename T>
@@ -270,28 +427,15 @@ lrd_status_t conv_bwd_data_t(const void* dout, const void* G, void* din, int64_t
                              cudaStream_t stream) {
     // M = input pixels, N = ci, K = taps * co, B = G regrouped as (tap, o) x i
     const int64_t P = B * g.H * g.W, K = (int64_t)g.k * g.k * co;
-    dim3 grid((unsigned)((ci + TN - 1) / TN), (unsigned)((P + TM - 1) / TM));
-    ConvBwdA<T> la{(const T*)dout, g, co};
-    CoreTransposedB<T> lb{(const T*)G, ci, co, g.k * g.k};
-    simt_gemm_kernel<T><<<grid, NT, 0, stream>>>(P, ci, K, la, lb, (T*)din, ci, (const T*)nullptr);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
+    return simt_product<T>(P, ci, K, ConvBwdA<T>{(const T*)dout, g, co}, CoreTransposedB<T>{(const T*)G, ci, co, g.k * g.k}, din, ci, nullptr, nullptr, stream);
 }
 
 template <typename T>
 lrd_status_t conv_filter_t(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int ci, int co,
                            cudaStream_t stream) {
-    const int taps = g.k * g.k;
-    const int64_t P = B * g.Ho * g.Wo;
-    dim3 grid((unsigned)((ci + TN - 1) / TN), (unsigned)((co + TM - 1) / TM));
-    for (int t = 0; t < taps; ++t) {   // one product per tap: M = co, N = ci, K = output pixels (single block owns all of K)
-        PlainA<T> la{(const T*)dout, co, 1};
-        ConvTapB<T> lb{(const T*)in, g, ci, t / g.k, t % g.k};
-        simt_gemm_kernel<T><<<grid, NT, 0, stream>>>(co, ci, P, la, lb, (T*)dG + (int64_t)t * ci, (int64_t)taps * ci,
-                                                     (const T*)nullptr);
-    }
-    count_launch(taps);
-    return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
+    // M = co, N = taps * ci, K = output pixels
+    const int64_t P = B * g.Ho * g.Wo, N = (int64_t)g.k * g.k * ci;
+    return simt_product<T>(co, N, P, PlainA<T, true>{(const T*)dout, co}, ConvTapsB<T>{(const T*)in, g, ci}, dG, N, nullptr, nullptr, stream);
 }
 
 }  // namespace
@@ -320,34 +464,6 @@ lrd_status_t simt_conv_bwd_filter(const void* dout, const void* in, void* dG, in
 int colsum_splits(int64_t M) {
     int64_t s = M / 64;
     return (int)(s < 1 ? 1 : (s > 64 ? 64 : s));
-}
-
-size_t colsum_scratch_bytes(int64_t M, int64_t N) {
-    const int s = colsum_splits(M);
-    return s > 1 ? align_up((size_t)s * (size_t)N * sizeof(float), 256) : 0;
-}
-
-lrd_status_t colsum(const void* A, int64_t lda, int64_t M, int64_t N, void* out, lrd_dtype_t dtype, float* scratch,
-                    size_t scratch_bytes, cudaStream_t stream) {
-    if (N <= 0) return LRD_OK;
-    const int s = colsum_splits(M);
-    if (s > 1 && scratch && scratch_bytes >= (size_t)s * (size_t)N * sizeof(float))
-        return dtype == LRD_F32 ? colsum_two_stage_t<float>(A, lda, M, N, out, scratch, s, stream)
-                                : colsum_two_stage_t<__nv_bfloat16>(A, lda, M, N, out, scratch, s, stream);
-    return simt_colsum(A, lda, M, N, out, dtype, stream);
-}
-
-lrd_status_t simt_colsum(const void* A, int64_t lda, int64_t M, int64_t N, void* out, lrd_dtype_t dtype,
-                         cudaStream_t stream) {
-    if (N <= 0) return LRD_OK;
-    const unsigned grid = (unsigned)((N + 31) / 32);
-    if (dtype == LRD_F32)
-        simt_colsum_kernel<float><<<grid, 256, 0, stream>>>((const float*)A, lda, M, N, (float*)out);
-    else
-        simt_colsum_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>((const __nv_bfloat16*)A, lda, M, N,
-                                                                     (__nv_bfloat16*)out);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
 }
 
 }  // namespace lrd
@@ -400,8 +516,7 @@ extern "C" lrd_status_t lrd_bias_grad_noalloc(const void* dY, int64_t ldy, int64
     float* scratch = nullptr;
     const lrd_status_t st = noalloc_scratch(&scratch);
     if (st != LRD_OK) return st;
-    // Same kernels and same row split as the workspace path (splits <= 64, so the partial sums fit);
-    // stage 1 writes every partial that stage 2 reads, so nothing left by an earlier call is ever used.
+    // At most 64 splits, so the partial sums fit; stage 1 writes every partial that stage 2 reads, so nothing left by an earlier call is ever used.
     const int splits = lrd::colsum_splits(M);
     return dtype == LRD_F32 ? lrd::colsum_two_stage_t<float>(dY, ldy, M, N, dbias, scratch, splits, stream)
                             : lrd::colsum_two_stage_t<__nv_bfloat16>(dY, ldy, M, N, dbias, scratch, splits, stream);

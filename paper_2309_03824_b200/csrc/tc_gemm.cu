@@ -659,15 +659,11 @@ size_t tc_split_workspace_bytes(int64_t M, int64_t N, int64_t K) {
     return need;
 }
 
-bool tc_gemm_colsum_ok(const GemmArgs& g) {
-    return tc_gemm_eligible(g) && g.a_mn_major && g.b_mn_major && (((uintptr_t)g.a_colsum & 1u) == 0);
-}
-
 lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_t partial_bytes,
                      cudaStream_t stream) {
     if (!tc_gemm_eligible(g)) return LRD_ERR_UNSUPPORTED;
     const bool ones = g.a_colsum != nullptr;
-    if (ones && !tc_gemm_colsum_ok(g)) return LRD_ERR_UNSUPPORTED;
+    if (ones && !(g.a_mn_major && g.b_mn_major)) return LRD_ERR_UNSUPPORTED;
     if (!allow_split && !ones) return tc_gemm_persistent(g, stream);   // data products: the persistent kernel
     int splits = 1, cluster = 1, bn;
     if (allow_split) {
