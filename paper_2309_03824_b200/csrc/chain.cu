@@ -183,16 +183,20 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
         const uint32_t idesc1 = idesc_bf16(p.RS, false, true);
         const uint64_t a_desc0 = smem_desc_sw128(0, 0, 1024);
         const uint64_t b_desc0 = smem_desc(0, p_box_bytes, 8u * p.swb, p.swb);
+        uint32_t ready = mbar_test_wait(smem_u32(&full1[0]), 0);
         for (int g = 0; g < ng1; ++g) {
-            ok = mbar_wait_uniform(smem_u32(&full1[s]), ph, ab);
+            ok = mbar_wait_peeked(ready, smem_u32(&full1[s]), ph, ab);
             if (!ok) break;
             tc_fence_after();
+            const uint32_t eb = smem_u32(&empty1[s]);
             const uint32_t in_src = ring1_base + s * p.stage1_bytes;
             const uint32_t p_src = in_src + p.G1 * kInTileBytes;
             const int nkb = min(p.G1, p.kb1 - g * p.G1);
             // descriptors differ only in the start-address field (bits 0-13, in 16-byte units)
             uint64_t ad = a_desc0 + ((in_src >> 4) & 0x3FFFu);
             uint64_t bd = b_desc0 + ((p_src >> 4) & 0x3FFFu);
+            if (++s == p.S1) { s = 0; ph ^= 1; }
+            ready = g + 1 < ng1 ? mbar_test_wait(smem_u32(&full1[s]), ph) : 0u;
             if (elect_one()) {
                 for (int i = 0; i < nkb; ++i) {
 #pragma unroll
@@ -201,10 +205,9 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
                     ad += kInTileBytes >> 4;
                     bd += (uint64_t)(4 * p.swb);              // 64 rows of swb bytes
                 }
-                mma_commit(smem_u32(&empty1[s]));
+                mma_commit(eb);
             }
             __syncwarp();
-            if (++s == p.S1) { s = 0; ph ^= 1; }
         }
         if (ok && elect_one()) mma_commit(smem_u32(&tacc_bar));
         __syncwarp();
@@ -224,6 +227,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
             tk_off[kk] = (((kk >> p.t_steps_lg) * t_atom_bytes) + (kk & ((1u << p.t_steps_lg) - 1u)) * 32u) >> 4;
         s = 0;
         ph = 0;
+        ready = 0;
         int i2 = 0;
         for (int j = c; j < p.n_chunks && ok; j += p.C, ++i2) {
             const uint32_t d_tmem = tmem_base + (uint32_t)(i2 & 1) * 256u;
@@ -242,22 +246,24 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
                     }
                     if (!ok) break;
                 }
-                ok = mbar_wait_uniform(smem_u32(&full2[s]), ph, ab);
+                ok = mbar_wait_peeked(ready, smem_u32(&full2[s]), ph, ab);
                 if (!ok) break;
                 tc_fence_after();
+                const uint32_t eb = smem_u32(&empty2[s]);
                 const uint32_t q_src = ring2_base + s * p.stage2_bytes;
                 const uint64_t bd = a_desc0 + ((q_src >> 4) & 0x3FFFu);
+                if (++s == p.S2) { s = 0; ph ^= 1; }
+                ready = mbar_test_wait(smem_u32(&full2[s]), ph);          // (after the last stage: not acted upon)
                 if (elect_one()) {
                     const uint64_t adk = t_desc0 + (uint32_t)kb * tk_stride;
                     const uint32_t acc = i > 0 ? 1u : 0u;
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)                        // 16-column steps within T
                         if (kk < nks) mma_bf16_ss(d_tmem, adk + tk_off[kk], bd + 2u * kk, idesc2, kk > 0 ? 1u : acc);
-                    mma_commit(smem_u32(&empty2[s]));
+                    mma_commit(eb);
                     if (i == p.kb2 - 1) mma_commit(smem_u32(&out_full[i2 & 1]));
                 }
                 __syncwarp();
-                if (++s == p.S2) { s = 0; ph ^= 1; }
             }
         }
         // a block without a chunk of its own still has to have received every slice before it passes barrier 2

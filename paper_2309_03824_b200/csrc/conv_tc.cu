@@ -180,11 +180,14 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
         int s = 0, cb = 0;
         uint32_t ph = 0;
         bool ok = true;
+        uint32_t ready = mbar_test_wait(smem_u32(&full_bar[0]), 0);
         for (int it = 0; it < iters; ++it) {
-            ok = mbar_wait_uniform(smem_u32(&full_bar[s]), ph, ab);
+            ok = mbar_wait_peeked(ready, smem_u32(&full_bar[s]), ph, ab);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t a_src = smem_base + s * stage_bytes, b_src = a_src + kTile;
+            const uint32_t a_src = smem_base + s * stage_bytes, b_src = a_src + kTile, eb = smem_u32(&empty_bar[s]);
+            if (++s == p.stages) { s = 0; ph ^= 1; }
+            ready = mbar_test_wait(smem_u32(&full_bar[s]), ph);              // (after the last stage: not acted upon)
             const int nks = min(4, (p.ka - cb * 64 + 15) / 16);              // 16-channel steps past ka hold zeros: not issued
             if (elect_one()) {
                 const uint64_t ad0 = smem_desc_sw128(a_src, 0, 1024);
@@ -192,10 +195,9 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)                               // the k-step moves the start address only
                     if (kk < nks) mma_bf16_ss(tmem_base, ad0 + 2u * kk, bd0 + (DGRAD ? 128u : 2u) * kk, idesc, (it > 0 || kk > 0) ? 1u : 0u);
-                mma_commit(smem_u32(&empty_bar[s]));
+                mma_commit(eb);
             }
             __syncwarp();
-            if (++s == p.stages) { s = 0; ph ^= 1; }
             if (++cb == p.nkc) cb = 0;
         }
         if (ok && elect_one()) mma_commit(smem_u32(&acc_bar));

@@ -38,6 +38,14 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok;
 }
 
+__device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity) {     // never suspends
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok;
+}
+
 // Bounded wait.  Returns false when the barrier did not flip within the limit or another
 // thread of the block has already given up; the caller then leaves its loop and the block
 // tears down in order.
@@ -65,6 +73,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const A
 __device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, const AbortCtx& ab) {
     const bool ok = mbar_wait(bar, parity, ab);
     return __all_sync(0xffffffffu, ok) != 0;
+}
+
+// The same for a barrier that was looked at before (`ready` = mbar_test_wait of this phase, issued ahead of other work so
+// that the hundred clocks a look takes pass beside it): waits only where that look came too early.
+__device__ __forceinline__ bool mbar_wait_peeked(uint32_t ready, uint32_t bar, uint32_t parity, const AbortCtx& ab) {
+    return __any_sync(0xffffffffu, ready == 0) ? mbar_wait_uniform(bar, parity, ab) : true;
 }
 
 // Warp-wide wait for the long waits of the epilogue warps: lane 0 polls with a sleep between tries

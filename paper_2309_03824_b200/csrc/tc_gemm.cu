@@ -38,14 +38,17 @@ using namespace ptx;
 
 constexpr int BM = 128, BK = 64;
 constexpr int kThreads = 224;                         // warp 6: second TMA producer (the B operand)
-constexpr uint32_t A_STAGE_BYTES = BM * BK * 2;
 constexpr int kMaxClusterSplits = 8;                 // portable cluster size
 
 // ONES: every stage carries one more 64-wide MN-major block of B that holds 1.0 everywhere and is never
 // overwritten; with N = BN + 16 the MMA then also forms sum_k A(m, k) in accumulator column BN (the bias
 // gradient falls out of the dU product: its A operand is dY).
+// G: 64-deep k-blocks per stage.  Two for the narrow tiles, whose MMAs take no longer than what a stage costs the issuing
+// warp beside them (see tc_gemm_persistent.cu), as long as three stages fit.
 template <int BN, bool ONES = false> struct Cfg {
-    static constexpr uint32_t B_STAGE_BYTES = BN * BK * 2 + (ONES ? 8192 : 0);
+    static constexpr int G = BN <= 64 || (BN <= 128 && !ONES) ? 2 : 1;
+    static constexpr uint32_t A_STAGE_BYTES = G * BM * BK * 2;
+    static constexpr uint32_t B_STAGE_BYTES = G * (BN * BK * 2 + (ONES ? 8192 : 0));
     static constexpr uint32_t STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
     static constexpr int STAGES_RAW = (200 * 1024) / STAGE_BYTES;
     static constexpr int STAGES = STAGES_RAW > 8 ? 8 : STAGES_RAW;
@@ -84,7 +87,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     static_assert(!ONES || (A_MN && B_MN && BN <= 192), "the ones block rides on an MN-major B of at most 192 columns");
     static_assert(!CONV || (A_MN && B_MN && !ONES && BN <= 192), "the filter gradient: both operands MN-major, split over a cluster or not at all");
     using C = Cfg<BN, ONES>;
-    constexpr int STAGES = C::STAGES;
+    constexpr int STAGES = C::STAGES, G = C::G;
+    constexpr uint32_t A_STAGE_BYTES = C::A_STAGE_BYTES, kBox = 8192u * G;        // MN-major box: 64 G k rows x 64 columns
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], acc_bar, red_bar;
     __shared__ uint32_t tmem_base_slot;
@@ -116,8 +120,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         fence_mbar_init();
     }
     if (ONES) {          // bf16 1.0 in every element of the extra block of each stage
-        for (uint32_t off = threadIdx.x * 16u; off < STAGES * 8192u; off += kThreads * 16u)
-            st_shared_v4(smem_base + (off / 8192u) * C::STAGE_BYTES + A_STAGE_BYTES + BN * 128u + (off % 8192u), 0x3F803F80u,
+        for (uint32_t off = threadIdx.x * 16u; off < STAGES * kBox; off += kThreads * 16u)
+            st_shared_v4(smem_base + (off / kBox) * C::STAGE_BYTES + A_STAGE_BYTES + BN * 128u * G + (off % kBox), 0x3F803F80u,
                          0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
         fence_proxy_async_smem();
     }
@@ -137,32 +141,31 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (warp == 0) {
         // TMA producer: the whole warp runs the loop, one elected lane issues (operands stay uniform)
         int it = 0;
-        for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
+        for (int kb = kb_begin; kb < kb_end; kb += G, ++it) {          // (a k-block past this block's share is loaded, not multiplied)
             const int s = it % STAGES;
             const uint32_t ph = (it / STAGES) & 1;
             if (!mbar_wait_uniform(smem_u32(&empty_bar[s]), ph ^ 1, ab)) break;
             const uint32_t fb = smem_u32(&full_bar[s]);
             const uint32_t a_dst = smem_base + s * C::STAGE_BYTES;
-            const uint32_t b_dst = a_dst + A_STAGE_BYTES;
             const int k0 = kb * BK;
             if (elect_one()) {
-                mbar_expect_tx(fb, A_STAGE_BYTES + BN * BK * 2);       // the whole stage: warp 6's copies complete on the same barrier
+                mbar_expect_tx(fb, A_STAGE_BYTES + G * BN * BK * 2);   // the whole stage: warp 6's copies complete on the same barrier
                 if (A_MN) {
 #pragma unroll
-                    for (int j = 0; j < BM / 64; ++j) tma_load_2d(a_dst + j * 8192, &tmA, fb, m0 + 64 * j, k0);
+                    for (int j = 0; j < BM / 64; ++j) tma_load_2d(a_dst + j * kBox, &tmA, fb, m0 + 64 * j, k0);
                 } else {
-                    tma_load_2d(a_dst, &tmA, fb, k0, m0);
+#pragma unroll
+                    for (int g = 0; g < G; ++g) tma_load_2d(a_dst + g * (BM * BK * 2), &tmA, fb, k0 + g * BK, m0);
                 }
             }
             __syncwarp();
-            (void)b_dst;
         }
         if (p.cluster_splits > 1) { cluster_arrive(); cluster_wait(); cluster_arrive_relaxed(); }   // barriers 1 and 2, see the epilogue
     } else if (warp == 6) {
         // second TMA producer: the B operand of every stage (its bytes are counted by warp 0's expect_tx; a copy that
         // lands before that arrival only makes the barrier's byte count negative for a moment)
         int it = 0;
-        for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
+        for (int kb = kb_begin; kb < kb_end; kb += G, ++it) {
             const int s = it % STAGES;
             const uint32_t ph = (it / STAGES) & 1;
             if (!mbar_wait_uniform(smem_u32(&empty_bar[s]), ph ^ 1, ab)) break;
@@ -170,23 +173,24 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t b_dst = smem_base + s * C::STAGE_BYTES + A_STAGE_BYTES;
             const int k0 = kb * BK;
             if (CONV) {
-                // 64 output pixels from pixel k0 on; a column block = 64 channels at one tap (blocks past the last tap load
+                // 64 G output pixels from pixel k0 on; a column block = 64 channels at one tap (blocks past the last tap load
                 // the last one again, their columns are never stored)
                 const int w = (k0 % p.cv_Wo) * p.cv_stride - p.cv_pad, hh = (k0 / p.cv_Wo) % p.cv_Ho, im = k0 / (p.cv_Wo * p.cv_Ho);
                 if (elect_one()) {
 #pragma unroll
                     for (int j = 0; j < BN / 64; ++j) {
                         const int blk = min(n0 / 64 + j, p.cv_nblk - 1), tap = blk / p.cv_nkc;
-                        tma_load_im2col(b_dst + j * 8192, &tmB, fb, (blk % p.cv_nkc) * 64, w, hh * p.cv_stride - p.cv_pad, im,
+                        tma_load_im2col(b_dst + j * kBox, &tmB, fb, (blk % p.cv_nkc) * 64, w, hh * p.cv_stride - p.cv_pad, im,
                                         (uint32_t)(tap % p.cv_k), (uint32_t)(tap / p.cv_k));
                     }
                 }
             } else if (elect_one()) {
                 if (B_MN) {
 #pragma unroll
-                    for (int j = 0; j < BN / 64; ++j) tma_load_2d(b_dst + j * 8192, &tmB, fb, n0 + 64 * j, k0);
+                    for (int j = 0; j < BN / 64; ++j) tma_load_2d(b_dst + j * kBox, &tmB, fb, n0 + 64 * j, k0);
                 } else {
-                    tma_load_2d(b_dst, &tmB, fb, k0, n0);
+#pragma unroll
+                    for (int g = 0; g < G; ++g) tma_load_2d(b_dst + g * (BN * BK * 2), &tmB, fb, k0 + g * BK, n0);
                 }
             }
             __syncwarp();
@@ -195,28 +199,31 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else if (warp == 1) {
         // MMA issuer: converged warp, elect.sync around the issue
         const uint32_t idesc = idesc_bf16(BN + ((ONES && blockIdx.x == 0) ? 16 : 0), A_MN, B_MN);
+        const uint64_t a_desc0 = A_MN ? smem_desc_sw128(smem_base, kBox, 1024) : smem_desc_sw128(smem_base, 0, 1024);
+        const uint64_t b_desc0 = B_MN ? smem_desc_sw128(smem_base + A_STAGE_BYTES, kBox, 1024) : smem_desc_sw128(smem_base + A_STAGE_BYTES, 0, 1024);
         int s = 0;
-        uint32_t ph = 0;
+        uint32_t ph = 0, ready = kb_begin < kb_end ? mbar_test_wait(smem_u32(&full_bar[0]), 0) : 0u;
         bool ok = true;
-        for (int kb = kb_begin; kb < kb_end; ++kb) {
-            ok = mbar_wait_uniform(smem_u32(&full_bar[s]), ph, ab);
+        for (int kb = kb_begin; kb < kb_end; kb += G) {
+            ok = mbar_wait_peeked(ready, smem_u32(&full_bar[s]), ph, ab);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t a_src = smem_base + s * C::STAGE_BYTES;
-            const uint32_t b_src = a_src + A_STAGE_BYTES;
+            const uint64_t ad = a_desc0 + (uint32_t)s * (C::STAGE_BYTES >> 4), bd = b_desc0 + (uint32_t)s * (C::STAGE_BYTES >> 4);
+            const uint32_t eb = smem_u32(&empty_bar[s]);
+            if (++s == STAGES) { s = 0; ph ^= 1; }
+            ready = kb + G < kb_end ? mbar_test_wait(smem_u32(&full_bar[s]), ph) : 0u;
             if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk) {
-                    const uint64_t ad = A_MN ? smem_desc_sw128(a_src + kk * 2048, 8192, 1024)
-                                             : smem_desc_sw128(a_src + kk * 32, 0, 1024);
-                    const uint64_t bd = B_MN ? smem_desc_sw128(b_src + kk * 2048, 8192, 1024)
-                                             : smem_desc_sw128(b_src + kk * 32, 0, 1024);
-                    mma_bf16_ss(tmem_base, ad, bd, idesc, (kb > kb_begin || kk > 0) ? 1u : 0u);
+                for (int g = 0; g < G; ++g) {
+                    if (g > 0 && kb + g >= kb_end) break;
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk)
+                        mma_bf16_ss(tmem_base, ad + (A_MN ? (g * 4 + kk) * 128u : g * (BM * BK * 2 >> 4) + kk * 2u),
+                                    bd + (B_MN ? (g * 4 + kk) * 128u : g * (BN * BK * 2 >> 4) + kk * 2u), idesc, g > 0 || kk > 0 ? 1u : (kb > kb_begin ? 1u : 0u));
                 }
-                mma_commit(smem_u32(&empty_bar[s]));
+                mma_commit(eb);
             }
             __syncwarp();
-            if (++s == STAGES) { s = 0; ph ^= 1; }
         }
         if (ok && elect_one()) mma_commit(smem_u32(&acc_bar));
         __syncwarp();
@@ -534,6 +541,15 @@ lrd_status_t launch_major(bool a_mn, bool b_mn, const CUtensorMap& tA, const CUt
 
 inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
+uint32_t stage_kblocks(int bn, bool ones) {
+    switch (bn) {
+        case 64:  return ones ? Cfg<64, true>::G : Cfg<64>::G;
+        case 128: return ones ? Cfg<128, true>::G : Cfg<128>::G;
+        default:  return 1;
+    }
+}
+static_assert(Cfg<192>::G == 1 && Cfg<192, true>::G == 1 && Cfg<256>::G == 1, "stage_kblocks");
+
 }  // namespace
 
 bool tc_gemm_eligible(const GemmArgs& g) {
@@ -636,7 +652,7 @@ static SplitPlan pick_split(int64_t M, int64_t N, int64_t K, bool ones, int max_
         for (int S = top; S >= 2; --S) {
             if (bn % (8 * S)) continue;
             if (tiles > max_active_clusters(S) || S > kb) continue;    // one wave: a second wave would double the time
-            const double per_block = (double)((kb + S - 1) / S) * (A_STAGE_BYTES + bn * BK * 2.0);
+            const double per_block = (double)((kb + S - 1) / S) * (BM * BK * 2.0 + bn * BK * 2.0);
             const double t = std::max(per_block / 110e9, per_block * (double)(tiles * S) / 11.5e12) + 2e-6 * bn / 192.0;
             if (t < best_t) { best_t = t; best.bn = bn; best.cluster = S; best.global = 1; }
             break;                                                // the largest feasible cluster for this width
@@ -682,9 +698,10 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     const int kb_per = (kb_total + zdim - 1) / zdim;
 
     CUtensorMap tA, tB;
-    bool ok = g.a_mn_major ? make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, BK, 64)
+    const uint32_t kbox = BK * stage_kblocks(bn, ones);             // k rows of an MN-major box
+    bool ok = g.a_mn_major ? make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, kbox, 64)
                            : make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda, BM, BK);
-    ok = ok && (g.b_mn_major ? make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb, BK, 64)
+    ok = ok && (g.b_mn_major ? make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb, kbox, 64)
                              : make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb, (uint32_t)bn, BK));
     if (!ok) return LRD_ERR_CUDA;
 
@@ -730,8 +747,9 @@ lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t 
     SplitPlan sp = pick_split(co, N, P, true);             // (tiles of at most 192 columns)
     if (sp.cluster < 2) sp.cluster = 1;                    // tiles enough to fill the GPU: each reduces over all pixels
     CUtensorMap tA, tB;
-    bool ok = make_tmap_2d_bf16(&tA, dout, (uint64_t)P, (uint64_t)co, (uint64_t)co, BK, 64);
-    ok = ok && make_tmap_im2col_bf16(&tB, in, (uint64_t)B, (uint64_t)g.H, (uint64_t)g.W, (uint64_t)ci, -g.pad, -g.pad, g.Ho, g.Wo, g.stride, BK);
+    const uint32_t kbox = BK * stage_kblocks(sp.bn, false);
+    bool ok = make_tmap_2d_bf16(&tA, dout, (uint64_t)P, (uint64_t)co, (uint64_t)co, kbox, 64);
+    ok = ok && make_tmap_im2col_bf16(&tB, in, (uint64_t)B, (uint64_t)g.H, (uint64_t)g.W, (uint64_t)ci, -g.pad, -g.pad, g.Ho, g.Wo, g.stride, kbox);
     if (!ok) return LRD_ERR_CUDA;
     TcParams p{};
     p.M = co; p.N = N; p.ldp = N;

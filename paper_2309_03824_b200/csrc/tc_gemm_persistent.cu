@@ -33,7 +33,14 @@ constexpr uint32_t kStagingBytes = 4 * 2 * kSlabBytes;
 
 template <int BN, int CG> struct PCfg {
     static constexpr int BNH = BN / CG;                      // columns of B this block loads
-    static constexpr uint32_t STAGE_BYTES = kATile + BNH * BK * 2;
+    // 64-deep k-blocks per stage.  A stage costs the issuing warp some 250 clocks beside its MMAs (a wait, an election, a
+    // commit); the four MMAs of a k-block of a narrow tile take no longer, so narrow tiles have two per stage.  One
+    // 128-row tile, 3072 -> 384: 13.3 us with one k-block per stage and each stage's barrier first looked at when it is
+    // needed, 10.7 with the look ahead, 9.1 with two k-blocks; pairs and wide tiles, paced by their MMAs and
+    // loads, are 1 % slower with two.
+    static constexpr int G = CG == 1 && BN <= 128 ? 2 : 1;
+    static constexpr uint32_t B_TILE = BNH * BK * 2;
+    static constexpr uint32_t STAGE_BYTES = G * (kATile + B_TILE);
     static constexpr int STAGES_RAW = (200 * 1024) / STAGE_BYTES;
     static constexpr int STAGES = STAGES_RAW > 8 ? 8 : STAGES_RAW;
     static constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + kStagingBytes + 1024;
@@ -62,7 +69,7 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     constexpr int BNH = C::BNH;
     static_assert(CG == 1 || CG == 2, "blocks per MMA");
     static_assert(CG == 1 || !B_MN || BNH % 64 == 0, "an MN-major half of B is made of 64-column boxes");
-    constexpr int STAGES = C::STAGES;
+    constexpr int STAGES = C::STAGES, G = C::G;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], out_full[2], out_empty[2];
     __shared__ uint32_t tmem_base_slot;
@@ -121,27 +128,29 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
         bool ok = true;
         for (int t = unit; t < n_tiles_total && ok; t += n_units) {
             const int m0 = (t % p.m_tiles) * (BM * CG) + h * BM, n0 = (t / p.m_tiles) * BN + h * BNH;
-            for (int kb = 0; kb < p.kb_total; ++kb) {
+            for (int kb = 0; kb < p.kb_total; kb += G) {         // k-blocks past the last read as zeros
                 ok = mbar_wait_uniform(smem_u32(&empty_bar[s]), ph, ab);
                 if (!ok) break;
                 // a pair's loads all complete on the even block's barrier, which its MMA warp waits on
                 const uint32_t fb_local = smem_u32(&full_bar[s]);
                 const uint32_t fb = CG == 2 ? map_to_cta(fb_local, 0) : fb_local;
-                const uint32_t a_dst = ring_base + s * C::STAGE_BYTES, b_dst = a_dst + kATile;
+                const uint32_t a_dst = ring_base + s * C::STAGE_BYTES, b_dst = a_dst + G * kATile;
                 const int k0 = kb * BK;
                 if (elect_one()) {
                     if (h == 0) mbar_expect_tx(fb_local, CG * C::STAGE_BYTES);
                     if (A_MN) {
 #pragma unroll
-                        for (int j = 0; j < BM / 64; ++j) load2d<CG>(a_dst + j * 8192, &tmA, fb, m0 + 64 * j, k0);
+                        for (int j = 0; j < BM / 64; ++j) load2d<CG>(a_dst + j * (8192 * G), &tmA, fb, m0 + 64 * j, k0);
                     } else {
-                        load2d<CG>(a_dst, &tmA, fb, k0, m0);
+#pragma unroll
+                        for (int g = 0; g < G; ++g) load2d<CG>(a_dst + g * kATile, &tmA, fb, k0 + g * BK, m0);
                     }
                     if (B_MN) {
 #pragma unroll
-                        for (int j = 0; j < BNH / 64; ++j) load2d<CG>(b_dst + j * 8192, &tmB, fb, n0 + 64 * j, k0);
+                        for (int j = 0; j < BNH / 64; ++j) load2d<CG>(b_dst + j * (8192 * G), &tmB, fb, n0 + 64 * j, k0);
                     } else {
-                        load2d<CG>(b_dst, &tmB, fb, k0, n0);
+#pragma unroll
+                        for (int g = 0; g < G; ++g) load2d<CG>(b_dst + g * C::B_TILE, &tmB, fb, k0 + g * BK, n0);
                     }
                 }
                 __syncwarp();
@@ -151,6 +160,10 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     } else if (warp == 1 && h == 0) {
         // ------------------------------------------------------------------ MMA issuer (the even block of a pair)
         constexpr uint32_t idesc = CG == 2 ? idesc_bf16_pair(BN, A_MN, B_MN) : idesc_bf16(BN, A_MN, B_MN);
+        // the descriptors of a stage differ from these in the start address only (bits 0-13, in 16-byte units); a k-step of
+        // 16 moves it by 2048 bytes (MN-major) or 32 (K-major: 32 within a k-block, then the next tile)
+        const uint64_t a_desc0 = A_MN ? smem_desc_sw128(ring_base, 8192 * G, 1024) : smem_desc_sw128(ring_base, 0, 1024);
+        const uint64_t b_desc0 = B_MN ? smem_desc_sw128(ring_base + G * kATile, 8192 * G, 1024) : smem_desc_sw128(ring_base + G * kATile, 0, 1024);
         int s = 0, i = 0;
         uint32_t ph = 0;
         bool ok = true;
@@ -158,31 +171,38 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
             const int buf = i & 1;
             const uint32_t d_tmem = tmem_base + (uint32_t)buf * C::BUF_COLS;
             ok = mbar_wait_uniform(smem_u32(&out_empty[buf]), ((i >> 1) & 1) ^ 1, ab);      // accumulator buffer drained
-            for (int kb = 0; kb < p.kb_total && ok; ++kb) {
-                ok = mbar_wait_uniform(smem_u32(&full_bar[s]), ph, ab);
+            uint32_t ready = mbar_test_wait(smem_u32(&full_bar[s]), ph);
+            for (int kb = 0; kb < p.kb_total && ok; kb += G) {
+                ok = mbar_wait_peeked(ready, smem_u32(&full_bar[s]), ph, ab);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t a_src = ring_base + s * C::STAGE_BYTES, b_src = a_src + kATile;
+                const uint64_t ad = a_desc0 + (uint32_t)s * (C::STAGE_BYTES >> 4), bd = b_desc0 + (uint32_t)s * (C::STAGE_BYTES >> 4);
+                const uint32_t eb = smem_u32(&empty_bar[s]);
+                const bool last = kb + G >= p.kb_total;
+                if (++s == STAGES) { s = 0; ph ^= 1; }
+                ready = last ? 0u : mbar_test_wait(smem_u32(&full_bar[s]), ph);
                 if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {
-                        const uint64_t ad = A_MN ? smem_desc_sw128(a_src + kk * 2048, 8192, 1024)
-                                                 : smem_desc_sw128(a_src + kk * 32, 0, 1024);
-                        const uint64_t bd = B_MN ? smem_desc_sw128(b_src + kk * 2048, 8192, 1024)
-                                                 : smem_desc_sw128(b_src + kk * 32, 0, 1024);
-                        if (CG == 2) mma_bf16_ss_pair(d_tmem, ad, bd, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-                        else mma_bf16_ss(d_tmem, ad, bd, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                    for (int g = 0; g < G; ++g) {
+                        if (g > 0 && kb + g >= p.kb_total) break;
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            const uint32_t ao = A_MN ? (g * 4 + kk) * 128u : g * (kATile >> 4) + kk * 2u;
+                            const uint32_t bo = B_MN ? (g * 4 + kk) * 128u : g * (C::B_TILE >> 4) + kk * 2u;
+                            const uint32_t acc = g > 0 || kk > 0 ? 1u : (kb > 0 ? 1u : 0u);
+                            if (CG == 2) mma_bf16_ss_pair(d_tmem, ad + ao, bd + bo, idesc, acc);
+                            else mma_bf16_ss(d_tmem, ad + ao, bd + bo, idesc, acc);
+                        }
                     }
                     if (CG == 2) {       // both blocks' stages are free, both blocks' accumulators are ready
-                        mma_commit_pair(smem_u32(&empty_bar[s]), 3);
-                        if (kb == p.kb_total - 1) mma_commit_pair(smem_u32(&out_full[buf]), 3);
+                        mma_commit_pair(eb, 3);
+                        if (last) mma_commit_pair(smem_u32(&out_full[buf]), 3);
                     } else {
-                        mma_commit(smem_u32(&empty_bar[s]));
-                        if (kb == p.kb_total - 1) mma_commit(smem_u32(&out_full[buf]));
+                        mma_commit(eb);
+                        if (last) mma_commit(smem_u32(&out_full[buf]));
                     }
                 }
                 __syncwarp();
-                if (++s == STAGES) { s = 0; ph ^= 1; }
             }
         }
     } else if (warp >= 2) {
@@ -353,9 +373,10 @@ lrd_status_t tc_gemm_persistent(const GemmArgs& g, cudaStream_t stream) {
     if (g_force_cg == 2 && sh.cg != 2) { g_force_cg = 0; sh = pick_shape_p(g.M, g.N); g_force_cg = 2; }
     const int bn = sh.bn, cg = sh.cg, bnh = bn / cg;
     CUtensorMap tA, tB, tC;
-    bool ok = g.a_mn_major ? make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, BK, 64)
+    const uint32_t kbox = BK * (cg == 1 && bn <= 128 ? 2 : 1);         // k rows of an MN-major box
+    bool ok = g.a_mn_major ? make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, kbox, 64)
                            : make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda, BM, BK);
-    ok = ok && (g.b_mn_major ? make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb, BK, 64)
+    ok = ok && (g.b_mn_major ? make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb, kbox, 64)
                              : make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb, (uint32_t)bnh, BK));
     ok = ok && make_tmap_2d_bf16(&tC, g.C, (uint64_t)g.M, (uint64_t)g.N, (uint64_t)g.ldc, 32, 32);
     if (!ok) return LRD_ERR_CUDA;

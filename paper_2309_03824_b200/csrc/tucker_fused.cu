@@ -155,13 +155,19 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         int s = 0;
         uint32_t ph = 0;
         bool ok = true;
+        uint32_t ready = mbar_test_wait(smem_u32(&full_bar[0]), 0);
+        auto advance = [&] {                                 // to the next stage, with a first look at its barrier
+            if (++s == kSlots) { s = 0; ph ^= 1; }
+            ready = mbar_test_wait(smem_u32(&full_bar[s]), ph);
+        };
         // phase A: T1 = In_halo P1
         const uint32_t idescA = idesc_bf16(p.nA, false, true);
         for (int st = 0; st < nkb1 && ok; ++st) {
-            ok = mbar_wait_uniform(smem_u32(&full_bar[s]), ph, ab);
+            ok = mbar_wait_peeked(ready, smem_u32(&full_bar[s]), ph, ab);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t a_src = ring_base + (uint32_t)s * kSlotBytes, b_src = a_src + kTile;
+            const uint32_t a_src = ring_base + (uint32_t)s * kSlotBytes, b_src = a_src + kTile, eb = smem_u32(&empty_bar[s]);
+            advance();
             const int nks = min(4, (p.c_in - st * 64 + 15) / 16);
             if (elect_one()) {
                 const uint64_t ad0 = smem_desc_sw128(a_src, 0, 1024);
@@ -169,10 +175,9 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                     if (kk < nks) mma_bf16_ss(tmem_base, ad0 + 2u * kk, bd0 + (uint64_t)(kk * p.swb), idescA, (st > 0 || kk > 0) ? 1u : 0u);
-                mma_commit(smem_u32(&empty_bar[s]));
+                mma_commit(eb);
             }
             __syncwarp();
-            if (++s == kSlots) { s = 0; ph ^= 1; }
         }
         if (ok && elect_one()) mma_commit(smem_u32(&acc_bar[0]));
         __syncwarp();
@@ -182,10 +187,11 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         const uint64_t z1_desc0 = smem_desc_plain(z1_base, slab_bytes, 128);
         const uint32_t ks_units = 2u * (slab_bytes >> 4);        // a 16-deep k-step = two slabs
         for (int tap = 0; tap < 9 && ok; ++tap) {
-            ok = mbar_wait_uniform(smem_u32(&full_bar[s]), ph, ab);
+            ok = mbar_wait_peeked(ready, smem_u32(&full_bar[s]), ph, ab);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t b_src = ring_base + (uint32_t)s * kSlotBytes;
+            const uint32_t b_src = ring_base + (uint32_t)s * kSlotBytes, eb = smem_u32(&empty_bar[s]);
+            advance();
             const int kh = tap / 3, kw = tap % 3;
             const uint32_t shift = DGRAD ? (uint32_t)((2 - kh) * p.PW + (2 - kw)) : (uint32_t)(kh * p.PW + kw);
             if (elect_one()) {
@@ -199,10 +205,9 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
                             mma_bf16_ss(tmem_base + kAcc2Col, z1_desc0 + shift + (uint32_t)(cb * 4 + kk) * ks_units,
                                         bd0 + (DGRAD ? 128u : 2u) * kk, idescB, (tap > 0 || cb > 0 || kk > 0) ? 1u : 0u);
                 }
-                mma_commit(smem_u32(&empty_bar[s]));
+                mma_commit(eb);
             }
             __syncwarp();
-            if (++s == kSlots) { s = 0; ph ^= 1; }
         }
         if (ok && elect_one()) mma_commit(smem_u32(&acc_bar[1]));
         __syncwarp();
@@ -210,10 +215,11 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         if (ok) ok = mbar_wait_uniform(smem_u32(&ready_bar[1]), 0, ab);
         const uint32_t idescC = idesc_bf16((p.n3 + 15) / 16 * 16, false, false);
         for (int kb = 0; kb < natC && ok; ++kb) {
-            ok = mbar_wait_uniform(smem_u32(&full_bar[s]), ph, ab);
+            ok = mbar_wait_peeked(ready, smem_u32(&full_bar[s]), ph, ab);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t b_src = ring_base + (uint32_t)s * kSlotBytes;
+            const uint32_t b_src = ring_base + (uint32_t)s * kSlotBytes, eb = smem_u32(&empty_bar[s]);
+            advance();
             const int nks = min(4, (p.nB - kb * 64) / 16);
             if (elect_one()) {
                 const uint64_t ad0 = smem_desc_sw128(z2_base + (uint32_t)kb * kTile, 0, 1024);
@@ -221,10 +227,9 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                     if (kk < nks) mma_bf16_ss(tmem_base + kAcc3Col, ad0 + 2u * kk, bd0 + 2u * kk, idescC, (kb > 0 || kk > 0) ? 1u : 0u);
-                mma_commit(smem_u32(&empty_bar[s]));
+                mma_commit(eb);
             }
             __syncwarp();
-            if (++s == kSlots) { s = 0; ph ^= 1; }
         }
         if (ok && elect_one()) mma_commit(smem_u32(&acc_bar[2]));
         __syncwarp();
