@@ -661,6 +661,25 @@ static SplitPlan pick_split(int64_t M, int64_t N, int64_t K, bool ones, int max_
     return best;
 }
 
+// A data product with few tiles and a long reduction (a short batch through a wide layer) is the latency of one tile's
+// k-blocks: about 0.13 us each for the narrow tiles such products run on, after some 3.3 us of launch, first loads and
+// epilogue.  Split over the blocks of a cluster it is a share of them and some 2.5 us more for the exchange.
+static bool split_data_product(const GemmArgs& g, SplitPlan* out) {
+    const int64_t mt = (g.M + BM - 1) / BM, kb = (g.K + BK - 1) / BK;
+    double best = 3.3 + 0.13 * (double)kb;
+    bool found = false;
+    for (int bn : {64, 128}) {
+        const int64_t tiles = mt * ((g.N + bn - 1) / bn);
+        for (int S = kMaxClusterSplits; S >= 2; S /= 2) {
+            if (tiles > max_active_clusters(S) || S > kb) continue;
+            const double t = 5.8 + 0.13 * (double)((kb + S - 1) / S) + 0.004 * bn;
+            if (t < 0.95 * best) { best = t; *out = SplitPlan{bn, S, 1}; found = true; }
+            break;
+        }
+    }
+    return found;
+}
+
 int tc_pick_splits(int64_t M, int64_t N, int64_t K) { return pick_split(M, N, K, false).global; }
 
 // fp32 partial tiles [splits][M][ldp], then (for the optional column sums) [splits][M]; nothing for a cluster split
@@ -680,9 +699,12 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     if (!tc_gemm_eligible(g)) return LRD_ERR_UNSUPPORTED;
     const bool ones = g.a_colsum != nullptr;
     if (ones && !(g.a_mn_major && g.b_mn_major)) return LRD_ERR_UNSUPPORTED;
-    if (!allow_split && !ones) return tc_gemm_persistent(g, stream);   // data products: the persistent kernel
     int splits = 1, cluster = 1, bn;
-    if (allow_split) {
+    SplitPlan dp;
+    if (!allow_split && !ones) {                           // data products: the persistent kernel, or a split of the reduction
+        if (!split_data_product(g, &dp)) return tc_gemm_persistent(g, stream);
+        bn = dp.bn; cluster = dp.cluster;
+    } else if (allow_split) {
         const SplitPlan sp = pick_split(g.M, g.N, g.K, ones, g.max_cluster_split);
         bn = sp.bn; cluster = sp.cluster; splits = sp.global;
     } else {
