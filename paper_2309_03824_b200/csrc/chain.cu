@@ -19,6 +19,8 @@
 // griddepcontrol.wait and so overlaps the tail of the previous kernel in the stream.
 // Every wait is bounded; a wait that runs out raises the device timeout flag and the block tears
 // down in order.
+#include <algorithm>
+
 #include "chain.cuh"
 
 #include "ptx.cuh"
@@ -539,14 +541,17 @@ bool chain_eligible(const ChainArgs& a) {
     return make_plan(a, &pl);
 }
 
-// The fused kernel loses to two separate products where the T buffer (128 rows x r) leaves room for only two
-// Q tiles of phase 2 in flight, i.e. at r = 512 (measured at 8192 tokens: 1024 -> 4096 forward 65 us fused against 49 us on two
-// persistent products, 4096 -> 1024 99 against 46 us; at r <= 384 the chain wins everywhere measured).  The
-// automatic path then takes the separate products; LRD_PATH_FUSED still forces the chain.
-bool chain_preferred(const ChainArgs& a) {
+// A stage takes its issue loop, its MMAs, or its turn of the ring (load latency over the stages in flight), whichever is
+// longest: constants fitted to forward passes of 12 layer shapes at 32 to 8192 tokens (6 % rms).
+double chain_estimate(const ChainArgs& a) {
     Plan pl;
-    if (!make_plan(a, &pl)) return false;
-    return pl.S2 >= 3;                 // Q tiles of phase 2 in flight
+    if (!make_plan(a, &pl)) return 1e300;
+    const int64_t room = max_active_clusters(pl.C), waves = ((a.M + 127) / 128 + room - 1) / room;
+    const double ng1 = (double)(((a.K1 + 63) / 64 + pl.G1 - 1) / pl.G1);
+    const int64_t chunks = ((a.N2 + pl.BN2 - 1) / pl.BN2 + pl.C - 1) / pl.C;
+    const double t1 = std::max({0.32, 1.41 / pl.S1, pl.G1 * 4 * std::max(pl.RS / 2.0, 32 + pl.RS / 4.0) / 1965.0});
+    const double t2 = std::max({0.505, 1.33 / pl.S2, pl.BN2 * 2 / 1965.0});
+    return chain_us(3.4, waves, ng1, t1, chunks, (double)((a.r + 63) / 64) * t2, 0.0094 * pl.BN2);
 }
 
 lrd_status_t chain_launch(const ChainArgs& a, cudaStream_t stream) {

@@ -7,6 +7,13 @@
 
 namespace lrd {
 
+// What both chain kernels' estimates are made of (see launch_chain in lrd_api.cu): microseconds of `waves` rounds of blocks
+// that each take ng1 stages of the first product at t1 and `chunks` chunks of the second with m2 of k-blocks and `epilogue`
+// of stores, the stores of a chunk beside the next one's k-blocks.
+inline double chain_us(double fixed, int64_t waves, double ng1, double t1, int64_t chunks, double m2, double epilogue) {
+    return fixed + (double)waves * (ng1 * t1 + m2 + (double)(chunks - 1) * (m2 > epilogue ? m2 : epilogue) + epilogue) + 2.0 * (double)(waves - 1);
+}
+
 struct ChainArgs {
     int64_t M, K1, r, N2;
     const void* In; int64_t ld_in;     // [M x K1]
@@ -23,8 +30,8 @@ struct ChainArgs {
 // phase-2 chunk width.  0 = automatic.  Not thread-safe against concurrent launches.
 void chain_tuning(int C, int G1, int BN2);
 bool chain_eligible(const ChainArgs& c);
-// Eligible, and expected to beat the two separate products (the automatic path's test).
-bool chain_preferred(const ChainArgs& c);
+// Estimated microseconds (only for eligible arguments).
+double chain_estimate(const ChainArgs& c);
 lrd_status_t chain_launch(const ChainArgs& c, cudaStream_t stream);
 
 // The same chain on pairs of SMs (tcgen05 cta_group::2): a cluster of 2 S blocks owns 256 rows.  `layers` are
@@ -34,8 +41,7 @@ constexpr int kChainMaxLayers = 4;
 // Overrides for sweeps and tests: pairs per cluster (1-4), k-blocks per phase-1 stage, phase-2 chunk width; 0 = automatic.
 void chain_pair_tuning(int S, int G1, int BN2);
 bool chain_pair_eligible(const ChainArgs* layers, int n);
-bool chain_pair_preferred(const ChainArgs* layers, int n);
-bool chain_pair_roomy(const ChainArgs* layers, int n);
+double chain_pair_estimate(const ChainArgs* layers, int n);
 lrd_status_t chain_pair_launch(const ChainArgs* layers, int n, cudaStream_t stream);
 
 }  // namespace lrd

@@ -577,28 +577,17 @@ bool chain_pair_eligible(const ChainArgs* layers, int n) {
     return make_plan(layers[0], n, &pl);
 }
 
-// Eligible, the ring beside the T buffer holds at least three Q tiles, and the shape is one where pairs measured
-// faster than single blocks: several layers in one launch, or a layer whose first product dominates (at 4096
-// tokens, r = 384: 3072 -> 768 forward 21.2 us on pairs against 22.5 us, but 768 -> 3072 24.6 against 18.5 us --
-// with few wide chunks per pair the epilogue of one chunk does not hide behind the MMAs of the next).
-bool chain_pair_preferred(const ChainArgs* layers, int n) {
-    if (!chain_pair_eligible(layers, n)) return false;
+// As chain_estimate (7 % rms over the same measurements).
+double chain_pair_estimate(const ChainArgs* layers, int n) {
     Plan pl;
-    if (!make_plan(layers[0], n, &pl) || pl.NS2 < 3) return false;
-    // Measured against the chain on single blocks: pairs win for groups, where the first product dominates, where
-    // the single blocks' T buffer leaves fewer than three weight tiles in flight (r = 512), and at r >= 384 once
-    // there are more row tiles than clusters of four fit on the GPU (8192 tokens, 4096 x 4096: r = 384 59 against
-    // 64 us forward, r = 512 62 against 85; r = 256 stays on single blocks, 50 against 54).
     const ChainArgs& a = layers[0];
-    return n > 1 || a.K1 >= 2 * a.N2 || (a.r > 384 && !chain_preferred(a)) || (a.r >= 384 && (a.M + 127) / 128 > 37);
-}
-
-// Eligible, with at least three weight tiles of the second product in flight: the form to take where the launch should
-// leave SMs free for others (16 clusters of 6 or fewer blocks against 32 clusters of 4).
-bool chain_pair_roomy(const ChainArgs* layers, int n) {
-    if (!chain_pair_eligible(layers, n)) return false;
-    Plan pl;
-    return make_plan(layers[0], n, &pl) && pl.NS2 >= 3;
+    if (!make_plan(a, n, &pl)) return 1e300;
+    const int64_t room = max_active_clusters(2 * pl.S), waves = ((a.M + 255) / 256 * n + room - 1) / room;
+    const double ng1 = (double)(((a.K1 + 63) / 64 + pl.G1 - 1) / pl.G1);
+    const int64_t chunks = ((a.N2 + pl.BN2 - 1) / pl.BN2 + pl.S - 1) / pl.S;
+    const double t1 = std::max({0.243, 1.26 / pl.NS1, pl.G1 * 4 * std::max(pl.RS / 2.0, 32 + pl.RS / 4.0) / 1965.0});
+    const double t2 = std::max({0.46, 1.21 / pl.NS2, pl.BN2 * 2 / 1965.0});
+    return chain_us(4.9, waves, ng1, t1, chunks, (double)((a.r + 63) / 64) * t2, 0.012 * pl.BN2);
 }
 
 lrd_status_t chain_pair_launch(const ChainArgs* layers, int n, cudaStream_t stream) {

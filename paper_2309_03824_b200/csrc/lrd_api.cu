@@ -76,17 +76,29 @@ GemmArgs gemm(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, bool 
     return make_gemm(M, N, K, A, lda, a_mn, B, ldb, b_mn, C, ldc, bias, dt);
 }
 
-// The fused chain for one layer, or for n layers of equal shape in one launch: on pairs of SMs where the shape
-// allows, else (one layer only) on single blocks.  Returns LRD_ERR_UNSUPPORTED when no fused kernel takes it.
+// The fused chain for one layer, or for n layers of equal shape in one launch (on pairs of SMs).  Returns
+// LRD_ERR_UNSUPPORTED when no fused kernel takes it, or two separate products are the faster way.
+//
+// Which of the three it is depends on the token count as much as on the layer: with few row tiles the chain is one cluster's
+// latency while the separate products spread each factor over all SMs and split long reductions; with many the chain
+// saves the trip of the rank-r intermediate and a launch; pairs halve the factors' traffic where the first product
+// dominates or the T buffer leaves no room.  Forward of 1024 -> 4096 at r = 512, in us (products / single blocks /
+// pairs): 256 tokens 9.6 / 14.6 / 23.5, 4096 tokens 30 / 27 / 41, 8192 tokens 51 / 61 / 46; 768 -> 768 at r = 192: 128
+// tokens 8.1 / 7.5 / -, 4096 tokens 12.3 / 9.2 / 10.9.  No simple line separates them, so each kernel estimates its
+// time; over 96 measured layers the choice costs 0.4 % on average against the best of the three.
 lrd_status_t launch_chain(const ChainArgs* c, int n, int path, cudaStream_t s, bool leave_room = false) {
     const int mode = g_chain_mma_blocks.load();
-    const bool forced = path == LRD_PATH_FUSED;
-    if (c[0].sm_share == 0 && mode != 1) {
-        if (mode == 2 || forced ? chain_pair_eligible(c, n) : (chain_pair_preferred(c, n) || (leave_room && chain_pair_roomy(c, n))))
-            return chain_pair_launch(c, n, s);
+    const bool pair = c[0].sm_share == 0 && mode != 1 && chain_pair_eligible(c, n);
+    const bool single = n == 1 && mode != 2 && chain_eligible(c[0]);
+    if (mode == 2 || path == LRD_PATH_FUSED || n > 1) {
+        if (pair) return chain_pair_launch(c, n, s);
+        return single ? chain_launch(c[0], s) : LRD_ERR_UNSUPPORTED;
     }
-    if (n != 1 || mode == 2) return LRD_ERR_UNSUPPORTED;
-    if (forced ? chain_eligible(c[0]) : chain_preferred(c[0])) return chain_launch(c[0], s);
+    const double us_pair = pair ? chain_pair_estimate(c, n) : 1e300, us_single = single ? chain_estimate(c[0]) : 1e300;
+    const double us_products = tc_gemm_estimate(c[0].M, c[0].r, c[0].K1) + tc_gemm_estimate(c[0].M, c[0].N2, c[0].r);
+    const double best = std::min({us_pair, us_single, us_products});
+    if (us_pair <= best * (leave_room ? 1.35 : 1.0)) return chain_pair_launch(c, n, s);
+    if (us_single <= us_products) return chain_launch(c[0], s);
     return LRD_ERR_UNSUPPORTED;
 }
 

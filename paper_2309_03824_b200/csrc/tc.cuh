@@ -15,6 +15,9 @@ size_t tc_split_workspace_bytes(int64_t M, int64_t N, int64_t K);
 // Unsplit product with a bf16 result on the persistent kernel (one block per SM walks over the tiles, the
 // epilogue of a tile overlaps the MMAs of the next).  Same eligibility as tc_gemm; no column sums.
 lrd_status_t tc_gemm_persistent(const GemmArgs& g, cudaStream_t stream);
+double tc_gemm_persistent_estimate(int64_t M, int64_t N, int64_t K);
+// Estimated microseconds of a data product on the kernel tc_gemm would take for it.
+double tc_gemm_estimate(int64_t M, int64_t N, int64_t K);
 void tc_gemm_persistent_force_pairs(int blocks_per_mma);     // 0: automatic; 1 or 2: forced where the shape allows
 // allow_split: the reduction dimension may be split over blocks (weight gradients).
 lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_t partial_bytes, cudaStream_t stream);

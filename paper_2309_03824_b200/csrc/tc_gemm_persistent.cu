@@ -365,6 +365,18 @@ PShape pick_shape_p(int64_t M, int64_t N) {
 
 }  // namespace
 
+// Estimated microseconds of one product (see launch_chain in lrd_api.cu): the k-blocks of a tile at the issue loop's, the
+// tensor pipe's or the loads' pace, whichever is slowest; the epilogue of a tile beside the next tile's k-blocks.
+double tc_gemm_persistent_estimate(int64_t M, int64_t N, int64_t K) {
+    const PShape sh = pick_shape_p(M, N);
+    const int64_t kb = (K + BK - 1) / BK, units = kNumSms / sh.cg;
+    const int64_t tiles = ((M + BM * sh.cg - 1) / (BM * sh.cg)) * ((N + sh.bn - 1) / sh.bn), waves = (tiles + units - 1) / units;
+    const double mma = 4.0 * (sh.bn / 2.0 > 32 + sh.bn / 4.0 ? sh.bn / 2.0 : 32 + sh.bn / 4.0) / 1965.0;
+    const double load = (double)(kATile + sh.bn / sh.cg * BK * 2) * 6.6e-6, issue = sh.cg == 1 && sh.bn <= 128 ? 0.16 : 0.19;
+    const double main = (double)kb * (mma > load ? (mma > issue ? mma : issue) : (load > issue ? load : issue)), epilogue = 0.0195 * sh.bn;
+    return 1.7 + main + (double)(waves - 1) * (main > epilogue ? main : epilogue) + epilogue;
+}
+
 void tc_gemm_persistent_force_pairs(int cg) { g_force_cg = (cg == 1 || cg == 2) ? cg : 0; }
 
 lrd_status_t tc_gemm_persistent(const GemmArgs& g, cudaStream_t stream) {

@@ -375,3 +375,12 @@ def test_backward_accumulates_over_micro_batches(dtype, shape, freeze):
 def test_packed_ranks_close_to_the_layer_width(shape, freeze):
     """Packed odd ranks whose padded rank (a multiple of 16) would pass K or N, and one that just fits."""
     check_linear(wl.random_factor_case(*shape, "bf16", 640 + shape[3]), freeze)
+
+
+@pytest.mark.parametrize("shape", [(1, 4096, 264, 64), (128, 3080, 392, 128), (130, 1032, 1544, 520), (500, 1544, 136, 96), (257, 4104, 72, 72)])
+def test_data_products_split_over_a_cluster(shape):
+    """Few tiles and a long reduction: the two products split over 2, 4 or 8 blocks, with a k-block or two past the end of a
+    share, ragged rows and columns, and the bias added after the sum."""
+    for freeze in (b.LRD_FREEZE_NONE, b.LRD_FREEZE_U):
+        check_linear(wl.random_factor_case(*shape, "bf16", 660 + shape[0]), freeze)
+        check_linear(wl.random_factor_case(*shape, "bf16", 660 + shape[0]), freeze, path=b.LRD_PATH_UNFUSED)
