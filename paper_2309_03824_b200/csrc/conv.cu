@@ -122,15 +122,13 @@ lrd_status_t tucker2_fwd(const lrd_tucker2_desc_t* d, const void* X, const void*
         const size_t inner = tucker2_workspace_bytes(&q, freeze, 0);
         const Repack o = repack_layout(t, inner);
         uint8_t* w = (uint8_t*)ws;
-        LRD_TRY(copy2d_bf16(w + o.A, q.r1, A, t.r1, t.C, t.r1, q.r1, s));
-        LRD_TRY(copy2d_bf16(w + o.G, q.r1, G, t.r1, t.r2 * t.taps, t.r1, q.r1, s));
-        LRD_TRY(zero_fill(w + o.G + (size_t)t.r2 * t.taps * q.r1 * 2, (q.r2 - t.r2) * t.taps, q.r1, q.r1, LRD_BF16, s));
-        LRD_TRY(copy2d_bf16(w + o.Bm, q.r2, Bm, t.r2, t.S, t.r2, q.r2, s));
+        const int r1 = (int)t.r1, r2 = (int)t.r2, p1 = (int)q.r1, p2 = (int)q.r2;
+        const Copy2d in[3] = {{w + o.A, p1, A, r1, t.C, t.C, r1, p1}, {w + o.G, p1, G, r1, r2 * t.taps, p2 * t.taps, r1, p1}, {w + o.Bm, p2, Bm, r2, t.S, t.S, r2, p2}};
+        LRD_TRY(copy2d_bf16(in, 3, s));
         LRD_TRY(tucker2_fwd(&q, X, w + o.A, w + o.G, w + o.Bm, bias, Y, Z1_save ? w + o.Z1 : nullptr, Z2_save ? w + o.Z2 : nullptr, freeze,
                             w, inner, path, s));
-        if (Z1_save) LRD_TRY(copy2d_bf16(Z1_save, t.r1, w + o.Z1, q.r1, t.P, q.r1, t.r1, s));
-        if (Z2_save) LRD_TRY(copy2d_bf16(Z2_save, t.r2, w + o.Z2, q.r2, t.Po, q.r2, t.r2, s));
-        return LRD_OK;
+        const Copy2d out[2] = {{Z1_save, r1, w + o.Z1, p1, t.P, Z1_save ? t.P : 0, r1, r1}, {Z2_save, r2, w + o.Z2, p2, t.Po, Z2_save ? t.Po : 0, r2, r2}};
+        return copy2d_bf16(out, 2, s);
     }
     // the whole forward in one launch where the shape allows: Z1 and Z2 stay on chip unless the caller saves them
     if (t.plain && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) && (!bias || ((uintptr_t)bias % 2) == 0) &&
@@ -166,22 +164,17 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
         const size_t inner = tucker2_workspace_bytes(&q, freeze, 1);
         const Repack o = repack_layout(t, inner);
         uint8_t* w = (uint8_t*)ws;
-        LRD_TRY(copy2d_bf16(w + o.A, q.r1, A, t.r1, t.C, t.r1, q.r1, s));
-        LRD_TRY(copy2d_bf16(w + o.G, q.r1, G, t.r1, t.r2 * t.taps, t.r1, q.r1, s));
-        LRD_TRY(zero_fill(w + o.G + (size_t)t.r2 * t.taps * q.r1 * 2, (q.r2 - t.r2) * t.taps, q.r1, q.r1, LRD_BF16, s));
-        LRD_TRY(copy2d_bf16(w + o.Bm, q.r2, Bm, t.r2, t.S, t.r2, q.r2, s));
-        if (core) LRD_TRY(copy2d_bf16(w + o.Z1, q.r1, Z1_save, t.r1, t.P, t.r1, q.r1, s));
-        if (factors) LRD_TRY(copy2d_bf16(w + o.Z2, q.r2, Z2_save, t.r2, t.Po, t.r2, q.r2, s));
+        const int r1 = (int)t.r1, r2 = (int)t.r2, p1 = (int)q.r1, p2 = (int)q.r2;
+        const Copy2d in[5] = {{w + o.A, p1, A, r1, t.C, t.C, r1, p1}, {w + o.G, p1, G, r1, r2 * t.taps, p2 * t.taps, r1, p1}, {w + o.Bm, p2, Bm, r2, t.S, t.S, r2, p2},
+                              {w + o.Z1, p1, Z1_save, r1, t.P, core ? t.P : 0, r1, p1}, {w + o.Z2, p2, Z2_save, r2, t.Po, factors ? t.Po : 0, r2, p2}};
+        LRD_TRY(copy2d_bf16(in, 5, s));
         // the frozen group's buffers were zero-filled above; the padded call gets none for them
         LRD_TRY(tucker2_bwd(&q, dY, X, w + o.A, w + o.G, w + o.Bm, core ? w + o.Z1 : nullptr, factors ? w + o.Z2 : nullptr, dX,
                             factors ? w + o.dA : nullptr, core ? w + o.dG : nullptr, factors ? w + o.dB : nullptr, factors ? dbias : nullptr,
                             freeze, w, inner, path, s));
-        if (factors) {
-            LRD_TRY(copy2d_bf16(dA, t.r1, w + o.dA, q.r1, t.C, q.r1, t.r1, s));
-            LRD_TRY(copy2d_bf16(dB, t.r2, w + o.dB, q.r2, t.S, q.r2, t.r2, s));
-        }
-        if (core) LRD_TRY(copy2d_bf16(dG, t.r1, w + o.dG, q.r1, t.r2 * t.taps, q.r1, t.r1, s));
-        return LRD_OK;
+        const Copy2d out[3] = {{dA, r1, w + o.dA, p1, t.C, factors ? t.C : 0, r1, r1}, {dB, r2, w + o.dB, p2, t.S, factors ? t.S : 0, r2, r2},
+                               {dG, r1, w + o.dG, p1, r2 * t.taps, core ? r2 * t.taps : 0, r1, r1}};
+        return copy2d_bf16(out, 3, s);
     }
 
     void* dZ1 = ws;

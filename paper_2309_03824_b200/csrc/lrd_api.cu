@@ -12,6 +12,7 @@
 #include "chain.cuh"
 #include "common.cuh"
 #include "conv.cuh"
+#include "ptx.cuh"
 #include "streams.cuh"
 #include "tc.cuh"
 
@@ -217,27 +218,64 @@ __global__ void add_into_kernel(T* __restrict__ dst, const T* __restrict__ src, 
 }  // namespace
 
 namespace {
-// dst[row][0 .. cols_dst) = src[row][0 .. min(cols_src, cols_dst)) followed by zeros, 2-byte elements, any
-// leading dimensions: the copy between a packed factor (rows that start at odd multiples of 2 bytes) and its copy
-// with rows padded to whole 16-byte groups.
-__global__ void copy2d_bf16_kernel(__nv_bfloat16* __restrict__ dst, int64_t ldd, const __nv_bfloat16* __restrict__ src, int64_t lds,
-                                   int64_t rows, int64_t cols_src, int64_t cols_dst) {
-    const int64_t n = rows * cols_dst;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / cols_dst, c = i % cols_dst;
-        dst[r * ldd + c] = c < cols_src ? src[r * lds + c] : __float2bfloat16_rn(0.f);
+// The copies between packed factors or activations (rows that start at odd multiples of 2 bytes) and their copies with rows
+// padded to whole 16-byte groups: a layer needs up to five of them at once, each a few microseconds of launch and
+// latency around a megabyte or two, so they share one launch.  A warp takes 128 columns of a row at a time, four
+// elements per lane in flight, consecutive lanes on consecutive elements: neither side needs any alignment.
+struct CopyBatch {
+    Copy2d job[kMaxCopies];
+    int64_t unit0[kMaxCopies + 1];       // first (row, 128-column piece) of each job
+    int n;
+};
+__global__ void __launch_bounds__(256) copy2d_bf16_kernel(const __grid_constant__ CopyBatch b) {
+    ptx::griddep_launch_dependents();
+    ptx::griddep_wait();
+    const int lane = threadIdx.x % 32;
+    const int64_t warps = (int64_t)gridDim.x * 8;
+    int j = 0;
+    for (int64_t u = (int64_t)blockIdx.x * 8 + threadIdx.x / 32; u < b.unit0[b.n]; u += warps) {
+        while (u >= b.unit0[j + 1]) ++j;
+        const Copy2d& c = b.job[j];
+        const uint32_t pieces = ((uint32_t)c.cols_dst + 127u) / 128u;
+        const int64_t local = u - b.unit0[j], row = local >> 32 ? local / pieces : (uint32_t)local / pieces;
+        const int col0 = (int)(local - row * pieces) * 128 + lane;
+        const uint16_t* src = (const uint16_t*)c.src + row * c.lds;
+        uint16_t* dst = (uint16_t*)c.dst + row * c.ldd;
+        const int cols = row < c.rows_src ? c.cols_src : 0;
+        uint16_t v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = col0 + 32 * e < cols ? src[col0 + 32 * e] : (uint16_t)0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (col0 + 32 * e < c.cols_dst) dst[col0 + 32 * e] = v[e];
     }
 }
 }  // namespace
 
-lrd_status_t copy2d_bf16(void* dst, int64_t ldd, const void* src, int64_t lds, int64_t rows, int64_t cols_src, int64_t cols_dst,
-                         cudaStream_t s) {
-    if (rows <= 0 || cols_dst <= 0) return LRD_OK;
-    const int64_t n = rows * cols_dst;
-    const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, 148 * 16);
-    copy2d_bf16_kernel<<<blocks, 256, 0, s>>>((__nv_bfloat16*)dst, ldd, (const __nv_bfloat16*)src, lds, rows, cols_src, cols_dst);
+lrd_status_t copy2d_bf16(const Copy2d* c, int n, cudaStream_t s) {
+    CopyBatch b;
+    b.n = 0;
+    b.unit0[0] = 0;
+    for (int i = 0; i < n; ++i) {
+        if (c[i].rows_dst <= 0 || c[i].cols_dst <= 0) continue;
+        if (b.n == kMaxCopies) return LRD_ERR_UNSUPPORTED;
+        b.job[b.n] = c[i];
+        b.unit0[b.n + 1] = b.unit0[b.n] + c[i].rows_dst * ((c[i].cols_dst + 127) / 128);
+        ++b.n;
+    }
+    if (b.n == 0) return LRD_OK;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>((b.unit0[b.n] + 7) / 8, kNumSms * 16), 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) before it touches global memory
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (!cuda_ok(cudaLaunchKernelEx(&cfg, copy2d_bf16_kernel, b), "cudaLaunchKernelEx(repack)")) return LRD_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
+    return LRD_OK;
 }
 
 lrd_status_t add_into(void* dst, const void* src, int64_t rows, int64_t cols, int64_t ld, lrd_dtype_t dt, cudaStream_t s) {
@@ -475,11 +513,12 @@ static lrd_status_t linear_fwd_on(const lrd_linear_desc_t* desc, const void* X, 
         const size_t inner = lrd_linear_workspace_bytes(&q, freeze, 0);
         const RepackLayout o = repack_layout(L, inner);
         uint8_t* w = (uint8_t*)workspace;
-        LRD_TRY(copy2d_bf16(w + o.Vp, q.r, V, L.ldv, L.K, L.r, q.r, s));
-        LRD_TRY(copy2d_bf16(w + o.Up, q.r, U, L.ldu, L.N, L.r, q.r, s));
+        const int r = (int)L.r, rp = (int)q.r;
+        const Copy2d in[2] = {{w + o.Vp, rp, V, L.ldv, L.K, L.K, r, rp}, {w + o.Up, rp, U, L.ldu, L.N, L.N, r, rp}};
+        LRD_TRY(copy2d_bf16(in, 2, s));
         LRD_TRY(linear_fwd_on(&q, X, w + o.Vp, w + o.Up, bias, Y, Z_save ? w + o.Zp : nullptr, freeze, w, inner, s, sm_share));
-        if (Z_save) LRD_TRY(copy2d_bf16(Z_save, L.ldz, w + o.Zp, q.r, L.M, L.r, L.r, s));
-        return LRD_OK;
+        const Copy2d out = {Z_save, L.ldz, w + o.Zp, rp, L.M, L.M, r, r};
+        return Z_save ? copy2d_bf16(&out, 1, s) : LRD_OK;
     }
 
     const int path = g_path.load();
@@ -550,17 +589,15 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
         const RepackLayout o = repack_layout(L, inner);
         uint8_t* w = (uint8_t*)workspace;
         const bool du = do_w && (plan & LRD_PLAN_DU) != 0, dv = do_w && (plan & LRD_PLAN_DV) != 0;
-        if (do_data) {
-            LRD_TRY(copy2d_bf16(w + o.Vp, q.r, V, L.ldv, L.K, L.r, q.r, s));
-            LRD_TRY(copy2d_bf16(w + o.Up, q.r, U, L.ldu, L.N, L.r, q.r, s));
-        }
-        if (du) LRD_TRY(copy2d_bf16(w + o.Zp, q.r, Z_save, L.ldz, L.M, L.r, q.r, s));
+        const int r = (int)L.r, rp = (int)q.r;
+        const Copy2d in[3] = {{w + o.Vp, rp, V, L.ldv, L.K, do_data ? L.K : 0, r, rp}, {w + o.Up, rp, U, L.ldu, L.N, do_data ? L.N : 0, r, rp},
+                              {w + o.Zp, rp, Z_save, L.ldz, L.M, du ? L.M : 0, r, rp}};
+        LRD_TRY(copy2d_bf16(in, 3, s));
         // the frozen factor's buffers were zero-filled above; the padded call gets none for them
         LRD_TRY(linear_bwd_on(&q, dY, X, w + o.Vp, w + o.Up, w + o.Zp, dX, w + o.dUp, w + o.dVp, du ? dbias : nullptr, freeze, w, inner, s,
                               nullptr, nullptr, sm_share, false, parts));
-        if (du) LRD_TRY(copy2d_bf16(dU, L.ldu, w + o.dUp, q.r, L.N, L.r, L.r, s));
-        if (dv) LRD_TRY(copy2d_bf16(dV, L.ldv, w + o.dVp, q.r, L.K, L.r, L.r, s));
-        return LRD_OK;
+        const Copy2d out[2] = {{dU, L.ldu, w + o.dUp, rp, L.N, du ? L.N : 0, r, r}, {dV, L.ldv, w + o.dVp, rp, L.K, dv ? L.K : 0, r, r}};
+        return copy2d_bf16(out, 2, s);
     }
 
     void* dZ = workspace;
