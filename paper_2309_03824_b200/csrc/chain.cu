@@ -4,15 +4,15 @@
 //   Phase 1  block c forms its r/C-column slice of T = In P in tensor memory (TMA-fed tcgen05.mma:
 //            In K-major, the slice of P MN-major), one or two 64-deep k-blocks per stage, as many
 //            stages as the shared memory beside the T buffer holds.
-//   Gather   four warps read the slice (tcgen05.ld), round it to bf16 and write it into this block's T
+//   Gather   eight warps read the slice (tcgen05.ld), round it to bf16 and write it into this block's T
 //            buffer (K-major, swizzled, slices are whole atoms = one contiguous range); one thread then
 //            copies the range into every peer's T buffer with bulk DSMEM copies that complete on the
 //            peer's barrier.  T never goes to global memory unless T_save asks.
 //   Phase 2  block c forms every C-th column chunk of Out = T Q^T (T from shared memory, Q by TMA, one
 //            64-deep tile per stage), double-buffered in tensor memory; each epilogue warp adds the
-//            bias (staged in shared memory while the MMAs run), rounds to bf16 and stores its 32 rows
+//            bias (fetched a chunk ahead), rounds to bf16 and stores its 32 rows
 //            through its own [32 x 32] slabs by TMA stores (which clip the ragged edges).
-// Warp 0: TMA producer.  Warp 1: tensor memory + MMA issue.  Warps 2-5: gather and epilogue.
+// Warp 0: TMA producer.  Warp 1: tensor memory + MMA issue.  Warps 2-9: gather and epilogue.
 // Two cluster barriers: the first (every block's barriers exist) is arrived at once and waited on only
 // where the first remote copy is near; the second (every block has received all slices sent to it) lets
 // no block leave while a peer may still be reading its shared memory.  The kernel's set-up runs before
@@ -32,18 +32,20 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 192;
+constexpr int kThreads = 320;             // TMA producer, MMA issuer, 8 x gather / epilogue
+constexpr int kEpiThreads = 256;
 constexpr int kMaxStages = 12;
 constexpr int kMaxCluster = 16;      // blocks per row tile (more than 8: a non-portable cluster size, allowed per function)
 constexpr int kMaxKb2 = 8;           // 64-column k-blocks of T (r <= 512)
 constexpr uint32_t kSmemLimit = 224 * 1024;         // dynamic shared memory; the rest is left for the barriers and the bias
 constexpr uint32_t kInTileBytes = 128 * 64 * 2;     // In tile of one k-block: 128 rows x 64 k
 constexpr uint32_t kSlabBytes = 32 * 32 * 2;        // epilogue slab of one warp: 32 rows x 32 columns of bf16
-constexpr uint32_t kStagingBytes = 4 * 2 * kSlabBytes;
+constexpr uint32_t kSlabsBytes = 8 * kSlabBytes;    // one slab for every epilogue warp; there are one or two sets
 
 struct ChainParams {
     int C, RS, swb, BN2, n_chunks, kb1, ks2, kb2, N2;
     int G1, S1, S2;           // k-blocks per phase-1 stage; stage counts of the two phases
+    int slabs;                // sets of epilogue slabs (1 or 2)
     uint32_t stage1_bytes, stage2_bytes, t_bytes;
     int taw;                  // columns per atom of the T buffer (64, 32 or 16; swizzle span = 2 * taw bytes)
     int t_steps_lg;           // log2 of the MMA k-steps (16 columns) per atom
@@ -62,7 +64,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full1[kMaxStages], empty1[kMaxStages], full2[kMaxStages], empty2[kMaxStages],
         tacc_bar, tready_bar[kMaxCluster], out_full[2], out_empty[2];
-    __shared__ __align__(16) float bias_s[2][256];
+    __shared__ __align__(16) uint16_t bias_s[2][256];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -74,7 +76,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
     const uint32_t t_base = smem_base;
     const uint32_t ring1_base = smem_base;
     const uint32_t staging_base = t_base + p.t_bytes;
-    const uint32_t ring2_base = staging_base + kStagingBytes;
+    const uint32_t ring2_base = staging_base + (uint32_t)p.slabs * kSlabsBytes;
     const AbortCtx ab{&abort_flag, p.timeout_flag};
     const uint32_t t_sw = 2u * (uint32_t)p.taw, t_atom_bytes = 128u * t_sw;   // T: atoms of [128 rows x taw columns]
     // The warp index is made provably warp-uniform, and the single-thread instructions (TMA, MMA, commit)
@@ -106,7 +108,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
         mbar_init(smem_u32(&tacc_bar), 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&out_full[i]), 1);
-            mbar_init(smem_u32(&out_empty[i]), 4);
+            mbar_init(smem_u32(&out_empty[i]), 8);
         }
         fence_mbar_init();
     }
@@ -276,8 +278,8 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
     } else {
         // ------------------------------------------------------------------ gather + epilogue
         const int q = warp % 4;                              // tensor-memory lanes [32 q, 32 q + 32)
+        const int hw = (warp - 2) / 4;                       // two warps share a quarter: they take alternate 32-column pieces
         const int row = q * 32 + lane;                       // row of the 128-row tile
-        const int et = (warp - 2) * 32 + lane;               // index among the 128 epilogue threads
         const bool lead_warp = (warp == 2);                  // issues this block's bulk copies and stores (elect.sync)
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
         bool ok = mbar_wait_uniform(smem_u32(&tacc_bar), 0, ab);   // warp-uniform from here on
@@ -285,7 +287,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
         cluster_arrive_relaxed();   // barrier 1: this block's phase-1 ring is dead (progress only, no data)
         if (ok) {
             // 32 columns per step (two tensor-memory loads in flight, one wait), a 16-column tail if RS / 16 is odd
-            for (int col = 0; col < p.RS; col += 32) {
+            for (int col = 32 * hw; col < p.RS; col += 64) {
                 uint32_t v[32];
                 const bool two = col + 32 <= p.RS;
                 tmem_ld_32x16(lane_addr + col, *reinterpret_cast<uint32_t(*)[16]>(&v[0]));
@@ -308,13 +310,13 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
             }
         }
         // The slice [c RS, (c+1) RS) is whole atoms, i.e. one contiguous range of this block's T buffer: after
-        // the four warps have written it, one thread copies it into every peer's buffer (bulk DSMEM copy that
+        // the warps have written it, one thread copies it into every peer's buffer (bulk DSMEM copy that
         // completes on the peer's barrier) and, if asked, stores it to T_save.  The accumulator columns of
         // the slice are free for phase 2 from here on.
         fence_proxy_async_smem();
         tc_fence_before();
         cluster_wait();        // barrier 1: the peers' barriers exist
-        ok = named_bar_and(2, 128, ok);    // the four warps go on, or give up, together
+        ok = named_bar_and(2, kEpiThreads, ok);    // the warps go on, or give up, together
         if (lead_warp) {
             if (ok && elect_one()) {
                 const uint32_t slice = t_base + (uint32_t)c * 256u * (uint32_t)p.RS;
@@ -331,54 +333,44 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
             }
             __syncwarp();
         }
-        // Epilogue: each warp on its own.  32 columns of its 32 rows at a time go through a [32 rows x 64 B]
-        // slab of the warp (64-byte swizzle, two slabs in rotation) and leave by one TMA store each.  The bias
-        // of a chunk is staged in shared memory while its MMAs run.
-        const uint32_t slab0 = staging_base + (uint32_t)(warp - 2) * 2u * kSlabBytes;
+        // Epilogue: each warp on its own.  32 columns of its 32 rows at a time go through a [32 rows x 64 B] slab of the warp
+        // (64-byte swizzle) and leave by one TMA store each; a piece is a chain of latencies (tensor memory, conversion, fence,
+        // the store's read of the slab), so eight warps share the chunk, and a chunk's bias is fetched while the chunk before it
+        // is stored.  8192 x 4096 output, r = 256: 48.7 us with four warps and the bias fetched at the chunk's own start, 44.5
+        // with eight and ahead; what is left of it is the write rate (67 MB at 5.4 TB/s, the rate of a memset: 12.4 us).
+        const uint32_t slab0 = staging_base + (uint32_t)(warp - 2) * kSlabBytes;
         const uint32_t row_off = (uint32_t)lane * 64u;
         const uint32_t row_xor = ((uint32_t)lane >> 1) & 3u;
         int i = 0, sb = 0;
         bool arrived2 = false;
+        uint16_t next_bias[4];
+        bias_fetch(next_bias, p.bias, (int64_t)c * p.BN2 + 32 * hw, p.N2);
         for (int j = c; j < p.n_chunks && ok; j += p.C, ++i) {
             const int buf = i & 1;
-            if (p.bias) {                                    // bias_s[buf] was last read two chunks ago, before a barrier
-                for (int e = et; e < p.BN2; e += 128) {
-                    const int col = j * p.BN2 + e;
-                    bias_s[buf][e] = col < p.N2 ? __bfloat162float(p.bias[col]) : 0.f;
-                }
-            }
             ok = mbar_wait_uniform(smem_u32(&out_full[buf]), (i >> 1) & 1, ab);
-            ok = named_bar_and(3, 128, ok);                  // the four warps go on, or give up, together (and see the bias)
             if (!ok) break;
+            if (p.bias) bias_put(&bias_s[buf][32 * hw], next_bias, p.BN2 / 64);
+            bias_fetch(next_bias, p.bias, (int64_t)(j + p.C) * p.BN2 + 32 * hw, p.N2);        // of the next chunk
             if (!arrived2) { cluster_arrive_relaxed(); arrived2 = true; }   // barrier 2 (T was complete before these MMAs)
             tc_fence_after();
             const uint32_t d_tmem = lane_addr + (uint32_t)buf * 256u;
-            for (int g = 0; g * 64 < p.BN2; ++g) {
-                const int col0 = j * p.BN2 + g * 64;
+            for (int c0 = hw; c0 * 32 < p.BN2; c0 += 4) {    // this warp's pieces, two at a time
+                const int col0 = j * p.BN2 + c0 * 32;
                 if (col0 >= p.N2) break;                     // (uniform) nothing of this piece is inside Out
-                uint32_t v[64];                              // both halves are loaded before the first is converted
-                tmem_ld_32x32(d_tmem + g * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-                tmem_ld_32x32(d_tmem + g * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+                const bool second = (c0 + 2) * 32 < p.BN2 && col0 + 64 < p.N2;
+                uint32_t v[64];                              // both pieces are loaded before the first is converted
+                tmem_ld_32x32(d_tmem + c0 * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                if (second) tmem_ld_32x32(d_tmem + c0 * 32 + 64, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
                 tmem_ld_wait();
 #pragma unroll
-                for (int h = 0; h < 2; ++h, ++sb) {
-                    if (col0 + 32 * h >= p.N2) break;        // (uniform)
-                    const uint32_t slab = slab0 + (uint32_t)(sb & 1) * kSlabBytes;
-                    if (sb >= 2) {                           // the store that last read this slab has finished reading
-                        tma_store_wait_read<1>();            // (only the lane that issued the stores has any to wait for)
-                        __syncwarp();
-                    }
-                    if (p.bias) {
-                        const float4* bp = reinterpret_cast<const float4*>(&bias_s[buf][g * 64 + h * 32]);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float4 b4 = bp[e];
-                            v[32 * h + 4 * e] = __float_as_uint(__uint_as_float(v[32 * h + 4 * e]) + b4.x);
-                            v[32 * h + 4 * e + 1] = __float_as_uint(__uint_as_float(v[32 * h + 4 * e + 1]) + b4.y);
-                            v[32 * h + 4 * e + 2] = __float_as_uint(__uint_as_float(v[32 * h + 4 * e + 2]) + b4.z);
-                            v[32 * h + 4 * e + 3] = __float_as_uint(__uint_as_float(v[32 * h + 4 * e + 3]) + b4.w);
-                        }
-                    }
+                for (int h = 0; h < 2; ++h) {
+                    if (h == 1 && !second) break;           // (uniform)
+                    const uint32_t slab = slab0 + (sb && p.slabs == 2 ? kSlabsBytes : 0u);
+                    sb ^= 1;
+                    if (p.slabs == 2) tma_store_wait_read<1>();      // the store that last read the slab has finished reading
+                    else tma_store_wait_read<0>();                   // (only the lane that issued the stores has any to wait for)
+                    __syncwarp();
+                    if (p.bias) bias_add(&v[32 * h], &bias_s[buf][32 * c0 + 64 * h]);
 #pragma unroll
                     for (int cc = 0; cc < 4; ++cc)
                         st_shared_v4(slab + row_off + ((((uint32_t)cc) ^ row_xor) << 4),
@@ -389,7 +381,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (elect_one()) {
-                        tma_store_2d(&tmOut, slab, col0 + 32 * h, m0 + q * 32);
+                        tma_store_2d(&tmOut, slab, col0 + 64 * h, m0 + q * 32);
                         tma_store_commit();
                     }
                     __syncwarp();
@@ -419,7 +411,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
 }
 
 struct Plan {
-    int C, RS, swb, BN2, G1, S1, S2;
+    int C, RS, swb, BN2, G1, S1, S2, slabs;
     uint32_t stage1_bytes, stage2_bytes, t_bytes, smem_bytes;
 };
 
@@ -495,8 +487,11 @@ bool make_plan(const ChainArgs& a, Plan* out) {
         const int swb = RS % 64 == 0 ? 128 : (RS % 32 == 0 ? 64 : 32);
         const int BN2 = pick_bn2(a.N2, C);
         const int64_t ring1 = (int64_t)kSmemLimit - 1024;                         // phase 1 has all of it
-        const int64_t ring2 = ring1 - t_bytes - (int64_t)kStagingBytes;
         const uint32_t kb1_bytes = kInTileBytes + 128u * RS, kb2_bytes = (uint32_t)BN2 * 128u;
+        // a second set of epilogue slabs where it does not cost the ring of Q tiles a slot that it needs
+        const int64_t room2 = ring1 - t_bytes;
+        const int slabs = (room2 - 2 * (int64_t)kSlabsBytes) / kb2_bytes >= std::min<int64_t>((room2 - (int64_t)kSlabsBytes) / kb2_bytes, 4) ? 2 : 1;
+        const int64_t ring2 = room2 - slabs * (int64_t)kSlabsBytes;
         if (ring2 < 2 * (int64_t)kb2_bytes) continue;
         // phase 1: two k-blocks per stage: what a stage costs the issuing threads beside its copies and MMAs (a wait,
         // an election, a commit: some 250 cycles) is then spread over eight MMAs of r / C columns, which by
@@ -510,9 +505,9 @@ bool make_plan(const ChainArgs& a, Plan* out) {
         if (S1 > kMaxStages) S1 = kMaxStages;
         if (S2 > kMaxStages) S2 = kMaxStages;
         const uint32_t s1b = (uint32_t)G1 * kb1_bytes;
-        const uint32_t used1 = (uint32_t)S1 * s1b, used2 = kStagingBytes + (uint32_t)S2 * kb2_bytes;
+        const uint32_t used1 = (uint32_t)S1 * s1b, used2 = (uint32_t)slabs * kSlabsBytes + (uint32_t)S2 * kb2_bytes;
         const uint32_t after1 = (uint32_t)t_bytes + used2;
-        Plan pl{C, RS, swb, BN2, G1, S1, S2, s1b, kb2_bytes, (uint32_t)t_bytes, 1024u + (used1 > after1 ? used1 : after1)};
+        Plan pl{C, RS, swb, BN2, G1, S1, S2, slabs, s1b, kb2_bytes, (uint32_t)t_bytes, 1024u + (used1 > after1 ? used1 : after1)};
         // prefer the largest cluster whose blocks are all resident at once (within this launch's share of the
         // SMs, when it runs beside other launches); else the smallest feasible.  With few row tiles the kernel is one
         // block's latency -- its share of P and Q through one SM -- so more blocks per tile shorten it: 768 -> 3072 at
@@ -575,7 +570,7 @@ lrd_status_t chain_launch(const ChainArgs& a, cudaStream_t stream) {
     p.ks2 = (int)a.r / 16;
     p.kb2 = (int)((a.r + 63) / 64);
     p.N2 = (int)a.N2;
-    p.G1 = pl.G1; p.S1 = pl.S1; p.S2 = pl.S2;
+    p.G1 = pl.G1; p.S1 = pl.S1; p.S2 = pl.S2; p.slabs = pl.slabs;
     p.stage1_bytes = pl.stage1_bytes; p.stage2_bytes = pl.stage2_bytes; p.t_bytes = pl.t_bytes;
     p.taw = pl.swb / 2;
     p.t_steps_lg = p.taw == 64 ? 2 : (p.taw == 32 ? 1 : 0);

@@ -24,7 +24,7 @@
 // barrier 1).
 // gridDim.z selects one of up to kMaxLayers independent layers of equal shape (a group launch).
 // Warp 0: TMA producer.  Warp 1: tensor memory; in the leader, MMA issue; in the odd block, forwarding
-// "slice landed" to the leader.  Warps 2-5: gather and epilogue.  Every wait is bounded; a wait that runs
+// "slice landed" to the leader.  Warps 2-9: gather and epilogue.  Every wait is bounded; a wait that runs
 // out raises the device timeout flag and the cluster tears down in order.
 #include <algorithm>
 
@@ -38,13 +38,14 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 192;
+constexpr int kThreads = 320;             // TMA producer, MMA issuer, 8 x gather / epilogue
+constexpr int kEpiThreads = 256;
 constexpr int kMaxSlots = 10;
 constexpr int kMaxS = 4;             // pairs per cluster
 constexpr uint32_t kSmemLimit = 224 * 1024;         // dynamic shared memory; the rest is left for the barriers and the bias
 constexpr uint32_t kInTileBytes = 128 * 64 * 2;     // In tile of one k-block: 128 rows x 64 k
 constexpr uint32_t kSlabBytes = 32 * 32 * 2;        // epilogue slab of one warp: 32 rows x 32 columns of bf16
-constexpr uint32_t kStagingBytes = 4 * 2 * kSlabBytes;
+constexpr uint32_t kSlabsBytes = 8 * kSlabBytes;    // one slab for every epilogue warp; there are one or two sets
 
 struct LayerMaps {
     CUtensorMap in, p, q, out, t;
@@ -56,6 +57,7 @@ struct PairGroup {
 struct PairParams {
     int S, RS, swb, BN2, n_chunks, kb1, ks2, kb2, N2, M;
     int G1, NS1, NS2;         // k-blocks per phase-1 stage; slots of the two rings
+    int slabs;                // sets of epilogue slabs (1 or 2)
     uint32_t stage1_bytes, stage2_bytes, t_bytes;
     int taw;                  // columns per atom of the T buffer (64, 32 or 16; swizzle span = 2 * taw bytes)
     int t_steps_lg;           // log2 of the MMA k-steps (16 columns) per atom
@@ -72,7 +74,7 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full1[kMaxSlots], empty1[kMaxSlots], full2[kMaxSlots], empty2[kMaxSlots], tacc_bar,
         tready_bar[kMaxS], pready_bar[kMaxS], out_full[2], out_empty[2];
-    __shared__ __align__(16) float bias_s[2][256];
+    __shared__ __align__(16) uint16_t bias_s[2][256];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -81,7 +83,7 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
     const uint32_t t_base = smem_base;
     const uint32_t ring1_base = smem_base;
     const uint32_t staging_base = t_base + p.t_bytes;
-    const uint32_t ring2_base = staging_base + kStagingBytes;
+    const uint32_t ring2_base = staging_base + (uint32_t)p.slabs * kSlabsBytes;
     const AbortCtx ab{&abort_flag, p.timeout_flag};
     const uint32_t t_sw = 2u * (uint32_t)p.taw, t_atom_bytes = 128u * t_sw;   // T: atoms of [128 rows x taw columns]
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0);
@@ -125,7 +127,7 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&out_full[i]), 1);
-            mbar_init(smem_u32(&out_empty[i]), 8);          // the epilogue warps of both blocks of the pair
+            mbar_init(smem_u32(&out_empty[i]), 16);          // the epilogue warps of both blocks of the pair
         }
         for (int j = 0; j < p.S; ++j)
             if (j != pr) mbar_expect_tx(smem_u32(&tready_bar[j]), 256u * (uint32_t)p.RS);
@@ -304,8 +306,8 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
     } else {
         // ------------------------------------------------------------------ gather + epilogue
         const int q = warp % 4;                              // tensor-memory lanes [32 q, 32 q + 32)
+        const int hw = (warp - 2) / 4;                       // two warps share a quarter: they take alternate 32-column pieces
         const int row = q * 32 + lane;                       // row of the 128-row tile
-        const int et = (warp - 2) * 32 + lane;               // index among the 128 epilogue threads
         const bool lead_warp = (warp == 2);                  // issues this block's bulk copies and stores (elect.sync)
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
         const bool rows_inside = m0 + q * 32 < p.M;          // (uniform) the odd block may hang over the last row tile
@@ -316,7 +318,7 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
         cluster_arrive_relaxed();
         if (ok) {
             // 32 columns per step (two tensor-memory loads in flight, one wait), a 16-column tail if RS / 16 is odd
-            for (int col = 0; col < p.RS; col += 32) {
+            for (int col = 32 * hw; col < p.RS; col += 64) {
                 uint32_t v[32];
                 const bool two = col + 32 <= p.RS;
                 tmem_ld_32x16(lane_addr + col, *reinterpret_cast<uint32_t(*)[16]>(&v[0]));
@@ -339,12 +341,12 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
             }
         }
         // The slice [pr RS, (pr + 1) RS) is whole atoms, i.e. one contiguous range of this block's T buffer: after the
-        // four warps have written it, one thread copies it into the buffers of the blocks with the same rows in the
+        // warps have written it, one thread copies it into the buffers of the blocks with the same rows in the
         // other pairs and, if asked, stores it to T_save.
         fence_proxy_async_smem();
         tc_fence_before();
         cluster_wait();                                      // barrier 1 complete: every peer's ring is dead
-        ok = named_bar_and(2, 128, ok);
+        ok = named_bar_and(2, kEpiThreads, ok);
         if (lead_warp) {
             if (ok && elect_one()) {
                 const uint32_t slice = t_base + (uint32_t)pr * 256u * (uint32_t)p.RS;
@@ -361,52 +363,38 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
             }
             __syncwarp();
         }
-        // Epilogue: each warp on its own.  32 columns of its 32 rows at a time go through a [32 rows x 64 B]
-        // slab of the warp (64-byte swizzle, two slabs in rotation) and leave by one TMA store each.  The bias
-        // of a chunk is staged in shared memory while its MMAs run.
-        const uint32_t slab0 = staging_base + (uint32_t)(warp - 2) * 2u * kSlabBytes;
+        // Epilogue: as in the single-block kernel, eight warps, the bias of a chunk fetched while the one before it is stored.
+        const uint32_t slab0 = staging_base + (uint32_t)(warp - 2) * kSlabBytes;
         const uint32_t row_off = (uint32_t)lane * 64u;
         const uint32_t row_xor = ((uint32_t)lane >> 1) & 3u;
         int i = 0, sb = 0;
+        uint16_t next_bias[4];
+        bias_fetch(next_bias, bias, (int64_t)pr * p.BN2 + 32 * hw, p.N2);
         for (int j = pr; j < p.n_chunks && ok; j += p.S, ++i) {
             const int buf = i & 1;
-            if (bias) {                                      // bias_s[buf] was last read two chunks ago, before a barrier
-                for (int e = et; e < p.BN2; e += 128) {
-                    const int col = j * p.BN2 + e;
-                    bias_s[buf][e] = col < p.N2 ? __bfloat162float(bias[col]) : 0.f;
-                }
-            }
             ok = mbar_wait_uniform(smem_u32(&out_full[buf]), (i >> 1) & 1, ab);
-            ok = named_bar_and(3, 128, ok);                  // the four warps go on, or give up, together (and see the bias)
             if (!ok) break;
+            if (bias) bias_put(&bias_s[buf][32 * hw], next_bias, p.BN2 / 64);
+            bias_fetch(next_bias, bias, (int64_t)(j + p.S) * p.BN2 + 32 * hw, p.N2);        // of the next chunk
             tc_fence_after();
             const uint32_t d_tmem = lane_addr + (uint32_t)buf * 256u;
-            for (int g = 0; g * 64 < p.BN2; ++g) {
-                const int col0 = j * p.BN2 + g * 64;
+            for (int c0 = hw; c0 * 32 < p.BN2; c0 += 4) {    // this warp's pieces, two at a time
+                const int col0 = j * p.BN2 + c0 * 32;
                 if (col0 >= p.N2) break;                     // (uniform) nothing of this piece is inside Out
-                uint32_t v[64];                              // both halves are loaded before the first is converted
-                tmem_ld_32x32(d_tmem + g * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-                tmem_ld_32x32(d_tmem + g * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+                const bool second = (c0 + 2) * 32 < p.BN2 && col0 + 64 < p.N2;
+                uint32_t v[64];                              // both pieces are loaded before the first is converted
+                tmem_ld_32x32(d_tmem + c0 * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                if (second) tmem_ld_32x32(d_tmem + c0 * 32 + 64, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
                 tmem_ld_wait();
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh, ++sb) {
-                    if (col0 + 32 * hh >= p.N2) break;       // (uniform)
-                    const uint32_t slab = slab0 + (uint32_t)(sb & 1) * kSlabBytes;
-                    if (sb >= 2) {                           // the store that last read this slab has finished reading
-                        tma_store_wait_read<1>();            // (only the lane that issued the stores has any to wait for)
-                        __syncwarp();
-                    }
-                    if (bias) {
-                        const float4* bp = reinterpret_cast<const float4*>(&bias_s[buf][g * 64 + hh * 32]);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float4 b4 = bp[e];
-                            v[32 * hh + 4 * e] = __float_as_uint(__uint_as_float(v[32 * hh + 4 * e]) + b4.x);
-                            v[32 * hh + 4 * e + 1] = __float_as_uint(__uint_as_float(v[32 * hh + 4 * e + 1]) + b4.y);
-                            v[32 * hh + 4 * e + 2] = __float_as_uint(__uint_as_float(v[32 * hh + 4 * e + 2]) + b4.z);
-                            v[32 * hh + 4 * e + 3] = __float_as_uint(__uint_as_float(v[32 * hh + 4 * e + 3]) + b4.w);
-                        }
-                    }
+                for (int hh = 0; hh < 2; ++hh) {
+                    if (hh == 1 && !second) break;           // (uniform)
+                    const uint32_t slab = slab0 + (sb && p.slabs == 2 ? kSlabsBytes : 0u);
+                    sb ^= 1;
+                    if (p.slabs == 2) tma_store_wait_read<1>();      // the store that last read the slab has finished reading
+                    else tma_store_wait_read<0>();                   // (only the lane that issued the stores has any to wait for)
+                    __syncwarp();
+                    if (bias) bias_add(&v[32 * hh], &bias_s[buf][32 * c0 + 64 * hh]);
 #pragma unroll
                     for (int cc = 0; cc < 4; ++cc)
                         st_shared_v4(slab + row_off + ((((uint32_t)cc) ^ row_xor) << 4),
@@ -417,7 +405,7 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (elect_one()) {
-                        if (rows_inside) tma_store_2d(&L.out, slab, col0 + 32 * hh, m0 + q * 32);
+                        if (rows_inside) tma_store_2d(&L.out, slab, col0 + 64 * hh, m0 + q * 32);
                         tma_store_commit();
                     }
                     __syncwarp();
@@ -448,7 +436,7 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
 }
 
 struct Plan {
-    int S, RS, swb, taw, BN2, G1, NS1, NS2;
+    int S, RS, swb, taw, BN2, G1, NS1, NS2, slabs;
     uint32_t stage1_bytes, stage2_bytes, t_bytes, smem_bytes;
 };
 
@@ -533,7 +521,10 @@ bool make_plan(const ChainArgs& a, int layers, Plan* out) {
         if (G1 > 4) G1 = 4;
         if (G1 > kb1) G1 = kb1;
         const int64_t all = (int64_t)kSmemLimit - 1024;
-        const int64_t ring2 = all - t_bytes - (int64_t)kStagingBytes;
+        // a second set of epilogue slabs where it does not cost the ring of Q tiles a slot that it needs
+        const int64_t room2 = all - t_bytes;
+        const int slabs = std::min<int64_t>((room2 - 2 * kSlabsBytes) / kb2_bytes, 6) >= std::min<int64_t>((room2 - kSlabsBytes) / kb2_bytes, 6) ? 2 : 1;
+        const int64_t ring2 = room2 - slabs * (int64_t)kSlabsBytes;
         const uint32_t s1b = (uint32_t)G1 * kb1_bytes;
         if (all < 2 * (int64_t)s1b || ring2 < 2 * (int64_t)kb2_bytes) continue;
         int NS1 = (int)(all / s1b), NS2 = (int)(ring2 / kb2_bytes);
@@ -548,8 +539,8 @@ bool make_plan(const ChainArgs& a, int layers, Plan* out) {
         const double cost = (double)waves * (std::max(fill1, mma1) + ph2 + 6000.0);
         if (cost < best_cost) {
             best_cost = cost;
-            const uint32_t used1 = (uint32_t)NS1 * s1b, used2 = (uint32_t)t_bytes + kStagingBytes + (uint32_t)NS2 * kb2_bytes;
-            best = Plan{S, RS, swb, taw, BN2, G1, NS1, NS2, s1b, kb2_bytes, (uint32_t)t_bytes, 1024u + std::max(used1, used2)};
+            const uint32_t used1 = (uint32_t)NS1 * s1b, used2 = (uint32_t)t_bytes + (uint32_t)slabs * kSlabsBytes + (uint32_t)NS2 * kb2_bytes;
+            best = Plan{S, RS, swb, taw, BN2, G1, NS1, NS2, slabs, s1b, kb2_bytes, (uint32_t)t_bytes, 1024u + std::max(used1, used2)};
         }
     }
     if (best_cost >= 1e300) return false;
@@ -619,7 +610,7 @@ lrd_status_t chain_pair_launch(const ChainArgs* layers, int n, cudaStream_t stre
     p.kb2 = (int)((a.r + 63) / 64);
     p.N2 = (int)a.N2;
     p.M = (int)a.M;
-    p.G1 = pl.G1; p.NS1 = pl.NS1; p.NS2 = pl.NS2;
+    p.G1 = pl.G1; p.NS1 = pl.NS1; p.NS2 = pl.NS2; p.slabs = pl.slabs;
     p.stage1_bytes = pl.stage1_bytes; p.stage2_bytes = pl.stage2_bytes; p.t_bytes = pl.t_bytes;
     p.taw = pl.taw;
     p.t_steps_lg = p.taw == 64 ? 2 : (p.taw == 32 ? 1 : 0);

@@ -292,6 +292,38 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
+// The bias of an epilogue warp's four 32-column pieces of a tile (columns col0 + 64 e + lane), fetched a tile ahead into
+// registers and put into shared memory (`at` = the place of col0) when the tile's turn comes.  Warps that share columns write
+// the same values to the same place and each reads behind its own write; two tiles' bias alternate, and a tile's is
+// written once its accumulator is complete, by when every warp is done with the tile two before it.
+__device__ __forceinline__ void bias_fetch(uint16_t (&b)[4], const __nv_bfloat16* bias, int64_t col0, int64_t n) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int64_t col = col0 + 64 * e + (threadIdx.x & 31);
+        b[e] = bias && col < n ? __bfloat16_as_ushort(bias[col]) : (uint16_t)0;
+    }
+}
+__device__ __forceinline__ void bias_put(uint16_t* at, const uint16_t (&b)[4], int pieces) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (e < pieces) at[64 * e + (threadIdx.x & 31)] = b[e];
+    __syncwarp();
+}
+// 32 accumulators += bias of their columns
+__device__ __forceinline__ void bias_add(uint32_t* v, const uint16_t* at) {
+    const uint4* bp = reinterpret_cast<const uint4*>(at);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const uint4 b4 = bp[x];
+        const uint32_t w[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+            v[8 * x + 2 * y] = __float_as_uint(__uint_as_float(v[8 * x + 2 * y]) + __uint_as_float(w[y] << 16));
+            v[8 * x + 2 * y + 1] = __float_as_uint(__uint_as_float(v[8 * x + 2 * y + 1]) + __uint_as_float(w[y] & 0xFFFF0000u));
+        }
+    }
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);

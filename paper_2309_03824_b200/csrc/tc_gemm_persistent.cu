@@ -2,11 +2,11 @@
 //   C[M x N] = op(A) op(B) (+ bias)
 // One block per SM walks over the 128 x BN output tiles (tile t -> row tile t % m_tiles, column tile
 // t / m_tiles, so that blocks working at the same time share the B operand in L2).  The accumulator is
-// double-buffered in tensor memory: while the four epilogue warps round tile i to bf16 and store it
-// (each warp its own 32 rows, through [32 x 32] shared-memory slabs and TMA stores that clip the ragged
+// double-buffered in tensor memory: while the eight epilogue warps round tile i to bf16 and store it
+// (each warp 32-column pieces of its own 32 rows, through [32 x 32] shared-memory slabs and TMA stores that clip the ragged
 // edges), the MMA warp already accumulates tile i + 1.  A short reduction (K of a few hundred, as in the
 // second product of an unfused decomposed layer) is otherwise all epilogue.
-// Warp 0: TMA producer.  Warp 1: tensor memory + MMA issue.  Warps 2-5: epilogue.  Single-thread
+// Warp 0: TMA producer.  Warp 1: tensor memory + MMA issue.  Warps 2-9: epilogue.  Single-thread
 // instructions are issued under elect.sync by a converged warp; every wait is bounded.
 //
 // CG = 2 runs the same loop on pairs of blocks (a cluster of two SMs, tcgen05 cta_group::2): a pair owns a
@@ -26,10 +26,10 @@ namespace {
 using namespace ptx;
 
 constexpr int BM = 128, BK = 64;
-constexpr int kThreads = 192;
+constexpr int kThreads = 320;                                // TMA producer, MMA issuer, 8 x epilogue
 constexpr uint32_t kATile = BM * BK * 2;
 constexpr uint32_t kSlabBytes = 32 * 32 * 2;                 // one warp's slab: 32 rows x 32 columns of bf16
-constexpr uint32_t kStagingBytes = 4 * 2 * kSlabBytes;
+constexpr uint32_t kStagingBytes = 8 * 2 * kSlabBytes;
 
 template <int BN, int CG> struct PCfg {
     static constexpr int BNH = BN / CG;                      // columns of B this block loads
@@ -41,7 +41,7 @@ template <int BN, int CG> struct PCfg {
     static constexpr int G = CG == 1 && BN <= 128 ? 2 : 1;
     static constexpr uint32_t B_TILE = BNH * BK * 2;
     static constexpr uint32_t STAGE_BYTES = G * (kATile + B_TILE);
-    static constexpr int STAGES_RAW = (200 * 1024) / STAGE_BYTES;
+    static constexpr int STAGES_RAW = (193 * 1024) / STAGE_BYTES;         // beside 32 KB of store slabs
     static constexpr int STAGES = STAGES_RAW > 8 ? 8 : STAGES_RAW;
     static constexpr uint32_t SMEM_BYTES = STAGES * STAGE_BYTES + kStagingBytes + 1024;
     static constexpr uint32_t TMEM_COLS = 2 * BN <= 128 ? 128 : (2 * BN <= 256 ? 256 : 512);
@@ -72,6 +72,7 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     constexpr int STAGES = C::STAGES, G = C::G;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], out_full[2], out_empty[2];
+    __shared__ __align__(16) uint16_t bias_s[2][256];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -94,7 +95,7 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&out_full[i]), 1);
-            mbar_init(smem_u32(&out_empty[i]), 4 * CG);       // the epilogue warps of every block of the pair
+            mbar_init(smem_u32(&out_empty[i]), 8 * CG);       // the epilogue warps of every block of the pair
         }
         fence_mbar_init();
     }
@@ -208,10 +209,12 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     } else if (warp >= 2) {
         // ------------------------------------------------------------------ epilogue
         const int q = warp % 4;                              // tensor-memory lanes [32 q, 32 q + 32)
+        const int hw = (warp - 2) / 4;                       // two warps share a quarter: they take alternate 32-column pieces
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
         const uint32_t slab0 = staging_base + (uint32_t)(warp - 2) * 2u * kSlabBytes;
         const uint32_t row_off = (uint32_t)lane * 64u, row_xor = ((uint32_t)lane >> 1) & 3u;
-        const bool bias_ok = p.bias && (((uintptr_t)p.bias & 15u) == 0);
+        uint16_t next_bias[4];
+        bias_fetch(next_bias, p.bias, (int64_t)(unit / p.m_tiles) * BN + 32 * hw, p.N);
         int i = 0, sb = 0;
         bool ok = true;
         for (int t = unit; t < n_tiles_total && ok; t += n_units, ++i) {
@@ -220,52 +223,44 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
             const bool rows_inside = m0 + q * 32 < p.M;      // (uniform) a pair's odd block may hang over the last row tile
             ok = mbar_wait_uniform(smem_u32(&out_full[buf]), (i >> 1) & 1, ab);
             if (!ok) break;
+            if (p.bias) bias_put(&bias_s[buf][32 * hw], next_bias, BN / 64);
+            bias_fetch(next_bias, p.bias, (int64_t)((t + n_units) / p.m_tiles) * BN + 32 * hw, p.N);        // of the next tile
             tc_fence_after();
             const uint32_t d_tmem = lane_addr + (uint32_t)buf * C::BUF_COLS;
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c, ++sb) {
-                const int col0 = n0 + c * 32;
-                if (col0 >= p.N) break;                      // (uniform) nothing of this piece is inside C
-                uint4 bv[4] = {};
-                const bool bvec = bias_ok && col0 + 32 <= p.N;
-                if (bvec) {
-                    const uint4* bp = reinterpret_cast<const uint4*>(p.bias + col0);
+            for (int c0 = hw; c0 < BN / 32; c0 += 4) {       // this warp's pieces, two at a time
+                if (n0 + c0 * 32 >= p.N) break;              // (uniform) nothing of this piece is inside C
+                const bool second = c0 + 2 < BN / 32 && n0 + c0 * 32 + 64 < p.N;
+                uint32_t v2[2][32];
+                tmem_ld_32x32(d_tmem + c0 * 32, v2[0]);
+                if (second) tmem_ld_32x32(d_tmem + c0 * 32 + 64, v2[1]);
+                tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) bv[e] = __ldg(bp + e);
-                }
-                uint32_t v[32];
-                tmem_ld_32x32(d_tmem + c * 32, v);
-                const uint32_t slab = slab0 + (uint32_t)(sb & 1) * kSlabBytes;
-                if (sb >= 2) {                               // the store that last read this slab has finished reading
-                    tma_store_wait_read<1>();
+                for (int h2 = 0; h2 < 2; ++h2, ++sb) {
+                    if (h2 == 1 && !second) break;           // (uniform)
+                    uint32_t (&v)[32] = v2[h2];
+                    const int col0 = n0 + (c0 + 2 * h2) * 32;
+                    if (p.bias) bias_add(v, &bias_s[buf][32 * c0 + 64 * h2]);
+                    const uint32_t slab = slab0 + (uint32_t)(sb & 1) * kSlabBytes;
+                    if (sb >= 2) {                           // the store that last read this slab has finished reading
+                        tma_store_wait_read<1>();
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc)
+                        st_shared_v4(slab + row_off + ((((uint32_t)cc) ^ row_xor) << 4),
+                                     pack_bf16(__uint_as_float(v[8 * cc]), __uint_as_float(v[8 * cc + 1])),
+                                     pack_bf16(__uint_as_float(v[8 * cc + 2]), __uint_as_float(v[8 * cc + 3])),
+                                     pack_bf16(__uint_as_float(v[8 * cc + 4]), __uint_as_float(v[8 * cc + 5])),
+                                     pack_bf16(__uint_as_float(v[8 * cc + 6]), __uint_as_float(v[8 * cc + 7])));
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (elect_one()) {
+                        if (rows_inside) tma_store_2d(&tmC, slab, col0, m0 + q * 32);
+                        tma_store_commit();
+                    }
                     __syncwarp();
                 }
-                tmem_ld_wait();
-                if (bvec) {
-                    const uint32_t* bw = reinterpret_cast<const uint32_t*>(bv);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        v[2 * e] = __float_as_uint(__uint_as_float(v[2 * e]) + __uint_as_float(bw[e] << 16));
-                        v[2 * e + 1] = __float_as_uint(__uint_as_float(v[2 * e + 1]) + __uint_as_float(bw[e] & 0xFFFF0000u));
-                    }
-                } else if (p.bias) {
-                    for (int e = 0; e < 32; ++e)
-                        if (col0 + e < p.N) v[e] = __float_as_uint(__uint_as_float(v[e]) + __bfloat162float(p.bias[col0 + e]));
-                }
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc)
-                    st_shared_v4(slab + row_off + ((((uint32_t)cc) ^ row_xor) << 4),
-                                 pack_bf16(__uint_as_float(v[8 * cc]), __uint_as_float(v[8 * cc + 1])),
-                                 pack_bf16(__uint_as_float(v[8 * cc + 2]), __uint_as_float(v[8 * cc + 3])),
-                                 pack_bf16(__uint_as_float(v[8 * cc + 4]), __uint_as_float(v[8 * cc + 5])),
-                                 pack_bf16(__uint_as_float(v[8 * cc + 6]), __uint_as_float(v[8 * cc + 7])));
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (elect_one()) {
-                    if (rows_inside) tma_store_2d(&tmC, slab, col0, m0 + q * 32);
-                    tma_store_commit();
-                }
-                __syncwarp();
             }
             tc_fence_before();
             __syncwarp();
