@@ -19,6 +19,9 @@ double tc_gemm_persistent_estimate(int64_t M, int64_t N, int64_t K);
 // Estimated microseconds of a data product on the kernel tc_gemm would take for it.
 double tc_gemm_estimate(int64_t M, int64_t N, int64_t K);
 void tc_gemm_persistent_force_pairs(int blocks_per_mma);     // 0: automatic; 1 or 2: forced where the shape allows
+// Weight gradients (both operands MN-major) on pairs of SMs; estimated microseconds, 1e300 where it does not apply.
+double tc_wgrad_pair_estimate(const GemmArgs& g);
+lrd_status_t tc_wgrad_pair(const GemmArgs& g, cudaStream_t stream);
 // allow_split: the reduction dimension may be split over blocks (weight gradients).
 lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_t partial_bytes, cudaStream_t stream);
 

@@ -661,6 +661,20 @@ static SplitPlan pick_split(int64_t M, int64_t N, int64_t K, bool ones, int max_
     return best;
 }
 
+// Estimated microseconds of a weight gradient under a plan, against the kernel on pairs of SMs (tc_wgrad_pair.cu).  Fitted to
+// 3072 x 384 over 4096 tokens (cluster of 2: 14.8 us, estimate 14.5; pairs 20.2), 4096 x 256 over 8192 (20; 20.2; pairs 21.9),
+// 4096 x 512 over 8192 (two shares through scratch memory: 37.1; 39.8; pairs 32.9), 4096 x 1024 over 1024 with sums (two waves
+// of tiles 192 wide: 16.2; 14.4; pairs 11.8).
+static double split_estimate(const SplitPlan& sp, int64_t M, int64_t N, int64_t K) {
+    const int64_t tiles = ((M + BM - 1) / BM) * ((N + sp.bn - 1) / sp.bn), kb = (K + BK - 1) / BK;
+    if (sp.cluster > 1) {
+        const double per_block = (double)((kb + sp.cluster - 1) / sp.cluster) * (BM * BK * 2.0 + sp.bn * BK * 2.0);
+        return 5.0 + 0.8e6 * std::max(per_block / 110e9, per_block * (double)(tiles * sp.cluster) / 14e12);
+    }
+    const int64_t waves = (tiles * sp.global + kNumSms - 1) / kNumSms;
+    return 4.0 + (double)(waves * ((kb + sp.global - 1) / sp.global)) * std::max(0.2, 0.0017 * sp.bn) + (sp.global > 1 ? 8.0 : 0.0);
+}
+
 // A data product with few tiles and a long reduction (a short batch through a wide layer) is the latency of one tile's
 // k-blocks: about 0.13 us each for the narrow tiles such products run on, after some 3.3 us of launch, first loads and
 // epilogue.  Split over the blocks of a cluster it is a share of them and the exchange: 128 tokens, 3072 -> 384 9.4 us
@@ -715,6 +729,8 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
         bn = dp.bn; cluster = dp.cluster;
     } else if (allow_split) {
         const SplitPlan sp = pick_split(g.M, g.N, g.K, ones, g.max_cluster_split);
+        // where the tiles leave no room for a cluster per tile
+        if (tc_wgrad_pair_estimate(g) < 0.95 * split_estimate(sp, g.M, g.N, g.K)) return tc_wgrad_pair(g, stream);
         bn = sp.bn; cluster = sp.cluster; splits = sp.global;
     } else {
         bn = pick_bn(g.M, g.N, false);
