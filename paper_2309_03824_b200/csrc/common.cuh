@@ -38,6 +38,8 @@ struct GemmArgs {
     int max_cluster_split = 0; // split weight gradients: largest cluster to split the reduction over (0 = automatic).  A
                                // launch meant to run BESIDE others asks for 2: clusters of 4 or 8 need that many free
                                // SMs inside one GPC, which a chain kernel on 128 of the 148 SMs never leaves
+    bool in_turn = false;      // weight gradients: started only when the launch before has ended (blocks that wait on an SM for
+                               // that end keep it from work in other streams)
 };
 
 // True when the CUDA call succeeded.  With the environment variable LRD_LOG_ERRORS set, a failure is also written to
@@ -57,6 +59,8 @@ lrd_status_t simt_gemm(const GemmArgs& g, cudaStream_t stream);
 // operands qualify, else the general kernel.
 lrd_status_t run_gemm(const GemmArgs& g, int path, bool allow_split, float* partials, size_t partial_bytes,
                       cudaStream_t s);
+// Several weight gradients (reduction split as above), independent of one another; their scratch may be shared.
+lrd_status_t run_wgrads(const GemmArgs* g, int n, int path, float* const* partials, const size_t* partial_bytes, cudaStream_t s);
 GemmArgs make_gemm(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
                    bool b_mn, void* C, int64_t ldc, const void* bias, lrd_dtype_t dt);
 lrd_status_t zero_fill(void* p, int64_t rows, int64_t cols, int64_t ld, lrd_dtype_t dt, cudaStream_t s);

@@ -189,20 +189,20 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     // nothing of each other; dB (+ db) needs only dY and Z2_save; dA needs the dZ1 the transposed core writes.  Every
     // launch here is a few microseconds of latency around little work, so the independent ones run side by side:
     // dB from the start and the filter gradient after dZ2 on library-owned streams, the data path and dA on the
-    // caller's stream, which waits for the other two before this function returns.
-    SideStreams* ss = g_tucker_overlap && (factors || core) ? side_streams() : nullptr;
-    cudaStream_t sB = ss && factors ? ss->aux[0] : s, sF = ss && core ? ss->aux[1] : s;
+    // caller's stream, which waits for the other two before this function returns.  With the core frozen there is no filter
+    // gradient, and dB and dA in one launch behind the data path need no second stream: 64 x 14 x 14, 256 -> 256 at rank 96
+    // 40.4 -> 38.5 us per step, 16 x 28 x 28, 128 -> 128 at 64 43.4 -> 41.8; with nothing frozen dB beside the data path
+    // remains the faster way (64 x 7 x 7, 512 -> 512 at 309 92.5 against 96.0).
+    SideStreams* ss = g_tucker_overlap && core ? side_streams() : nullptr;
+    cudaStream_t sB = ss && factors ? ss->aux[0] : s, sF = ss ? ss->aux[1] : s;
     lrd_status_t st = LRD_OK;
     auto keep = [&st](lrd_status_t x) { if (st == LRD_OK) st = x; };
     if (sB != s) {
         if (!stream_after(sB, s, ss->fork)) return LRD_ERR_CUDA;
     }
-    auto launch_dB = [&]() {
-        GemmArgs gb = make_gemm(t.S, t.r2, t.Po, dY, t.S, true, Z2_save, t.r2, true, dB, t.r2, nullptr, t.dt);
-        gb.a_colsum = dbias;                              // the bias gradient rides on the dB product (A = dY)
-        keep(run_gemm(gb, path, true, pB, reg.dB, sB));
-    };
-    if (factors && sB != s) launch_dB();
+    GemmArgs dB_product = make_gemm(t.S, t.r2, t.Po, dY, t.S, true, Z2_save, t.r2, true, dB, t.r2, nullptr, t.dt);
+    dB_product.a_colsum = dbias;                          // the bias gradient rides on the dB product (A = dY)
+    if (factors && sB != s) keep(run_gemm(dB_product, path, true, pB, reg.dB, sB));
 
     auto launch_filter = [&](cudaStream_t st_f) {
         keep(conv_bwd_filter(dZ2, Z1_save, dG, t.B, t.g, t.r1, t.r2, t.dt, path, st_f));
@@ -231,8 +231,10 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     else if (dX || factors) keep(conv_bwd_data(dZ2, G, dZ1, t.B, t.g, t.r1, t.r2, t.dt, path, s));
     if (dX && !fuse_dx && !one_launch) keep(run_gemm(make_gemm(t.P, t.C, t.r1, dZ1, t.r1, false, A, t.r1, false, dX, t.C, nullptr, t.dt), path, false, nullptr, 0, s));
     if (factors) {
-        if (sB == s) launch_dB();
-        keep(run_gemm(make_gemm(t.C, t.r1, t.P, X, t.C, true, dZ1, t.r1, true, dA, t.r1, nullptr, t.dt), path, true, pA, reg.dA, s));
+        const GemmArgs gw[2] = {make_gemm(t.C, t.r1, t.P, X, t.C, true, dZ1, t.r1, true, dA, t.r1, nullptr, t.dt), dB_product};
+        float* const scratch[2] = {pA, pB};
+        const size_t scratch_bytes[2] = {reg.dA, reg.dB};
+        keep(run_wgrads(gw, sB == s ? 2 : 1, path, scratch, scratch_bytes, s));
     }
     if (core && sF == s) launch_filter(s);
     // join even after a failed launch, so that a capture in progress is left whole

@@ -199,6 +199,17 @@ lrd_status_t run_gemm(const GemmArgs& g, int path, bool allow_split, float* part
     return simt_gemm(g, s);
 }
 
+lrd_status_t run_wgrads(const GemmArgs* g, int n, int path, float* const* partials, const size_t* partial_bytes, cudaStream_t s) {
+    bool tc = path != LRD_PATH_GENERAL;
+    for (int i = 0; i < n; ++i) tc = tc && g[i].M > 0 && g[i].N > 0 && tc_gemm_eligible(g[i]);
+    if (tc) return tc_wgrads(g, n, partials, partial_bytes, s);
+    for (int i = 0; i < n; ++i) {
+        const lrd_status_t st = run_gemm(g[i], path, true, partials[i], partial_bytes[i], s);
+        if (st != LRD_OK) return st;
+    }
+    return LRD_OK;
+}
+
 lrd_status_t zero_fill(void* p, int64_t rows, int64_t cols, int64_t ld, lrd_dtype_t dt, cudaStream_t s) {
     if (!p || rows <= 0 || cols <= 0) return LRD_OK;
     const size_t e = elem_size(dt);
@@ -539,6 +550,19 @@ static lrd_status_t lrd_linear_fwd_impl(const lrd_linear_desc_t* desc, const voi
     return linear_fwd_on(desc, X, V, U, bias, Y, Z_save, freeze, workspace, workspace_bytes, (cudaStream_t)cuda_stream, 0);
 }
 
+// The weight gradients `plan` asks for, dU (+ db) before dV; returns how many.
+static int linear_wgrads(const Linear& L, uint32_t plan, const void* dY, const void* X, const void* Z_save, const void* dZ, void* dU, void* dV,
+                         void* dbias, int max_cluster, GemmArgs* g) {
+    int n = 0;
+    if (plan & LRD_PLAN_DU) {
+        g[n] = gemm(L.N, L.r, L.M, dY, L.ldy, true, Z_save, L.ldz, true, dU, L.ldu, nullptr, L.dt);
+        g[n++].a_colsum = dbias;           // db rides on the dU product (A = dY): no second pass over dY
+    }
+    if (plan & LRD_PLAN_DV) g[n++] = gemm(L.K, L.r, L.M, X, L.ldx, true, dZ, L.r, true, dV, L.ldv, nullptr, L.dt);
+    for (int i = 0; i < n; ++i) g[i].max_cluster_split = max_cluster;
+    return n;
+}
+
 // One layer's backward on stream s.  With a side stream, the dU (+ db) product, which needs nothing the data
 // chain produces, runs there beside the chain; the caller has made `side` wait for s's earlier work and makes s
 // wait for `side` afterwards.  dV follows the chain (it reads the dZ the chain spills) and, when dU is computed too,
@@ -622,22 +646,17 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
         if (dX)
             LRD_TRY(run_gemm(gemm(L.M, L.K, L.r, dZ, L.r, false, V, L.ldv, false, dX, L.ldx, nullptr, L.dt), false, nullptr, 0, s));
     }
-    if (do_w && (plan & LRD_PLAN_DU)) {
-        GemmArgs gu = gemm(L.N, L.r, L.M, dY, L.ldy, true, Z_save, L.ldz, true, dU, L.ldu, nullptr, L.dt);
-        gu.max_cluster_split = wsplit;
-        gu.a_colsum = dbias;               // db rides on the dU product (A = dY): no second pass over dY
-        cudaStream_t su = side ? side : s;
-        LRD_TRY(run_gemm(gu, true, partials, partial_bytes, su));
-        if (side && (plan & LRD_PLAN_DV)) {
-            if (cudaEventRecord(side_done, side) != cudaSuccess || cudaStreamWaitEvent(s, side_done, 0) != cudaSuccess) return LRD_ERR_CUDA;
-        }
+    if (!do_w) return LRD_OK;
+    GemmArgs gw[2];
+    const int n = linear_wgrads(L, plan, dY, X, Z_save, dZ, dU, dV, dbias, wsplit, gw);
+    if (side && n == 2) {
+        LRD_TRY(run_gemm(gw[0], true, partials, partial_bytes, side));
+        if (cudaEventRecord(side_done, side) != cudaSuccess || cudaStreamWaitEvent(s, side_done, 0) != cudaSuccess) return LRD_ERR_CUDA;
+        return run_gemm(gw[1], true, partials, partial_bytes, s);
     }
-    if (do_w && (plan & LRD_PLAN_DV)) {
-        GemmArgs gv = gemm(L.K, L.r, L.M, X, L.ldx, true, dZ, L.r, true, dV, L.ldv, nullptr, L.dt);
-        gv.max_cluster_split = wsplit;
-        LRD_TRY(run_gemm(gv, true, partials, partial_bytes, s));
-    }
-    return LRD_OK;
+    float* const scratch[2] = {partials, partials};
+    const size_t scratch_bytes[2] = {partial_bytes, partial_bytes};
+    return run_wgrads(gw, n, path, scratch, scratch_bytes, side && (plan & LRD_PLAN_DU) ? side : s);
 }
 
 static lrd_status_t lrd_linear_bwd_data_impl(const lrd_linear_desc_t* desc, const void* dY, const void* V, const void* U, void* dX,
@@ -748,18 +767,14 @@ static lrd_status_t lrd_linear_group_bwd_impl(int n, const lrd_linear_desc_t* de
     for (int i = 0; i < n; ++i)
         LRD_TRY(linear_bwd_on(&descs[i], dY[i], at(X, i), V[i], U[i], at(Z_save, i), at_w(dX, i), at_w(dU, i), at_w(dV, i),
                               at_w(dbias, i), freeze, workspace[i], workspace_bytes[i], s, nullptr, nullptr, 0, true));
-    SideStreams* ss = side_streams();
-    if (!ss) return LRD_ERR_CUDA;
-    if (cudaEventRecord(ss->fork, s) != cudaSuccess) return LRD_ERR_CUDA;
-    const bool du_aside = (lrd_linear_bwd_plan(freeze) & LRD_PLAN_DU) != 0;
-    // layers of one shape: their data chains (dZ, dX) in one launch on pairs of SMs, the layer picked by gridDim.z;
-    // the weight gradients then run side by side as below
-    bool data_done = false;
+    // layers of one shape: their data chains (dZ, dX) in one launch on pairs of SMs, the layer picked by gridDim.z, then all
+    // their weight gradients in one more
+    const uint32_t plan = lrd_linear_bwd_plan(freeze);
     const int path = g_path.load();
     if (n > 1 && n <= kChainMaxLayers && dX && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) && g_chain_mma_blocks.load() != 1) {
         ChainArgs c[kChainMaxLayers];
         bool ok = true;
-        const bool need_dz = (lrd_linear_bwd_plan(freeze) & LRD_PLAN_DV) != 0;
+        const bool need_dz = (plan & LRD_PLAN_DV) != 0;
         for (int i = 0; i < n && ok; ++i) {
             Linear L;
             ok = parse_linear(&descs[i], &L, false) == LRD_OK && L.M > 0 && dX[i] != nullptr;
@@ -767,10 +782,37 @@ static lrd_status_t lrd_linear_group_bwd_impl(int n, const lrd_linear_desc_t* de
         }
         if (ok && chain_pair_eligible(c, n)) {
             LRD_TRY(chain_pair_launch(c, n, s));
-            data_done = true;
-            if (!cuda_ok(cudaEventRecord(ss->mid, s), "cudaEventRecord(group mid)")) return LRD_ERR_CUDA;
+            GemmArgs gw[2 * kChainMaxLayers];
+            float* scratch[2 * kChainMaxLayers];
+            size_t scratch_bytes[2 * kChainMaxLayers];
+            int m = 0;
+            for (int i = 0; i < n; ++i) {
+                Linear L;
+                LRD_TRY(parse_linear(&descs[i], &L, false));
+                // the frozen factor's gradient buffer, if the caller passed one, reads as zero
+                if (!(plan & LRD_PLAN_DU)) {
+                    LRD_TRY(zero_fill(at_w(dU, i), L.N, L.r, L.ldu, L.dt, s));
+                    LRD_TRY(zero_fill(at_w(dbias, i), 1, L.N, L.N, L.dt, s));
+                }
+                if (!(plan & LRD_PLAN_DV)) LRD_TRY(zero_fill(at_w(dV, i), L.K, L.r, L.ldv, L.dt, s));
+                const int k = linear_wgrads(L, plan, dY[i], at(X, i), at(Z_save, i), workspace[i], at_w(dU, i), at_w(dV, i), at_w(dbias, i), 0, gw + m);
+                for (int j = 0; j < k; ++j, ++m) {
+                    scratch[m] = (float*)((uint8_t*)workspace[i] + linear_z_bytes(L));
+                    scratch_bytes[m] = workspace_bytes[i] - linear_z_bytes(L);
+                }
+            }
+            // (the side stream of a caller that overlaps weight gradients may still be busy: blocks of this launch that wait
+            // on their SMs for the data chains to end would be in its way.  A block of 768-wide layers, 4096 tokens: 202 us
+            // waiting ahead, 185 in turn, 193 with the gradients on three streams)
+            for (int i = 0; i < m; ++i) gw[i].in_turn = true;
+            return run_wgrads(gw, m, path, scratch, scratch_bytes, s);
         }
     }
+    // otherwise every layer on a stream of its own
+    SideStreams* ss = side_streams();
+    if (!ss) return LRD_ERR_CUDA;
+    if (cudaEventRecord(ss->fork, s) != cudaSuccess) return LRD_ERR_CUDA;
+    const bool du_aside = (plan & LRD_PLAN_DU) != 0;
     // The data chains are shaped for twice their even share: the weight-gradient launches that follow each of them
     // fill the machine anyway, and a chain of 2 blocks per row tile finishes sooner than one of 1 (three
     // 768 -> 768, r = 192 layers at 4096 tokens, U frozen: 32.9 us against 35.3 us).
@@ -779,11 +821,11 @@ static lrd_status_t lrd_linear_group_bwd_impl(int n, const lrd_linear_desc_t* de
     for (int i = 0; i < n; ++i) {
         cudaStream_t si = i == 0 ? s : ss->layer[i - 1];
         cudaStream_t sd = du_aside ? ss->aux[i] : nullptr;
-        if (i > 0 && !cuda_ok(cudaStreamWaitEvent(si, data_done ? ss->mid : ss->fork, 0), "cudaStreamWaitEvent(group layer)")) { st = LRD_ERR_CUDA; continue; }
+        if (i > 0 && !cuda_ok(cudaStreamWaitEvent(si, ss->fork, 0), "cudaStreamWaitEvent(group layer)")) { st = LRD_ERR_CUDA; continue; }
         if (sd && cudaStreamWaitEvent(sd, ss->fork, 0) != cudaSuccess) { st = LRD_ERR_CUDA; continue; }
         const lrd_status_t sti = linear_bwd_on(&descs[i], dY[i], at(X, i), V[i], U[i], at(Z_save, i), at_w(dX, i), at_w(dU, i),
                                                at_w(dV, i), at_w(dbias, i), freeze, workspace[i], workspace_bytes[i], si, sd,
-                                               ss->aux_done[i], share, false, data_done ? 2 : 3);
+                                               ss->aux_done[i], share, false);
         if (sti != LRD_OK) st = sti;
         if (sd && !stream_after(s, sd, ss->aux_done[i])) st = LRD_ERR_CUDA;
         if (i > 0 && !stream_after(s, si, ss->join[i - 1])) st = LRD_ERR_CUDA;

@@ -19,9 +19,13 @@ double tc_gemm_persistent_estimate(int64_t M, int64_t N, int64_t K);
 // Estimated microseconds of a data product on the kernel tc_gemm would take for it.
 double tc_gemm_estimate(int64_t M, int64_t N, int64_t K);
 void tc_gemm_persistent_force_pairs(int blocks_per_mma);     // 0: automatic; 1 or 2: forced where the shape allows
-// Weight gradients (both operands MN-major) on pairs of SMs; estimated microseconds, 1e300 where it does not apply.
-double tc_wgrad_pair_estimate(const GemmArgs& g);
-lrd_status_t tc_wgrad_pair(const GemmArgs& g, cudaStream_t stream);
+// Weight gradients (both operands MN-major), up to kMaxWgrads of them in one launch.  Estimated microseconds on pairs of
+// SMs (1e300 where that does not apply); all of them on pairs; all of them the fastest way (partials: scratch of each,
+// which may be shared).
+constexpr int kMaxWgrads = 8;
+double tc_wgrad_pair_estimate(const GemmArgs* g, int n);
+lrd_status_t tc_wgrad_pair(const GemmArgs* g, int n, cudaStream_t stream);
+lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const size_t* partial_bytes, cudaStream_t stream);
 // allow_split: the reduction dimension may be split over blocks (weight gradients).
 lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_t partial_bytes, cudaStream_t stream);
 

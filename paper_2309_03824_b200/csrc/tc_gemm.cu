@@ -24,6 +24,7 @@
 // and a block of B is 64 consecutive output pixels' input channels at one tap, fetched by TMA in im2col mode.  The
 // reduction runs over all pixels whatever the image size.
 #include <algorithm>
+#include <climits>
 
 #include "common.cuh"
 #include "conv.cuh"
@@ -75,15 +76,30 @@ struct TcParams {
     unsigned int* timeout_flag;
 };
 
+// What one launch computes: a product, or NP independent ones (weight gradients) whose row tiles follow one another in
+// gridDim.y; every product takes the tile width and the cluster size of the launch.
+template <int NP> struct TcLaunch {
+    int row0[NP];       // first row tile of each product (INT_MAX: none)
+    TcParams p[NP];
+    CUtensorMap tA[NP], tB[NP];
+};
+
 // CONV: column of dG (= tap * ci + channel) that column `col` of the product belongs to; -1: padding
 __device__ __forceinline__ int conv_col(const TcParams& p, int col) {
     const int blk = col / 64, c = (blk % p.cv_nkc) * 64 + col % 64;
     return blk < p.cv_nblk && c < p.cv_ci ? (blk / p.cv_nkc) * p.cv_ci + c : -1;
 }
 
-template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false>
+template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1>
 __global__ void __launch_bounds__(kThreads, 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcParams p) {
+tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
+    int prod = 0;
+#pragma unroll
+    for (int i = 1; i < NP; ++i)
+        if ((int)blockIdx.y >= L.row0[i]) prod = i;
+    const CUtensorMap &tmA = L.tA[prod], &tmB = L.tB[prod];
+    const TcParams p = L.p[prod];
+    if (NP > 1 && (int64_t)blockIdx.x * BN >= p.N) return;         // (the whole cluster: its blocks share x and y)
     static_assert(!ONES || (A_MN && B_MN && BN <= 192), "the ones block rides on an MN-major B of at most 192 columns");
     static_assert(!CONV || (A_MN && B_MN && !ONES && BN <= 192), "the filter gradient: both operands MN-major, split over a cluster or not at all");
     using C = Cfg<BN, ONES>;
@@ -97,7 +113,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const AbortCtx ab{&abort_flag, p.timeout_flag};
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int m0 = ((int)blockIdx.y - (NP > 1 ? L.row0[prod] : 0)) * BM, n0 = blockIdx.x * BN;
+    const bool with_colsum = ONES && blockIdx.x == 0 && (NP == 1 || p.colsum_out);
     const int kb_begin = blockIdx.z * p.kb_per_split;
     const int kb_end = min(kb_begin + p.kb_per_split, p.kb_total);
 
@@ -114,7 +131,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (p.cluster_splits > 1) {                        // bytes the peers will send this block
             const uint32_t S = (uint32_t)p.cluster_splits;
             uint32_t tx = (S - 1u) * 128u * (BN / S) * 4u;
-            if (ONES && blockIdx.x == 0 && cluster_ctarank() == 0) tx += (S - 1u) * 512u;
+            if (with_colsum && cluster_ctarank() == 0) tx += (S - 1u) * 512u;
             mbar_expect_tx(smem_u32(&red_bar), tx);
         }
         fence_mbar_init();
@@ -198,7 +215,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (p.cluster_splits > 1) { cluster_arrive(); cluster_wait(); cluster_arrive_relaxed(); }
     } else if (warp == 1) {
         // MMA issuer: converged warp, elect.sync around the issue
-        const uint32_t idesc = idesc_bf16(BN + ((ONES && blockIdx.x == 0) ? 16 : 0), A_MN, B_MN);
+        const uint32_t idesc = idesc_bf16(BN + (with_colsum ? 16 : 0), A_MN, B_MN);
         const uint64_t a_desc0 = A_MN ? smem_desc_sw128(smem_base, kBox, 1024) : smem_desc_sw128(smem_base, 0, 1024);
         const uint64_t b_desc0 = B_MN ? smem_desc_sw128(smem_base + A_STAGE_BYTES, kBox, 1024) : smem_desc_sw128(smem_base + A_STAGE_BYTES, 0, 1024);
         int s = 0;
@@ -237,7 +254,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint32_t chunk_bytes = 128u * cs * 4u, ngrp = cs / 4u;
         const uint32_t stage_base = smem_base, recv_base = smem_base + 128u * BN * 4u;
         const uint32_t cs_stage = recv_base + 128u * BN * 4u, cs_recv = cs_stage + 512u;
-        const bool with_colsum = ONES && blockIdx.x == 0;
         bool ok = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         // barrier 1: this block's pipeline ring is dead (all its MMAs have completed).  Progress only: what the peers
@@ -381,7 +397,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const int64_t row = (int64_t)m0 + quarter * 32 + lane;
             const bool row_ok = row < p.M;
             const bool bias_vec_ok = p.bias && (((uintptr_t)p.bias & 15u) == 0);
-            if (ONES && blockIdx.x == 0) {                 // accumulator column BN = sum over k of A(row, k)
+            if (with_colsum) {                             // accumulator column BN = sum over k of A(row, k)
                 uint32_t cs[16];
                 tmem_ld_32x16(tmem_base + ((uint32_t)(quarter * 32) << 16) + BN, cs);
                 tmem_ld_wait();
@@ -503,9 +519,10 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
         }
 }
 
-template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false>
-lrd_status_t launch(const CUtensorMap& tA, const CUtensorMap& tB, const TcParams& p, dim3 grid, cudaStream_t stream) {
-    auto kern = tc_gemm_kernel<BN, A_MN, B_MN, ONES, CONV>;
+template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1>
+lrd_status_t launch(const TcLaunch<NP>& L, dim3 grid, cudaStream_t stream, bool wait_ahead = true) {
+    auto kern = tc_gemm_kernel<BN, A_MN, B_MN, ONES, CONV, NP>;
+    const TcParams& p = L.p[0];
     static bool configured_on[kMaxDevices] = {};     // per instantiation; the attribute is sticky per function
     bool& configured = configured_on[device_slot()];
     if (!configured) {
@@ -524,19 +541,18 @@ lrd_status_t launch(const CUtensorMap& tA, const CUtensorMap& tB, const TcParams
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = p.cluster_splits > 1 ? (unsigned)p.cluster_splits : 1u;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) before it touches global memory
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].val.programmaticStreamSerializationAllowed = wait_ahead ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, kern, tA, tB, p) != cudaSuccess) return LRD_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, kern, L) != cudaSuccess) return LRD_ERR_CUDA;
     count_launch();
     return LRD_OK;
 }
 
 template <int BN>
-lrd_status_t launch_major(bool a_mn, bool b_mn, const CUtensorMap& tA, const CUtensorMap& tB, const TcParams& p,
-                          dim3 grid, cudaStream_t s) {
-    if (a_mn) return b_mn ? launch<BN, true, true>(tA, tB, p, grid, s) : launch<BN, true, false>(tA, tB, p, grid, s);
-    return b_mn ? launch<BN, false, true>(tA, tB, p, grid, s) : launch<BN, false, false>(tA, tB, p, grid, s);
+lrd_status_t launch_major(bool a_mn, bool b_mn, const TcLaunch<1>& L, dim3 grid, cudaStream_t s) {
+    if (a_mn) return b_mn ? launch<BN, true, true>(L, grid, s) : launch<BN, true, false>(L, grid, s);
+    return b_mn ? launch<BN, false, true>(L, grid, s) : launch<BN, false, false>(L, grid, s);
 }
 
 inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -730,7 +746,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     } else if (allow_split) {
         const SplitPlan sp = pick_split(g.M, g.N, g.K, ones, g.max_cluster_split);
         // where the tiles leave no room for a cluster per tile
-        if (tc_wgrad_pair_estimate(g) < 0.95 * split_estimate(sp, g.M, g.N, g.K)) return tc_wgrad_pair(g, stream);
+        if (tc_wgrad_pair_estimate(&g, 1) < 0.95 * split_estimate(sp, g.M, g.N, g.K)) return tc_wgrad_pair(&g, 1, stream);
         bn = sp.bn; cluster = sp.cluster; splits = sp.global;
     } else {
         bn = pick_bn(g.M, g.N, false);
@@ -744,7 +760,8 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     const int zdim = cluster > 1 ? cluster : splits;
     const int kb_per = (kb_total + zdim - 1) / zdim;
 
-    CUtensorMap tA, tB;
+    TcLaunch<1> L{};
+    CUtensorMap &tA = L.tA[0], &tB = L.tB[0];
     const uint32_t kbox = BK * stage_kblocks(bn, ones);             // k rows of an MN-major box
     bool ok = g.a_mn_major ? make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, kbox, 64)
                            : make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda, BM, BK);
@@ -752,7 +769,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
                              : make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb, (uint32_t)bn, BK));
     if (!ok) return LRD_ERR_CUDA;
 
-    TcParams p{};
+    TcParams& p = L.p[0];
     p.M = g.M; p.N = g.N; p.ldp = ldp; p.kb_total = kb_total; p.kb_per_split = kb_per;
     p.partial = splits > 1 ? 1 : 0;
     p.cluster_splits = cluster;
@@ -766,16 +783,16 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     lrd_status_t st;
     if (ones) {
         switch (bn) {
-            case 192: st = launch<192, true, true, true>(tA, tB, p, grid, stream); break;
-            case 128: st = launch<128, true, true, true>(tA, tB, p, grid, stream); break;
-            default:  st = launch<64, true, true, true>(tA, tB, p, grid, stream); break;
+            case 192: st = launch<192, true, true, true>(L, grid, stream); break;
+            case 128: st = launch<128, true, true, true>(L, grid, stream); break;
+            default:  st = launch<64, true, true, true>(L, grid, stream); break;
         }
     } else
     switch (bn) {
-        case 256: st = launch_major<256>(g.a_mn_major, g.b_mn_major, tA, tB, p, grid, stream); break;
-        case 192: st = launch_major<192>(g.a_mn_major, g.b_mn_major, tA, tB, p, grid, stream); break;
-        case 128: st = launch_major<128>(g.a_mn_major, g.b_mn_major, tA, tB, p, grid, stream); break;
-        default:  st = launch_major<64>(g.a_mn_major, g.b_mn_major, tA, tB, p, grid, stream); break;
+        case 256: st = launch_major<256>(g.a_mn_major, g.b_mn_major, L, grid, stream); break;
+        case 192: st = launch_major<192>(g.a_mn_major, g.b_mn_major, L, grid, stream); break;
+        case 128: st = launch_major<128>(g.a_mn_major, g.b_mn_major, L, grid, stream); break;
+        default:  st = launch_major<64>(g.a_mn_major, g.b_mn_major, L, grid, stream); break;
     }
     if (st != LRD_OK || splits == 1) return st;
     const int64_t work = g.M * ((g.N + 3) / 4) + (ones ? g.M : 0);
@@ -786,6 +803,89 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
 }
 
+// Estimated microseconds of one launch for all of g's products, one 128 x bn tile and cluster of S blocks each (S = 1: waves
+// of single blocks), by the same terms as split_estimate.
+static double group_estimate(const GemmArgs* g, int n, int bn, int S) {
+    int64_t tiles = 0, deepest = 0;
+    double bytes = 0.0;
+    const double kb_bytes = BM * BK * 2.0 + bn * BK * 2.0;
+    for (int i = 0; i < n; ++i) {
+        const int64_t t = ((g[i].M + BM - 1) / BM) * ((g[i].N + bn - 1) / bn), kb = ((g[i].K + BK - 1) / BK + S - 1) / S;
+        tiles += t;
+        deepest = std::max(deepest, kb);
+        bytes += (double)(t * S * kb) * kb_bytes;
+    }
+    if (S > 1) return tiles > max_active_clusters(S) ? 1e300 : 5.0 + 0.8e6 * std::max((double)deepest * kb_bytes / 110e9, bytes / 14e12);
+    return 4.0 + (double)((tiles + kNumSms - 1) / kNumSms * deepest) * std::max(0.2, 0.0017 * bn);
+}
+
+template <int BN, bool ONES>
+static lrd_status_t launch_group(const GemmArgs* g, int n, int S, cudaStream_t stream) {
+    TcLaunch<kMaxWgrads> L{};
+    unsigned nx = 0, ny = 0;
+    const uint32_t kbox = BK * Cfg<BN, ONES>::G;
+    for (int i = 0; i < kMaxWgrads; ++i) {
+        L.row0[i] = i < n ? (int)ny : INT_MAX;
+        if (i >= n) continue;
+        if (!make_tmap_2d_bf16(&L.tA[i], g[i].A, (uint64_t)g[i].K, (uint64_t)g[i].M, (uint64_t)g[i].lda, kbox, 64) ||
+            !make_tmap_2d_bf16(&L.tB[i], g[i].B, (uint64_t)g[i].K, (uint64_t)g[i].N, (uint64_t)g[i].ldb, kbox, 64))
+            return LRD_ERR_CUDA;
+        TcParams& p = L.p[i];
+        p.M = g[i].M; p.N = g[i].N; p.ldp = g[i].N;
+        p.kb_total = (int)((g[i].K + BK - 1) / BK);
+        p.kb_per_split = (p.kb_total + S - 1) / S;
+        p.cluster_splits = S;
+        p.timeout_flag = device_timeout_flag();
+        p.C = g[i].C; p.ldc = g[i].ldc;
+        p.colsum_out = (__nv_bfloat16*)g[i].a_colsum;
+        nx = std::max(nx, (unsigned)((g[i].N + BN - 1) / BN));
+        ny += (unsigned)((g[i].M + BM - 1) / BM);
+    }
+    return launch<BN, true, true, ONES, false, kMaxWgrads>(L, dim3(nx, ny, (unsigned)S), stream, !g[0].in_turn);
+}
+
+// The weight gradients of one backward pass.  Each alone has few output tiles and one pays for its launch, its first loads and
+// its exchange over a chip that is mostly idle, so as many as the caller has at hand go into one launch, on single SMs
+// (a cluster per tile) or on pairs, when the estimate is below the sum of theirs.  Forward and backward of a layer with nothing
+// frozen, each alone / together: 4096 -> 4096 at rank 512, 8192 tokens 189 / 182 us; rank 256 142 / 132; 768 -> 3072 at 384,
+// 4096 tokens 73 / 62; 1024 -> 4096 at 512, 1024 tokens 48 / 42; 768 -> 768 at 192, 300 tokens 30 / 21.
+lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const size_t* partial_bytes, cudaStream_t stream) {
+    bool ones = false, together = n > 1 && n <= kMaxWgrads;
+    int64_t rows = 0;
+    double separate = 0.0;
+    for (int i = 0; i < n && together; ++i) {
+        together = tc_gemm_eligible(g[i]) && g[i].a_mn_major && g[i].b_mn_major && !g[i].bias && g[i].max_cluster_split == g[0].max_cluster_split;
+        if (!together) break;
+        ones = ones || g[i].a_colsum;
+        rows += (g[i].M + BM - 1) / BM;
+        separate += std::min(split_estimate(pick_split(g[i].M, g[i].N, g[i].K, g[i].a_colsum != nullptr, g[i].max_cluster_split), g[i].M, g[i].N, g[i].K),
+                             tc_wgrad_pair_estimate(&g[i], 1));
+    }
+    if (together && rows <= 65535) {
+        const int top = g[0].max_cluster_split >= 2 && g[0].max_cluster_split < kMaxClusterSplits ? g[0].max_cluster_split : kMaxClusterSplits;
+        int bn = 0, S = 1;
+        double us = separate;
+        for (int b : {192, 128, 64})
+            for (int c = top; c >= 1; --c) {
+                if (b % (8 * c)) continue;
+                const double t = group_estimate(g, n, b, c);
+                if (t < us) { us = t; bn = b; S = c; }
+            }
+        if (tc_wgrad_pair_estimate(g, n) < us) return tc_wgrad_pair(g, n, stream);
+        switch (bn) {
+            case 192: return ones ? launch_group<192, true>(g, n, S, stream) : launch_group<192, false>(g, n, S, stream);
+            case 128: return ones ? launch_group<128, true>(g, n, S, stream) : launch_group<128, false>(g, n, S, stream);
+            case 64:  return ones ? launch_group<64, true>(g, n, S, stream) : launch_group<64, false>(g, n, S, stream);
+            default:  break;
+        }
+    }
+    for (int i = 0; i < n; ++i) {
+        const lrd_status_t st = tc_gemm(g[i], true, partials[i], partial_bytes[i], stream);
+        if (st != LRD_OK) return st;
+    }
+    return LRD_OK;
+}
+
 // Filter gradient (see CONV above): M = co, N = taps x 64-column blocks, K = output pixels.
 lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co,
                             cudaStream_t stream) {
@@ -793,12 +893,13 @@ lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t 
     const int64_t P = B * g.Ho * g.Wo, taps = (int64_t)g.k * g.k, nkc = (ci + 63) / 64, N = taps * nkc * 64;
     SplitPlan sp = pick_split(co, N, P, true);             // (tiles of at most 192 columns)
     if (sp.cluster < 2) sp.cluster = 1;                    // tiles enough to fill the GPU: each reduces over all pixels
-    CUtensorMap tA, tB;
+    TcLaunch<1> L{};
+    CUtensorMap &tA = L.tA[0], &tB = L.tB[0];
     const uint32_t kbox = BK * stage_kblocks(sp.bn, false);
     bool ok = make_tmap_2d_bf16(&tA, dout, (uint64_t)P, (uint64_t)co, (uint64_t)co, kbox, 64);
     ok = ok && make_tmap_im2col_bf16(&tB, in, (uint64_t)B, (uint64_t)g.H, (uint64_t)g.W, (uint64_t)ci, -g.pad, -g.pad, g.Ho, g.Wo, g.stride, kbox);
     if (!ok) return LRD_ERR_CUDA;
-    TcParams p{};
+    TcParams& p = L.p[0];
     p.M = co; p.N = N; p.ldp = N;
     p.kb_total = (int)((P + BK - 1) / BK);
     p.kb_per_split = (p.kb_total + sp.cluster - 1) / sp.cluster;
@@ -809,9 +910,9 @@ lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t 
     p.cv_Ho = g.Ho; p.cv_Wo = g.Wo; p.cv_stride = g.stride; p.cv_pad = g.pad;
     dim3 grid((unsigned)((N + sp.bn - 1) / sp.bn), (unsigned)((co + BM - 1) / BM), (unsigned)sp.cluster);
     switch (sp.bn) {
-        case 192: return launch<192, true, true, false, true>(tA, tB, p, grid, stream);
-        case 128: return launch<128, true, true, false, true>(tA, tB, p, grid, stream);
-        default:  return launch<64, true, true, false, true>(tA, tB, p, grid, stream);
+        case 192: return launch<192, true, true, false, true>(L, grid, stream);
+        case 128: return launch<128, true, true, false, true>(L, grid, stream);
+        default:  return launch<64, true, true, false, true>(L, grid, stream);
     }
 }
 

@@ -17,6 +17,7 @@
 // Warp 0: TMA producer.  Warp 1: tensor memory, in the even block MMA issue.  Warps 2-9: reduction and stores.
 // Every wait is bounded; a wait that runs out raises the device timeout flag and the cluster tears down in order.
 #include <algorithm>
+#include <climits>
 
 #include "common.cuh"
 #include "ptx_pair.cuh"
@@ -44,10 +45,17 @@ template <int BN> struct Cfg {
 
 struct WgradParams {
     int64_t M, N, ldc;
-    int kb_total, kb_per_pair, pairs;
+    int kb_total, kb_per_pair;
     __nv_bfloat16* C;
     __nv_bfloat16* colsum;        // [M] or nullptr
+};
+// NP independent products at most: their row tiles follow one another in gridDim.z.
+template <int NP> struct WgradLaunch {
     unsigned int* timeout_flag;
+    int pairs;
+    int row0[NP];                 // first row tile of each (INT_MAX: none)
+    WgradParams p[NP];
+    CUtensorMap tA[NP], tB[NP];
 };
 
 // 16 columns of one row, rounded once
@@ -75,9 +83,16 @@ __device__ __forceinline__ void store16(const WgradParams& p, int64_t row, int64
 }
 
 // grid: (2 pairs = one cluster, column tiles, row tiles of 256)
-template <int BN>
+template <int BN, int NP>
 __global__ void __launch_bounds__(kThreads, 1)
-wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const WgradParams p) {
+wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
+    int prod = 0;
+#pragma unroll
+    for (int i = 1; i < NP; ++i)
+        if ((int)blockIdx.z >= L.row0[i]) prod = i;
+    const CUtensorMap &tmA = L.tA[prod], &tmB = L.tB[prod];
+    const WgradParams p = L.p[prod];
+    if (NP > 1 && (int64_t)blockIdx.y * BN >= p.N) return;         // (the whole cluster: its blocks share y and z)
     using C = Cfg<BN>;
     constexpr int STAGES = C::STAGES, G = C::G;
     extern __shared__ uint8_t smem_raw[];
@@ -85,13 +100,13 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
     const uint32_t ring_base = (smem_u32(smem_raw) + 1023u) & ~1023u, ones_base = ring_base + kRingBytes;
-    const AbortCtx ab{&abort_flag, p.timeout_flag};
+    const AbortCtx ab{&abort_flag, L.timeout_flag};
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
     const uint32_t crank = cluster_ctarank();
-    const int S = p.pairs, pr = (int)(crank >> 1), h = (int)(crank & 1u);
+    const int S = L.pairs, pr = (int)(crank >> 1), h = (int)(crank & 1u);
     const uint32_t lead_rank = crank & ~1u;
     const uint16_t pair_mask = (uint16_t)(3u << lead_rank);
-    const int m0 = (int)blockIdx.z * 256 + h * 128, n0 = (int)blockIdx.y * BN;
+    const int m0 = ((int)blockIdx.z - (NP > 1 ? L.row0[prod] : 0)) * 256 + h * 128, n0 = (int)blockIdx.y * BN;
     const int kb_begin = min(pr * p.kb_per_pair, p.kb_total), kb_end = min(kb_begin + p.kb_per_pair, p.kb_total);
     const bool sums = p.colsum != nullptr && blockIdx.y == 0;
     const uint32_t cs = (uint32_t)(BN / S), chunk_bytes = 128u * cs * 4u;       // columns this block owns; one slice of them
@@ -312,8 +327,9 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 }
 
 bool set_attributes() {
-    return cudaFuncSetAttribute(wgrad_pair_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) == cudaSuccess &&
-           cudaFuncSetAttribute(wgrad_pair_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) == cudaSuccess;
+    auto one = [](const void* f) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) == cudaSuccess; };
+    return one((const void*)wgrad_pair_kernel<256, 1>) && one((const void*)wgrad_pair_kernel<128, 1>) &&
+           one((const void*)wgrad_pair_kernel<256, kMaxWgrads>);
 }
 
 // Clusters of n blocks that can be resident at once.
@@ -333,7 +349,7 @@ int max_active_clusters(int n) {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (!set_attributes() || cudaOccupancyMaxActiveClusters(&cnt, wgrad_pair_kernel<256>, &cfg) != cudaSuccess || cnt < 1) {
+        if (!set_attributes() || cudaOccupancyMaxActiveClusters(&cnt, wgrad_pair_kernel<256, 1>, &cfg) != cudaSuccess || cnt < 1) {
             cudaGetLastError();
             cnt = (kNumSms - 20) / n;
         }
@@ -346,13 +362,20 @@ struct Plan { int bn, pairs; double us; };
 
 // Estimated microseconds: 3 of launch and first loads, the k-blocks of a pair's share, 1.5 of stores, 2.5 of exchange (measured
 // at 4096 x 512 over 8192 tokens: 256 wide one pair 54.9, two 33.3, 128 wide one pair 36.0).
-Plan make_plan(int64_t M, int64_t N, int64_t K, bool sums, int max_cluster) {
+Plan make_plan(const GemmArgs* g, int n) {
     Plan best{0, 0, 1e300};
-    const int64_t kb = (K + BK - 1) / BK;
+    bool sums = false;
+    int64_t kb = 0;
+    for (int i = 0; i < n; ++i) {
+        sums = sums || g[i].a_colsum;
+        kb = std::max(kb, (g[i].K + BK - 1) / BK);
+    }
     for (int bn : {256, 128}) {
-        const int64_t tiles = ((M + 255) / 256) * ((N + bn - 1) / bn);
+        if (n > 1 && bn == 128) continue;                 // several products fill the narrow tiles' SMs better as single blocks
+        int64_t tiles = 0;
+        for (int i = 0; i < n; ++i) tiles += ((g[i].M + 255) / 256) * ((g[i].N + bn - 1) / bn);
         for (int S = kMaxPairs; S >= 1; S /= 2) {
-            if ((max_cluster && 2 * S > max_cluster) || S > kb) continue;
+            if ((g[0].max_cluster_split && 2 * S > g[0].max_cluster_split) || S > kb) continue;
             const int64_t room = max_active_clusters(2 * S), waves = (tiles + room - 1) / room;
             if (S > 1 && waves > 1) continue;
             const double per = (bn == 256 ? 0.40 : 0.25) + (sums ? 0.01 : 0.0);
@@ -365,27 +388,38 @@ Plan make_plan(int64_t M, int64_t N, int64_t K, bool sums, int max_cluster) {
 
 }  // namespace
 
-double tc_wgrad_pair_estimate(const GemmArgs& g) {
-    if (!tc_gemm_eligible(g) || !g.a_mn_major || !g.b_mn_major || g.bias || g.M > (int64_t)65535 * 256 || g.N > (int64_t)65535 * 128) return 1e300;
-    return make_plan(g.M, g.N, g.K, g.a_colsum != nullptr, g.max_cluster_split).us;
+double tc_wgrad_pair_estimate(const GemmArgs* g, int n) {
+    int64_t rows = 0;
+    if (n > kMaxWgrads) return 1e300;
+    for (int i = 0; i < n; ++i) {
+        if (!tc_gemm_eligible(g[i]) || !g[i].a_mn_major || !g[i].b_mn_major || g[i].bias || g[i].N > (int64_t)65535 * 128) return 1e300;
+        rows += (g[i].M + 255) / 256;
+    }
+    return rows > 65535 ? 1e300 : make_plan(g, n).us;
 }
 
-lrd_status_t tc_wgrad_pair(const GemmArgs& g, cudaStream_t stream) {
-    if (tc_wgrad_pair_estimate(g) >= 1e300) return LRD_ERR_UNSUPPORTED;
-    const Plan pl = make_plan(g.M, g.N, g.K, g.a_colsum != nullptr, g.max_cluster_split);
+template <int NP>
+static lrd_status_t launch(const GemmArgs* g, int n, const Plan& pl, cudaStream_t stream) {
     const uint32_t box = BK * (uint32_t)(pl.bn == 256 ? Cfg<256>::G : Cfg<128>::G);
-    CUtensorMap tA, tB;
-    if (!make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, box, 64) ||
-        !make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb, box, 64))
-        return LRD_ERR_CUDA;
-    WgradParams p{};
-    p.M = g.M; p.N = g.N; p.ldc = g.ldc;
-    p.kb_total = (int)((g.K + BK - 1) / BK);
-    p.pairs = pl.pairs;
-    p.kb_per_pair = (p.kb_total + pl.pairs - 1) / pl.pairs;
-    p.C = (__nv_bfloat16*)g.C;
-    p.colsum = (__nv_bfloat16*)g.a_colsum;
-    p.timeout_flag = device_timeout_flag();
+    WgradLaunch<NP> L{};
+    unsigned ny = 0, nz = 0;
+    for (int i = 0; i < NP; ++i) {
+        L.row0[i] = i < n ? (int)nz : INT_MAX;
+        if (i >= n) continue;
+        if (!make_tmap_2d_bf16(&L.tA[i], g[i].A, (uint64_t)g[i].K, (uint64_t)g[i].M, (uint64_t)g[i].lda, box, 64) ||
+            !make_tmap_2d_bf16(&L.tB[i], g[i].B, (uint64_t)g[i].K, (uint64_t)g[i].N, (uint64_t)g[i].ldb, box, 64))
+            return LRD_ERR_CUDA;
+        WgradParams& p = L.p[i];
+        p.M = g[i].M; p.N = g[i].N; p.ldc = g[i].ldc;
+        p.kb_total = (int)((g[i].K + BK - 1) / BK);
+        p.kb_per_pair = (p.kb_total + pl.pairs - 1) / pl.pairs;
+        p.C = (__nv_bfloat16*)g[i].C;
+        p.colsum = (__nv_bfloat16*)g[i].a_colsum;
+        ny = std::max(ny, (unsigned)((g[i].N + pl.bn - 1) / pl.bn));
+        nz += (unsigned)((g[i].M + 255) / 256);
+    }
+    L.pairs = pl.pairs;
+    L.timeout_flag = device_timeout_flag();
     static bool configured_on[kMaxDevices] = {};
     bool& configured = configured_on[device_slot()];
     if (!configured) {
@@ -393,7 +427,7 @@ lrd_status_t tc_wgrad_pair(const GemmArgs& g, cudaStream_t stream) {
         configured = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * pl.pairs), (unsigned)((g.N + pl.bn - 1) / pl.bn), (unsigned)((g.M + 255) / 256));
+    cfg.gridDim = dim3((unsigned)(2 * pl.pairs), ny, nz);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = stream;
@@ -403,13 +437,21 @@ lrd_status_t tc_wgrad_pair(const GemmArgs& g, cudaStream_t stream) {
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) before it touches global memory
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].val.programmaticStreamSerializationAllowed = g[0].in_turn ? 0 : 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const cudaError_t e = pl.bn == 256 ? cudaLaunchKernelEx(&cfg, wgrad_pair_kernel<256>, tA, tB, p) : cudaLaunchKernelEx(&cfg, wgrad_pair_kernel<128>, tA, tB, p);
+    cudaError_t e;
+    if constexpr (NP == 1) e = pl.bn == 256 ? cudaLaunchKernelEx(&cfg, wgrad_pair_kernel<256, 1>, L) : cudaLaunchKernelEx(&cfg, wgrad_pair_kernel<128, 1>, L);
+    else e = cudaLaunchKernelEx(&cfg, wgrad_pair_kernel<256, NP>, L);
     if (!cuda_ok(e, "cudaLaunchKernelEx(weight gradient on pairs)")) return LRD_ERR_CUDA;
     count_launch();
     return LRD_OK;
+}
+
+lrd_status_t tc_wgrad_pair(const GemmArgs* g, int n, cudaStream_t stream) {
+    if (tc_wgrad_pair_estimate(g, n) >= 1e300) return LRD_ERR_UNSUPPORTED;
+    const Plan pl = make_plan(g, n);
+    return n == 1 ? launch<1>(g, n, pl, stream) : launch<kMaxWgrads>(g, n, pl, stream);
 }
 
 }  // namespace lrd
