@@ -649,46 +649,46 @@ struct SplitPlan {
     int global;      // > 1: global split (partials in scratch memory + reduce kernel)
 };
 
-// Cluster split: the time of one block is its operand traffic (every block streams its share of A and
-// B through one SM's memory port); all blocks together must not exceed what L2 delivers.  The
-// candidates are tile widths that the reduction buffers fit (<= 192) and cluster sizes that divide
-// the tile into slices of whole 16-byte groups.
-static SplitPlan pick_split(int64_t M, int64_t N, int64_t K, bool ones, int max_cluster = 0) {
+// Estimated microseconds of weight gradients in one launch: `tiles` of 128 x bn, each in a cluster of S blocks (1: waves of
+// single blocks), `deepest` k-blocks in the longest share and `kblocks` in all.  A block's time is its operand traffic (every
+// block streams its share of A and B through one SM's memory port, all together through what L2 delivers), and a split adds
+// the exchange, which grows with the tile.  Measured / estimated: 3072 x 384 over 4096 tokens (192 wide, 2 blocks) 14.8 / 15.3;
+// over 16384 40.8 / 40.4; 768 x 192 over 4096 (64, 4) 7.1 / 6.7; 1536 x 384 over 2048 (192, 4) 9.4 / 9.1; 4096 x 256 over 8192
+// (128, 2) 19.9 / 18.9.  Short reductions and many tiles are better left whole (no exchange): 3072 x 384 over 4096 tokens 14.9 us
+// in clusters of 2, 12.5 in 144 blocks 64 wide; over 512 6.8 / 5.1; 1536 x 384 over 2048 9.6 / 7.0.
+static double split_us(int bn, int S, int64_t tiles, int64_t deepest, int64_t kblocks) {
+    const double kb_bytes = BM * BK * 2.0 + bn * BK * 2.0;
+    if (S > 1) return 4.2 + 0.022 * (bn - 64) + std::max(0.7e6 * (double)deepest * kb_bytes / 110e9, 0.8e6 * (double)kblocks * kb_bytes / 14e12);
+    const int64_t waves = (tiles + kNumSms - 1) / kNumSms;
+    return 2.5 + 0.006 * (bn - 64) + (double)(waves * deepest) * std::max(0.2, 0.0017 * bn) + 3.0 * (double)(waves - 1);
+}
+
+// One weight gradient: the candidates are tile widths that the reduction buffers fit (<= 192) and cluster sizes that divide
+// the tile into slices of whole 16-byte groups; where no cluster per tile fits, single blocks or shares through scratch memory.
+// A launch that runs beside a data chain (clusters of at most 2) gets some 50 SMs: few wide blocks, always split, leave most
+// of them to others (step of a block of 768-wide layers, U frozen: 182 us with the plans of a launch that runs alone, 178.5 so).
+static SplitPlan pick_split(int64_t M, int64_t N, int64_t K, bool ones, int max_cluster = 0, double* us = nullptr) {
     const int top = max_cluster >= 2 && max_cluster < kMaxClusterSplits ? max_cluster : kMaxClusterSplits;
     const int64_t mt = (M + BM - 1) / BM, kb = (K + BK - 1) / BK;
     SplitPlan best{pick_bn(M, N, true), 1, 1};
     if (ones && best.bn > 192) best.bn = 192;
     best.global = global_splits(M, N, K, best.bn);
-    double best_t = 1e300;
-    const int bns[3] = {192, 128, 64};
-    for (int bn : bns) {
-        const int64_t nt = (N + bn - 1) / bn;
+    const int64_t tiles0 = mt * ((N + best.bn - 1) / best.bn), share = (kb + best.global - 1) / best.global;
+    double best_t = split_us(best.bn, 1, tiles0 * best.global, share, 0) + (best.global > 1 ? 8.0 + 8e6 * (double)(best.global * M * N) / 5e12 : 0.0);     // + partials out and in, one more launch
+    for (int bn : {192, 128, 64}) {
+        const int64_t nt = (N + bn - 1) / bn, tiles = mt * nt;
         if (nt * bn >= N + 64 && bn > 64) continue;              // a narrower width covers N with less waste
-        const int64_t tiles = mt * nt;
-        for (int S = top; S >= 2; --S) {
-            if (bn % (8 * S)) continue;
-            if (tiles > max_active_clusters(S) || S > kb) continue;    // one wave: a second wave would double the time
-            const double per_block = (double)((kb + S - 1) / S) * (BM * BK * 2.0 + bn * BK * 2.0);
-            const double t = std::max(per_block / 110e9, per_block * (double)(tiles * S) / 11.5e12) + 2e-6 * bn / 192.0;
+        for (int S = top; S >= 1; --S) {
+            if (bn % (8 * S) || S > kb || (S == 1 && top == 2)) continue;
+            if (S > 1 && tiles > max_active_clusters(S)) continue;     // one wave: a second wave would double the time
+            const int64_t per = (kb + S - 1) / S;
+            double t = split_us(bn, S, tiles, per, tiles * S * per);
+            if (top == 2) t = 3.0 + 0.8e6 * std::max((double)per * (BM + bn) * 128.0 / 110e9, (double)(tiles * S * per) * (BM + bn) * 128.0 / 11.5e12) + bn / 120.0;
             if (t < best_t) { best_t = t; best.bn = bn; best.cluster = S; best.global = 1; }
-            break;                                                // the largest feasible cluster for this width
         }
     }
+    if (us) *us = best_t;
     return best;
-}
-
-// Estimated microseconds of a weight gradient under a plan, against the kernel on pairs of SMs (tc_wgrad_pair.cu).  Fitted to
-// 3072 x 384 over 4096 tokens (cluster of 2: 14.8 us, estimate 14.5; pairs 20.2), 4096 x 256 over 8192 (20; 20.2; pairs 21.9),
-// 4096 x 512 over 8192 (two shares through scratch memory: 37.1; 39.8; pairs 32.9), 4096 x 1024 over 1024 with sums (two waves
-// of tiles 192 wide: 16.2; 14.4; pairs 11.8).
-static double split_estimate(const SplitPlan& sp, int64_t M, int64_t N, int64_t K) {
-    const int64_t tiles = ((M + BM - 1) / BM) * ((N + sp.bn - 1) / sp.bn), kb = (K + BK - 1) / BK;
-    if (sp.cluster > 1) {
-        const double per_block = (double)((kb + sp.cluster - 1) / sp.cluster) * (BM * BK * 2.0 + sp.bn * BK * 2.0);
-        return 5.0 + 0.8e6 * std::max(per_block / 110e9, per_block * (double)(tiles * sp.cluster) / 14e12);
-    }
-    const int64_t waves = (tiles * sp.global + kNumSms - 1) / kNumSms;
-    return 4.0 + (double)(waves * ((kb + sp.global - 1) / sp.global)) * std::max(0.2, 0.0017 * sp.bn) + (sp.global > 1 ? 8.0 : 0.0);
 }
 
 // A data product with few tiles and a long reduction (a short batch through a wide layer) is the latency of one tile's
@@ -744,9 +744,10 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
         if (!split_data_product(g.M, g.N, g.K, &dp, &us)) return tc_gemm_persistent(g, stream);
         bn = dp.bn; cluster = dp.cluster;
     } else if (allow_split) {
-        const SplitPlan sp = pick_split(g.M, g.N, g.K, ones, g.max_cluster_split);
+        double us;
+        const SplitPlan sp = pick_split(g.M, g.N, g.K, ones, g.max_cluster_split, &us);
         // where the tiles leave no room for a cluster per tile
-        if (tc_wgrad_pair_estimate(&g, 1) < 0.95 * split_estimate(sp, g.M, g.N, g.K)) return tc_wgrad_pair(&g, 1, stream);
+        if (tc_wgrad_pair_estimate(&g, 1) < 0.95 * us) return tc_wgrad_pair(&g, 1, stream);
         bn = sp.bn; cluster = sp.cluster; splits = sp.global;
     } else {
         bn = pick_bn(g.M, g.N, false);
@@ -803,20 +804,16 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
 }
 
-// Estimated microseconds of one launch for all of g's products, one 128 x bn tile and cluster of S blocks each (S = 1: waves
-// of single blocks), by the same terms as split_estimate.
+// Estimated microseconds of one launch for all of g's products, with one width and cluster size.
 static double group_estimate(const GemmArgs* g, int n, int bn, int S) {
-    int64_t tiles = 0, deepest = 0;
-    double bytes = 0.0;
-    const double kb_bytes = BM * BK * 2.0 + bn * BK * 2.0;
+    int64_t tiles = 0, deepest = 0, kblocks = 0;
     for (int i = 0; i < n; ++i) {
         const int64_t t = ((g[i].M + BM - 1) / BM) * ((g[i].N + bn - 1) / bn), kb = ((g[i].K + BK - 1) / BK + S - 1) / S;
         tiles += t;
         deepest = std::max(deepest, kb);
-        bytes += (double)(t * S * kb) * kb_bytes;
+        kblocks += t * S * kb;
     }
-    if (S > 1) return tiles > max_active_clusters(S) ? 1e300 : 5.0 + 0.8e6 * std::max((double)deepest * kb_bytes / 110e9, bytes / 14e12);
-    return 4.0 + (double)((tiles + kNumSms - 1) / kNumSms * deepest) * std::max(0.2, 0.0017 * bn);
+    return S > 1 && tiles > max_active_clusters(S) ? 1e300 : split_us(bn, S, tiles, deepest, kblocks);
 }
 
 template <int BN, bool ONES>
@@ -858,8 +855,9 @@ lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const s
         if (!together) break;
         ones = ones || g[i].a_colsum;
         rows += (g[i].M + BM - 1) / BM;
-        separate += std::min(split_estimate(pick_split(g[i].M, g[i].N, g[i].K, g[i].a_colsum != nullptr, g[i].max_cluster_split), g[i].M, g[i].N, g[i].K),
-                             tc_wgrad_pair_estimate(&g[i], 1));
+        double us;
+        pick_split(g[i].M, g[i].N, g[i].K, g[i].a_colsum != nullptr, g[i].max_cluster_split, &us);
+        separate += std::min(us, tc_wgrad_pair_estimate(&g[i], 1));
     }
     if (together && rows <= 65535) {
         const int top = g[0].max_cluster_split >= 2 && g[0].max_cluster_split < kMaxClusterSplits ? g[0].max_cluster_split : kMaxClusterSplits;

@@ -11,8 +11,8 @@ from helpers import check_linear, run_linear
 pytestmark = pytest.mark.gpu
 
 
-# the estimates send these to (tile width, pairs): 128 x 1, 256 x 1, 128 x 2, 256 x 2, 128 x 4, 256 x 4 (twice)
-@pytest.mark.parametrize("shape", [(130, 520, 2056), (300, 3528, 1000), (2050, 264, 2056), (5000, 3528, 264), (9000, 1032, 248), (1021, 1032, 520), (1000, 2600, 248)])
+# the estimates send these to (tile width, pairs): 128 x 1, 256 x 1, 256 x 1, 256 x 2, 256 x 4
+@pytest.mark.parametrize("shape", [(60, 1032, 4096), (300, 3528, 1000), (1021, 4096, 1288), (5000, 264, 4096), (5000, 1032, 520)])
 def test_dense_weight_gradient(shape):
     """The undecomposed layer's dW and bias gradient."""
     M, K, N = shape
