@@ -38,6 +38,8 @@ struct GemmArgs {
     int max_cluster_split = 0; // split weight gradients: largest cluster to split the reduction over (0 = automatic).  A
                                // launch meant to run BESIDE others asks for 2: clusters of 4 or 8 need that many free
                                // SMs inside one GPC, which a chain kernel on 128 of the 148 SMs never leaves
+    bool add = false;          // weight gradients on the tensor-core kernels: C (and a_colsum) += the product, rounded to the storage
+                               // type before the fp32 sum and after it
     bool in_turn = false;      // weight gradients: started only when the launch before has ended (blocks that wait on an SM for
                                // that end keep it from work in other streams)
 };

@@ -329,5 +329,14 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// two bf16 sums, each fp32 and rounded once
+__device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
+    return pack_bf16(__uint_as_float(a << 16) + __uint_as_float(b << 16), __uint_as_float(a & 0xFFFF0000u) + __uint_as_float(b & 0xFFFF0000u));
+}
+__device__ __forceinline__ void add_into_bf16(__nv_bfloat16* dst, float x) {
+    *dst = __float2bfloat16_rn(__bfloat162float(*dst) + __bfloat162float(__float2bfloat16_rn(x)));
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 }  // namespace ptx
 }  // namespace lrd

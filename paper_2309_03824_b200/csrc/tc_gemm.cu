@@ -68,6 +68,7 @@ struct TcParams {
     int64_t ldc;
     const __nv_bfloat16* bias;
     int partial;        // 1: write fp32 partials
+    int add;            // C += the product rounded to bf16 (fp32 sum, one more rounding) instead of C = it; column sums too
     int cluster_splits; // > 1: the gridDim.z blocks of a tile are one cluster and reduce through shared memory
     // CONV: input channels, 64-column blocks of a tap and of all taps, k of the k x k taps, output grid, stride, pad
     int cv_ci, cv_nkc, cv_nblk, cv_k, cv_Ho, cv_Wo, cv_stride, cv_pad;
@@ -83,6 +84,10 @@ template <int NP> struct TcLaunch {
     TcParams p[NP];
     CUtensorMap tA[NP], tB[NP];
 };
+
+__device__ __forceinline__ uint4 add_bf16x8(const uint4& a, const uint4& b) {
+    return make_uint4(add_bf16x2(a.x, b.x), add_bf16x2(a.y, b.y), add_bf16x2(a.z, b.z), add_bf16x2(a.w, b.w));
+}
 
 // CONV: column of dG (= tap * ci + channel) that column `col` of the product belongs to; -1: padding
 __device__ __forceinline__ int conv_col(const TcParams& p, int col) {
@@ -254,6 +259,11 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         const uint32_t chunk_bytes = 128u * cs * 4u, ngrp = cs / 4u;
         const uint32_t stage_base = smem_base, recv_base = smem_base + 128u * BN * 4u;
         const uint32_t cs_stage = recv_base + 128u * BN * 4u, cs_recv = cs_stage + 512u;
+        if (p.add) {           // what this block's slice adds to, on its way while the products are formed
+            const int64_t grow = (int64_t)m0 + row, gcol0 = (int64_t)n0 + self * cs;
+            for (uint32_t c = 0; c < cs; c += 64)
+                if (grow < p.M && gcol0 + c < p.N) prefetch_l2((const __nv_bfloat16*)p.C + grow * p.ldc + gcol0 + c);
+        }
         bool ok = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         // barrier 1: this block's pipeline ring is dead (all its MMAs have completed).  Progress only: what the peers
@@ -352,10 +362,15 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                 if (CONV && at < 0) return;
                 __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + at;
                 if (CONV || col + 8 <= p.N) {
-                    *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+                    uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+                    if (!CONV && p.add) v = add_bf16x8(v, *reinterpret_cast<const uint4*>(dst));
+                    *reinterpret_cast<uint4*>(dst) = v;
                 } else {
                     for (int e = 0; e < 8; ++e)
-                        if (col + e < p.N) dst[e] = __float2bfloat16_rn(acc[e]);
+                        if (col + e < p.N) {
+                            if (p.add) add_into_bf16(dst + e, acc[e]);
+                            else dst[e] = __float2bfloat16_rn(acc[e]);
+                        }
                 }
             };
             // 16 columns (one whole 32-byte sector) per store instruction where the layout allows, else two 16-byte stores
@@ -371,6 +386,12 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                     const int64_t at = CONV ? conv_col(p, (int)col) : col;
                     if (CONV && at < 0) continue;
                     __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + at;
+                    if (!CONV && p.add) {
+                        const uint4 o0 = reinterpret_cast<const uint4*>(dst)[0], o1 = reinterpret_cast<const uint4*>(dst)[1];
+                        const uint4 s0 = add_bf16x8(make_uint4(w0[0], w0[1], w0[2], w0[3]), o0), s1 = add_bf16x8(make_uint4(w1[0], w1[1], w1[2], w1[3]), o1);
+                        w0[0] = s0.x; w0[1] = s0.y; w0[2] = s0.z; w0[3] = s0.w;
+                        w1[0] = s1.x; w1[1] = s1.y; w1[2] = s1.z; w1[3] = s1.w;
+                    }
                     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                                  ::"l"(dst), "r"(w0[0]), "r"(w0[1]), "r"(w0[2]), "r"(w0[3]), "r"(w1[0]), "r"(w1[1]), "r"(w1[2]), "r"(w1[3]) : "memory");
                 } else {
@@ -386,11 +407,17 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(src));
                     t += x;
                 }
-                p.colsum_out[grow] = __float2bfloat16_rn(t);
+                if (p.add) add_into_bf16(p.colsum_out + grow, t);
+                else p.colsum_out[grow] = __float2bfloat16_rn(t);
             }
         }
     } else {
         const int quarter = warp % 4;                      // lanes [32 q, 32 q + 32) of tensor memory
+        if (p.add && !p.partial) {
+            const int64_t row = (int64_t)m0 + quarter * 32 + lane;
+            for (int c = 0; c < BN; c += 64)
+                if (row < p.M && n0 + c < p.N) prefetch_l2((const __nv_bfloat16*)p.C + row * p.ldc + n0 + c);
+        }
         const bool ready = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         if (ready) {
@@ -403,6 +430,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                 tmem_ld_wait();
                 if (row_ok) {
                     if (p.partial) p.colsum_partial[(int64_t)blockIdx.z * p.M + row] = __uint_as_float(cs[0]);
+                    else if (p.colsum_out && p.add) add_into_bf16(p.colsum_out + row, __uint_as_float(cs[0]));
                     else if (p.colsum_out) p.colsum_out[row] = __float2bfloat16_rn(__uint_as_float(cs[0]));
                 }
             }
@@ -454,11 +482,15 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                             }
                         }
                         if (col0 + g * 8 + 8 <= p.N) {
-                            *reinterpret_cast<uint4*>(dst + g * 8) = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]),
-                                                                                 pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+                            uint4 x = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+                            if (p.add) x = add_bf16x8(x, *reinterpret_cast<const uint4*>(dst + g * 8));
+                            *reinterpret_cast<uint4*>(dst + g * 8) = x;
                         } else {
                             for (int e = 0; e < 8; ++e)
-                                if (col0 + g * 8 + e < p.N) dst[g * 8 + e] = __float2bfloat16_rn(f[e]);
+                                if (col0 + g * 8 + e < p.N) {
+                                    if (p.add) add_into_bf16(dst + g * 8 + e, f[e]);
+                                    else dst[g * 8 + e] = __float2bfloat16_rn(f[e]);
+                                }
                         }
                     }
                 }
@@ -486,7 +518,7 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
                                                             const __nv_bfloat16* __restrict__ bias,
                                                             __nv_bfloat16* __restrict__ C, int64_t ldc,
                                                             const float* __restrict__ colsum_partial,
-                                                            __nv_bfloat16* __restrict__ colsum_out) {
+                                                            __nv_bfloat16* __restrict__ colsum_out, int add) {
     const int64_t n4 = (N + 3) / 4;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= M * n4) {                                // trailing threads: the column sums, one row each
@@ -494,7 +526,8 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
         if (colsum_out && m < M) {
             float t = 0.f;
             for (int z = 0; z < splits; ++z) t += colsum_partial[(int64_t)z * M + m];
-            colsum_out[m] = __float2bfloat16_rn(t);
+            if (add) add_into_bf16(colsum_out + m, t);
+            else colsum_out[m] = __float2bfloat16_rn(t);
         }
         return;
     }
@@ -515,7 +548,8 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
         if (n + e < N) {
             float v = acc[e];
             if (bias) v += __bfloat162float(bias[n + e]);
-            C[m * ldc + n + e] = __float2bfloat16_rn(v);
+            if (add) add_into_bf16(C + m * ldc + n + e, v);
+            else C[m * ldc + n + e] = __float2bfloat16_rn(v);
         }
 }
 
@@ -773,6 +807,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     TcParams& p = L.p[0];
     p.M = g.M; p.N = g.N; p.ldp = ldp; p.kb_total = kb_total; p.kb_per_split = kb_per;
     p.partial = splits > 1 ? 1 : 0;
+    p.add = g.add;
     p.cluster_splits = cluster;
     p.timeout_flag = device_timeout_flag();
     p.C = splits > 1 ? (void*)partials : g.C;
@@ -799,7 +834,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     const int64_t work = g.M * ((g.N + 3) / 4) + (ones ? g.M : 0);
     splitk_reduce_kernel<<<(unsigned)((work + 255) / 256), 256, 0, stream>>>(
         partials, splits, g.M, g.N, ldp, (const __nv_bfloat16*)g.bias, (__nv_bfloat16*)g.C, g.ldc, p.colsum_partial,
-        ones ? (__nv_bfloat16*)g.a_colsum : nullptr);
+        ones ? (__nv_bfloat16*)g.a_colsum : nullptr, g.add);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
 }
@@ -833,7 +868,7 @@ static lrd_status_t launch_group(const GemmArgs* g, int n, int S, cudaStream_t s
         p.kb_per_split = (p.kb_total + S - 1) / S;
         p.cluster_splits = S;
         p.timeout_flag = device_timeout_flag();
-        p.C = g[i].C; p.ldc = g[i].ldc;
+        p.C = g[i].C; p.ldc = g[i].ldc; p.add = g[i].add;
         p.colsum_out = (__nv_bfloat16*)g[i].a_colsum;
         nx = std::max(nx, (unsigned)((g[i].N + BN - 1) / BN));
         ny += (unsigned)((g[i].M + BM - 1) / BM);

@@ -46,6 +46,7 @@ template <int BN> struct Cfg {
 struct WgradParams {
     int64_t M, N, ldc;
     int kb_total, kb_per_pair;
+    int add;                      // C (and colsum) += the result rounded to bf16, see tc_gemm.cu
     __nv_bfloat16* C;
     __nv_bfloat16* colsum;        // [M] or nullptr
 };
@@ -66,6 +67,12 @@ __device__ __forceinline__ void store16(const WgradParams& p, int64_t row, int64
 #pragma unroll
     for (int e = 0; e < 8; ++e) w[e] = pack_bf16(f[2 * e], f[2 * e + 1]);
     if (col + 16 <= p.N && sectors) {
+        if (p.add) {
+            const uint4 o0 = reinterpret_cast<const uint4*>(dst)[0], o1 = reinterpret_cast<const uint4*>(dst)[1];
+            const uint32_t o[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) w[e] = add_bf16x2(w[e], o[e]);
+        }
         asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                      ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
         return;
@@ -73,11 +80,19 @@ __device__ __forceinline__ void store16(const WgradParams& p, int64_t row, int64
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (col + 8 * h + 8 <= p.N) {
+            if (p.add) {
+                const uint4 o = *reinterpret_cast<const uint4*>(dst + 8 * h);
+                w[4 * h] = add_bf16x2(w[4 * h], o.x); w[4 * h + 1] = add_bf16x2(w[4 * h + 1], o.y);
+                w[4 * h + 2] = add_bf16x2(w[4 * h + 2], o.z); w[4 * h + 3] = add_bf16x2(w[4 * h + 3], o.w);
+            }
             *reinterpret_cast<uint4*>(dst + 8 * h) = make_uint4(w[4 * h], w[4 * h + 1], w[4 * h + 2], w[4 * h + 3]);
         } else {
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                if (col + 8 * h + e < p.N) dst[8 * h + e] = __float2bfloat16_rn(f[8 * h + e]);
+                if (col + 8 * h + e < p.N) {
+                    if (p.add) add_into_bf16(dst + 8 * h + e, f[8 * h + e]);
+                    else dst[8 * h + e] = __float2bfloat16_rn(f[8 * h + e]);
+                }
         }
     }
 }
@@ -206,6 +221,10 @@ wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
         const bool has_work = kb_begin < kb_end;             // a pair past the end of the reduction contributes zeros
         const bool sectors = p.ldc % 16 == 0 && ((uintptr_t)p.C & 31u) == 0;
         const uint32_t ngrp = cs / 4u, rot = (uint32_t)row % ngrp;   // 16-byte groups of a row, rotated by the row: no two rows of a warp hit the same banks
+        if (p.add && grow < p.M) {       // what this block's columns add to, on its way while the products are formed
+            for (uint32_t c = (uint32_t)hw * 64u; c < cs; c += 128u)
+                if ((int64_t)n0 + pr * cs + c < p.N) prefetch_l2(p.C + grow * p.ldc + n0 + pr * cs + c);
+        }
         bool ok = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         cluster_arrive_relaxed();      // barrier 1: this block's ring is dead (progress only)
@@ -308,7 +327,8 @@ wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
                     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(cs_recv + (uint32_t)(k - 1) * 512u + (uint32_t)row * 4u));
                     t += x;
                 }
-                p.colsum[grow] = __float2bfloat16_rn(t);
+                if (p.add) add_into_bf16(p.colsum + grow, t);
+                else p.colsum[grow] = __float2bfloat16_rn(t);
             }
         }
         tc_fence_before();
@@ -414,6 +434,7 @@ static lrd_status_t launch(const GemmArgs* g, int n, const Plan& pl, cudaStream_
         p.kb_total = (int)((g[i].K + BK - 1) / BK);
         p.kb_per_pair = (p.kb_total + pl.pairs - 1) / pl.pairs;
         p.C = (__nv_bfloat16*)g[i].C;
+        p.add = g[i].add;
         p.colsum = (__nv_bfloat16*)g[i].a_colsum;
         ny = std::max(ny, (unsigned)((g[i].N + pl.bn - 1) / pl.bn));
         nz += (unsigned)((g[i].M + 255) / 256);

@@ -48,3 +48,26 @@ def test_group_of_layers(n, tokens, stride_rank):
         for k in ("dX", "dU", "dV", "db"):
             # dZ is rounded to bf16 after sums in another order: an ulp of some of its values, then one rounding of each result
             assert rel_err(out[k][i], alone[i][k].double().cpu().numpy()) <= 2 ** -7
+
+
+# freeze mask V: one product (64 wide, pairs, shares through scratch memory, cluster); none: several in one launch
+@pytest.mark.parametrize("shape,freeze", [((1021, 1024, 4096, 512), "V"), ((300, 1000, 3528, 1000), "V"), ((5000, 1032, 520, 520), "V"), ((9000, 264, 4096, 264), "V"),
+                                          ((4097, 768, 776, 200), "V"), ((130, 264, 328, 64), "U"), ((1000, 520, 1000, 136), "NONE"), ((70, 4096, 4096, 504), "NONE")],
+                         ids=lambda x: "x".join(map(str, x)) if isinstance(x, tuple) else x)
+def test_adding_to_the_callers_gradients(shape, freeze):
+    """The accumulating backward gives exactly the sum of what the buffers held and the plain backward's gradients."""
+    M, K, N, r = shape
+    f = getattr(b, "LRD_FREEZE_" + freeze)
+    g = torch.Generator(device="cuda").manual_seed(M)
+    X, dY, V, U, Z = (torch.randn(*s, device="cuda", generator=g).to(torch.bfloat16) for s in ((M, K), (M, N), (K, r), (N, r), (M, r)))
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16)
+    ws = torch.empty(b.lrd_linear_workspace_bytes(desc, f, 2), dtype=torch.uint8, device="cuda")
+    start = [torch.randn(*s, device="cuda", generator=g).mul_(M ** 0.5).to(torch.bfloat16) for s in ((N, r), (K, r), (N,))]
+    plain, summed = [torch.zeros_like(t) for t in start], [t.clone() for t in start]
+    dX = torch.empty_like(X)
+    x, z = None if freeze == "V" else X, None if freeze == "U" else Z
+    b.lrd_linear_bwd(desc, dY, x, V, U, z, dX, *plain, f, ws)
+    b.lrd_linear_bwd_accumulate(desc, dY, x, V, U, z, dX, *summed, f, ws)
+    assert b.lrd_check_device_status() == b.LRD_OK
+    for s, p, q in zip(start, plain, summed):
+        assert torch.equal(q, (s.float() + p.float()).to(torch.bfloat16))
