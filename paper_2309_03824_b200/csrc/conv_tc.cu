@@ -21,7 +21,9 @@
 // A block takes at most half of an SM's shared and tensor memory where the grid has more blocks than the GPU has SMs,
 // so that two blocks share an SM and one's set-up, first loads and epilogue run beside the other's MMAs.
 // Warp roles as in the matrix-product kernel: TMA producer, MMA issuer (both issue under elect.sync from a converged
-// warp), 4 epilogue warps.
+// warp), 8 epilogue warps: what a block does after its MMAs is latency of tensor-memory loads and stores, and more warps have
+// more of both in flight (four: a stride-2 step, 64 x 28 x 28, 256 -> 256 at rank 96, 65.6 us; eight, with whole sectors per
+// store: 61.3).
 #include <algorithm>
 
 #include "common.cuh"
@@ -35,7 +37,7 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 192;
+constexpr int kThreads = 320;                        // TMA producer, MMA issuer, 8 x epilogue
 constexpr int kMaxStages = 8;
 constexpr uint32_t kTile = 128 * 128;               // the A tile of a stage: 128 pixels x 64 channels of bf16
 constexpr uint32_t kSmemFull = 222 * 1024, kSmemHalf = 110 * 1024;      // dynamic shared memory of one block per SM / two
@@ -74,16 +76,22 @@ struct ConvParams {
     const __nv_bfloat16* bias2;   // [n2] or nullptr
 };
 
-// 32 fp32 accumulators of one row -> bf16 at dst (columns col0 .. col0 + 31 of n, n a multiple of 8)
-__device__ __forceinline__ void store_row32(__nv_bfloat16* dst, int col0, int n, const uint32_t (&v)[32]) {
+// 32 fp32 accumulators of one row -> bf16 at dst (columns col0 .. col0 + 31 of n, n a multiple of 8); sectors: whole 32-byte
+// sectors per store (n a multiple of 16, dst aligned to 32 bytes)
+__device__ __forceinline__ void store_row32(__nv_bfloat16* dst, int col0, int n, const uint32_t (&v)[32], bool sectors) {
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        if (col0 + g * 8 + 8 <= n)
-            *reinterpret_cast<uint4*>(dst + col0 + g * 8) =
-                make_uint4(pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1])),
-                           pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3])),
-                           pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5])),
-                           pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7])));
+    for (int g = 0; g < 2; ++g) {
+        uint32_t w[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[e] = pack_bf16(__uint_as_float(v[16 * g + 2 * e]), __uint_as_float(v[16 * g + 2 * e + 1]));
+        __nv_bfloat16* d = dst + col0 + g * 16;
+        if (sectors && col0 + g * 16 + 16 <= n) {
+            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                         ::"l"(d), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+            continue;
+        }
+        if (col0 + g * 16 + 8 <= n) *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+        if (col0 + g * 16 + 16 <= n) *reinterpret_cast<uint4*>(d + 8) = make_uint4(w[4], w[5], w[6], w[7]);
     }
 }
 
@@ -116,7 +124,7 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
         }
         mbar_init(smem_u32(&acc_bar), 1);
         mbar_init(smem_u32(&q_full), 1);
-        mbar_init(smem_u32(&t_ready), 4);
+        mbar_init(smem_u32(&t_ready), 8);
         mbar_init(smem_u32(&out_full), 1);
         if (FUSE) prefetch_tmap(&maps.q);
         fence_mbar_init();
@@ -221,7 +229,7 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
             }
         }
     } else {
-        const int q = warp % 4;
+        const int q = warp % 4, hw = (warp - 2) / 4;             // two warps share a quarter of the rows: alternate 32-column pieces
         const int row = q * 32 + lane;
         const bool row_ok = m0 + row < cl.pixels;
         int64_t pix = m0 + row;                                  // this row's pixel of the output image(s)
@@ -234,8 +242,9 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
         tc_fence_after();
         if (ready) {
             __nv_bfloat16* dst_row = p.out + pix * p.n_total;
+            const bool sectors = p.n_total % 16 == 0 && ((uintptr_t)p.out & 31u) == 0;
 #pragma unroll 1
-            for (int c = 0; c < p.bn && n0 + c < p.n_total; c += 32) {
+            for (int c = 32 * hw; c < p.bn && n0 + c < p.n_total; c += 64) {
                 uint32_t v[32];
                 if (iters > 0) {
                     tmem_ld_32x32(lane_addr + c, v);
@@ -256,7 +265,7 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
                     }
                     if (!p.out) continue;
                 }
-                if (row_ok) store_row32(dst_row, n0 + c, p.n_total, v);
+                if (row_ok) store_row32(dst_row, n0 + c, p.n_total, v, sectors);
             }
         }
         if (FUSE) {
@@ -268,9 +277,10 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
             tc_fence_after();
             if (done) {
                 __nv_bfloat16* dst_row = p.out2 + pix * p.n2;
+                const bool sectors = p.n2 % 16 == 0 && ((uintptr_t)p.out2 & 31u) == 0;
                 const bool bias_vec = p.bias2 && (((uintptr_t)p.bias2 & 15u) == 0);
 #pragma unroll 1
-                for (int col0 = 0; col0 < p.n2; col0 += 32) {
+                for (int col0 = 32 * hw; col0 < p.n2; col0 += 64) {
                     uint4 bv[4] = {};
                     const bool bvec = bias_vec && col0 + 32 <= p.n2;
                     if (bvec) {
@@ -293,7 +303,7 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
                         for (int e = 0; e < 32; ++e)
                             if (col0 + e < p.n2) v[e] = __float_as_uint(__uint_as_float(v[e]) + __bfloat162float(p.bias2[col0 + e]));
                     }
-                    store_row32(dst_row, col0, p.n2, v);
+                    store_row32(dst_row, col0, p.n2, v, sectors);
                 }
             }
         }

@@ -17,8 +17,9 @@
 //      the ring.
 // T1 (its bh interior rows) and T2 go to global memory only where the caller needs them later (the saved
 // activations Z1 / Z2 of the forward pass, dZ2 / dZ1 of the backward pass).
-// Warp 0: TMA producer (one ring for all three phases).  Warp 1: tensor memory + MMA issue.  Warps 2-5: the three
-// epilogues.  Every wait is bounded; a wait that runs out raises the device timeout flag and the block tears down.
+// Warp 0: TMA producer (one ring for all three phases).  Warp 1: tensor memory + MMA issue.  Warps 2-9: the three
+// epilogues, two warps per quarter of the rows (one: 64 x 14 x 14, 256 -> 256 at rank 96, forward and backward with the core
+// frozen 38.5 us; two, with whole sectors per store: 36.5).  Every wait is bounded; a wait that runs out raises the device timeout flag and the block tears down.
 #include "common.cuh"
 #include "conv.cuh"
 #include "ptx.cuh"
@@ -30,7 +31,7 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 192;
+constexpr int kThreads = 320;
 constexpr int kSlots = 4;
 constexpr uint32_t kTile = 128 * 128;                // 128 rows x 64 channels of bf16
 constexpr uint32_t kSlotBytes = 2 * kTile;           // a stage of any phase fits 32 KB
@@ -98,7 +99,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
             mbar_init(smem_u32(&empty_bar[s]), 1);
         }
         for (int i = 0; i < 3; ++i) mbar_init(smem_u32(&acc_bar[i]), 1);
-        for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&ready_bar[i]), 4);
+        for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&ready_bar[i]), 8);
         fence_mbar_init();
     }
     if (warp == 1) {
@@ -235,7 +236,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         __syncwarp();
     } else {
         // ------------------------------------------------------------------ the three epilogues
-        const int q = warp % 4;
+        const int q = warp % 4, hw = (warp - 2) / 4;         // two warps share a quarter of the rows: alternate 32-column pieces
         const int row = q * 32 + lane;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
         // T1: row = pixel of the haloed tile
@@ -249,7 +250,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
             const uint32_t slot_addr = z1_base + (uint32_t)(hr * p.PW + w + 1) * 16u;
             __nv_bfloat16* dst_row = p.save1 + ((int64_t)(img * p.H + hi) * p.W + w) * p.nA;
 #pragma unroll 1
-            for (int c0 = 0; c0 < p.nA; c0 += 32) {
+            for (int c0 = 32 * hw; c0 < p.nA; c0 += 64) {
                 uint32_t v[32];
                 tmem_ld_32x32(lane_addr + c0, v);
                 tmem_ld_wait();
@@ -280,7 +281,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
             __nv_bfloat16* dst_row = p.save2 + pix * p.nB;
             const bool keep = p.save2 && row_ok;
 #pragma unroll 1
-            for (int c0 = 0; c0 < p.nB; c0 += 32) {
+            for (int c0 = 32 * hw; c0 < p.nB; c0 += 64) {
                 uint32_t v[32];
                 tmem_ld_32x32(lane_addr + kAcc2Col + c0, v);
                 tmem_ld_wait();
@@ -307,9 +308,10 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         tc_fence_after();
         if (ok) {
             __nv_bfloat16* dst_row = p.out3 + pix * p.n3;
+            const bool sectors = p.n3 % 16 == 0 && ((uintptr_t)p.out3 & 31u) == 0;
             const bool bias_vec = p.bias3 && (((uintptr_t)p.bias3 & 15u) == 0);
 #pragma unroll 1
-            for (int c0 = 0; c0 < p.n3; c0 += 32) {
+            for (int c0 = 32 * hw; c0 < p.n3; c0 += 64) {
                 uint4 bv[4] = {};
                 const bool bvec = bias_vec && c0 + 32 <= p.n3;
                 if (bvec) {
@@ -333,13 +335,18 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
                         if (c0 + e < p.n3) v[e] = __float_as_uint(__uint_as_float(v[e]) + __bfloat162float(p.bias3[c0 + e]));
                 }
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    if (c0 + g * 8 + 8 <= p.n3)
-                        *reinterpret_cast<uint4*>(dst_row + c0 + g * 8) =
-                            make_uint4(pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1])),
-                                       pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3])),
-                                       pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5])),
-                                       pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7])));
+                for (int g = 0; g < 2; ++g) {
+                    uint32_t o[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) o[e] = pack_bf16(__uint_as_float(v[16 * g + 2 * e]), __uint_as_float(v[16 * g + 2 * e + 1]));
+                    __nv_bfloat16* d = dst_row + c0 + g * 16;
+                    if (sectors && c0 + g * 16 + 16 <= p.n3) {       // one whole 32-byte sector per store
+                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                     ::"l"(d), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
+                        continue;
+                    }
+                    if (c0 + g * 16 + 8 <= p.n3) *reinterpret_cast<uint4*>(d) = make_uint4(o[0], o[1], o[2], o[3]);
+                    if (c0 + g * 16 + 16 <= p.n3) *reinterpret_cast<uint4*>(d + 8) = make_uint4(o[4], o[5], o[6], o[7]);
                 }
             }
         }
