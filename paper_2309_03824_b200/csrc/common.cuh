@@ -56,6 +56,7 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // General fp32-FMA path (any shape, any alignment).
 lrd_status_t simt_gemm(const GemmArgs& g, cudaStream_t stream);
+lrd_status_t simt_wgrads(const GemmArgs& a, const GemmArgs& b, cudaStream_t s);
 
 // One product on the path chosen by `path` (an lrd_path_t): the tensor-core kernel when the
 // operands qualify, else the general kernel.

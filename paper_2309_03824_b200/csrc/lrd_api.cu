@@ -203,6 +203,7 @@ lrd_status_t run_wgrads(const GemmArgs* g, int n, int path, float* const* partia
     bool tc = path != LRD_PATH_GENERAL;
     for (int i = 0; i < n; ++i) tc = tc && g[i].M > 0 && g[i].N > 0 && tc_gemm_eligible(g[i]);
     if (tc) return tc_wgrads(g, n, partials, partial_bytes, s);
+    if (n == 2 && (path == LRD_PATH_GENERAL || (!tc_gemm_eligible(g[0]) && !tc_gemm_eligible(g[1])))) return simt_wgrads(g[0], g[1], s);
     for (int i = 0; i < n; ++i) {
         const lrd_status_t st = run_gemm(g[i], path, true, partials[i], partial_bytes[i], s);
         if (st != LRD_OK) return st;
