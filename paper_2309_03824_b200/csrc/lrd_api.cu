@@ -200,7 +200,8 @@ lrd_status_t run_gemm(const GemmArgs& g, int path, bool allow_split, float* part
 }
 
 lrd_status_t run_wgrads(const GemmArgs* g, int n, int path, float* const* partials, const size_t* partial_bytes, cudaStream_t s) {
-    bool tc = path != LRD_PATH_GENERAL;
+    // (the forced fused path launches each gradient by itself: its launch count tells which chains ran)
+    bool tc = path != LRD_PATH_GENERAL && path != LRD_PATH_FUSED;
     for (int i = 0; i < n; ++i) tc = tc && g[i].M > 0 && g[i].N > 0 && tc_gemm_eligible(g[i]);
     if (tc) return tc_wgrads(g, n, partials, partial_bytes, s);
     if (n == 2 && (path == LRD_PATH_GENERAL || (!tc_gemm_eligible(g[0]) && !tc_gemm_eligible(g[1])))) return simt_wgrads(g[0], g[1], s);
