@@ -68,7 +68,6 @@ struct TcParams {
     int64_t ldc;
     const __nv_bfloat16* bias;
     int partial;        // 1: write fp32 partials
-    int add;            // C += the product rounded to bf16 (fp32 sum, one more rounding) instead of C = it; column sums too
     int cluster_splits; // > 1: the gridDim.z blocks of a tile are one cluster and reduce through shared memory
     // CONV: input channels, 64-column blocks of a tap and of all taps, k of the k x k taps, output grid, stride, pad
     int cv_ci, cv_nkc, cv_nblk, cv_k, cv_Ho, cv_Wo, cv_stride, cv_pad;
@@ -95,7 +94,11 @@ __device__ __forceinline__ int conv_col(const TcParams& p, int col) {
     return blk < p.cv_nblk && c < p.cv_ci ? (blk / p.cv_nkc) * p.cv_ci + c : -1;
 }
 
-template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1>
+// ADD: C += the product rounded to bf16 (fp32 sum, one more rounding) instead of C = it; column sums too.  A variant of its own:
+// as a flag that every launch tests, its code stands between the stores of all of them, and a launch behind another kernel
+// fetches it cold.  Backward passes in a graph, flag / variant: 768 -> 768 at rank 192, 4096 tokens, V frozen 18.05 / 17.33 us;
+// 1024 -> 4096 at 512, 1021 tokens 23.7 / 22.7; 768 -> 3072 at 384, 600 tokens 18.95 / 18.10.
+template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1, bool ADD = false>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     int prod = 0;
@@ -106,6 +109,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     const TcParams p = L.p[prod];
     if (NP > 1 && (int64_t)blockIdx.x * BN >= p.N) return;         // (the whole cluster: its blocks share x and y)
     static_assert(!ONES || (A_MN && B_MN && BN <= 192), "the ones block rides on an MN-major B of at most 192 columns");
+    static_assert(!ADD || !CONV, "only weight gradients add");
     static_assert(!CONV || (A_MN && B_MN && !ONES && BN <= 192), "the filter gradient: both operands MN-major, split over a cluster or not at all");
     using C = Cfg<BN, ONES>;
     constexpr int STAGES = C::STAGES, G = C::G;
@@ -259,7 +263,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         const uint32_t chunk_bytes = 128u * cs * 4u, ngrp = cs / 4u;
         const uint32_t stage_base = smem_base, recv_base = smem_base + 128u * BN * 4u;
         const uint32_t cs_stage = recv_base + 128u * BN * 4u, cs_recv = cs_stage + 512u;
-        if (p.add) {           // what this block's slice adds to, on its way while the products are formed
+        if (ADD) {             // what this block's slice adds to, on its way while the products are formed
             const int64_t grow = (int64_t)m0 + row, gcol0 = (int64_t)n0 + self * cs;
             for (uint32_t c = 0; c < cs; c += 64)
                 if (grow < p.M && gcol0 + c < p.N) prefetch_l2((const __nv_bfloat16*)p.C + grow * p.ldc + gcol0 + c);
@@ -363,12 +367,12 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                 __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + at;
                 if (CONV || col + 8 <= p.N) {
                     uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-                    if (!CONV && p.add) v = add_bf16x8(v, *reinterpret_cast<const uint4*>(dst));
+                    if (ADD) v = add_bf16x8(v, *reinterpret_cast<const uint4*>(dst));
                     *reinterpret_cast<uint4*>(dst) = v;
                 } else {
                     for (int e = 0; e < 8; ++e)
                         if (col + e < p.N) {
-                            if (p.add) add_into_bf16(dst + e, acc[e]);
+                            if (ADD) add_into_bf16(dst + e, acc[e]);
                             else dst[e] = __float2bfloat16_rn(acc[e]);
                         }
                 }
@@ -386,7 +390,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                     const int64_t at = CONV ? conv_col(p, (int)col) : col;
                     if (CONV && at < 0) continue;
                     __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + at;
-                    if (!CONV && p.add) {
+                    if (ADD) {
                         const uint4 o0 = reinterpret_cast<const uint4*>(dst)[0], o1 = reinterpret_cast<const uint4*>(dst)[1];
                         const uint4 s0 = add_bf16x8(make_uint4(w0[0], w0[1], w0[2], w0[3]), o0), s1 = add_bf16x8(make_uint4(w1[0], w1[1], w1[2], w1[3]), o1);
                         w0[0] = s0.x; w0[1] = s0.y; w0[2] = s0.z; w0[3] = s0.w;
@@ -407,13 +411,13 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(src));
                     t += x;
                 }
-                if (p.add) add_into_bf16(p.colsum_out + grow, t);
+                if (ADD) add_into_bf16(p.colsum_out + grow, t);
                 else p.colsum_out[grow] = __float2bfloat16_rn(t);
             }
         }
     } else {
         const int quarter = warp % 4;                      // lanes [32 q, 32 q + 32) of tensor memory
-        if (p.add && !p.partial) {
+        if (ADD) {
             const int64_t row = (int64_t)m0 + quarter * 32 + lane;
             for (int c = 0; c < BN; c += 64)
                 if (row < p.M && n0 + c < p.N) prefetch_l2((const __nv_bfloat16*)p.C + row * p.ldc + n0 + c);
@@ -430,7 +434,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                 tmem_ld_wait();
                 if (row_ok) {
                     if (p.partial) p.colsum_partial[(int64_t)blockIdx.z * p.M + row] = __uint_as_float(cs[0]);
-                    else if (p.colsum_out && p.add) add_into_bf16(p.colsum_out + row, __uint_as_float(cs[0]));
+                    else if (ADD && p.colsum_out) add_into_bf16(p.colsum_out + row, __uint_as_float(cs[0]));
                     else if (p.colsum_out) p.colsum_out[row] = __float2bfloat16_rn(__uint_as_float(cs[0]));
                 }
             }
@@ -483,12 +487,12 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                         }
                         if (col0 + g * 8 + 8 <= p.N) {
                             uint4 x = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
-                            if (p.add) x = add_bf16x8(x, *reinterpret_cast<const uint4*>(dst + g * 8));
+                            if (ADD) x = add_bf16x8(x, *reinterpret_cast<const uint4*>(dst + g * 8));
                             *reinterpret_cast<uint4*>(dst + g * 8) = x;
                         } else {
                             for (int e = 0; e < 8; ++e)
                                 if (col0 + g * 8 + e < p.N) {
-                                    if (p.add) add_into_bf16(dst + g * 8 + e, f[e]);
+                                    if (ADD) add_into_bf16(dst + g * 8 + e, f[e]);
                                     else dst[g * 8 + e] = __float2bfloat16_rn(f[e]);
                                 }
                         }
@@ -553,9 +557,9 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
         }
 }
 
-template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1>
+template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1, bool ADD = false>
 lrd_status_t launch(const TcLaunch<NP>& L, dim3 grid, cudaStream_t stream, bool wait_ahead = true) {
-    auto kern = tc_gemm_kernel<BN, A_MN, B_MN, ONES, CONV, NP>;
+    auto kern = tc_gemm_kernel<BN, A_MN, B_MN, ONES, CONV, NP, ADD>;
     const TcParams& p = L.p[0];
     static bool configured_on[kMaxDevices] = {};     // per instantiation; the attribute is sticky per function
     bool& configured = configured_on[device_slot()];
@@ -581,6 +585,11 @@ lrd_status_t launch(const TcLaunch<NP>& L, dim3 grid, cudaStream_t stream, bool 
     if (cudaLaunchKernelEx(&cfg, kern, L) != cudaSuccess) return LRD_ERR_CUDA;
     count_launch();
     return LRD_OK;
+}
+
+template <int BN, bool ONES, int NP = 1>
+lrd_status_t launch_wgrad(bool add, const TcLaunch<NP>& L, dim3 grid, cudaStream_t s, bool wait_ahead = true) {
+    return add ? launch<BN, true, true, ONES, false, NP, true>(L, grid, s, wait_ahead) : launch<BN, true, true, ONES, false, NP>(L, grid, s, wait_ahead);
 }
 
 template <int BN>
@@ -807,7 +816,6 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     TcParams& p = L.p[0];
     p.M = g.M; p.N = g.N; p.ldp = ldp; p.kb_total = kb_total; p.kb_per_split = kb_per;
     p.partial = splits > 1 ? 1 : 0;
-    p.add = g.add;
     p.cluster_splits = cluster;
     p.timeout_flag = device_timeout_flag();
     p.C = splits > 1 ? (void*)partials : g.C;
@@ -817,11 +825,19 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     p.colsum_out = (ones && splits == 1) ? (__nv_bfloat16*)g.a_colsum : nullptr;
     dim3 grid((unsigned)((g.N + bn - 1) / bn), (unsigned)((g.M + BM - 1) / BM), (unsigned)zdim);
     lrd_status_t st;
+    const bool add = g.add && splits == 1;                 // (shares through scratch memory: the second kernel adds)
     if (ones) {
         switch (bn) {
-            case 192: st = launch<192, true, true, true>(L, grid, stream); break;
-            case 128: st = launch<128, true, true, true>(L, grid, stream); break;
-            default:  st = launch<64, true, true, true>(L, grid, stream); break;
+            case 192: st = launch_wgrad<192, true>(add, L, grid, stream); break;
+            case 128: st = launch_wgrad<128, true>(add, L, grid, stream); break;
+            default:  st = launch_wgrad<64, true>(add, L, grid, stream); break;
+        }
+    } else if (g.a_mn_major && g.b_mn_major) {
+        switch (bn) {
+            case 256: st = launch_wgrad<256, false>(add, L, grid, stream); break;
+            case 192: st = launch_wgrad<192, false>(add, L, grid, stream); break;
+            case 128: st = launch_wgrad<128, false>(add, L, grid, stream); break;
+            default:  st = launch_wgrad<64, false>(add, L, grid, stream); break;
         }
     } else
     switch (bn) {
@@ -868,12 +884,12 @@ static lrd_status_t launch_group(const GemmArgs* g, int n, int S, cudaStream_t s
         p.kb_per_split = (p.kb_total + S - 1) / S;
         p.cluster_splits = S;
         p.timeout_flag = device_timeout_flag();
-        p.C = g[i].C; p.ldc = g[i].ldc; p.add = g[i].add;
+        p.C = g[i].C; p.ldc = g[i].ldc;
         p.colsum_out = (__nv_bfloat16*)g[i].a_colsum;
         nx = std::max(nx, (unsigned)((g[i].N + BN - 1) / BN));
         ny += (unsigned)((g[i].M + BM - 1) / BM);
     }
-    return launch<BN, true, true, ONES, false, kMaxWgrads>(L, dim3(nx, ny, (unsigned)S), stream, !g[0].in_turn);
+    return launch_wgrad<BN, ONES>(g[0].add, L, dim3(nx, ny, (unsigned)S), stream, !g[0].in_turn);
 }
 
 // The weight gradients of one backward pass.  Each alone has few output tiles and one pays for its launch, its first loads and
@@ -886,7 +902,8 @@ lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const s
     int64_t rows = 0;
     double separate = 0.0;
     for (int i = 0; i < n && together; ++i) {
-        together = tc_gemm_eligible(g[i]) && g[i].a_mn_major && g[i].b_mn_major && !g[i].bias && g[i].max_cluster_split == g[0].max_cluster_split;
+        together = tc_gemm_eligible(g[i]) && g[i].a_mn_major && g[i].b_mn_major && !g[i].bias && g[i].max_cluster_split == g[0].max_cluster_split &&
+                   g[i].add == g[0].add;
         if (!together) break;
         ones = ones || g[i].a_colsum;
         rows += (g[i].M + BM - 1) / BM;

@@ -46,7 +46,6 @@ template <int BN> struct Cfg {
 struct WgradParams {
     int64_t M, N, ldc;
     int kb_total, kb_per_pair;
-    int add;                      // C (and colsum) += the result rounded to bf16, see tc_gemm.cu
     __nv_bfloat16* C;
     __nv_bfloat16* colsum;        // [M] or nullptr
 };
@@ -59,7 +58,8 @@ template <int NP> struct WgradLaunch {
     CUtensorMap tA[NP], tB[NP];
 };
 
-// 16 columns of one row, rounded once
+// 16 columns of one row, rounded once (ADD: added to what C holds, see tc_gemm.cu)
+template <bool ADD>
 __device__ __forceinline__ void store16(const WgradParams& p, int64_t row, int64_t col, const float (&f)[16], bool sectors) {
     if (row >= p.M || col >= p.N) return;
     __nv_bfloat16* dst = p.C + row * p.ldc + col;
@@ -67,7 +67,7 @@ __device__ __forceinline__ void store16(const WgradParams& p, int64_t row, int64
 #pragma unroll
     for (int e = 0; e < 8; ++e) w[e] = pack_bf16(f[2 * e], f[2 * e + 1]);
     if (col + 16 <= p.N && sectors) {
-        if (p.add) {
+        if (ADD) {
             const uint4 o0 = reinterpret_cast<const uint4*>(dst)[0], o1 = reinterpret_cast<const uint4*>(dst)[1];
             const uint32_t o[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
 #pragma unroll
@@ -80,7 +80,7 @@ __device__ __forceinline__ void store16(const WgradParams& p, int64_t row, int64
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (col + 8 * h + 8 <= p.N) {
-            if (p.add) {
+            if (ADD) {
                 const uint4 o = *reinterpret_cast<const uint4*>(dst + 8 * h);
                 w[4 * h] = add_bf16x2(w[4 * h], o.x); w[4 * h + 1] = add_bf16x2(w[4 * h + 1], o.y);
                 w[4 * h + 2] = add_bf16x2(w[4 * h + 2], o.z); w[4 * h + 3] = add_bf16x2(w[4 * h + 3], o.w);
@@ -90,7 +90,7 @@ __device__ __forceinline__ void store16(const WgradParams& p, int64_t row, int64
 #pragma unroll
             for (int e = 0; e < 8; ++e)
                 if (col + 8 * h + e < p.N) {
-                    if (p.add) add_into_bf16(dst + 8 * h + e, f[8 * h + e]);
+                    if (ADD) add_into_bf16(dst + 8 * h + e, f[8 * h + e]);
                     else dst[8 * h + e] = __float2bfloat16_rn(f[8 * h + e]);
                 }
         }
@@ -98,7 +98,7 @@ __device__ __forceinline__ void store16(const WgradParams& p, int64_t row, int64
 }
 
 // grid: (2 pairs = one cluster, column tiles, row tiles of 256)
-template <int BN, int NP>
+template <int BN, int NP, bool ADD>
 __global__ void __launch_bounds__(kThreads, 1)
 wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
     int prod = 0;
@@ -221,7 +221,7 @@ wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
         const bool has_work = kb_begin < kb_end;             // a pair past the end of the reduction contributes zeros
         const bool sectors = p.ldc % 16 == 0 && ((uintptr_t)p.C & 31u) == 0;
         const uint32_t ngrp = cs / 4u, rot = (uint32_t)row % ngrp;   // 16-byte groups of a row, rotated by the row: no two rows of a warp hit the same banks
-        if (p.add && grow < p.M) {       // what this block's columns add to, on its way while the products are formed
+        if (ADD && grow < p.M) {       // what this block's columns add to, on its way while the products are formed
             for (uint32_t c = (uint32_t)hw * 64u; c < cs; c += 128u)
                 if ((int64_t)n0 + pr * cs + c < p.N) prefetch_l2(p.C + grow * p.ldc + n0 + pr * cs + c);
         }
@@ -317,7 +317,7 @@ wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
                             f[4 * g] += x.x; f[4 * g + 1] += x.y; f[4 * g + 2] += x.z; f[4 * g + 3] += x.w;
                         }
                     }
-                    store16(p, grow, (int64_t)n0 + pr * cs + c0 + 16 * half, f, sectors);
+                    store16<ADD>(p, grow, (int64_t)n0 + pr * cs + c0 + 16 * half, f, sectors);
                 }
             }
             if (sums && hw == 0 && pr == 0 && grow < p.M) {
@@ -327,7 +327,7 @@ wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
                     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(cs_recv + (uint32_t)(k - 1) * 512u + (uint32_t)row * 4u));
                     t += x;
                 }
-                if (p.add) add_into_bf16(p.colsum + grow, t);
+                if (ADD) add_into_bf16(p.colsum + grow, t);
                 else p.colsum[grow] = __float2bfloat16_rn(t);
             }
         }
@@ -348,8 +348,9 @@ wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
 
 bool set_attributes() {
     auto one = [](const void* f) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) == cudaSuccess; };
-    return one((const void*)wgrad_pair_kernel<256, 1>) && one((const void*)wgrad_pair_kernel<128, 1>) &&
-           one((const void*)wgrad_pair_kernel<256, kMaxWgrads>);
+    return one((const void*)wgrad_pair_kernel<256, 1, false>) && one((const void*)wgrad_pair_kernel<128, 1, false>) &&
+           one((const void*)wgrad_pair_kernel<256, kMaxWgrads, false>) && one((const void*)wgrad_pair_kernel<256, 1, true>) &&
+           one((const void*)wgrad_pair_kernel<128, 1, true>) && one((const void*)wgrad_pair_kernel<256, kMaxWgrads, true>);
 }
 
 // Clusters of n blocks that can be resident at once.
@@ -369,7 +370,7 @@ int max_active_clusters(int n) {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (!set_attributes() || cudaOccupancyMaxActiveClusters(&cnt, wgrad_pair_kernel<256, 1>, &cfg) != cudaSuccess || cnt < 1) {
+        if (!set_attributes() || cudaOccupancyMaxActiveClusters(&cnt, wgrad_pair_kernel<256, 1, false>, &cfg) != cudaSuccess || cnt < 1) {
             cudaGetLastError();
             cnt = (kNumSms - 20) / n;
         }
@@ -434,7 +435,6 @@ static lrd_status_t launch(const GemmArgs* g, int n, const Plan& pl, cudaStream_
         p.kb_total = (int)((g[i].K + BK - 1) / BK);
         p.kb_per_pair = (p.kb_total + pl.pairs - 1) / pl.pairs;
         p.C = (__nv_bfloat16*)g[i].C;
-        p.add = g[i].add;
         p.colsum = (__nv_bfloat16*)g[i].a_colsum;
         ny = std::max(ny, (unsigned)((g[i].N + pl.bn - 1) / pl.bn));
         nz += (unsigned)((g[i].M + 255) / 256);
@@ -461,9 +461,10 @@ static lrd_status_t launch(const GemmArgs* g, int n, const Plan& pl, cudaStream_
     attr[1].val.programmaticStreamSerializationAllowed = g[0].in_turn ? 0 : 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e;
-    if constexpr (NP == 1) e = pl.bn == 256 ? cudaLaunchKernelEx(&cfg, wgrad_pair_kernel<256, 1>, L) : cudaLaunchKernelEx(&cfg, wgrad_pair_kernel<128, 1>, L);
-    else e = cudaLaunchKernelEx(&cfg, wgrad_pair_kernel<256, NP>, L);
+    auto kern = g[0].add ? wgrad_pair_kernel<256, NP, true> : wgrad_pair_kernel<256, NP, false>;
+    if constexpr (NP == 1)
+        if (pl.bn == 128) kern = g[0].add ? wgrad_pair_kernel<128, 1, true> : wgrad_pair_kernel<128, 1, false>;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, L);
     if (!cuda_ok(e, "cudaLaunchKernelEx(weight gradient on pairs)")) return LRD_ERR_CUDA;
     count_launch();
     return LRD_OK;
