@@ -45,9 +45,11 @@ constexpr int kMaxClusterSplits = 8;                 // portable cluster size
 // overwritten; with N = BN + 16 the MMA then also forms sum_k A(m, k) in accumulator column BN (the bias
 // gradient falls out of the dU product: its A operand is dY).
 // G: 64-deep k-blocks per stage.  Two for the narrow tiles, whose MMAs take no longer than what a stage costs the issuing
-// warp beside them (see tc_gemm_persistent.cu), as long as three stages fit.
+// warp beside them (see tc_gemm_persistent.cu).  One with the ones block: two leave three stages of 64 KB, and the first MMA
+// waits for twice the bytes (768 x 192 over 4096 tokens with the bias gradient 8.06 us with two, 7.88 with one; in clusters of
+// two as the two-call backward runs it 10.78 / 10.36; over 9000 tokens, 264 x 264, the same).
 template <int BN, bool ONES = false> struct Cfg {
-    static constexpr int G = BN <= 64 || (BN <= 128 && !ONES) ? 2 : 1;
+    static constexpr int G = BN <= 128 && !ONES ? 2 : 1;
     static constexpr uint32_t A_STAGE_BYTES = G * BM * BK * 2;
     static constexpr uint32_t B_STAGE_BYTES = G * (BN * BK * 2 + (ONES ? 8192 : 0));
     static constexpr uint32_t STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
