@@ -64,7 +64,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full1[kMaxStages], empty1[kMaxStages], full2[kMaxStages], empty2[kMaxStages],
         tacc_bar, tready_bar[kMaxCluster], out_full[2], out_empty[2];
-    __shared__ __align__(16) uint16_t bias_s[2][256];
+    __shared__ __align__(16) float bias_s[2][256];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -336,8 +336,10 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
         // Epilogue: each warp on its own.  32 columns of its 32 rows at a time go through a [32 rows x 64 B] slab of the warp
         // (64-byte swizzle) and leave by one TMA store each; a piece is a chain of latencies (tensor memory, conversion, fence,
         // the store's read of the slab), so eight warps share the chunk, and a chunk's bias is fetched while the chunk before it
-        // is stored.  8192 x 4096 output, r = 256: 48.7 us with four warps and the bias fetched at the chunk's own start, 44.5
-        // with eight and ahead; what is left of it is the write rate (67 MB at 5.4 TB/s, the rate of a memset: 12.4 us).
+        // is stored.  8192 tokens, 1024 -> 4096 at r = 256: 34.3 us with four warps and the bias fetched at the chunk's own start,
+        // 27.3 with eight and ahead; the 67 MB of output alone take 12.4 at the rate of a memset.  (A variant without the bias
+        // code for backward passes: each launch alone 0.2 us faster, but forward and backward no longer share their
+        // instructions, 768 -> 768 at r = 192, 4096 tokens 26.2 -> 28.5 us a step.)
         const uint32_t slab0 = staging_base + (uint32_t)(warp - 2) * kSlabBytes;
         const uint32_t row_off = (uint32_t)lane * 64u;
         const uint32_t row_xor = ((uint32_t)lane >> 1) & 3u;

@@ -74,7 +74,7 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full1[kMaxSlots], empty1[kMaxSlots], full2[kMaxSlots], empty2[kMaxSlots], tacc_bar,
         tready_bar[kMaxS], pready_bar[kMaxS], out_full[2], out_empty[2];
-    __shared__ __align__(16) uint16_t bias_s[2][256];
+    __shared__ __align__(16) float bias_s[2][256];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 

@@ -309,6 +309,25 @@ __device__ __forceinline__ void bias_put(uint16_t* at, const uint16_t (&b)[4], i
         if (e < pieces) at[64 * e + (threadIdx.x & 31)] = b[e];
     __syncwarp();
 }
+// The same with the bias kept as fp32: twice the shared memory, half the instructions per piece, which a block of one or two
+// chunks waits for (chain forward, 700 tokens, 512 -> 512 at rank 128: 6.53 us with bf16, 6.44 with fp32, 6.26 without a bias).
+__device__ __forceinline__ void bias_put(float* at, const uint16_t (&b)[4], int pieces) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (e < pieces) at[64 * e + (threadIdx.x & 31)] = __uint_as_float((uint32_t)b[e] << 16);
+    __syncwarp();
+}
+__device__ __forceinline__ void bias_add(uint32_t* v, const float* at) {
+    const float4* bp = reinterpret_cast<const float4*>(at);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const float4 b4 = bp[e];
+        v[4 * e] = __float_as_uint(__uint_as_float(v[4 * e]) + b4.x);
+        v[4 * e + 1] = __float_as_uint(__uint_as_float(v[4 * e + 1]) + b4.y);
+        v[4 * e + 2] = __float_as_uint(__uint_as_float(v[4 * e + 2]) + b4.z);
+        v[4 * e + 3] = __float_as_uint(__uint_as_float(v[4 * e + 3]) + b4.w);
+    }
+}
 // 32 accumulators += bias of their columns
 __device__ __forceinline__ void bias_add(uint32_t* v, const uint16_t* at) {
     const uint4* bp = reinterpret_cast<const uint4*>(at);
