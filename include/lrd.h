@@ -282,14 +282,16 @@ lrd_status_t lrd_linear_bwd_accumulate(const lrd_linear_desc_t* desc, const void
  * outputs and workspaces must not overlap one another (every layer writes its own dX: the caller adds
  * them up where the layers share X).  One mask applies to the whole group.
  *
- * The layers are enqueued side by side: layer 0 on `cuda_stream`, the others on streams the library
- * owns (created on first use, one set per host thread and device, never freed), which start after the work already in
- * `cuda_stream` and which `cuda_stream` waits for before the call returns - so to the caller the group
- * behaves like n single-layer calls on `cuda_stream`, and it may be captured into a CUDA graph.  Each
- * launch is shaped for 1/n of the SMs.  In the backward, a layer's dU (+ dbias) product runs beside its
- * data chain.  Z_save, dU, dV and dbias have the bits of the single-layer calls; Y and dX agree with them to
- * rounding (the fused kernel sums over the rank in an order that depends on its cluster size, which follows
- * the launch's share of the SMs).  n = 1 is allowed (then only the dU overlap differs from lrd_linear_bwd).
+ * To the caller a group behaves like n single-layer calls on `cuda_stream`, and it may be captured into a CUDA graph.  2 to 4
+ * layers of one shape that the fused chain takes on pairs of SMs run in one launch on `cuda_stream` (in the backward their
+ * weight gradients follow there).  Otherwise the layers are enqueued side by side: layer 0 on `cuda_stream`, the others on
+ * streams the library owns (created on first use, one set per host thread and device, never freed), which start after the
+ * work already in `cuda_stream` and which `cuda_stream` waits for before the call returns; each launch is then shaped for
+ * 1/n of the SMs, and in the backward a layer's dU (+ dbias) product runs beside its data chain.  Z_save has the bits of the
+ * single-layer call.  Y, dX, dU, dV and dbias agree with it to rounding: the fused kernel sums over the rank in an order that
+ * depends on its cluster size, and the weight gradients of a group share the SMs, so their sums over the tokens are split
+ * differently.  The same group call always gives the same bits.  n = 1 is allowed (then only the dU overlap differs from
+ * lrd_linear_bwd).
  *
  * Errors: LRD_ERR_INVALID_ARG for n outside [0, LRD_MAX_GROUP] or a NULL required array; otherwise the
  * first failing layer's status.  All layers are validated before anything is enqueued.  Every host

@@ -40,6 +40,7 @@ struct GemmArgs {
                                // SMs inside one GPC, which a chain kernel on 128 of the 148 SMs never leaves
     bool add = false;          // weight gradients on the tensor-core kernels: C (and a_colsum) += the product, rounded to the storage
                                // type before the fp32 sum and after it
+    bool whole = false;        // data products: the reduction is not split over a cluster
     bool in_turn = false;      // weight gradients: started only when the launch before has ended (blocks that wait on an SM for
                                // that end keep it from work in other streams)
 };

@@ -87,20 +87,32 @@ GemmArgs gemm(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, bool 
 // pairs): 256 tokens 9.6 / 14.6 / 23.5, 4096 tokens 30 / 27 / 41, 8192 tokens 51 / 61 / 46; 768 -> 768 at r = 192: 128
 // tokens 8.1 / 7.5 / -, 4096 tokens 12.3 / 9.2 / 10.9.  No simple line separates them, so each kernel estimates its
 // time; over 96 measured layers the choice costs 0.4 % on average against the best of the three.
-lrd_status_t launch_chain(const ChainArgs* c, int n, int path, cudaStream_t s, bool leave_room = false) {
+enum class Form { products, single, pair };
+// whole_t: the separate products would have to form T in one piece
+Form choose_form(const ChainArgs* c, int n, int path, bool leave_room, bool whole_t) {
+    if (path != LRD_PATH_AUTO && path != LRD_PATH_FUSED) return Form::products;
     const int mode = g_chain_mma_blocks.load();
     const bool pair = c[0].sm_share == 0 && mode != 1 && chain_pair_eligible(c, n);
     const bool single = n == 1 && mode != 2 && chain_eligible(c[0]);
-    if (mode == 2 || path == LRD_PATH_FUSED || n > 1) {
-        if (pair) return chain_pair_launch(c, n, s);
-        return single ? chain_launch(c[0], s) : LRD_ERR_UNSUPPORTED;
-    }
+    if (mode == 2 || path == LRD_PATH_FUSED || n > 1) return pair ? Form::pair : single ? Form::single : Form::products;
     const double us_pair = pair ? chain_pair_estimate(c, n) : 1e300, us_single = single ? chain_estimate(c[0]) : 1e300;
-    const double us_products = tc_gemm_estimate(c[0].M, c[0].r, c[0].K1) + tc_gemm_estimate(c[0].M, c[0].N2, c[0].r);
+    const double us_products = tc_gemm_estimate(c[0].M, c[0].r, c[0].K1, whole_t) + tc_gemm_estimate(c[0].M, c[0].N2, c[0].r);
     const double best = std::min({us_pair, us_single, us_products});
-    if (us_pair <= best * (leave_room ? 1.35 : 1.0)) return chain_pair_launch(c, n, s);
-    if (us_single <= us_products) return chain_launch(c[0], s);
-    return LRD_ERR_UNSUPPORTED;
+    if (us_pair <= best * (leave_room ? 1.35 : 1.0)) return Form::pair;
+    return us_single <= us_products ? Form::single : Form::products;
+}
+
+lrd_status_t launch_chain(const ChainArgs* c, int n, int path, cudaStream_t s, bool leave_room = false, bool whole_t = false) {
+    const Form form = choose_form(c, n, path, leave_room, whole_t);
+    if (form == Form::products) return LRD_ERR_UNSUPPORTED;
+    return form == Form::pair ? chain_pair_launch(c, n, s) : chain_launch(c[0], s);
+}
+
+// Whether the layer's own call, with the GPU to itself, runs as two products and splits the reduction of the first: the only form
+// in which T is not summed over K1 in one piece.
+bool alone_splits_t(ChainArgs c, int path) {
+    c.sm_share = 0;
+    return path != LRD_PATH_GENERAL && choose_form(&c, 1, path, false, false) == Form::products && tc_splits_data_product(c.M, c.r, c.K1);
 }
 
 ChainArgs fwd_chain_args(const Linear& L, const void* X, const void* V, const void* U, const void* bias, void* Y, void* Z_save,
@@ -535,14 +547,18 @@ static lrd_status_t linear_fwd_on(const lrd_linear_desc_t* desc, const void* X, 
     }
 
     const int path = g_path.load();
-    if (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) {
-        const ChainArgs c = fwd_chain_args(L, X, V, U, bias, Y, Z_save, sm_share);
-        const lrd_status_t st = launch_chain(&c, 1, path, s);
-        if (st != LRD_ERR_UNSUPPORTED) return st;
-    }
+    ChainArgs c = fwd_chain_args(L, X, V, U, bias, Y, Z_save, sm_share);
+    // Beside other layers a saved Z still has the bits of the layer's own call: it is split where that call splits it (which is
+    // then the form to run: few tiles, most of the GPU is left to the others), and nowhere else
+    const bool as_alone = sm_share > 0 && Z_save && alone_splits_t(c, path), whole = sm_share > 0 && Z_save && !as_alone;
+    if (as_alone) c.sm_share = 0;
+    const lrd_status_t st = launch_chain(&c, 1, path, s, false, whole);
+    if (st != LRD_ERR_UNSUPPORTED) return st;
     void* Z = Z_save ? Z_save : workspace;
     const int64_t ldz = Z_save ? L.ldz : L.r;
-    LRD_TRY(run_gemm(gemm(L.M, L.r, L.K, X, L.ldx, false, V, L.ldv, true, Z, ldz, nullptr, L.dt), false, nullptr, 0, s));
+    GemmArgs first = gemm(L.M, L.r, L.K, X, L.ldx, false, V, L.ldv, true, Z, ldz, nullptr, L.dt);
+    first.whole = whole;
+    LRD_TRY(run_gemm(first, false, nullptr, 0, s));
     return run_gemm(gemm(L.M, L.N, L.r, Z, ldz, false, U, L.ldu, false, Y, L.ldy, bias, L.dt), false, nullptr, 0, s);
 }
 
@@ -758,7 +774,9 @@ static lrd_status_t lrd_linear_group_fwd_impl(int n, const lrd_linear_desc_t* de
             ok = parse_linear(&descs[i], &L, false) == LRD_OK && L.M > 0;
             if (ok) c[i] = fwd_chain_args(L, X[i], V[i], U[i], bias ? bias[i] : nullptr, Y[i], Z_save ? Z_save[i] : nullptr, 0);
         }
-        if (ok && chain_pair_eligible(c, n)) return chain_pair_launch(c, n, s);
+        // (not where the layers' own calls split the reduction of a saved Z, whose bits a group keeps; that costs three layers
+        // 4096 -> 1024 at r = 384 nothing at 256 tokens, 22.2 us in one launch, 22.9 side by side, and at 512 22.2 / 29.0)
+        if (ok && !(Z_save && alone_splits_t(c[0], path)) && chain_pair_eligible(c, n)) return chain_pair_launch(c, n, s);
     }
     SideStreams* ss = n > 1 ? side_streams() : nullptr;
     if (n > 1 && !ss) return LRD_ERR_CUDA;

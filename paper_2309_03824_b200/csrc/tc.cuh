@@ -16,8 +16,10 @@ size_t tc_split_workspace_bytes(int64_t M, int64_t N, int64_t K);
 // epilogue of a tile overlaps the MMAs of the next).  Same eligibility as tc_gemm; no column sums.
 lrd_status_t tc_gemm_persistent(const GemmArgs& g, cudaStream_t stream);
 double tc_gemm_persistent_estimate(int64_t M, int64_t N, int64_t K);
-// Estimated microseconds of a data product on the kernel tc_gemm would take for it.
-double tc_gemm_estimate(int64_t M, int64_t N, int64_t K);
+// Estimated microseconds of a data product on the kernel tc_gemm would take for it (whole: without a split of the reduction),
+// and whether it would split it.
+double tc_gemm_estimate(int64_t M, int64_t N, int64_t K, bool whole = false);
+bool tc_splits_data_product(int64_t M, int64_t N, int64_t K);
 void tc_gemm_persistent_force_pairs(int blocks_per_mma);     // 0: automatic; 1 or 2: forced where the shape allows
 // Weight gradients (both operands MN-major), up to kMaxWgrads of them in one launch.  Estimated microseconds on pairs of
 // SMs (1e300 where that does not apply); all of them on pairs; all of them the fastest way (partials: scratch of each,

@@ -757,10 +757,16 @@ static bool split_data_product(int64_t M, int64_t N, int64_t K, SplitPlan* out, 
     return found;
 }
 
-double tc_gemm_estimate(int64_t M, int64_t N, int64_t K) {
+bool tc_splits_data_product(int64_t M, int64_t N, int64_t K) {
     SplitPlan sp;
     double us;
-    return split_data_product(M, N, K, &sp, &us) ? us : tc_gemm_persistent_estimate(M, N, K);
+    return split_data_product(M, N, K, &sp, &us);
+}
+
+double tc_gemm_estimate(int64_t M, int64_t N, int64_t K, bool whole) {
+    SplitPlan sp;
+    double us;
+    return !whole && split_data_product(M, N, K, &sp, &us) ? us : tc_gemm_persistent_estimate(M, N, K);
 }
 
 int tc_pick_splits(int64_t M, int64_t N, int64_t K) { return pick_split(M, N, K, false).global; }
@@ -786,7 +792,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     SplitPlan dp;
     if (!allow_split && !ones) {                           // data products: the persistent kernel, or a split of the reduction
         double us;
-        if (!split_data_product(g.M, g.N, g.K, &dp, &us)) return tc_gemm_persistent(g, stream);
+        if (g.whole || !split_data_product(g.M, g.N, g.K, &dp, &us)) return tc_gemm_persistent(g, stream);
         bn = dp.bn; cluster = dp.cluster;
     } else if (allow_split) {
         double us;

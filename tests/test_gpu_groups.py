@@ -184,3 +184,14 @@ def test_groups_from_two_host_threads_at_once():
     assert not errors, errors
     for g in gs:
         g.check(single=False)
+
+
+@pytest.mark.parametrize("shapes", [[(256, 4096, 1024, 384)] * 3, [(300, 3072, 768, 250)] * 2, [(700, 1024, 1024, 256), (130, 3072, 768, 288), (1021, 1280, 640, 96)]],
+                         ids=["equal", "packed_rank", "mixed"])
+def test_saved_intermediate_where_a_single_layer_splits_the_reduction(shapes):
+    """Few row tiles and a long reduction: alone, these layers run as two products and the first is split over a cluster (the
+    last shape of the mixed group is not split).  The Z of the group still has the bits of the single-layer calls."""
+    g = Group(make_group(shapes, 1800 + len(shapes)), b.LRD_FREEZE_V)
+    g.fwd()
+    g.bwd()
+    g.check()
