@@ -202,7 +202,8 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     }
     GemmArgs dB_product = make_gemm(t.S, t.r2, t.Po, dY, t.S, true, Z2_save, t.r2, true, dB, t.r2, nullptr, t.dt);
     dB_product.a_colsum = dbias;                          // the bias gradient rides on the dB product (A = dY)
-    if (factors && sB != s) keep(run_gemm(dB_product, path, true, pB, reg.dB, sB));
+    // (by itself with the switch off too: one launch with dA would share the pixels out differently, and the switch changes no bits)
+    if (factors && core) keep(run_gemm(dB_product, path, true, pB, reg.dB, sB));
 
     auto launch_filter = [&](cudaStream_t st_f) {
         keep(conv_bwd_filter(dZ2, Z1_save, dG, t.B, t.g, t.r1, t.r2, t.dt, path, st_f));
@@ -234,7 +235,7 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
         const GemmArgs gw[2] = {make_gemm(t.C, t.r1, t.P, X, t.C, true, dZ1, t.r1, true, dA, t.r1, nullptr, t.dt), dB_product};
         float* const scratch[2] = {pA, pB};
         const size_t scratch_bytes[2] = {reg.dA, reg.dB};
-        keep(run_wgrads(gw, sB == s ? 2 : 1, path, scratch, scratch_bytes, s));
+        keep(run_wgrads(gw, core ? 1 : 2, path, scratch, scratch_bytes, s));
     }
     if (core && sF == s) launch_filter(s);
     // join even after a failed launch, so that a capture in progress is left whole

@@ -162,6 +162,22 @@ def test_backward_launches_side_by_side_or_in_a_row_give_the_same_bits(geom, fre
                 assert torch.equal(v, row[k]), k
 
 
+@pytest.mark.parametrize("geom", [(64, 7, 7, 512, 512, 309, 309), (64, 14, 14, 256, 256, 96, 96)])
+def test_side_by_side_or_in_a_row_with_long_reductions(geom):
+    """Nothing frozen and thousands of pixels: dA and dB reduce over shares of them, the same shares with the switch off (with
+    the core frozen the switch changes nothing: dA and dB share one launch either way)."""
+    B, H, W, C, S, r1, r2 = geom
+    case = wl.random_tucker_case(B, H, W, C, S, r1, r2, 3, "bf16", 650 + C)
+    try:
+        b.lrd_tucker2_overlap(False)
+        row = run_tucker(case, b.LRD_TK_FREEZE_NONE)
+    finally:
+        b.lrd_tucker2_overlap(True)
+    side = run_tucker(case, b.LRD_TK_FREEZE_NONE)
+    for k, v in side.items():
+        assert torch.equal(v, row[k]), k
+
+
 @pytest.mark.parametrize("freeze", [b.LRD_TK_FREEZE_CORE, b.LRD_TK_FREEZE_FACTORS])
 def test_c3_resnet_stage3_shape_full_size(freeze):
     c = wl.C3_TUCKER
