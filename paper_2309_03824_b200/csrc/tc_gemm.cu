@@ -836,16 +836,16 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     const bool add = g.add && splits == 1;                 // (shares through scratch memory: the second kernel adds)
     if (ones) {
         switch (bn) {
-            case 192: st = launch_wgrad<192, true>(add, L, grid, stream); break;
-            case 128: st = launch_wgrad<128, true>(add, L, grid, stream); break;
-            default:  st = launch_wgrad<64, true>(add, L, grid, stream); break;
+            case 192: st = launch_wgrad<192, true>(add, L, grid, stream, !g.in_turn); break;
+            case 128: st = launch_wgrad<128, true>(add, L, grid, stream, !g.in_turn); break;
+            default:  st = launch_wgrad<64, true>(add, L, grid, stream, !g.in_turn); break;
         }
     } else if (g.a_mn_major && g.b_mn_major) {
         switch (bn) {
-            case 256: st = launch_wgrad<256, false>(add, L, grid, stream); break;
-            case 192: st = launch_wgrad<192, false>(add, L, grid, stream); break;
-            case 128: st = launch_wgrad<128, false>(add, L, grid, stream); break;
-            default:  st = launch_wgrad<64, false>(add, L, grid, stream); break;
+            case 256: st = launch_wgrad<256, false>(add, L, grid, stream, !g.in_turn); break;
+            case 192: st = launch_wgrad<192, false>(add, L, grid, stream, !g.in_turn); break;
+            case 128: st = launch_wgrad<128, false>(add, L, grid, stream, !g.in_turn); break;
+            default:  st = launch_wgrad<64, false>(add, L, grid, stream, !g.in_turn); break;
         }
     } else
     switch (bn) {

@@ -195,3 +195,32 @@ def test_saved_intermediate_where_a_single_layer_splits_the_reduction(shapes):
     g.fwd()
     g.bwd()
     g.check()
+
+
+@pytest.mark.parametrize("path", [b.LRD_PATH_AUTO, b.LRD_PATH_FUSED])
+def test_weight_gradients_of_a_group_start_in_turn(path):
+    """The gradients behind a group's one data launch must not wait for its end on SMs that other streams could use: no launch of
+    the captured backward depends on another programmatically (= starts before that one has ended)."""
+    import ctypes
+    g = Group(make_group(QKV, 1900, shared_x=True), b.LRD_FREEZE_NONE)
+    g.fwd()
+    g.bwd()
+    torch.cuda.synchronize()
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph(keep_graph=True)
+    b.lrd_set_path(path)
+    try:
+        n0 = b.lrd_launch_count()
+        with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side):
+            g.bwd()
+        launches = b.lrd_launch_count() - n0
+    finally:
+        b.lrd_set_path(b.LRD_PATH_AUTO)
+
+    class Edge(ctypes.Structure):
+        _fields_ = [("from_port", ctypes.c_ubyte), ("to_port", ctypes.c_ubyte), ("type", ctypes.c_ubyte), ("reserved", ctypes.c_ubyte * 5)]
+
+    cu, count = ctypes.CDLL("libcuda.so.1"), ctypes.c_size_t(64)
+    nodes, edges = [(ctypes.c_void_p * 64)() for _ in range(2)], (Edge * 64)()
+    assert cu.cuGraphGetEdges_v2(ctypes.c_void_p(graph.raw_cuda_graph()), nodes[0], nodes[1], edges, ctypes.byref(count)) == 0
+    assert count.value == launches - 1 and launches == (2 if path == b.LRD_PATH_AUTO else 7)
+    assert [e.type for e in edges[:count.value]] == [0] * count.value
