@@ -9,7 +9,9 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblrd_b200.so")
-NATIVE = os.path.join(HERE, "_native.so")         # the binding's call marshalling (a CPython extension linked to LIB)
+# the binding's call marshalling: a CPython extension linked to LIB, named for the interpreter it is built for (another one
+# does not find it and builds its own)
+NATIVE = os.path.join(HERE, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["lrd_api.cu", "simt.cu", "tma.cu", "tc_gemm.cu", "tc_gemm_persistent.cu", "tc_wgrad_pair.cu", "chain.cu", "chain_pair.cu", "conv.cu", "conv_tc.cu", "tucker_fused.cu", "streams.cu", "selftest.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "-cudart", "static"]

@@ -3,8 +3,8 @@
  * A step of a small layer is a few launches of some ten microseconds each, and marshalling a call through ctypes objects
  * took the interpreter 7 to 9 microseconds (linear_fwd / linear_bwd) -- as long as the GPU takes for a launch.  Here a
  * call costs 1.0 / 2.3: tensors are asked for their data_ptr(), descriptors (ctypes structures) are read through the
- * buffer protocol, the current stream comes from torch's own lookup.  No state is kept from one call to the next.  The
- * GIL is released around the library call, as ctypes does.
+ * buffer protocol, the current stream comes from torch's own lookup.  Nothing of a call is kept for the next;
+ * the two stream functions of torch are looked up once.  The GIL is released around the library call, as ctypes does.
  */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>

@@ -1,11 +1,15 @@
 """The native call marshalling against the plain ctypes call: same status for the same arguments, and Python errors for
 arguments that are not what the call takes.  Only calls that the library refuses before it looks for a device."""
 import ctypes
+import importlib.machinery
+import os
+import sysconfig
 
 import pytest
 import torch
 
 from paper_2309_03824_b200 import binding as b
+from paper_2309_03824_b200 import build
 
 T = torch.zeros(64, dtype=torch.bfloat16)
 ODD = torch.zeros(65, dtype=torch.uint8)[1:]           # not aligned to a bf16 element
@@ -43,3 +47,11 @@ def test_groups_take_lists_and_none():
     assert b.lrd_linear_group_bwd([d], [T], None, [T], [T], None, [T], None, [T], None, 1, [WS], stream=0, check=False) == b.LRD_ERR_INVALID_ARG
     n = 9                                              # one more than a group may have
     assert b.lrd_linear_group_fwd([d] * n, [T] * n, [T] * n, [T] * n, None, [T] * n, None, 1, [WS] * n, stream=0, check=False) == b.LRD_ERR_INVALID_ARG
+
+
+def test_extension_is_named_for_its_interpreter():
+    """Only the interpreter that it was built for imports it: the plain ".so" that every CPython takes is not its name."""
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    assert suffix in importlib.machinery.EXTENSION_SUFFIXES and suffix != ".so"
+    assert os.path.basename(build.NATIVE) == "_native" + suffix
+    assert os.path.samefile(b._native.__file__, build.NATIVE)
