@@ -145,6 +145,7 @@ def _stream_source():
 
 
 _native.set_stream_source(_stream_source)
+_native.set_descriptor_types(lrd_linear_desc_t, lrd_tucker2_desc_t)
 
 
 def _ws(workspace):

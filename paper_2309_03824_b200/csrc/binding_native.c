@@ -15,6 +15,7 @@
 static PyObject *s_data_ptr, *s_numel, *s_element_size;      /* interned method names */
 static PyObject* stream_source;                              /* () -> (current device, device -> its current raw stream) */
 static PyObject *fn_device, *fn_stream;
+static PyTypeObject *linear_type, *tucker2_type;             /* the binding's two descriptor structures */
 
 typedef struct {
     PyObject* const* v;      /* the call's arguments */
@@ -84,9 +85,14 @@ static void* stream(Args* a, int i) {
     return p;
 }
 
-static void descriptor(Args* a, PyObject* o, void* out, size_t size) {
+static void descriptor(Args* a, PyObject* o, PyTypeObject* type, void* out, size_t size) {
     Py_buffer b;
     if (a->bad) return;
+    if (!PyObject_TypeCheck(o, type)) {
+        PyErr_Format(PyExc_TypeError, "expected %s, not %s", type->tp_name, Py_TYPE(o)->tp_name);
+        a->bad = 1;
+        return;
+    }
     if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) { a->bad = 1; return; }
     if ((size_t)b.len == size) {
         memcpy(out, b.buf, size);
@@ -113,7 +119,7 @@ static void descriptor(Args* a, PyObject* o, void* out, size_t size) {
 
 ENTRY(linear_fwd, 10)      /* desc X V U bias Y Z_save freeze workspace stream */
     lrd_linear_desc_t d;
-    descriptor(a, v[0], &d, sizeof d);
+    descriptor(a, v[0], linear_type, &d, sizeof d);
     void *X = ptr(a, 1), *V = ptr(a, 2), *U = ptr(a, 3), *bias = ptr(a, 4), *Y = ptr(a, 5), *Z = ptr(a, 6), *w = ptr(a, 8), *s = stream(a, 9);
     const lrd_freeze_t f = (lrd_freeze_t)num(a, 7);
     const size_t nb = nbytes(a, 8);
@@ -122,7 +128,7 @@ CALL(lrd_linear_fwd(&d, X, V, U, bias, Y, Z, f, w, nb, s))
 #define BACKWARD(name)     /* desc dY X V U Z_save dX dU dV dbias freeze workspace stream */                                   \
     ENTRY(name, 13)                                                                                                            \
     lrd_linear_desc_t d;                                                                                                       \
-    descriptor(a, v[0], &d, sizeof d);                                                                                         \
+    descriptor(a, v[0], linear_type, &d, sizeof d);                                                                            \
     void *dY = ptr(a, 1), *X = ptr(a, 2), *V = ptr(a, 3), *U = ptr(a, 4), *Z = ptr(a, 5), *dX = ptr(a, 6), *dU = ptr(a, 7),     \
          *dV = ptr(a, 8), *db = ptr(a, 9), *w = ptr(a, 11), *s = stream(a, 12);                                                \
     const lrd_freeze_t f = (lrd_freeze_t)num(a, 10);                                                                           \
@@ -133,7 +139,7 @@ BACKWARD(linear_bwd_accumulate)
 
 ENTRY(linear_bwd_data, 8)  /* desc dY V U dX freeze workspace stream */
     lrd_linear_desc_t d;
-    descriptor(a, v[0], &d, sizeof d);
+    descriptor(a, v[0], linear_type, &d, sizeof d);
     void *dY = ptr(a, 1), *V = ptr(a, 2), *U = ptr(a, 3), *dX = ptr(a, 4), *w = ptr(a, 6), *s = stream(a, 7);
     const lrd_freeze_t f = (lrd_freeze_t)num(a, 5);
     const size_t nb = nbytes(a, 6);
@@ -141,7 +147,7 @@ CALL(lrd_linear_bwd_data(&d, dY, V, U, dX, f, w, nb, s))
 
 ENTRY(linear_bwd_weights, 10)      /* desc dY X Z_save dU dV dbias freeze workspace stream */
     lrd_linear_desc_t d;
-    descriptor(a, v[0], &d, sizeof d);
+    descriptor(a, v[0], linear_type, &d, sizeof d);
     void *dY = ptr(a, 1), *X = ptr(a, 2), *Z = ptr(a, 3), *dU = ptr(a, 4), *dV = ptr(a, 5), *db = ptr(a, 6), *w = ptr(a, 8), *s = stream(a, 9);
     const lrd_freeze_t f = (lrd_freeze_t)num(a, 7);
     const size_t nb = nbytes(a, 8);
@@ -149,21 +155,21 @@ CALL(lrd_linear_bwd_weights(&d, dY, X, Z, dU, dV, db, f, w, nb, s))
 
 ENTRY(dense_fwd, 7)        /* desc X W bias Y workspace stream */
     lrd_linear_desc_t d;
-    descriptor(a, v[0], &d, sizeof d);
+    descriptor(a, v[0], linear_type, &d, sizeof d);
     void *X = ptr(a, 1), *W = ptr(a, 2), *bias = ptr(a, 3), *Y = ptr(a, 4), *w = ptr(a, 5), *s = stream(a, 6);
     const size_t nb = nbytes(a, 5);
 CALL(lrd_dense_fwd(&d, X, W, bias, Y, w, nb, s))
 
 ENTRY(dense_bwd, 9)        /* desc dY X W dX dW dbias workspace stream */
     lrd_linear_desc_t d;
-    descriptor(a, v[0], &d, sizeof d);
+    descriptor(a, v[0], linear_type, &d, sizeof d);
     void *dY = ptr(a, 1), *X = ptr(a, 2), *W = ptr(a, 3), *dX = ptr(a, 4), *dW = ptr(a, 5), *db = ptr(a, 6), *w = ptr(a, 7), *s = stream(a, 8);
     const size_t nb = nbytes(a, 7);
 CALL(lrd_dense_bwd(&d, dY, X, W, dX, dW, db, w, nb, s))
 
 ENTRY(tucker2_fwd, 12)     /* desc X A G Bm bias Y Z1_save Z2_save freeze workspace stream */
     lrd_tucker2_desc_t d;
-    descriptor(a, v[0], &d, sizeof d);
+    descriptor(a, v[0], tucker2_type, &d, sizeof d);
     void *X = ptr(a, 1), *A = ptr(a, 2), *G = ptr(a, 3), *B = ptr(a, 4), *bias = ptr(a, 5), *Y = ptr(a, 6), *Z1 = ptr(a, 7), *Z2 = ptr(a, 8),
          *w = ptr(a, 10), *s = stream(a, 11);
     const lrd_tucker_freeze_t f = (lrd_tucker_freeze_t)num(a, 9);
@@ -172,7 +178,7 @@ CALL(lrd_tucker2_fwd(&d, X, A, G, B, bias, Y, Z1, Z2, f, w, nb, s))
 
 ENTRY(tucker2_bwd, 16)     /* desc dY X A G Bm Z1_save Z2_save dX dA dG dB dbias freeze workspace stream */
     lrd_tucker2_desc_t d;
-    descriptor(a, v[0], &d, sizeof d);
+    descriptor(a, v[0], tucker2_type, &d, sizeof d);
     void *dY = ptr(a, 1), *X = ptr(a, 2), *A = ptr(a, 3), *G = ptr(a, 4), *B = ptr(a, 5), *Z1 = ptr(a, 6), *Z2 = ptr(a, 7), *dX = ptr(a, 8),
          *dA = ptr(a, 9), *dG = ptr(a, 10), *dB = ptr(a, 11), *db = ptr(a, 12), *w = ptr(a, 14), *s = stream(a, 15);
     const lrd_tucker_freeze_t f = (lrd_tucker_freeze_t)num(a, 13);
@@ -201,7 +207,7 @@ static void group_parse(Args* a, Group* g, int lists, int at_ws) {
     if (!g->block) { PyErr_NoMemory(); a->bad = 1; Py_DECREF(ds); return; }
     g->descs = (lrd_linear_desc_t*)g->block;
     void** at = (void**)(g->descs + n);
-    for (Py_ssize_t i = 0; i < n; ++i) descriptor(a, PySequence_Fast_GET_ITEM(ds, i), &g->descs[i], sizeof g->descs[i]);
+    for (Py_ssize_t i = 0; i < n; ++i) descriptor(a, PySequence_Fast_GET_ITEM(ds, i), linear_type, &g->descs[i], sizeof g->descs[i]);
     Py_DECREF(ds);
     for (int k = 0; k <= lists && !a->bad; ++k, at += n) {
         PyObject* arg = a->v[k < lists ? k + 1 : at_ws];
@@ -254,11 +260,21 @@ static PyObject* py_set_stream_source(PyObject* self, PyObject* f) {
     Py_RETURN_NONE;
 }
 
+static PyObject* py_set_descriptor_types(PyObject* self, PyObject* args) {
+    PyTypeObject *linear, *tucker2;
+    (void)self;
+    if (!PyArg_ParseTuple(args, "O!O!", &PyType_Type, &linear, &PyType_Type, &tucker2)) return NULL;
+    Py_XSETREF(linear_type, (PyTypeObject*)Py_NewRef(linear));
+    Py_XSETREF(tucker2_type, (PyTypeObject*)Py_NewRef(tucker2));
+    Py_RETURN_NONE;
+}
+
 #define METHOD(name) {#name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, NULL}
 static PyMethodDef methods[] = {METHOD(linear_fwd), METHOD(linear_bwd), METHOD(linear_bwd_accumulate), METHOD(linear_bwd_data),
                                 METHOD(linear_bwd_weights), METHOD(dense_fwd), METHOD(dense_bwd), METHOD(tucker2_fwd), METHOD(tucker2_bwd),
                                 METHOD(linear_group_fwd), METHOD(linear_group_bwd),
-                                {"set_stream_source", py_set_stream_source, METH_O, NULL}, {NULL, NULL, 0, NULL}};
+                                {"set_stream_source", py_set_stream_source, METH_O, NULL},
+                                {"set_descriptor_types", py_set_descriptor_types, METH_VARARGS, NULL}, {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", NULL, -1, methods, NULL, NULL, NULL, NULL};
 
 PyMODINIT_FUNC PyInit__native(void) {

@@ -35,6 +35,11 @@ def test_arguments_of_the_wrong_kind_raise():
     d, t = b.linear_desc(256, 64, 64, 16, b.LRD_BF16), b.tucker2_desc(1, 4, 4, 8, 8, 4, 4, b.LRD_BF16)
     with pytest.raises(TypeError):
         b.lrd_linear_fwd(t, T, T, T, None, T, T, 0, WS, stream=0)
+    for not_a_descriptor in (bytes(d), memoryview(bytes(d)), bytearray(bytes(d))):       # the right size is not enough
+        with pytest.raises(TypeError):
+            b.lrd_linear_fwd(not_a_descriptor, T, T, T, None, T, T, 0, WS, stream=0)
+        with pytest.raises(TypeError):
+            b.lrd_linear_group_fwd([not_a_descriptor], [T], [T], [T], None, [T], [T], 0, [WS], stream=0)
     with pytest.raises(AttributeError):
         b.lrd_linear_fwd(d, 5, T, T, None, T, T, 0, WS, stream=0)
     with pytest.raises(ValueError):
