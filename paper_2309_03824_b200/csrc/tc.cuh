@@ -8,12 +8,10 @@ constexpr int kNumSms = 148;   // B200: tile and split choices are made against 
 
 // bf16, 16-byte aligned bases, leading dimensions multiples of 8 elements.
 bool tc_gemm_eligible(const GemmArgs& g);
-int tc_pick_bn(int64_t M, int64_t N);
-int tc_pick_splits(int64_t M, int64_t N, int64_t K);
 // fp32 partial-tile scratch a split product of this shape needs (0 when it is not split).
 size_t tc_split_workspace_bytes(int64_t M, int64_t N, int64_t K);
 // Unsplit product with a bf16 result on the persistent kernel (one block per SM walks over the tiles, the
-// epilogue of a tile overlaps the MMAs of the next).  Same eligibility as tc_gemm; no column sums.
+// epilogue of a tile overlaps the MMAs of the next).  A K-major; no column sums.
 lrd_status_t tc_gemm_persistent(const GemmArgs& g, cudaStream_t stream);
 double tc_gemm_persistent_estimate(int64_t M, int64_t N, int64_t K);
 // Estimated microseconds of a data product on the kernel tc_gemm would take for it (whole: without a split of the reduction),
@@ -28,7 +26,8 @@ constexpr int kMaxWgrads = 8;
 double tc_wgrad_pair_estimate(const GemmArgs* g, int n);
 lrd_status_t tc_wgrad_pair(const GemmArgs* g, int n, cudaStream_t stream);
 lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const size_t* partial_bytes, cudaStream_t stream);
-// allow_split: the reduction dimension may be split over blocks (weight gradients).
+// allow_split: a weight gradient (both operands MN-major), whose reduction may be split over blocks; else a data product (A
+// K-major, no column sums).
 lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_t partial_bytes, cudaStream_t stream);
 
 }  // namespace lrd

@@ -15,9 +15,9 @@
 // B operand (issuing a copy costs a thread about a hundred clocks, and an MN-major operand takes one copy per
 // 64 columns: one warp alone issues a 40 KB stage in about 0.4 us, less than the memory system delivers),
 // warp 1 owns tensor memory and issues the MMAs, warps 2-5 read the accumulator (each its own quarter of the
-// 128 lanes) and store.  The single-thread instructions are issued under elect.sync by a converged warp.  Both
-// operands may be K-major (reduction index contiguous) or MN-major (row / column index contiguous),
-// which covers every product of the forward and backward pass without a transposed copy.
+// 128 lanes) and store.  The single-thread instructions are issued under elect.sync by a converged warp.  Weight
+// gradients have both operands MN-major (row / column index contiguous), data products A K-major (reduction index contiguous)
+// and B either way: no product of the forward or backward pass needs a transposed copy.
 //
 // CONV: the filter gradient of a k x k convolution, dG[o][tap][i] = sum_p dout[p][o] in[p stride + tap - pad][i], is
 // the same product with the taps side by side as columns (a tap takes whole 64-column blocks): A = dout[pixels x co],
@@ -594,12 +594,6 @@ lrd_status_t launch_wgrad(bool add, const TcLaunch<NP>& L, dim3 grid, cudaStream
     return add ? launch<BN, true, true, ONES, false, NP, true>(L, grid, s, wait_ahead) : launch<BN, true, true, ONES, false, NP>(L, grid, s, wait_ahead);
 }
 
-template <int BN>
-lrd_status_t launch_major(bool a_mn, bool b_mn, const TcLaunch<1>& L, dim3 grid, cudaStream_t s) {
-    if (a_mn) return b_mn ? launch<BN, true, true>(L, grid, s) : launch<BN, true, false>(L, grid, s);
-    return b_mn ? launch<BN, false, true>(L, grid, s) : launch<BN, false, false>(L, grid, s);
-}
-
 inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 uint32_t stage_kblocks(int bn, bool ones) {
@@ -624,24 +618,18 @@ bool tc_gemm_eligible(const GemmArgs& g) {
 // Tile width.  Every MMA of a tile reads its 128 x 16 block of A from shared memory whatever its width, and
 // every tile streams its own copy of A, so a narrow tile pays the same A traffic for fewer columns: below
 // about 154 columns the cost of a k-block is taken as constant, above as proportional to the width.
-//   split = false: blocks run in waves over the SMs -> minimise waves x per-tile cost;
-//   split = true:  the reduction is split until the machine is full -> minimise tiles x per-tile cost.
-static int pick_bn(int64_t M, int64_t N, bool split) {
-    const int cands[4] = {256, 192, 128, 64};
+// The reduction is split until the machine is full -> minimise tiles x per-tile cost.
+static int pick_bn(int64_t M, int64_t N) {
     const int64_t mt = (M + BM - 1) / BM;
     int best = 64;
     double best_cost = 1e300;
-    for (int bn : cands) {
+    for (int bn : {256, 192, 128, 64}) {
         if (bn == 64 && N > 64) continue;
-        const int64_t tiles = mt * ((N + bn - 1) / bn);
-        const double per_tile = bn < 154 ? 154.0 : (double)bn;
-        const double cost = split ? (double)tiles * per_tile : (double)((tiles + kNumSms - 1) / kNumSms) * (per_tile + 32);
+        const double cost = (double)(mt * ((N + bn - 1) / bn)) * (bn < 154 ? 154.0 : (double)bn);
         if (cost < best_cost) { best_cost = cost; best = bn; }
     }
     return best;
 }
-
-int tc_pick_bn(int64_t M, int64_t N) { return pick_bn(M, N, false); }
 
 static int global_splits(int64_t M, int64_t N, int64_t K, int bn) {
     const int64_t tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
@@ -715,7 +703,7 @@ static double split_us(int bn, int S, int64_t tiles, int64_t deepest, int64_t kb
 static SplitPlan pick_split(int64_t M, int64_t N, int64_t K, bool ones, int max_cluster = 0, double* us = nullptr) {
     const int top = max_cluster >= 2 && max_cluster < kMaxClusterSplits ? max_cluster : kMaxClusterSplits;
     const int64_t mt = (M + BM - 1) / BM, kb = (K + BK - 1) / BK;
-    SplitPlan best{pick_bn(M, N, true), 1, 1};
+    SplitPlan best{pick_bn(M, N), 1, 1};
     if (ones && best.bn > 192) best.bn = 192;
     best.global = global_splits(M, N, K, best.bn);
     const int64_t tiles0 = mt * ((N + best.bn - 1) / best.bn), share = (kb + best.global - 1) / best.global;
@@ -769,8 +757,6 @@ double tc_gemm_estimate(int64_t M, int64_t N, int64_t K, bool whole) {
     return !whole && split_data_product(M, N, K, &sp, &us) ? us : tc_gemm_persistent_estimate(M, N, K);
 }
 
-int tc_pick_splits(int64_t M, int64_t N, int64_t K) { return pick_split(M, N, K, false).global; }
-
 // fp32 partial tiles [splits][M][ldp], then (for the optional column sums) [splits][M]; nothing for a cluster split
 size_t tc_split_workspace_bytes(int64_t M, int64_t N, int64_t K) {
     size_t need = 0;
@@ -787,22 +773,20 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
                      cudaStream_t stream) {
     if (!tc_gemm_eligible(g)) return LRD_ERR_UNSUPPORTED;
     const bool ones = g.a_colsum != nullptr;
-    if (ones && !(g.a_mn_major && g.b_mn_major)) return LRD_ERR_UNSUPPORTED;
-    int splits = 1, cluster = 1, bn;
-    SplitPlan dp;
-    if (!allow_split && !ones) {                           // data products: the persistent kernel, or a split of the reduction
-        double us;
-        if (g.whole || !split_data_product(g.M, g.N, g.K, &dp, &us)) return tc_gemm_persistent(g, stream);
-        bn = dp.bn; cluster = dp.cluster;
-    } else if (allow_split) {
+    int splits = 1, cluster, bn;
+    if (allow_split) {                                     // weight gradients
+        if (!g.a_mn_major || !g.b_mn_major) return LRD_ERR_UNSUPPORTED;
         double us;
         const SplitPlan sp = pick_split(g.M, g.N, g.K, ones, g.max_cluster_split, &us);
         // where the tiles leave no room for a cluster per tile
         if (tc_wgrad_pair_estimate(&g, 1) < 0.95 * us) return tc_wgrad_pair(&g, 1, stream);
         bn = sp.bn; cluster = sp.cluster; splits = sp.global;
-    } else {
-        bn = pick_bn(g.M, g.N, false);
-        if (ones && bn > 192) bn = 192;                // the ones block needs 16 accumulator columns beside the tile
+    } else {                                               // data products: the persistent kernel, or a split of the reduction
+        if (g.a_mn_major || ones) return LRD_ERR_UNSUPPORTED;
+        SplitPlan dp;
+        double us;
+        if (g.whole || !split_data_product(g.M, g.N, g.K, &dp, &us)) return tc_gemm_persistent(g, stream);
+        bn = dp.bn; cluster = dp.cluster;
     }
     const int64_t ldp = (g.N + 3) / 4 * 4;
     const size_t tile_bytes = align_up((size_t)splits * g.M * ldp * sizeof(float), 256);
@@ -840,19 +824,17 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
             case 128: st = launch_wgrad<128, true>(add, L, grid, stream, !g.in_turn); break;
             default:  st = launch_wgrad<64, true>(add, L, grid, stream, !g.in_turn); break;
         }
-    } else if (g.a_mn_major && g.b_mn_major) {
+    } else if (allow_split) {
         switch (bn) {
             case 256: st = launch_wgrad<256, false>(add, L, grid, stream, !g.in_turn); break;
             case 192: st = launch_wgrad<192, false>(add, L, grid, stream, !g.in_turn); break;
             case 128: st = launch_wgrad<128, false>(add, L, grid, stream, !g.in_turn); break;
             default:  st = launch_wgrad<64, false>(add, L, grid, stream, !g.in_turn); break;
         }
-    } else
-    switch (bn) {
-        case 256: st = launch_major<256>(g.a_mn_major, g.b_mn_major, L, grid, stream); break;
-        case 192: st = launch_major<192>(g.a_mn_major, g.b_mn_major, L, grid, stream); break;
-        case 128: st = launch_major<128>(g.a_mn_major, g.b_mn_major, L, grid, stream); break;
-        default:  st = launch_major<64>(g.a_mn_major, g.b_mn_major, L, grid, stream); break;
+    } else if (bn == 128) {
+        st = g.b_mn_major ? launch<128, false, true>(L, grid, stream) : launch<128, false, false>(L, grid, stream);
+    } else {
+        st = g.b_mn_major ? launch<64, false, true>(L, grid, stream) : launch<64, false, false>(L, grid, stream);
     }
     if (st != LRD_OK || splits == 1) return st;
     const int64_t work = g.M * ((g.N + 3) / 4) + (ones ? g.M : 0);

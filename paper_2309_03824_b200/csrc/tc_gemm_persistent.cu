@@ -1,5 +1,5 @@
 // Persistent tensor-core matrix product for sm_100a (unsplit products with a bf16 result):
-//   C[M x N] = op(A) op(B) (+ bias)
+//   C[M x N] = A op(B) (+ bias), A K-major
 // One block per SM walks over the 128 x BN output tiles (tile t -> row tile t % m_tiles, column tile
 // t / m_tiles, so that blocks working at the same time share the B operand in L2).  The accumulator is
 // double-buffered in tensor memory: while the eight epilogue warps round tile i to bf16 and store it
@@ -61,7 +61,7 @@ struct PParams {
     unsigned int* timeout_flag;
 };
 
-template <int BN, bool A_MN, bool B_MN, int CG>
+template <int BN, bool B_MN, int CG>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                           const __grid_constant__ CUtensorMap tmC, const PParams p) {
@@ -139,13 +139,8 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
                 const int k0 = kb * BK;
                 if (elect_one()) {
                     if (h == 0) mbar_expect_tx(fb_local, CG * C::STAGE_BYTES);
-                    if (A_MN) {
 #pragma unroll
-                        for (int j = 0; j < BM / 64; ++j) load2d<CG>(a_dst + j * (8192 * G), &tmA, fb, m0 + 64 * j, k0);
-                    } else {
-#pragma unroll
-                        for (int g = 0; g < G; ++g) load2d<CG>(a_dst + g * kATile, &tmA, fb, k0 + g * BK, m0);
-                    }
+                    for (int g = 0; g < G; ++g) load2d<CG>(a_dst + g * kATile, &tmA, fb, k0 + g * BK, m0);
                     if (B_MN) {
 #pragma unroll
                         for (int j = 0; j < BNH / 64; ++j) load2d<CG>(b_dst + j * (8192 * G), &tmB, fb, n0 + 64 * j, k0);
@@ -160,10 +155,10 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
         }
     } else if (warp == 1 && h == 0) {
         // ------------------------------------------------------------------ MMA issuer (the even block of a pair)
-        constexpr uint32_t idesc = CG == 2 ? idesc_bf16_pair(BN, A_MN, B_MN) : idesc_bf16(BN, A_MN, B_MN);
+        constexpr uint32_t idesc = CG == 2 ? idesc_bf16_pair(BN, false, B_MN) : idesc_bf16(BN, false, B_MN);
         // the descriptors of a stage differ from these in the start address only (bits 0-13, in 16-byte units); a k-step of
         // 16 moves it by 2048 bytes (MN-major) or 32 (K-major: 32 within a k-block, then the next tile)
-        const uint64_t a_desc0 = A_MN ? smem_desc_sw128(ring_base, 8192 * G, 1024) : smem_desc_sw128(ring_base, 0, 1024);
+        const uint64_t a_desc0 = smem_desc_sw128(ring_base, 0, 1024);
         const uint64_t b_desc0 = B_MN ? smem_desc_sw128(ring_base + G * kATile, 8192 * G, 1024) : smem_desc_sw128(ring_base + G * kATile, 0, 1024);
         int s = 0, i = 0;
         uint32_t ph = 0;
@@ -188,7 +183,7 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
                         if (g > 0 && kb + g >= p.kb_total) break;
 #pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk) {
-                            const uint32_t ao = A_MN ? (g * 4 + kk) * 128u : g * (kATile >> 4) + kk * 2u;
+                            const uint32_t ao = g * (kATile >> 4) + kk * 2u;
                             const uint32_t bo = B_MN ? (g * 4 + kk) * 128u : g * (C::B_TILE >> 4) + kk * 2u;
                             const uint32_t acc = g > 0 || kk > 0 ? 1u : (kb > 0 ? 1u : 0u);
                             if (CG == 2) mma_bf16_ss_pair(d_tmem, ad + ao, bd + bo, idesc, acc);
@@ -293,10 +288,10 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     }
 }
 
-template <int BN, bool A_MN, bool B_MN, int CG>
+template <int BN, bool B_MN, int CG>
 lrd_status_t launch_p(const CUtensorMap& tA, const CUtensorMap& tB, const CUtensorMap& tC, const PParams& p, unsigned blocks,
                       cudaStream_t stream) {
-    auto kern = tc_gemm_persistent_kernel<BN, A_MN, B_MN, CG>;
+    auto kern = tc_gemm_persistent_kernel<BN, B_MN, CG>;
     static bool configured_on[kMaxDevices] = {};     // per instantiation; the attribute is sticky per function
     bool& configured = configured_on[device_slot()];
     if (!configured) {
@@ -324,10 +319,9 @@ lrd_status_t launch_p(const CUtensorMap& tA, const CUtensorMap& tB, const CUtens
 }
 
 template <int BN, int CG>
-lrd_status_t launch_p_major(bool a_mn, bool b_mn, const CUtensorMap& tA, const CUtensorMap& tB, const CUtensorMap& tC,
-                            const PParams& p, unsigned blocks, cudaStream_t s) {
-    if (a_mn) return b_mn ? launch_p<BN, true, true, CG>(tA, tB, tC, p, blocks, s) : launch_p<BN, true, false, CG>(tA, tB, tC, p, blocks, s);
-    return b_mn ? launch_p<BN, false, true, CG>(tA, tB, tC, p, blocks, s) : launch_p<BN, false, false, CG>(tA, tB, tC, p, blocks, s);
+lrd_status_t launch_p_major(bool b_mn, const CUtensorMap& tA, const CUtensorMap& tB, const CUtensorMap& tC, const PParams& p, unsigned blocks,
+                            cudaStream_t s) {
+    return b_mn ? launch_p<BN, true, CG>(tA, tB, tC, p, blocks, s) : launch_p<BN, false, CG>(tA, tB, tC, p, blocks, s);
 }
 
 // Tile shape.  Per k-block a block streams (A tile + its part of the B tile) from L2 at about 64 B/clk and
@@ -375,14 +369,13 @@ double tc_gemm_persistent_estimate(int64_t M, int64_t N, int64_t K) {
 void tc_gemm_persistent_force_pairs(int cg) { g_force_cg = (cg == 1 || cg == 2) ? cg : 0; }
 
 lrd_status_t tc_gemm_persistent(const GemmArgs& g, cudaStream_t stream) {
-    if (!tc_gemm_eligible(g) || g.a_colsum) return LRD_ERR_UNSUPPORTED;
+    if (!tc_gemm_eligible(g) || g.a_colsum || g.a_mn_major) return LRD_ERR_UNSUPPORTED;
     PShape sh = pick_shape_p(g.M, g.N);
     if (g_force_cg == 2 && sh.cg != 2) { g_force_cg = 0; sh = pick_shape_p(g.M, g.N); g_force_cg = 2; }
     const int bn = sh.bn, cg = sh.cg, bnh = bn / cg;
     CUtensorMap tA, tB, tC;
     const uint32_t kbox = BK * (cg == 1 && bn <= 128 ? 2 : 1);         // k rows of an MN-major box
-    bool ok = g.a_mn_major ? make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, kbox, 64)
-                           : make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda, BM, BK);
+    bool ok = make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda, BM, BK);
     ok = ok && (g.b_mn_major ? make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb, kbox, 64)
                              : make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb, (uint32_t)bnh, BK));
     ok = ok && make_tmap_2d_bf16(&tC, g.C, (uint64_t)g.M, (uint64_t)g.N, (uint64_t)g.ldc, 32, 32);
@@ -399,14 +392,14 @@ lrd_status_t tc_gemm_persistent(const GemmArgs& g, cudaStream_t stream) {
     const int64_t waves = (tiles + units_max - 1) / units_max;
     const unsigned blocks = (unsigned)((tiles + waves - 1) / waves) * (unsigned)cg;
     if (cg == 2) {
-        if (bn == 256) return launch_p_major<256, 2>(g.a_mn_major, g.b_mn_major, tA, tB, tC, p, blocks, stream);
-        return launch_p_major<128, 2>(g.a_mn_major, g.b_mn_major, tA, tB, tC, p, blocks, stream);
+        if (bn == 256) return launch_p_major<256, 2>(g.b_mn_major, tA, tB, tC, p, blocks, stream);
+        return launch_p_major<128, 2>(g.b_mn_major, tA, tB, tC, p, blocks, stream);
     }
     switch (bn) {
-        case 256: return launch_p_major<256, 1>(g.a_mn_major, g.b_mn_major, tA, tB, tC, p, blocks, stream);
-        case 192: return launch_p_major<192, 1>(g.a_mn_major, g.b_mn_major, tA, tB, tC, p, blocks, stream);
-        case 128: return launch_p_major<128, 1>(g.a_mn_major, g.b_mn_major, tA, tB, tC, p, blocks, stream);
-        default:  return launch_p_major<64, 1>(g.a_mn_major, g.b_mn_major, tA, tB, tC, p, blocks, stream);
+        case 256: return launch_p_major<256, 1>(g.b_mn_major, tA, tB, tC, p, blocks, stream);
+        case 192: return launch_p_major<192, 1>(g.b_mn_major, tA, tB, tC, p, blocks, stream);
+        case 128: return launch_p_major<128, 1>(g.b_mn_major, tA, tB, tC, p, blocks, stream);
+        default:  return launch_p_major<64, 1>(g.b_mn_major, tA, tB, tC, p, blocks, stream);
     }
 }
 
