@@ -162,15 +162,16 @@ const char* lrd_status_string(lrd_status_t s);
 lrd_status_t lrd_set_path(lrd_path_t path);
 
 /* Launch-shape overrides of the fused chain kernel, for measurement sweeps (no counterpart in the
- * paper): blocks per cluster (1, 2 or 4), 64-deep k-blocks per pipeline stage of the first product
+ * paper): blocks per cluster (1 to 4; automatically up to 16), 64-deep k-blocks per pipeline stage of the first product
  * (1..4), column-chunk width of the second product (64, 128, 192 or 256).  0 = automatic (the default).
  * A shape the override makes infeasible falls back to the unfused products.  Process-wide, not
  * thread-safe against concurrent launches.  Returns LRD_ERR_INVALID_ARG for values outside the lists. */
 lrd_status_t lrd_chain_tuning(int cluster_blocks, int kblocks_per_stage, int chunk_columns);
 
 /* The fused chain also runs on pairs of SMs (a cluster of 2 S blocks owns 256 rows; the two blocks of a
- * pair share every MMA and each loads half of the weights): it is taken automatically for layers of more than
- * 128 rows whose rank splits into S slices of whole 32-column groups.  Overrides for measurement sweeps and
+ * pair share every MMA and each loads half of the weights).  It takes layers of more than 128 rows whose rank splits
+ * into S slices of whole 32-column groups; automatically for a group of such layers of one shape, and for one layer where
+ * its estimated time is below those of the single-block chain and of two separate products.  Overrides for measurement sweeps and
  * tests (no counterpart in the paper): blocks_per_mma 1 = single-block chain only, 2 = pairs wherever the shape
  * allows (else the unfused products), 0 = automatic; pairs_per_cluster S (1..4), 64-deep k-blocks per
  * pipeline stage of the first product (1..4), column-chunk width of the second product (64, 128, 192, 256);
@@ -185,6 +186,19 @@ lrd_status_t lrd_chain_pair_tuning(int blocks_per_mma, int pairs_per_cluster, in
  * 128 rows.  Process-wide, not thread-safe against concurrent launches.  Returns LRD_ERR_INVALID_ARG for
  * other values. */
 lrd_status_t lrd_gemm_tuning(int blocks_per_mma);
+
+/* Launch-shape overrides for tests, of the CALLING HOST THREAD only (no counterpart in the paper).  The library picks the form
+ * of a weight gradient, and whether a data product splits its reduction, by estimates; these pick it instead, so that
+ * every form can be run at any size.  0 everywhere = automatic (the default).
+ * lrd_wgrad_tuning: blocks_per_mma 1 (single SMs; tiles of 64, 128 or 192 columns; the reduction split over 1 to 8 blocks that
+ *   divide the tile into multiples of 8 columns; the filter gradient of a convolution too) or 2 (pairs of SMs; 128 or 256 columns;
+ *   1, 2 or 4 pairs).  Several gradients at hand still share a launch; pairs do that with 256 columns only, and a call that
+ *   would need another form returns LRD_ERR_UNSUPPORTED.
+ * lrd_data_split_tuning: every data product on the tensor-core kernels is split over 2, 4 or 8 blocks, tiles of 64 or 128 columns
+ *   (the fused chain, where it is taken, has no such products: LRD_PATH_UNFUSED).
+ * LRD_ERR_INVALID_ARG for values outside the lists. */
+lrd_status_t lrd_wgrad_tuning(int blocks_per_mma, int columns, int split);
+lrd_status_t lrd_data_split_tuning(int columns, int split);
 
 /* With the core unfrozen, lrd_tucker2_bwd enqueues its independent launches side by side (the dB + dbias product from the
  * start, the core's filter gradient once dZ2 exists, both on streams the library owns; the data path and dA on the

@@ -31,7 +31,7 @@ EXPORTS = [
     "lrd_rank_quantize", "lrd_freeze_for_epoch", "lrd_tucker_freeze_for_epoch", "lrd_linear_bwd_plan",
     "lrd_status_string", "lrd_launch_count", "lrd_set_path", "lrd_check_device_status", "lrd_linear_workspace_bytes",
     "lrd_tucker2_workspace_bytes", "lrd_dense_workspace_bytes", "lrd_linear_fwd", "lrd_linear_bwd",
-    "lrd_dense_fwd", "lrd_dense_bwd", "lrd_tucker2_fwd", "lrd_tucker2_bwd", "lrd_bias_grad_noalloc", "lrd_chain_tuning", "lrd_chain_pair_tuning", "lrd_selftest_wait_timeout", "lrd_gemm_tuning", "lrd_tucker2_overlap", "lrd_rank_search", "lrd_rank_multiple", "lrd_svd_rank", "lrd_tucker_rank", "lrd_tucker_rank_min", "lrd_conv3x3_workspace_bytes", "lrd_conv3x3_fwd", "lrd_conv3x3_bwd", "lrd_linear_group_fwd", "lrd_linear_group_bwd", "lrd_linear_bwd_accumulate", "lrd_linear_bwd_data", "lrd_linear_bwd_weights",
+    "lrd_dense_fwd", "lrd_dense_bwd", "lrd_tucker2_fwd", "lrd_tucker2_bwd", "lrd_bias_grad_noalloc", "lrd_chain_tuning", "lrd_chain_pair_tuning", "lrd_selftest_wait_timeout", "lrd_gemm_tuning", "lrd_wgrad_tuning", "lrd_data_split_tuning", "lrd_tucker2_overlap", "lrd_rank_search", "lrd_rank_multiple", "lrd_svd_rank", "lrd_tucker_rank", "lrd_tucker_rank_min", "lrd_conv3x3_workspace_bytes", "lrd_conv3x3_fwd", "lrd_conv3x3_bwd", "lrd_linear_group_fwd", "lrd_linear_group_bwd", "lrd_linear_bwd_accumulate", "lrd_linear_bwd_data", "lrd_linear_bwd_weights",
 ]
 
 
@@ -88,6 +88,10 @@ _lib.lrd_linear_group_bwd.restype = _int
 _lib.lrd_linear_group_bwd.argtypes = [_int, C.POINTER(lrd_linear_desc_t)] + [_pp] * 9 + [_int, _pp, C.POINTER(C.c_size_t), C.c_void_p]
 _lib.lrd_gemm_tuning.restype = _int
 _lib.lrd_gemm_tuning.argtypes = [_int]
+_lib.lrd_wgrad_tuning.restype = _int
+_lib.lrd_wgrad_tuning.argtypes = [_int] * 3
+_lib.lrd_data_split_tuning.restype = _int
+_lib.lrd_data_split_tuning.argtypes = [_int] * 2
 _lib.lrd_tucker2_overlap.restype = _int
 _lib.lrd_tucker2_overlap.argtypes = [_int]
 _lib.lrd_check_device_status.restype = _int
@@ -261,6 +265,14 @@ def lrd_chain_pair_tuning(blocks_per_mma=0, pairs_per_cluster=0, kblocks_per_sta
 
 def lrd_gemm_tuning(blocks_per_mma=0):
     _check(_lib.lrd_gemm_tuning(blocks_per_mma))
+
+
+def lrd_wgrad_tuning(blocks_per_mma=0, columns=0, split=0):
+    _check(_lib.lrd_wgrad_tuning(blocks_per_mma, columns, split))
+
+
+def lrd_data_split_tuning(columns=0, split=0):
+    _check(_lib.lrd_data_split_tuning(columns, split))
 
 
 def lrd_tucker2_overlap(on=True):

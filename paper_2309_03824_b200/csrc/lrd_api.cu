@@ -474,6 +474,21 @@ lrd_status_t lrd_gemm_tuning(int blocks_per_mma) {
     return LRD_OK;
 }
 
+lrd_status_t lrd_wgrad_tuning(int blocks_per_mma, int columns, int split) {
+    const bool automatic = blocks_per_mma == 0 && columns == 0 && split == 0;
+    const bool single = blocks_per_mma == 1 && (columns == 64 || columns == 128 || columns == 192) && split >= 1 && split <= 8 && columns % (8 * split) == 0;
+    const bool pairs = blocks_per_mma == 2 && (columns == 128 || columns == 256) && (split == 1 || split == 2 || split == 4);
+    if (!automatic && !single && !pairs) return LRD_ERR_INVALID_ARG;
+    tc_wgrad_form() = WgradForm{blocks_per_mma, columns, split};
+    return LRD_OK;
+}
+
+lrd_status_t lrd_data_split_tuning(int columns, int split) {
+    if (!(columns == 0 && split == 0) && !((columns == 64 || columns == 128) && (split == 2 || split == 4 || split == 8))) return LRD_ERR_INVALID_ARG;
+    tc_data_split_form(columns, split);
+    return LRD_OK;
+}
+
 lrd_status_t lrd_tucker2_overlap(int on) {
     tucker2_overlap(on != 0);
     return LRD_OK;

@@ -23,8 +23,14 @@ void tc_gemm_persistent_force_pairs(int blocks_per_mma);     // 0: automatic; 1 
 // SMs (1e300 where that does not apply); all of them on pairs; all of them the fastest way (partials: scratch of each,
 // which may be shared).
 constexpr int kMaxWgrads = 8;
+// Test hooks of the calling host thread: weight gradients on `blocks` blocks per MMA (1: single SMs, 2: pairs; 0: automatic) with
+// tiles of `columns`, the reduction split over `split` blocks or pairs of a cluster; split data products likewise.  A product
+// that no kernel runs in the form asked for is LRD_ERR_UNSUPPORTED.
+struct WgradForm { int blocks, columns, split; };
+WgradForm& tc_wgrad_form();
+void tc_data_split_form(int columns, int split);
 double tc_wgrad_pair_estimate(const GemmArgs* g, int n);
-lrd_status_t tc_wgrad_pair(const GemmArgs* g, int n, cudaStream_t stream);
+lrd_status_t tc_wgrad_pair(const GemmArgs* g, int n, cudaStream_t stream);       // (in the form of the test hook where that asks for pairs)
 lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const size_t* partial_bytes, cudaStream_t stream);
 // allow_split: a weight gradient (both operands MN-major), whose reduction may be split over blocks; else a data product (A
 // K-major, no column sums).

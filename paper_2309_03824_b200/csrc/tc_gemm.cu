@@ -724,6 +724,13 @@ static SplitPlan pick_split(int64_t M, int64_t N, int64_t K, bool ones, int max_
     return best;
 }
 
+WgradForm& tc_wgrad_form() {
+    static thread_local WgradForm form{0, 0, 0};
+    return form;
+}
+static thread_local int t_data_columns = 0, t_data_split = 0;
+void tc_data_split_form(int columns, int split) { t_data_columns = columns; t_data_split = split; }
+
 // A data product with few tiles and a long reduction (a short batch through a wide layer) is the latency of one tile's
 // k-blocks: about 0.13 us each for the narrow tiles such products run on, after some 3.3 us of launch, first loads and
 // epilogue.  Split over the blocks of a cluster it is a share of them and the exchange: 128 tokens, 3072 -> 384 9.4 us
@@ -732,6 +739,11 @@ static bool split_data_product(int64_t M, int64_t N, int64_t K, SplitPlan* out, 
     const int64_t mt = (M + BM - 1) / BM, kb = (K + BK - 1) / BK;
     double best = 3.3 + 0.13 * (double)kb;
     bool found = false;
+    if (t_data_columns) {
+        *us = best;
+        *out = SplitPlan{t_data_columns, t_data_split, 1};
+        return true;
+    }
     for (int bn : {64, 128}) {
         const int64_t tiles = mt * ((N + bn - 1) / bn);
         for (int S = kMaxClusterSplits; S >= 2; S /= 2) {
@@ -777,9 +789,10 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     if (allow_split) {                                     // weight gradients
         if (!g.a_mn_major || !g.b_mn_major) return LRD_ERR_UNSUPPORTED;
         double us;
-        const SplitPlan sp = pick_split(g.M, g.N, g.K, ones, g.max_cluster_split, &us);
-        // where the tiles leave no room for a cluster per tile
-        if (tc_wgrad_pair_estimate(&g, 1) < 0.95 * us) return tc_wgrad_pair(&g, 1, stream);
+        const WgradForm& form = tc_wgrad_form();
+        const SplitPlan sp = form.blocks ? SplitPlan{form.columns, form.split, 1} : pick_split(g.M, g.N, g.K, ones, g.max_cluster_split, &us);
+        // pairs where the tiles leave no room for a cluster per tile
+        if (form.blocks ? form.blocks == 2 : tc_wgrad_pair_estimate(&g, 1) < 0.95 * us) return tc_wgrad_pair(&g, 1, stream);
         bn = sp.bn; cluster = sp.cluster; splits = sp.global;
     } else {                                               // data products: the persistent kernel, or a split of the reduction
         if (g.a_mn_major || ones) return LRD_ERR_UNSUPPORTED;
@@ -888,6 +901,7 @@ static lrd_status_t launch_group(const GemmArgs* g, int n, int S, cudaStream_t s
 // frozen, each alone / together: 4096 -> 4096 at rank 512, 8192 tokens 189 / 182 us; rank 256 142 / 132; 768 -> 3072 at 384,
 // 4096 tokens 73 / 62; 1024 -> 4096 at 512, 1024 tokens 48 / 42; 768 -> 768 at 192, 300 tokens 30 / 21.
 lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const size_t* partial_bytes, cudaStream_t stream) {
+    const WgradForm& form = tc_wgrad_form();
     bool ones = false, together = n > 1 && n <= kMaxWgrads;
     int64_t rows = 0;
     double separate = 0.0;
@@ -911,7 +925,8 @@ lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const s
                 const double t = group_estimate(g, n, b, c);
                 if (t < us) { us = t; bn = b; S = c; }
             }
-        if (tc_wgrad_pair_estimate(g, n) < us) return tc_wgrad_pair(g, n, stream);
+        if (form.blocks) { bn = form.columns; S = form.split; }
+        if (form.blocks ? form.blocks == 2 : tc_wgrad_pair_estimate(g, n) < us) return tc_wgrad_pair(g, n, stream);
         switch (bn) {
             case 192: return ones ? launch_group<192, true>(g, n, S, stream) : launch_group<192, false>(g, n, S, stream);
             case 128: return ones ? launch_group<128, true>(g, n, S, stream) : launch_group<128, false>(g, n, S, stream);
@@ -932,6 +947,7 @@ lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t 
     if (!tc_conv_eligible(B, g, ci, co, LRD_BF16, dout, in, dG)) return LRD_ERR_UNSUPPORTED;
     const int64_t P = B * g.Ho * g.Wo, taps = (int64_t)g.k * g.k, nkc = (ci + 63) / 64, N = taps * nkc * 64;
     SplitPlan sp = pick_split(co, N, P, true);             // (tiles of at most 192 columns)
+    if (tc_wgrad_form().blocks == 1) sp = SplitPlan{tc_wgrad_form().columns, tc_wgrad_form().split, 1};
     if (sp.cluster < 2) sp.cluster = 1;                    // tiles enough to fill the GPU: each reduces over all pixels
     TcLaunch<1> L{};
     CUtensorMap &tA = L.tA[0], &tB = L.tB[0];

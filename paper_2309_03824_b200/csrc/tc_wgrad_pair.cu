@@ -472,7 +472,9 @@ static lrd_status_t launch(const GemmArgs* g, int n, const Plan& pl, cudaStream_
 
 lrd_status_t tc_wgrad_pair(const GemmArgs* g, int n, cudaStream_t stream) {
     if (tc_wgrad_pair_estimate(g, n) >= 1e300) return LRD_ERR_UNSUPPORTED;
-    const Plan pl = make_plan(g, n);
+    const WgradForm& form = tc_wgrad_form();
+    const Plan pl = form.blocks == 2 ? Plan{form.columns, form.split, 0.0} : make_plan(g, n);
+    if (n > 1 && pl.bn != 256) return LRD_ERR_UNSUPPORTED;
     return n == 1 ? launch<1>(g, n, pl, stream) : launch<kMaxWgrads>(g, n, pl, stream);
 }
 

@@ -2,6 +2,8 @@
 gradients where some blocks of a cluster get no share of the reduction, and of layers launched back to back
 whose inputs are the previous launch's outputs (the kernels start early under programmatic dependent launch and
 must still wait for their producers)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -57,6 +59,30 @@ def test_chain_kernel_clusters_of_up_to_sixteen(shape):
     case = wl.random_factor_case(*shape, "bf16", 960 + shape[0])
     for freeze in (b.LRD_FREEZE_NONE, b.LRD_FREEZE_U):
         check_linear(case, freeze, path=b.LRD_PATH_FUSED)
+
+
+class _KernelNode(ctypes.Structure):
+    _fields_ = [("func", ctypes.c_void_p)] + [(n, ctypes.c_uint) for n in ("gx", "gy", "gz", "bx", "by", "bz", "smem")] + \
+               [(n, ctypes.c_void_p) for n in ("params", "extra", "kern", "ctx")]
+
+
+@pytest.mark.parametrize("cluster,shape", [(12, (100, 776, 520, 192)), (12, (64, 768, 3072, 384)), (16, (128, 264, 1000, 256)), (16, (300, 520, 520, 512)),
+                                           (7, (1, 136, 136, 112)), (10, (700, 256, 264, 160)), (8, (1500, 520, 520, 128))])
+def test_cluster_sizes_that_the_plan_chooses(cluster, shape):
+    """The grid of the captured forward is (blocks per cluster, row tiles): the largest cluster whose row tiles are all resident."""
+    M, K, N, r = shape
+    b.lrd_chain_pair_tuning(1, 0, 0, 0)
+    b.lrd_set_path(b.LRD_PATH_FUSED)
+    X, V, U, Y = (torch.zeros(*s, dtype=torch.bfloat16, device="cuda") for s in ((M, K), (K, r), (N, r), (M, N)))
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16)
+    ws = workspace(b.lrd_linear_workspace_bytes(desc, b.LRD_FREEZE_U, 0))
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side):
+        b.lrd_linear_fwd(desc, X, V, U, None, Y, None, b.LRD_FREEZE_U, ws)
+    cu, node, count, p = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_size_t(1), _KernelNode()
+    assert cu.cuGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.byref(node), ctypes.byref(count)) == 0 and count.value == 1
+    assert cu.cuGraphKernelNodeGetParams_v2(node, ctypes.byref(p)) == 0
+    assert (p.gx, p.gy) == (cluster, (M + 127) // 128)
 
 
 @pytest.mark.parametrize("mode", [(2, 1, 0, 0), (2, 2, 0, 0), (2, 3, 0, 0), (2, 4, 0, 0), (2, 0, 1, 0), (2, 0, 2, 0), (2, 2, 1, 128), (2, 1, 3, 64),

@@ -11,7 +11,8 @@ from helpers import check_linear, run_linear
 pytestmark = pytest.mark.gpu
 
 
-# the estimates send these to (tile width, pairs): 128 x 1, 256 x 1, 256 x 1, 256 x 2, 256 x 4
+# shapes where the estimates choose pairs, when this was written (tile width, pairs): 128 x 1, 256 x 1, 256 x 1, 256 x 2, 256 x 4
+# (every form by name: test_gpu_forms.py)
 @pytest.mark.parametrize("shape", [(60, 1032, 4096), (300, 3528, 1000), (1021, 4096, 1288), (5000, 264, 4096), (5000, 1032, 520)])
 def test_dense_weight_gradient(shape):
     """The undecomposed layer's dW and bias gradient."""

@@ -10,7 +10,8 @@ from helpers import check_linear, rel_err, run_linear
 
 pytestmark = pytest.mark.gpu
 
-# tokens, K, N, r; the estimates send them to (width, blocks per tile): 192 x 2, 192 x 1, 64 x 1, 192 x 8, 64 x 4, 128 x 1, 128 x 8, 64 x 8, pairs 256 wide
+# tokens, K, N, r; what the estimates choose, when this was written (width, blocks per tile): 192 x 2, 192 x 1, 64 x 1, 192 x 8, 64 x 4,
+# 128 x 1, 128 x 8, 64 x 8, pairs 256 wide (every form by name: test_gpu_forms.py)
 SHAPES = [(4096, 768, 3072, 384), (1024, 1024, 4096, 520), (70, 264, 200, 56), (5000, 520, 1000, 136), (2000, 264, 520, 248),
           (70, 1000, 4096, 200), (9000, 264, 520, 72), (9000, 264, 392, 40), (70, 4096, 4096, 504)]
 
