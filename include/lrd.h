@@ -76,7 +76,8 @@ typedef enum {
     LRD_PATH_AUTO = 0,     /* library chooses */
     LRD_PATH_GENERAL = 1,  /* fp32-FMA kernels for every shape and alignment */
     LRD_PATH_UNFUSED = 2,  /* tensor-core GEMMs, rank-r intermediate through the workspace */
-    LRD_PATH_FUSED = 3     /* fused tensor-core chain where the shape allows, else UNFUSED */
+    LRD_PATH_FUSED = 3     /* fused tensor-core chain where the shape allows, else UNFUSED; every weight gradient a launch of
+                            * its own (automatically, several share one) */
 } lrd_path_t;
 
 typedef struct {
@@ -89,8 +90,10 @@ typedef struct {
     int64_t B, H, W, C, S, r1, r2;  /* NHWC activations [B][H][W][C] -> [B][H][W][S] */
     int64_t k, stride, pad;         /* k x k core: k odd, 1..7; stride 1 or 2 (on the core); pad = (k - 1) / 2.
                                      * The output is [B][Ho][Wo][S] with Ho = (H - 1) / stride + 1, Wo likewise.
-                                     * bf16 runs the core on the tensor-core kernels whatever its k and stride (ranks off a
-                                     * multiple of 8 are repacked), fp32 on the general FMA kernels.
+                                     * bf16 runs the core on the tensor-core kernels whatever its k and stride where its bases
+                                     * are 16-byte aligned, its images have fewer than 2^30 pixels, and both ranks are multiples
+                                     * of 8 or C and S are (other ranks are then repacked); the rest, and fp32, run on the
+                                     * general FMA kernels.
                                      * Anything else: LRD_ERR_UNSUPPORTED. */
     int32_t dtype;
 } lrd_tucker2_desc_t;
@@ -148,7 +151,7 @@ int64_t lrd_tucker_rank_min(int64_t C, int64_t S, int64_t k, double alpha, doubl
 /* The undecomposed 3 x 3 convolution (stride 1, zero padding 1, NHWC; kernel Wk[S][3][3][C]) that a Tucker-2 layer
  * replaces (Eq. 4): the comparison layer of the convolutional workloads and the T of Algorithm 1's closing test.
  * Forward Y = conv(X, Wk); backward dX (nullable: skipped) and dW.  Same conventions as the other entry points;
- * the workspace holds the split partial sums of the filter gradient. */
+ * the workspace (256 bytes) is not used at present. */
 size_t lrd_conv3x3_workspace_bytes(int64_t B, int64_t H, int64_t W, int64_t C, int64_t S, int dtype);
 lrd_status_t lrd_conv3x3_fwd(int64_t B, int64_t H, int64_t W, int64_t C, int64_t S, int dtype, const void* X, const void* Wk,
                              void* Y, void* cuda_stream);
@@ -279,8 +282,9 @@ lrd_status_t lrd_linear_bwd_weights(const lrd_linear_desc_t* desc, const void* d
 /* Backward with gradient accumulation: as lrd_linear_bwd, but the unfrozen factor's dU, dbias and dV are ADDED to
  * what the buffers hold (gradient accumulation over micro-batches) instead of overwritten; dX is overwritten as
  * usual.  A frozen factor's gradient buffers are not touched at all (its gradient is zero), and may be NULL.
- * This step's gradients are formed in scratch at the end of the workspace, rounded to the storage type, then
- * added in fp32 and rounded once more.  Workspace: lrd_linear_workspace_bytes(desc, freeze, 2).  The paper's
+ * This step's gradients are rounded to the storage type, then added in fp32 and rounded once more: by the weight-gradient
+ * kernels themselves where they run on the tensor cores (bf16, ranks and strides multiples of 8, 16-byte aligned bases), else
+ * from scratch at the end of the workspace.  Workspace: lrd_linear_workspace_bytes(desc, freeze, 2).  The paper's
  * Section 2.2 trains with plain steps; accumulation is a convenience with no counterpart there. */
 lrd_status_t lrd_linear_bwd_accumulate(const lrd_linear_desc_t* desc, const void* dY, const void* X, const void* V,
                                        const void* U, const void* Z_save, void* dX, void* dU, void* dV, void* dbias,
