@@ -539,7 +539,8 @@ bool chain_eligible(const ChainArgs& a) {
 }
 
 // A stage takes its issue loop, its MMAs, or its turn of the ring (load latency over the stages in flight), whichever is
-// longest: constants fitted to forward passes of 12 layer shapes at 32 to 8192 tokens (6 % rms).
+// longest: constants fitted to forward passes of 12 layer shapes at 32 to 8192 tokens (over 336 others, 64 to 8192 tokens and ranks
+// 32 to 512, 7.5 % rms).
 double chain_estimate(const ChainArgs& a) {
     Plan pl;
     if (!make_plan(a, &pl)) return 1e300;

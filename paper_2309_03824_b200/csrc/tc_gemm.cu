@@ -688,12 +688,16 @@ struct SplitPlan {
 // the exchange, which grows with the tile.  Measured / estimated: 3072 x 384 over 4096 tokens (192 wide, 2 blocks) 14.8 / 15.3;
 // over 16384 40.8 / 40.4; 768 x 192 over 4096 (64, 4) 7.1 / 6.7; 1536 x 384 over 2048 (192, 4) 9.4 / 9.1; 4096 x 256 over 8192
 // (128, 2) 19.9 / 18.9.  Short reductions and many tiles are better left whole (no exchange): 3072 x 384 over 4096 tokens 14.9 us
-// in clusters of 2, 12.5 in 144 blocks 64 wide; over 512 6.8 / 5.1; 1536 x 384 over 2048 9.6 / 7.0.
+// in clusters of 2, 12.5 in 144 blocks 64 wide; over 512 6.8 / 5.1; 1536 x 384 over 2048 9.6 / 7.0.  Many waves want wide tiles:
+// 4096 x 4096 over 8192 tokens, 64 / 128 / 192 wide 426 / 299 / 274 us (without L2's limit the 128 wide ones looked best), 274 on
+// pairs; 4096 x 1024 115 / 74 / 90, on pairs 63.
 static double split_us(int bn, int S, int64_t tiles, int64_t deepest, int64_t kblocks) {
     const double kb_bytes = BM * BK * 2.0 + bn * BK * 2.0;
     if (S > 1) return 4.2 + 0.022 * (bn - 64) + std::max(0.7e6 * (double)deepest * kb_bytes / 110e9, 0.8e6 * (double)kblocks * kb_bytes / 14e12);
+    // single blocks: the issue loop's or the MMAs' pace, or, once every SM has a block, what L2 delivers to all of them
     const int64_t waves = (tiles + kNumSms - 1) / kNumSms;
-    return 2.5 + 0.006 * (bn - 64) + (double)(waves * deepest) * std::max(0.2, 0.0017 * bn) + 3.0 * (double)(waves - 1);
+    const double pace = std::max({0.2, 0.0017 * bn, (double)std::min<int64_t>(tiles, kNumSms) * kb_bytes / 18.5e6});
+    return 2.5 + 0.006 * (bn - 64) + (double)(waves * deepest) * pace + 3.0 * (double)(waves - 1);
 }
 
 // One weight gradient: the candidates are tile widths that the reduction buffers fit (<= 192) and cluster sizes that divide

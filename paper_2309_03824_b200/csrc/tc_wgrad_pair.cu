@@ -382,7 +382,8 @@ int max_active_clusters(int n) {
 struct Plan { int bn, pairs; double us; };
 
 // Estimated microseconds: 3 of launch and first loads, the k-blocks of a pair's share, 1.5 of stores, 2.5 of exchange (measured
-// at 4096 x 512 over 8192 tokens: 256 wide one pair 54.9, two 33.3, 128 wide one pair 36.0).
+// at 4096 x 512 over 8192 tokens: 256 wide one pair 54.9, two 33.3, 128 wide one pair 36.0); every further wave pays for its
+// first loads too (4096 x 4096 over 2048 tokens, four waves: 73.0, as 192 wide tiles of single SMs 69.1).
 Plan make_plan(const GemmArgs* g, int n) {
     Plan best{0, 0, 1e300};
     bool sums = false;
@@ -400,7 +401,7 @@ Plan make_plan(const GemmArgs* g, int n) {
             const int64_t room = max_active_clusters(2 * S), waves = (tiles + room - 1) / room;
             if (S > 1 && waves > 1) continue;
             const double per = (bn == 256 ? 0.40 : 0.25) + (sums ? 0.01 : 0.0);
-            const double us = (double)waves * ((double)((kb + S - 1) / S) * per + (S > 1 ? 4.0 : 1.5)) + 3.0;
+            const double us = (double)waves * ((double)((kb + S - 1) / S) * per + (S > 1 ? 4.0 : 1.5)) + 3.0 * (double)waves;
             if (us < best.us) best = Plan{bn, S, us};
         }
     }
