@@ -84,9 +84,10 @@ GemmArgs gemm(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, bool 
 // latency while the separate products spread each factor over all SMs and split long reductions; with many the chain
 // saves the trip of the rank-r intermediate and a launch; pairs halve the factors' traffic where the first product
 // dominates or the T buffer leaves no room.  Forward of 1024 -> 4096 at r = 512, in us (products / single blocks /
-// pairs): 256 tokens 9.6 / 14.6 / 23.5, 4096 tokens 30 / 27 / 41, 8192 tokens 51 / 61 / 46; 768 -> 768 at r = 192: 128
-// tokens 8.1 / 7.5 / -, 4096 tokens 12.3 / 9.2 / 10.9.  No simple line separates them, so each kernel estimates its
-// time; over 96 measured layers the choice costs 0.4 % on average against the best of the three.
+// pairs): 256 tokens 10.5 / 15.2 / 24.0, 4096 tokens 27 / 33 / 38, 8192 tokens 42 / 61 / 42; 768 -> 768 at r = 192: 128
+// tokens 8.9 / 7.9 / -, 4096 tokens 12.0 / 9.5 / 11.4.  No simple line separates them, so each kernel estimates its
+// time; over 336 measured forward passes (64 to 8192 tokens, 11 layers, two ranks each) the choice costs 0.7 % on average
+// against the best of the three.
 enum class Form { products, single, pair };
 // whole_t: the separate products would have to form T in one piece
 Form choose_form(const ChainArgs* c, int n, int path, bool leave_room, bool whole_t) {
@@ -789,6 +790,7 @@ static lrd_status_t lrd_linear_group_fwd_impl(int n, const lrd_linear_desc_t* de
             ok = parse_linear(&descs[i], &L, false) == LRD_OK && L.M > 0;
             if (ok) c[i] = fwd_chain_args(L, X[i], V[i], U[i], bias ? bias[i] : nullptr, Y[i], Z_save ? Z_save[i] : nullptr, 0);
         }
+        // Three layers 768 -> 768 at r = 192, in one launch / side by side: 200 tokens 10.2 / 10.4 us, 512 tokens 10.5 / 18.3.
         // (not where the layers' own calls split the reduction of a saved Z, whose bits a group keeps; that costs three layers
         // 4096 -> 1024 at r = 384 nothing at 256 tokens, 22.2 us in one launch, 22.9 side by side, and at 512 22.2 / 29.0)
         if (ok && !(Z_save && alone_splits_t(c[0], path)) && chain_pair_eligible(c, n)) return chain_pair_launch(c, n, s);
