@@ -903,12 +903,13 @@ static lrd_status_t launch_group(const GemmArgs* g, int n, int S, cudaStream_t s
 // its exchange over a chip that is mostly idle, so as many as the caller has at hand go into one launch, on single SMs
 // (a cluster per tile) or on pairs, when the estimate is below the sum of theirs.  Forward and backward of a layer with nothing
 // frozen, each alone / together: 4096 -> 4096 at rank 512, 8192 tokens 189 / 182 us; rank 256 142 / 132; 768 -> 3072 at 384,
-// 4096 tokens 73 / 62; 1024 -> 4096 at 512, 1024 tokens 48 / 42; 768 -> 768 at 192, 300 tokens 30 / 21.
+// 4096 tokens 73 / 62; 1024 -> 4096 at 512, 1024 tokens 48 / 42; 768 -> 768 at 192, 300 tokens 30 / 21.  Two launches cost 2 us
+// more than their times alone (backward of the first layer at rank 1000, 2 x 64 tiles on pairs: two launches 256 us, one of two waves 242).
 lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const size_t* partial_bytes, cudaStream_t stream) {
     const WgradForm& form = tc_wgrad_form();
     bool ones = false, together = n > 1 && n <= kMaxWgrads;
     int64_t rows = 0;
-    double separate = 0.0;
+    double separate = 2.0 * (n - 1);           // a launch behind another one drains and fills the SMs anew
     for (int i = 0; i < n && together; ++i) {
         together = tc_gemm_eligible(g[i]) && g[i].a_mn_major && g[i].b_mn_major && !g[i].bias && g[i].max_cluster_split == g[0].max_cluster_split &&
                    g[i].add == g[0].add;
