@@ -142,7 +142,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
         uint32_t ph = 1;                                     // parity to wait on for an empty stage
         bool ok = true;
         const int atom_cols = p.swb / 2;
-        const int n_pbox = p.RS / atom_cols;
+        const int n_pbox = (p.RS + atom_cols - 1) / atom_cols;     // (the last box may reach into the next slice)
         for (int g = 0; g < ng1 && ok; ++g) {
             const uint32_t fb = smem_u32(&full1[s]);
             ok = mbar_wait_uniform(smem_u32(&empty1[s]), ph, ab);
@@ -413,7 +413,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
 }
 
 struct Plan {
-    int C, RS, swb, BN2, G1, S1, S2, slabs;
+    int C, RS, swb, taw, BN2, G1, S1, S2, slabs;
     uint32_t stage1_bytes, stage2_bytes, t_bytes, smem_bytes;
 };
 
@@ -486,10 +486,12 @@ bool make_plan(const ChainArgs& a, Plan* out) {
         if (a.r % (16 * C)) continue;
         const int RS = (int)a.r / C;
         if (RS > 256) continue;
-        const int swb = RS % 64 == 0 ? 128 : (RS % 32 == 0 ? 64 : 32);
+        const int taw = RS % 64 == 0 ? 64 : (RS % 32 == 0 ? 32 : 16);
+        const int swb = p_box_span(RS);
+        const uint32_t p_cols = (uint32_t)((RS + swb / 2 - 1) / (swb / 2) * (swb / 2));
         const int BN2 = pick_bn2(a.N2, C);
         const int64_t ring1 = (int64_t)kSmemLimit - 1024;                         // phase 1 has all of it
-        const uint32_t kb1_bytes = kInTileBytes + 128u * RS, kb2_bytes = (uint32_t)BN2 * 128u;
+        const uint32_t kb1_bytes = kInTileBytes + 128u * p_cols, kb2_bytes = (uint32_t)BN2 * 128u;
         // a second set of epilogue slabs where it does not cost the ring of Q tiles a slot that it needs
         const int64_t room2 = ring1 - t_bytes;
         const int slabs = (room2 - 2 * (int64_t)kSlabsBytes) / kb2_bytes >= std::min<int64_t>((room2 - (int64_t)kSlabsBytes) / kb2_bytes, 4) ? 2 : 1;
@@ -509,7 +511,7 @@ bool make_plan(const ChainArgs& a, Plan* out) {
         const uint32_t s1b = (uint32_t)G1 * kb1_bytes;
         const uint32_t used1 = (uint32_t)S1 * s1b, used2 = (uint32_t)slabs * kSlabsBytes + (uint32_t)S2 * kb2_bytes;
         const uint32_t after1 = (uint32_t)t_bytes + used2;
-        Plan pl{C, RS, swb, BN2, G1, S1, S2, slabs, s1b, kb2_bytes, (uint32_t)t_bytes, 1024u + (used1 > after1 ? used1 : after1)};
+        Plan pl{C, RS, swb, taw, BN2, G1, S1, S2, slabs, s1b, kb2_bytes, (uint32_t)t_bytes, 1024u + (used1 > after1 ? used1 : after1)};
         // prefer the largest cluster whose blocks are all resident at once (within this launch's share of the
         // SMs, when it runs beside other launches); else the smallest feasible.  With few row tiles the kernel is one
         // block's latency -- its share of P and Q through one SM -- so more blocks per tile shorten it: 768 -> 3072 at
@@ -561,7 +563,7 @@ lrd_status_t chain_launch(const ChainArgs& a, cudaStream_t stream) {
     ok = ok && make_tmap_2d_bf16(&tQ, a.Q, (uint64_t)a.N2, (uint64_t)a.r, (uint64_t)a.ldq, (uint32_t)pl.BN2, 64);
     ok = ok && make_tmap_2d_bf16(&tOut, a.Out, (uint64_t)a.M, (uint64_t)a.N2, (uint64_t)a.ld_out, 32, 32);
     if (a.T_save)
-        ok = ok && make_tmap_2d_bf16(&tT, a.T_save, (uint64_t)a.M, (uint64_t)a.r, (uint64_t)a.ldt, 128, (uint32_t)pl.swb / 2);
+        ok = ok && make_tmap_2d_bf16(&tT, a.T_save, (uint64_t)a.M, (uint64_t)a.r, (uint64_t)a.ldt, 128, (uint32_t)pl.taw);
     else
         tT = tOut;
     if (!ok) return LRD_ERR_CUDA;
@@ -575,7 +577,7 @@ lrd_status_t chain_launch(const ChainArgs& a, cudaStream_t stream) {
     p.N2 = (int)a.N2;
     p.G1 = pl.G1; p.S1 = pl.S1; p.S2 = pl.S2; p.slabs = pl.slabs;
     p.stage1_bytes = pl.stage1_bytes; p.stage2_bytes = pl.stage2_bytes; p.t_bytes = pl.t_bytes;
-    p.taw = pl.swb / 2;
+    p.taw = pl.taw;
     p.t_steps_lg = p.taw == 64 ? 2 : (p.taw == 32 ? 1 : 0);
     p.bias = (const __nv_bfloat16*)a.bias;
     p.has_tsave = a.T_save ? 1 : 0;

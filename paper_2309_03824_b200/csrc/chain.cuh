@@ -14,6 +14,12 @@ inline double chain_us(double fixed, int64_t waves, double ng1, double t1, int64
     return fixed + (double)waves * (ng1 * t1 + m2 + (double)(chunks - 1) * (m2 > epilogue ? m2 : epilogue) + epilogue) + 2.0 * (double)(waves - 1);
 }
 
+// Row length in bytes (= swizzle span) of the boxes a block's `cols` columns of P are loaded in.  A box costs the TMA unit its
+// rows, however short they are: columns that fill no whole 64-wide boxes are loaded in boxes 64 wide all the same, whose last
+// one brings columns that nobody multiplies, rather than in three to seven boxes of 32- or 64-byte rows.  768 -> 768 at r = 192
+// (slices of 48), 4096 tokens: forward 9.01 -> 8.80 us, backward with V frozen 16.6 -> 16.2; other widths within 1 %.
+inline int p_box_span(int cols) { return cols > 32 ? 128 : cols > 16 ? 64 : 32; }
+
 struct ChainArgs {
     int64_t M, K1, r, N2;
     const void* In; int64_t ld_in;     // [M x K1]

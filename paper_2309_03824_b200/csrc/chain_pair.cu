@@ -155,7 +155,7 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
         uint32_t ph = 1;                                     // parity to wait on for an empty slot
         bool ok = true;
         const int atom_cols = p.swb / 2;
-        const int n_pbox = RSL / atom_cols;
+        const int n_pbox = (RSL + atom_cols - 1) / atom_cols;     // (the last box may reach past this block's columns)
         const int p_col0 = pr * p.RS + h * RSL;              // first column of P this block loads
         cluster_arrive_relaxed();                            // barrier 1 (this warp has nothing to tell)
         for (int g = 0; g < ng1 && ok; ++g) {
@@ -510,11 +510,12 @@ bool make_plan(const ChainArgs& a, int layers, Plan* out) {
         if (a.r % (32 * S)) continue;
         const int RS = (int)a.r / S, RSL = RS / 2;
         if (RS > 256) continue;
-        const int swb = RSL % 64 == 0 ? 128 : (RSL % 32 == 0 ? 64 : 32);
+        const int swb = p_box_span(RSL);
+        const uint32_t p_cols = (uint32_t)((RSL + swb / 2 - 1) / (swb / 2) * (swb / 2));
         const int taw = RS % 64 == 0 ? 64 : (RS % 32 == 0 ? 32 : 16);
         const int BN2 = pick_bn2(a.N2, S);
         if (BN2 % 32) continue;
-        const uint32_t kb1_bytes = kInTileBytes + 128u * (uint32_t)RSL, kb2_bytes = (uint32_t)(BN2 / 2) * 128u;
+        const uint32_t kb1_bytes = kInTileBytes + 128u * p_cols, kb2_bytes = (uint32_t)(BN2 / 2) * 128u;
         // two k-blocks per phase-1 stage where they are small: the MMA warp's work per stage (a wait, a commit)
         // is then spread over eight MMAs
         int G1 = g_tune_G1 ? g_tune_G1 : (kb1_bytes <= 28 * 1024 ? 2 : 1);

@@ -210,3 +210,17 @@ def test_gemm_tuning_rejects_values_outside_the_list():
         with pytest.raises(b.LrdError):
             b.lrd_gemm_tuning(bad)
     b.lrd_gemm_tuning(0)
+
+
+@pytest.mark.parametrize("blocks,shape", [(4, (300, 264, 520, 192)), (3, (200, 264, 328, 240)), (2, (130, 328, 264, 224)), (4, (260, 392, 520, 384)), (1, (129, 72, 136, 48))])
+def test_slices_that_fill_no_whole_boxes(blocks, shape):
+    """Slices of 48, 80, 112, 96 and 48 columns: the last 64-wide box of the first factor reaches into the next slice, or past the rank."""
+    b.lrd_chain_tuning(blocks, 0, 0)
+    b.lrd_chain_pair_tuning(1, 0, 0, 0)
+    check_linear(wl.random_factor_case(*shape, "bf16", 970 + shape[3]), b.LRD_FREEZE_NONE, path=b.LRD_PATH_FUSED)
+
+
+@pytest.mark.parametrize("pairs,rank", [(1, 96), (1, 160), (2, 192), (3, 288)])
+def test_slices_of_a_pair_that_fill_no_whole_boxes(pairs, rank):
+    b.lrd_chain_pair_tuning(2, pairs, 0, 0)                             # 48, 80, 48 and 48 columns for each block
+    check_linear(wl.random_factor_case(300, 328, 520, rank, "bf16", 980 + rank), b.LRD_FREEZE_NONE)
