@@ -73,6 +73,7 @@ struct TcParams {
     int cluster_splits; // > 1: the gridDim.z blocks of a tile are one cluster and reduce through shared memory
     // CONV: input channels, 64-column blocks of a tap and of all taps, k of the k x k taps, output grid, stride, pad
     int cv_ci, cv_nkc, cv_nblk, cv_k, cv_Ho, cv_Wo, cv_stride, cv_pad;
+    int has_c_map;      // the result goes out by TMA
     float* colsum_partial;        // ONES, split: [splits][M] partial sums over k of A
     __nv_bfloat16* colsum_out;    // ONES, not split: [M]
     unsigned int* timeout_flag;
@@ -83,12 +84,8 @@ struct TcParams {
 template <int NP> struct TcLaunch {
     int row0[NP];       // first row tile of each product (INT_MAX: none)
     TcParams p[NP];
-    CUtensorMap tA[NP], tB[NP];
+    CUtensorMap tA[NP], tB[NP], tC[NP];        // tC: boxes of 32 rows x 64 columns (tiles of one block) or one block's columns (cluster split, ADD)
 };
-
-__device__ __forceinline__ uint4 add_bf16x8(const uint4& a, const uint4& b) {
-    return make_uint4(add_bf16x2(a.x, b.x), add_bf16x2(a.y, b.y), add_bf16x2(a.z, b.z), add_bf16x2(a.w, b.w));
-}
 
 // CONV: column of dG (= tap * ci + channel) that column `col` of the product belongs to; -1: padding
 __device__ __forceinline__ int conv_col(const TcParams& p, int col) {
@@ -107,7 +104,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
 #pragma unroll
     for (int i = 1; i < NP; ++i)
         if ((int)blockIdx.y >= L.row0[i]) prod = i;
-    const CUtensorMap &tmA = L.tA[prod], &tmB = L.tB[prod];
+    const CUtensorMap &tmA = L.tA[prod], &tmB = L.tB[prod], &tmC = L.tC[prod];
     const TcParams p = L.p[prod];
     if (NP > 1 && (int64_t)blockIdx.x * BN >= p.N) return;         // (the whole cluster: its blocks share x and y)
     static_assert(!ONES || (A_MN && B_MN && BN <= 192), "the ones block rides on an MN-major B of at most 192 columns");
@@ -133,6 +130,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         abort_flag = 0;
         prefetch_tmap(&tmA);
         prefetch_tmap(&tmB);
+        if (p.has_c_map) prefetch_tmap(&tmC);
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 1);
             mbar_init(smem_u32(&empty_bar[s]), 1);
@@ -265,11 +263,6 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         const uint32_t chunk_bytes = 128u * cs * 4u, ngrp = cs / 4u;
         const uint32_t stage_base = smem_base, recv_base = smem_base + 128u * BN * 4u;
         const uint32_t cs_stage = recv_base + 128u * BN * 4u, cs_recv = cs_stage + 512u;
-        if (ADD) {             // what this block's slice adds to, on its way while the products are formed
-            const int64_t grow = (int64_t)m0 + row, gcol0 = (int64_t)n0 + self * cs;
-            for (uint32_t c = 0; c < cs; c += 64)
-                if (grow < p.M && gcol0 + c < p.N) prefetch_l2((const __nv_bfloat16*)p.C + grow * p.ldc + gcol0 + c);
-        }
         bool ok = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         // barrier 1: this block's pipeline ring is dead (all its MMAs have completed).  Progress only: what the peers
@@ -368,42 +361,47 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                 if (CONV && at < 0) return;
                 __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + at;
                 if (CONV || col + 8 <= p.N) {
-                    uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-                    if (ADD) v = add_bf16x8(v, *reinterpret_cast<const uint4*>(dst));
-                    *reinterpret_cast<uint4*>(dst) = v;
+                    *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
                 } else {
                     for (int e = 0; e < 8; ++e)
-                        if (col + e < p.N) {
-                            if (ADD) add_into_bf16(dst + e, acc[e]);
-                            else dst[e] = __float2bfloat16_rn(acc[e]);
-                        }
+                        if (col + e < p.N) dst[e] = __float2bfloat16_rn(acc[e]);
                 }
             };
             // 16 columns (one whole 32-byte sector) per store instruction where the layout allows, else two 16-byte stores
             const bool sectors = (p.ldc % 16 == 0) && (((uintptr_t)p.C & 31u) == 0) && (gcol0 % 16 == 0) && (!CONV || p.cv_ci % 16 == 0);
+            const uint32_t slab = recv_base + self * chunk_bytes + (uint32_t)row * cs * 2u;        // (ADD; nobody sends to the own slot)
             for (uint32_t c4 = 0; c4 < cs; c4 += 16) {
                 uint32_t w0[4], w1[4];
                 float a0[8], a1[8];
                 sum8(c4, w0, a0);
                 const bool second = c4 + 8 < cs;
                 if (second) sum8(c4 + 8, w1, a1);
+                if (ADD) {
+                    st_shared_v4(slab + c4 * 2u, w0[0], w0[1], w0[2], w0[3]);
+                    if (second) st_shared_v4(slab + c4 * 2u + 16u, w1[0], w1[1], w1[2], w1[3]);
+                    continue;
+                }
                 const int64_t col = gcol0 + c4;
                 if (sectors && second && grow < p.M && col + 16 <= p.N) {
                     const int64_t at = CONV ? conv_col(p, (int)col) : col;
                     if (CONV && at < 0) continue;
                     __nv_bfloat16* dst = (__nv_bfloat16*)p.C + grow * p.ldc + at;
-                    if (ADD) {
-                        const uint4 o0 = reinterpret_cast<const uint4*>(dst)[0], o1 = reinterpret_cast<const uint4*>(dst)[1];
-                        const uint4 s0 = add_bf16x8(make_uint4(w0[0], w0[1], w0[2], w0[3]), o0), s1 = add_bf16x8(make_uint4(w1[0], w1[1], w1[2], w1[3]), o1);
-                        w0[0] = s0.x; w0[1] = s0.y; w0[2] = s0.z; w0[3] = s0.w;
-                        w1[0] = s1.x; w1[1] = s1.y; w1[2] = s1.z; w1[3] = s1.w;
-                    }
                     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                                  ::"l"(dst), "r"(w0[0]), "r"(w0[1]), "r"(w0[2]), "r"(w0[3]), "r"(w1[0]), "r"(w1[1]), "r"(w1[2]), "r"(w1[3]) : "memory");
                 } else {
                     store8(c4, w0, a0);
                     if (second) store8(c4 + 8, w1, a1);
                 }
+            }
+            if (ADD) {
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (elect_one()) {
+                    if (m0 + quarter * 32 < p.M && gcol0 < p.N) tma_add_2d(&tmC, recv_base + self * chunk_bytes + quarter * 32u * cs * 2u, (int)gcol0, m0 + quarter * 32);
+                    tma_store_commit();
+                    tma_store_wait_read<0>();
+                }
+                __syncwarp();
             }
             if (with_colsum && self == 0 && p.colsum_out && grow < p.M) {
                 float t = 0.f;
@@ -419,20 +417,15 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         }
     } else {
         const int quarter = warp % 4;                      // lanes [32 q, 32 q + 32) of tensor memory
-        if (ADD) {
-            const int64_t row = (int64_t)m0 + quarter * 32 + lane;
-            for (int c = 0; c < BN; c += 64)
-                if (row < p.M && n0 + c < p.N) prefetch_l2((const __nv_bfloat16*)p.C + row * p.ldc + n0 + c);
-        }
         const bool ready = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         if (ready) {
+            const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
             const int64_t row = (int64_t)m0 + quarter * 32 + lane;
             const bool row_ok = row < p.M;
-            const bool bias_vec_ok = p.bias && (((uintptr_t)p.bias & 15u) == 0);
             if (with_colsum) {                             // accumulator column BN = sum over k of A(row, k)
                 uint32_t cs[16];
-                tmem_ld_32x16(tmem_base + ((uint32_t)(quarter * 32) << 16) + BN, cs);
+                tmem_ld_32x16(lane_addr + BN, cs);
                 tmem_ld_wait();
                 if (row_ok) {
                     if (p.partial) p.colsum_partial[(int64_t)blockIdx.z * p.M + row] = __uint_as_float(cs[0]);
@@ -440,14 +433,14 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                     else if (p.colsum_out) p.colsum_out[row] = __float2bfloat16_rn(__uint_as_float(cs[0]));
                 }
             }
+            if (p.partial) {
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-                uint32_t v[32];
-                tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + c * 32, v);
-                tmem_ld_wait();
-                const int64_t col0 = (int64_t)n0 + c * 32;
-                if (!row_ok || col0 >= p.N) continue;
-                if (p.partial) {
+                for (int c = 0; c < BN / 32; ++c) {
+                    uint32_t v[32];
+                    tmem_ld_32x32(lane_addr + c * 32, v);
+                    tmem_ld_wait();
+                    const int64_t col0 = (int64_t)n0 + c * 32;
+                    if (!row_ok || col0 >= p.N) continue;
                     float* dst = (float*)p.C + ((int64_t)blockIdx.z * p.M + row) * p.ldp + col0;
 #pragma unroll
                     for (int g = 0; g < 8; ++g) {
@@ -458,48 +451,51 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                                 if (col0 + g * 4 + e < p.N) dst[g * 4 + e] = __uint_as_float(v[4 * g + e]);
                         }
                     }
-                } else {
-                    __nv_bfloat16* dst = (__nv_bfloat16*)p.C + row * p.ldc + col0;
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        if (CONV) {                        // 8 columns of one tap, inside or outside together
-                            const int at = conv_col(p, (int)col0 + g * 8);
-                            if (at >= 0)
-                                *reinterpret_cast<uint4*>((__nv_bfloat16*)p.C + row * p.ldc + at) =
-                                    make_uint4(pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1])), pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3])),
-                                               pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5])), pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7])));
-                            continue;
-                        }
-                        float f[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * g + e]);
-                        if (p.bias) {
-                            if (bias_vec_ok && col0 + g * 8 + 8 <= p.N) {       // one 16-byte load for 8 columns
-                                const uint4 b4 = __ldg(reinterpret_cast<const uint4*>(p.bias + col0 + g * 8));
-                                const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    f[2 * e] += __uint_as_float(bw[e] << 16);
-                                    f[2 * e + 1] += __uint_as_float(bw[e] & 0xFFFF0000u);
-                                }
-                            } else {
-                                for (int e = 0; e < 8; ++e)
-                                    if (col0 + g * 8 + e < p.N) f[e] += __bfloat162float(p.bias[col0 + g * 8 + e]);
-                            }
-                        }
-                        if (col0 + g * 8 + 8 <= p.N) {
-                            uint4 x = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
-                            if (ADD) x = add_bf16x8(x, *reinterpret_cast<const uint4*>(dst + g * 8));
-                            *reinterpret_cast<uint4*>(dst + g * 8) = x;
-                        } else {
-                            for (int e = 0; e < 8; ++e)
-                                if (col0 + g * 8 + e < p.N) {
-                                    if (ADD) add_into_bf16(dst + g * 8 + e, f[e]);
-                                    else dst[g * 8 + e] = __float2bfloat16_rn(f[e]);
-                                }
-                        }
-                    }
                 }
+            } else {
+                // 64 columns of the warp's 32 rows at a time through a slab of their own in the dead ring (128-byte swizzle), then
+                // out by one TMA store, or, ADD, by one that adds in L2 (the fp32 sum of two bf16 values, rounded once).  Stores
+                // straight from the registers, each lane a row of its own, were four dependent steps of scattered 16-byte
+                // accesses, and reading C for them as many trips to memory: 4096 x 512 over 1021 tokens, accumulating, 128 blocks
+                // 128 wide: 6 us behind the last MMA, the pass 41.9 us, now 37.0; 768 x 192 over 128 tokens, a pass 19.0 -> 18.5.
+                const uint32_t slab0 = smem_base + (uint32_t)quarter * (BN / 64 * 4096u), row_off = (uint32_t)lane * 128u, row_xor = (uint32_t)lane & 7u;
+#pragma unroll 1
+                for (int c = 0; c < BN / 64; ++c) {
+                    const int col0 = n0 + c * 64;
+                    if (col0 >= p.N && !CONV) break;       // (uniform)
+                    uint32_t v[64];
+                    tmem_ld_32x32(lane_addr + c * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                    tmem_ld_32x32(lane_addr + c * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+                    tmem_ld_wait();
+                    uint32_t w[32];
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) w[e] = pack_bf16(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+                    if (CONV) {                            // 8 columns of one tap, inside or outside together
+#pragma unroll
+                        for (int g = 0; g < 8; ++g) {
+                            const int at = col0 < p.N ? conv_col(p, col0 + g * 8) : -1;
+                            if (row_ok && at >= 0)
+                                *reinterpret_cast<uint4*>((__nv_bfloat16*)p.C + row * p.ldc + at) = make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+                        }
+                        continue;
+                    }
+                    const uint32_t slab = slab0 + (uint32_t)c * 4096u;
+#pragma unroll
+                    for (int g = 0; g < 8; ++g)
+                        st_shared_v4(slab + row_off + (((uint32_t)g ^ row_xor) << 4), w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (elect_one()) {
+                        if (m0 + quarter * 32 < p.M) {
+                            if (ADD) tma_add_2d(&tmC, slab, col0, m0 + quarter * 32);
+                            else tma_store_2d(&tmC, slab, col0, m0 + quarter * 32);
+                        }
+                        tma_store_commit();
+                    }
+                    __syncwarp();
+                }
+                tma_store_wait_read<0>();                  // shared memory may go once the stores have read it
+                __syncwarp();
             }
         }
     }
@@ -595,6 +591,12 @@ lrd_status_t launch_wgrad(bool add, const TcLaunch<NP>& L, dim3 grid, cudaStream
 }
 
 inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+
+// Tensor map of the result where it leaves by TMA.
+bool result_map(const GemmArgs& g, bool add, int bn, int cluster, bool partial, CUtensorMap* t, TcParams* p) {
+    p->has_c_map = !partial && (cluster <= 1 || add);
+    return !p->has_c_map || make_tmap_2d_bf16(t, g.C, (uint64_t)g.M, (uint64_t)g.N, (uint64_t)g.ldc, 32, cluster > 1 ? (uint32_t)(bn / cluster) : 64u, cluster <= 1);
+}
 
 uint32_t stage_kblocks(int bn, bool ones) {
     switch (bn) {
@@ -820,9 +822,10 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
                            : make_tmap_2d_bf16(&tA, g.A, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda, BM, BK);
     ok = ok && (g.b_mn_major ? make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb, kbox, 64)
                              : make_tmap_2d_bf16(&tB, g.B, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb, (uint32_t)bn, BK));
+    TcParams& p = L.p[0];
+    ok = ok && result_map(g, g.add && splits == 1, bn, cluster, splits > 1, &L.tC[0], &p);
     if (!ok) return LRD_ERR_CUDA;
 
-    TcParams& p = L.p[0];
     p.M = g.M; p.N = g.N; p.ldp = ldp; p.kb_total = kb_total; p.kb_per_split = kb_per;
     p.partial = splits > 1 ? 1 : 0;
     p.cluster_splits = cluster;
@@ -886,6 +889,7 @@ static lrd_status_t launch_group(const GemmArgs* g, int n, int S, cudaStream_t s
             !make_tmap_2d_bf16(&L.tB[i], g[i].B, (uint64_t)g[i].K, (uint64_t)g[i].N, (uint64_t)g[i].ldb, kbox, 64))
             return LRD_ERR_CUDA;
         TcParams& p = L.p[i];
+        if (!result_map(g[i], g[i].add, BN, S, false, &L.tC[i], &p)) return LRD_ERR_CUDA;
         p.M = g[i].M; p.N = g[i].N; p.ldp = g[i].N;
         p.kb_total = (int)((g[i].K + BK - 1) / BK);
         p.kb_per_split = (p.kb_total + S - 1) / S;

@@ -8,10 +8,10 @@
 namespace lrd {
 
 // 2-D bf16 tensor [rows x cols], row stride ld elements, box [box_rows x box_cols]; the swizzle
-// span equals the box row (128, 64 or 32 bytes; none otherwise); zero fill outside the tensor.
+// span equals the box row (128, 64 or 32 bytes; none otherwise, or where asked for); zero fill outside the tensor.
 // Returns false on failure.
 bool make_tmap_2d_bf16(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld_elems,
-                       uint32_t box_rows, uint32_t box_cols);
+                       uint32_t box_rows, uint32_t box_cols, bool swizzled = true);
 
 // 4-D bf16 NHWC tensor [B][H][W][C], box [1][box_h][box_w][box_c], 128-byte swizzle, zero fill.
 bool make_tmap_nhwc_bf16(CUtensorMap* out, const void* base, uint64_t B, uint64_t H, uint64_t W, uint64_t C,

@@ -112,3 +112,28 @@ def test_override_values():
     for bad in [(192, 2), (64, 3), (64, 0), (0, 2)]:
         with pytest.raises(b.LrdError):
             b.lrd_data_split_tuning(*bad)
+
+
+@gpu
+@pytest.mark.parametrize("form", SINGLE, ids=lambda f: "x".join(map(str, f)))
+@pytest.mark.parametrize("shape", SHAPES + [(130, 72, 1000, 8)], ids=lambda s: "x".join(map(str, s)))
+def test_adding_leaves_the_rest_alone(form, shape, forms):
+    """Gradients added to buffers with a leading dimension of their own: ragged rows and columns, and nothing outside them."""
+    M, K, N, r = shape
+    case = wl.random_factor_case(M, K, N, r, "bf16", 570 + M)
+    X, V, U, dY = (torch.from_numpy(case[k]).to("cuda", torch.bfloat16) for k in ("X", "V", "U", "dY"))
+    Z, ld = (X.float() @ V.float()).to(torch.bfloat16), r + 24
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16)
+    desc.ldu = ld
+    Up, dU = (torch.full((N, ld), 3.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    Up[:, :r] = U
+    db, dX = torch.ones(N, dtype=torch.bfloat16, device="cuda"), torch.empty_like(X)
+    ws = torch.empty(b.lrd_linear_workspace_bytes(desc, b.LRD_FREEZE_V, 2), dtype=torch.uint8, device="cuda")
+    b.lrd_wgrad_tuning(*form)
+    b.lrd_linear_bwd_accumulate(desc, dY, None, V, Up, Z, dX, dU, None, db, b.LRD_FREEZE_V, ws)
+    assert b.lrd_check_device_status() == b.LRD_OK
+    ref = dY.double().T @ Z.double()
+    # one rounding of the product, one of the sum
+    assert float((dU[:, :r].double() - ref - 3).abs().max() / (ref.abs().max() + 3)) <= 2 ** -7
+    assert float((db.double() - dY.double().sum(0) - 1).abs().max() / dY.double().sum(0).abs().max()) <= 2 ** -7
+    assert bool((dU[:, r:] == 3).all())
