@@ -133,8 +133,8 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
     const uint32_t tmem_base = tmem_base_slot;
     // Everything above touched only this block's own shared and tensor memory, so it may overlap the tail
     // of the previous kernel in the stream; global memory is first read (and written) below this line.
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();       // (in this order: see GemmArgs::a_early)
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer

@@ -232,7 +232,9 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     else if (dX || factors) keep(conv_bwd_data(dZ2, G, dZ1, t.B, t.g, t.r1, t.r2, t.dt, path, s));
     if (dX && !fuse_dx && !one_launch) keep(run_gemm(make_gemm(t.P, t.C, t.r1, dZ1, t.r1, false, A, t.r1, false, dX, t.C, nullptr, t.dt), path, false, nullptr, 0, s));
     if (factors) {
-        const GemmArgs gw[2] = {make_gemm(t.C, t.r1, t.P, X, t.C, true, dZ1, t.r1, true, dA, t.r1, nullptr, t.dt), dB_product};
+        GemmArgs gw[2] = {make_gemm(t.C, t.r1, t.P, X, t.C, true, dZ1, t.r1, true, dA, t.r1, nullptr, t.dt), dB_product};
+        // the data path stands before them on this stream, and writes dZ1 alone of their operands
+        gw[0].a_early = gw[1].a_early = gw[1].b_early = true;
         float* const scratch[2] = {pA, pB};
         const size_t scratch_bytes[2] = {reg.dA, reg.dB};
         keep(run_wgrads(gw, core ? 1 : 2, path, scratch, scratch_bytes, s));

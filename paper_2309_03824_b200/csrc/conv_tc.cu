@@ -139,8 +139,8 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only this block's own shared and tensor memory: under programmatic dependent launch it
     // overlaps the tail of the previous kernel in the stream; global memory is first touched below this line
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();       // (in this order: see GemmArgs::a_early)
     // fused: once the core's MMAs are done the ring is dead; it then holds [T: one atom of 128 rows x 64 columns per 64
     // columns of the core's result | Q: one [n2 rows x 64 k] tile per 64 columns of the core's result]
     const int nq = (p.n_total + 63) / 64;

@@ -254,8 +254,8 @@ struct CopyBatch {
     int n;
 };
 __global__ void __launch_bounds__(256) copy2d_bf16_kernel(const __grid_constant__ CopyBatch b) {
-    ptx::griddep_launch_dependents();
     ptx::griddep_wait();
+    ptx::griddep_launch_dependents();
     const int lane = threadIdx.x % 32;
     const int64_t warps = (int64_t)gridDim.x * 8;
     int j = 0;
@@ -684,6 +684,12 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
     GemmArgs gw[2];
     const int n = linear_wgrads(L, plan, dY, X, Z_save, dZ, dU, dV, dbias, wsplit, gw);
     for (int i = 0; i < n; ++i) gw[i].add = accumulate;
+    // behind a launch of this call the gradients' operands that the data half does not write need not wait for it
+    if (!side && do_data && (dX || need_dz_in_memory))
+        for (int i = 0; i < n; ++i) {
+            gw[i].a_early = true;
+            gw[i].b_early = gw[i].B != dZ;
+        }
     if (side && n == 2) {
         LRD_TRY(run_gemm(gw[0], true, partials, partial_bytes, side));
         if (cudaEventRecord(side_done, side) != cudaSuccess || cudaStreamWaitEvent(s, side_done, 0) != cudaSuccess) return LRD_ERR_CUDA;

@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(NT, 2) simt_gemm_kernel(const __grid_constant_
     __shared__ __align__(16) float smem[C_::kSmem];
     float* As = smem;
     float* Bs = smem + TK * LDA;
-    ptx::griddep_launch_dependents();
     ptx::griddep_wait();
+    ptx::griddep_launch_dependents();       // (in this order: see GemmArgs::a_early)
     const int t = threadIdx.x;
     const int64_t n_tiles = (N + TN - 1) / TN;
     const int64_t m0 = (int64_t)(tile / n_tiles) * TM, n0 = (int64_t)(tile % n_tiles) * TN;

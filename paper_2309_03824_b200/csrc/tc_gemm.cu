@@ -73,6 +73,8 @@ struct TcParams {
     int cluster_splits; // > 1: the gridDim.z blocks of a tile are one cluster and reduce through shared memory
     // CONV: input channels, 64-column blocks of a tap and of all taps, k of the k x k taps, output grid, stride, pad
     int cv_ci, cv_nkc, cv_nblk, cv_k, cv_Ho, cv_Wo, cv_stride, cv_pad;
+    // Operands that no launch of the same call still in flight writes are loaded before this launch's turn (griddepcontrol.wait)
+    int a_early, b_early;
     int has_c_map;      // the result goes out by TMA
     float* colsum_partial;        // ONES, split: [splits][M] partial sums over k of A
     __nv_bfloat16* colsum_out;    // ONES, not split: [M]
@@ -106,7 +108,10 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         if ((int)blockIdx.y >= L.row0[i]) prod = i;
     const CUtensorMap &tmA = L.tA[prod], &tmB = L.tB[prod], &tmC = L.tC[prod];
     const TcParams p = L.p[prod];
-    if (NP > 1 && (int64_t)blockIdx.x * BN >= p.N) return;         // (the whole cluster: its blocks share x and y)
+    if (NP > 1 && (int64_t)blockIdx.x * BN >= p.N) {               // (the whole cluster: its blocks share x and y)
+        griddep_wait();
+        return;
+    }
     static_assert(!ONES || (A_MN && B_MN && BN <= 192), "the ones block rides on an MN-major B of at most 192 columns");
     static_assert(!ADD || !CONV, "only weight gradients add");
     static_assert(!CONV || (A_MN && B_MN && !ONES && BN <= 192), "the filter gradient: both operands MN-major, split over a cluster or not at all");
@@ -160,12 +165,13 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only this block's own shared and tensor memory: it may overlap the tail of the
-    // previous kernel in the stream; global memory is first touched below this line
+    // previous kernel in the stream; global memory is first touched below this line, by the producers and then by the epilogue
+    if (!A_MN) griddep_wait();         // (in this order: see GemmArgs::a_early)
     griddep_launch_dependents();
-    griddep_wait();
 
     if (warp == 0) {
         // TMA producer: the whole warp runs the loop, one elected lane issues (operands stay uniform)
+        if (!p.a_early) griddep_wait();
         int it = 0;
         for (int kb = kb_begin; kb < kb_end; kb += G, ++it) {          // (a k-block past this block's share is loaded, not multiplied)
             const int s = it % STAGES;
@@ -190,6 +196,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     } else if (warp == 6) {
         // second TMA producer: the B operand of every stage (its bytes are counted by warp 0's expect_tx; a copy that
         // lands before that arrival only makes the barrier's byte count negative for a moment)
+        if (!p.b_early) griddep_wait();
         int it = 0;
         for (int kb = kb_begin; kb < kb_end; kb += G, ++it) {
             const int s = it % STAGES;
@@ -263,6 +270,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         const uint32_t chunk_bytes = 128u * cs * 4u, ngrp = cs / 4u;
         const uint32_t stage_base = smem_base, recv_base = smem_base + 128u * BN * 4u;
         const uint32_t cs_stage = recv_base + 128u * BN * 4u, cs_recv = cs_stage + 512u;
+        if (ADD) griddep_wait();
         bool ok = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         // barrier 1: this block's pipeline ring is dead (all its MMAs have completed).  Progress only: what the peers
@@ -417,6 +425,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         }
     } else {
         const int quarter = warp % 4;                      // lanes [32 q, 32 q + 32) of tensor memory
+        if (ADD) griddep_wait();
         const bool ready = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         if (ready) {
@@ -500,6 +509,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         }
     }
 
+    griddep_wait();        // (early loads: this launch ends no sooner than the one before it, on which the launches behind it rely)
     // cluster split, barrier 2: no block leaves while a peer may still be reading its slice out of this
     // block's shared memory
     if (p.cluster_splits > 1) cluster_wait();
@@ -592,9 +602,10 @@ lrd_status_t launch_wgrad(bool add, const TcLaunch<NP>& L, dim3 grid, cudaStream
 
 inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-// Tensor map of the result where it leaves by TMA.
+// Tensor map of the result where it leaves by TMA, and the early operands.
 bool result_map(const GemmArgs& g, bool add, int bn, int cluster, bool partial, CUtensorMap* t, TcParams* p) {
     p->has_c_map = !partial && (cluster <= 1 || add);
+    p->a_early = g.a_early; p->b_early = g.b_early;
     return !p->has_c_map || make_tmap_2d_bf16(t, g.C, (uint64_t)g.M, (uint64_t)g.N, (uint64_t)g.ldc, 32, cluster > 1 ? (uint32_t)(bn / cluster) : 64u, cluster <= 1);
 }
 

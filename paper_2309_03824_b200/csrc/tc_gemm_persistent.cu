@@ -119,8 +119,8 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only this block's own shared and tensor memory: it may overlap the tail of the
     // previous kernel in the stream; global memory is first touched below this line
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();       // (in this order: see GemmArgs::a_early)
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer

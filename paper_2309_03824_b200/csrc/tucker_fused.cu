@@ -112,8 +112,8 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only this block's own shared and tensor memory: under programmatic dependent launch it
     // overlaps the tail of the previous kernel in the stream; global memory is first touched below this line
-    griddep_launch_dependents();
     griddep_wait();
+    griddep_launch_dependents();       // (in this order: see GemmArgs::a_early)
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer: phases A, B, C through one ring

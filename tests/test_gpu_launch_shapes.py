@@ -224,3 +224,44 @@ def test_slices_that_fill_no_whole_boxes(blocks, shape):
 def test_slices_of_a_pair_that_fill_no_whole_boxes(pairs, rank):
     b.lrd_chain_pair_tuning(2, pairs, 0, 0)                             # 48, 80, 48 and 48 columns for each block
     check_linear(wl.random_factor_case(300, 328, 520, rank, "bf16", 980 + rank), b.LRD_FREEZE_NONE)
+
+
+@pytest.mark.parametrize("freeze", [b.LRD_FREEZE_V, b.LRD_FREEZE_U, b.LRD_FREEZE_NONE])
+@pytest.mark.parametrize("shape", [(4096, 768, 768, 192), (128, 768, 768, 192), (1021, 1024, 1024, 512), (300, 520, 520, 250), (2000, 264, 264, 64)])
+@pytest.mark.parametrize("path", [b.LRD_PATH_AUTO, b.LRD_PATH_UNFUSED])
+def test_gradients_that_start_beside_their_data_pass(shape, freeze, path):
+    """Weight gradients load what their own call's data pass does not write before that pass has ended: their operands are made
+    right before the call, by another kernel or by another layer's backward pass, and overwritten right behind it."""
+    M, K, N, r = shape
+    b.lrd_set_path(path)
+    case = wl.random_factor_case(M, K, N, r, "bf16", 990 + M)
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16)
+    X, V, U, dY0 = (dev(case[k], "bf16") for k in ("X", "V", "U", "dY"))
+    Z0 = (X.float() @ V.float()).to(torch.bfloat16)
+    ws = workspace(b.lrd_linear_workspace_bytes(desc, freeze, 1))
+
+    def chain_of_calls(wait):
+        dY, Z, Xc = torch.empty_like(dY0), torch.empty_like(Z0), torch.empty_like(X)
+        dX = torch.empty_like(X)
+        out = []
+        for i in range(6):
+            if i % 2 == 0:
+                torch.mul(dY0, 1.0 + i, out=dY)
+            else:
+                dY.copy_(dX)                                            # (K = N)
+            torch.mul(Z0, 1.0 + i, out=Z)
+            torch.mul(X, 1.0 - i, out=Xc)
+            g = [torch.empty(s, dtype=torch.bfloat16, device="cuda") for s in ((N, r), (K, r), (N,))]
+            for _ in range(2):                                          # the second call's data pass behind the first one's gradients
+                b.lrd_linear_bwd(desc, dY, Xc, V, U, Z, dX, g[0], g[1], g[2], freeze, ws)
+                if wait:
+                    torch.cuda.synchronize()
+            for t in (dY, Z, Xc):
+                t.zero_()
+            out += g + [dX.clone()]
+        torch.cuda.synchronize()
+        return out
+
+    for a, c in zip(chain_of_calls(False), chain_of_calls(True)):
+        assert torch.equal(a, c)
+    assert b.lrd_check_device_status() == b.LRD_OK
