@@ -22,8 +22,8 @@
 // so that two blocks share an SM and one's set-up, first loads and epilogue run beside the other's MMAs.
 // Warp roles as in the matrix-product kernel: TMA producer, MMA issuer (both issue under elect.sync from a converged
 // warp), 8 epilogue warps: what a block does after its MMAs is latency of tensor-memory loads and stores, and more warps have
-// more of both in flight (four: a stride-2 step, 64 x 28 x 28, 256 -> 256 at rank 96, 65.6 us; eight, with whole sectors per
-// store: 61.3).
+// more of both in flight.  A stride-2 step, 64 x 28 x 28, 256 -> 256 at rank 96: 65.6 us with four warps, 61.3 with eight and whole
+// sectors per store; beside each other, sectors / whole lines out of shared memory 62.0 / 60.2 (replayed 56.6 / 54.7).
 #include <algorithm>
 
 #include "common.cuh"
@@ -76,31 +76,13 @@ struct ConvParams {
     const __nv_bfloat16* bias2;   // [n2] or nullptr
 };
 
-// 32 fp32 accumulators of one row -> bf16 at dst (columns col0 .. col0 + 31 of n, n a multiple of 8); sectors: whole 32-byte
-// sectors per store (n a multiple of 16, dst aligned to 32 bytes)
-__device__ __forceinline__ void store_row32(__nv_bfloat16* dst, int col0, int n, const uint32_t (&v)[32], bool sectors) {
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-        uint32_t w[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) w[e] = pack_bf16(__uint_as_float(v[16 * g + 2 * e]), __uint_as_float(v[16 * g + 2 * e + 1]));
-        __nv_bfloat16* d = dst + col0 + g * 16;
-        if (sectors && col0 + g * 16 + 16 <= n) {
-            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                         ::"l"(d), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-            continue;
-        }
-        if (col0 + g * 16 + 8 <= n) *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
-        if (col0 + g * 16 + 16 <= n) *reinterpret_cast<uint4*>(d + 8) = make_uint4(w[4], w[5], w[6], w[7]);
-    }
-}
-
 // grid: (tiles of all classes, column tiles of bn); fused: one column tile
 template <bool DGRAD, bool FUSE>
 __global__ void __launch_bounds__(kThreads, 2)
 conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], acc_bar, q_full, t_ready, out_full;
+    __shared__ __align__(16) float bias_s[FUSE ? 256 : 1];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -230,42 +212,40 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
         }
     } else {
         const int q = warp % 4, hw = (warp - 2) / 4;             // two warps share a quarter of the rows: alternate 32-column pieces
-        const int row = q * 32 + lane;
-        const bool row_ok = m0 + row < cl.pixels;
-        int64_t pix = m0 + row;                                  // this row's pixel of the output image(s)
-        if (p.step > 1 && row_ok) {
-            const int m = m0 + row, w = m % cl.Wc, h = (m / cl.Wc) % cl.Hc, im = m / (cl.Wc * cl.Hc);
-            pix = ((int64_t)im * p.H + cl.ph + h * p.step) * p.W + cl.pw + w * p.step;
+        const int m = m0 + q * 32 + lane;
+        int pix = m < cl.pixels ? m : -1;                        // this lane's pixel of the output image(s); -1: none
+        if (p.step > 1 && pix >= 0) {
+            const int w = m % cl.Wc, h = (m / cl.Wc) % cl.Hc, im = m / (cl.Wc * cl.Hc);
+            pix = (im * p.H + cl.ph + h * p.step) * p.W + cl.pw + w * p.step;
         }
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+        if (FUSE)
+            for (int n = threadIdx.x - 64; n < 256; n += 256) bias_s[n] = p.bias2 && n < p.n2 ? __bfloat162float(p.bias2[n]) : 0.f;
         const bool ready = mbar_wait_uniform(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
+        // Blocks of 64 columns per warp, through shared memory: the T tile of the second product (rows past the tile hold garbage that
+        // only reaches output rows nobody stores), or a slab of the warp in the dead ring; out of it to memory in whole lines.
+        const uint32_t slab = smem_base + (uint32_t)(warp - 2) * 4096u;
         if (ready) {
-            __nv_bfloat16* dst_row = p.out + pix * p.n_total;
-            const bool sectors = p.n_total % 16 == 0 && ((uintptr_t)p.out & 31u) == 0;
 #pragma unroll 1
-            for (int c = 32 * hw; c < p.bn && n0 + c < p.n_total; c += 64) {
-                uint32_t v[32];
+            for (int c = 64 * hw; c < p.bn && n0 + c < p.n_total; c += 128) {
+                uint32_t v[64];
                 if (iters > 0) {
-                    tmem_ld_32x32(lane_addr + c, v);
+                    tmem_ld_32x32(lane_addr + c, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                    tmem_ld_32x32(lane_addr + c + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
                     tmem_ld_wait();
                 } else {                                         // a class that meets no tap (k = 1, stride 2)
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] = 0u;
+                    for (int e = 0; e < 64; ++e) v[e] = 0u;
                 }
-                if (FUSE) {                                      // bf16 tile T for the second product (rows past the tile hold
-#pragma unroll                                                   // garbage that only reaches output rows nobody stores)
-                    for (int g = 0; g < 4; ++g) {
-                        const uint32_t col = (uint32_t)(c + g * 8);
-                        st_shared_v4(t_base + (col / 64u) * kTile + (uint32_t)row * 128u + ((((col % 64u) / 8u) ^ ((uint32_t)row & 7u)) << 4),
-                                     pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1])),
-                                     pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3])),
-                                     pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5])),
-                                     pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7])));
-                    }
-                    if (!p.out) continue;
+                if (FUSE) {
+                    put_row64(t_base + (uint32_t)(c / 64) * kTile + (uint32_t)q * 4096u, v);
+                } else {
+                    put_row64(slab, v);
+                    __syncwarp();
+                    store_rows64(slab, p.out, pix, n0 + c, p.n_total);
+                    __syncwarp();
                 }
-                if (row_ok) store_row32(dst_row, n0 + c, p.n_total, v, sectors);
             }
         }
         if (FUSE) {
@@ -273,37 +253,27 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&t_ready));
+            if (ready && p.out)                              // the core's result, where it is wanted, while the second product runs
+#pragma unroll 1
+                for (int c = 64 * hw; c < p.n_total; c += 128) store_rows64(t_base + (uint32_t)(c / 64) * kTile + (uint32_t)q * 4096u, p.out, pix, c, p.n_total);
             const bool done = ready && mbar_wait_uniform(smem_u32(&out_full), 0, ab);
             tc_fence_after();
+            named_bar_sync(2, 256);                          // (the bias is in shared memory, and every warp is done with T)
             if (done) {
-                __nv_bfloat16* dst_row = p.out2 + pix * p.n2;
-                const bool sectors = p.n2 % 16 == 0 && ((uintptr_t)p.out2 & 31u) == 0;
-                const bool bias_vec = p.bias2 && (((uintptr_t)p.bias2 & 15u) == 0);
 #pragma unroll 1
-                for (int col0 = 32 * hw; col0 < p.n2; col0 += 64) {
-                    uint4 bv[4] = {};
-                    const bool bvec = bias_vec && col0 + 32 <= p.n2;
-                    if (bvec) {
-                        const uint4* bp = reinterpret_cast<const uint4*>(p.bias2 + col0);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) bv[e] = __ldg(bp + e);
-                    }
-                    uint32_t v[32];
-                    tmem_ld_32x32(lane_addr + col0, v);
+                for (int col0 = 64 * hw; col0 < p.n2; col0 += 128) {
+                    uint32_t v[64];
+                    tmem_ld_32x32(lane_addr + col0, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                    if (col0 + 32 < p.n2) tmem_ld_32x32(lane_addr + col0 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
                     tmem_ld_wait();
-                    if (!row_ok) continue;
-                    if (bvec) {
-                        const uint32_t* bw = reinterpret_cast<const uint32_t*>(bv);
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            v[2 * e] = __float_as_uint(__uint_as_float(v[2 * e]) + __uint_as_float(bw[e] << 16));
-                            v[2 * e + 1] = __float_as_uint(__uint_as_float(v[2 * e + 1]) + __uint_as_float(bw[e] & 0xFFFF0000u));
-                        }
-                    } else if (p.bias2) {
-                        for (int e = 0; e < 32; ++e)
-                            if (col0 + e < p.n2) v[e] = __float_as_uint(__uint_as_float(v[e]) + __bfloat162float(p.bias2[col0 + e]));
+                    if (p.bias2) {
+                        bias_add(&v[0], &bias_s[col0]);
+                        bias_add(&v[32], &bias_s[col0 + 32]);
                     }
-                    store_row32(dst_row, col0, p.n2, v, sectors);
+                    put_row64(slab, v);
+                    __syncwarp();
+                    store_rows64(slab, p.out2, pix, col0, p.n2);
+                    __syncwarp();
                 }
             }
         }

@@ -353,6 +353,34 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// One warp's 32 rows x 64 columns of bf16 out of shared memory (rows of 128 bytes, 16-byte groups swizzled by the row) to rows of
+// `dst` (ld = cols of them, a multiple of 8): lane r's `row` is where row r goes, -1: nowhere.  Eight lanes share a row, so that an
+// instruction writes four whole lines; stored straight from the registers, a lane a row, it touches 32.
+__device__ __forceinline__ void store_rows64(uint32_t src, __nv_bfloat16* dst, int row, int col0, int cols) {
+    const int lane = threadIdx.x & 31, col = col0 + 8 * (lane & 7);
+    uint4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t r = 4u * i + ((uint32_t)lane >> 3);
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w) : "r"(src + r * 128u + ((((uint32_t)lane & 7u) ^ (r & 7u)) << 4)));
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int to = __shfl_sync(0xffffffffu, row, 4 * i + (lane >> 3));
+        if (to >= 0 && col < cols) *reinterpret_cast<uint4*>(dst + (int64_t)to * cols + col) = v[i];
+    }
+}
+// 64 accumulators of this lane's row -> bf16, into the warp's rows of such a buffer
+__device__ __forceinline__ void put_row64(uint32_t dst, const uint32_t (&v)[64]) {
+    const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+    for (uint32_t g = 0; g < 8; ++g)
+        st_shared_v4(dst + lane * 128u + ((g ^ (lane & 7u)) << 4), pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1])),
+                     pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3])), pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5])),
+                     pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7])));
+}
+
 // two bf16 sums, each fp32 and rounded once
 __device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
     return pack_bf16(__uint_as_float(a << 16) + __uint_as_float(b << 16), __uint_as_float(a & 0xFFFF0000u) + __uint_as_float(b & 0xFFFF0000u));

@@ -19,7 +19,9 @@
 // activations Z1 / Z2 of the forward pass, dZ2 / dZ1 of the backward pass).
 // Warp 0: TMA producer (one ring for all three phases).  Warp 1: tensor memory + MMA issue.  Warps 2-9: the three
 // epilogues, two warps per quarter of the rows (one: 64 x 14 x 14, 256 -> 256 at rank 96, forward and backward with the core
-// frozen 38.5 us; two, with whole sectors per store: 36.5).  Every wait is bounded; a wait that runs out raises the device timeout flag and the block tears down.
+// frozen 38.5 us; two, with whole sectors per store: 36.5; with whole lines out of
+// shared memory, the bias fetched ahead and the saved T2 stored behind the arrival 36.1 -> 35.3, beside each other).  Every wait is
+// bounded; a wait that runs out raises the device timeout flag and the block tears down.
 #include "common.cuh"
 #include "conv.cuh"
 #include "ptx.cuh"
@@ -69,6 +71,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
                     const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmP3, const FusedParams p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kSlots], empty_bar[kSlots], acc_bar[3], ready_bar[2];
+    __shared__ __align__(16) uint16_t bias_s[256];           // (bf16)
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -236,34 +239,31 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         __syncwarp();
     } else {
         // ------------------------------------------------------------------ the three epilogues
-        const int q = warp % 4, hw = (warp - 2) / 4;         // two warps share a quarter of the rows: alternate 32-column pieces
+        // Blocks of 64 columns of its 32 rows at a time per warp.  What goes to global memory goes behind the arrival that lets the next
+        // product start, out of shared memory in whole lines (store_rows64).
+        const int q = warp % 4, hw = (warp - 2) / 4;         // two warps share a quarter of the rows: alternate 64-column blocks
         const int row = q * 32 + lane;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+        for (int n = threadIdx.x - 64; n < 256; n += 256) bias_s[n] = p.bias3 && n < p.n3 ? __bfloat16_as_ushort(p.bias3[n]) : (uint16_t)0;
         // T1: row = pixel of the haloed tile
         bool ok = mbar_wait_uniform(smem_u32(&acc_bar[0]), 0, ab);
         tc_fence_after();
+        const int hr = row / p.W, w1 = row % p.W, hi = h0 - 1 + hr;
+        const uint32_t slot_addr = z1_base + (uint32_t)(hr * p.PW + w1 + 1) * 16u;
         if (ok) {
-            const int hr = row / p.W, w = row % p.W;
-            const bool in_tile = row < HR;
-            const int hi = h0 - 1 + hr;
-            const bool keep = p.save1 && in_tile && hr >= 1 && hr <= p.bh && hi < p.H;
-            const uint32_t slot_addr = z1_base + (uint32_t)(hr * p.PW + w + 1) * 16u;
-            __nv_bfloat16* dst_row = p.save1 + ((int64_t)(img * p.H + hi) * p.W + w) * p.nA;
 #pragma unroll 1
-            for (int c0 = 32 * hw; c0 < p.nA; c0 += 64) {
-                uint32_t v[32];
-                tmem_ld_32x32(lane_addr + c0, v);
+            for (int c0 = 64 * hw; c0 < p.nA; c0 += 128) {
+                uint32_t v[64];
+                tmem_ld_32x32(lane_addr + c0, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                if (c0 + 32 < p.nA) tmem_ld_32x32(lane_addr + c0 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
                 tmem_ld_wait();
-                if (!in_tile) continue;
+                if (row >= HR) continue;
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
+                for (int g = 0; g < 8; ++g) {
                     if (c0 + g * 8 >= p.nA) break;
-                    const uint32_t w0 = pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1]));
-                    const uint32_t w1 = pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3]));
-                    const uint32_t w2 = pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5]));
-                    const uint32_t w3 = pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7]));
-                    st_shared_v4(slot_addr + (uint32_t)(c0 / 8 + g) * slab_bytes, w0, w1, w2, w3);
-                    if (keep) *reinterpret_cast<uint4*>(dst_row + c0 + g * 8) = make_uint4(w0, w1, w2, w3);
+                    st_shared_v4(slot_addr + (uint32_t)(c0 / 8 + g) * slab_bytes, pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1])),
+                                 pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3])), pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5])),
+                                 pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7])));
                 }
             }
         }
@@ -271,83 +271,63 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ready_bar[0]));
+        if (ok && p.save1) {
+            const bool keep = row < HR && hr >= 1 && hr <= p.bh && hi < p.H;
+            __nv_bfloat16* dst_row = p.save1 + ((int64_t)(img * p.H + hi) * p.W + w1) * p.nA;
+#pragma unroll 1
+            for (int c0 = 64 * hw; c0 < p.nA && keep; c0 += 128)
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    if (c0 + g * 8 >= p.nA) break;
+                    uint4 x;
+                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "r"(slot_addr + (uint32_t)(c0 / 8 + g) * slab_bytes));
+                    *reinterpret_cast<uint4*>(dst_row + c0 + g * 8) = x;
+                }
+        }
         // T2: row = pixel slot of the output rows, W + 2 wide
         const int ho = row / p.PW, wo = row % p.PW;
-        const bool row_ok = ho < p.bh && wo < p.W && h0 + ho < p.H;
-        const int64_t pix = (int64_t)(img * p.H + h0 + ho) * p.W + wo;
+        const int pix = ho < p.bh && wo < p.W && h0 + ho < p.H ? ho * p.W + wo : -1;       // within the tile
+        const int64_t pix0 = (int64_t)(img * p.H + h0) * p.W;
         if (ok) ok = mbar_wait_uniform(smem_u32(&acc_bar[1]), 0, ab);
         tc_fence_after();
         if (ok) {
-            __nv_bfloat16* dst_row = p.save2 + pix * p.nB;
-            const bool keep = p.save2 && row_ok;
 #pragma unroll 1
-            for (int c0 = 32 * hw; c0 < p.nB; c0 += 64) {
-                uint32_t v[32];
-                tmem_ld_32x32(lane_addr + kAcc2Col + c0, v);
+            for (int c0 = 64 * hw; c0 < p.nB; c0 += 128) {   // (columns past nB hold leftovers that no MMA reads)
+                uint32_t v[64];
+                tmem_ld_32x32(lane_addr + kAcc2Col + c0, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                tmem_ld_32x32(lane_addr + kAcc2Col + c0 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
                 tmem_ld_wait();
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    if (c0 + g * 8 >= p.nB) break;
-                    const uint32_t col = (uint32_t)(c0 + g * 8);
-                    const uint32_t w0 = pack_bf16(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1]));
-                    const uint32_t w1 = pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3]));
-                    const uint32_t w2 = pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5]));
-                    const uint32_t w3 = pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7]));
-                    st_shared_v4(z2_base + (col / 64u) * kTile + (uint32_t)row * 128u + ((((col % 64u) / 8u) ^ ((uint32_t)row & 7u)) << 4),
-                                 w0, w1, w2, w3);
-                    if (keep) *reinterpret_cast<uint4*>(dst_row + col) = make_uint4(w0, w1, w2, w3);
-                }
+                put_row64(z2_base + (uint32_t)(c0 / 64) * kTile + (uint32_t)q * 4096u, v);
             }
         }
         fence_proxy_async_smem();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ready_bar[1]));
-        // Out
+        if (ok && p.save2)
+#pragma unroll 1
+            for (int c0 = 64 * hw; c0 < p.nB; c0 += 128) store_rows64(z2_base + (uint32_t)(c0 / 64) * kTile + (uint32_t)q * 4096u, p.save2 + pix0 * p.nB, pix, c0, p.nB);
+        // Out, through a slab of this warp in the ring, which is dead by then
         if (ok) ok = mbar_wait_uniform(smem_u32(&acc_bar[2]), 0, ab);
         tc_fence_after();
+        named_bar_sync(2, 256);                              // (the bias is in shared memory)
         if (ok) {
-            __nv_bfloat16* dst_row = p.out3 + pix * p.n3;
-            const bool sectors = p.n3 % 16 == 0 && ((uintptr_t)p.out3 & 31u) == 0;
-            const bool bias_vec = p.bias3 && (((uintptr_t)p.bias3 & 15u) == 0);
+            const uint32_t slab = ring_base + (uint32_t)(warp - 2) * 4096u;
 #pragma unroll 1
-            for (int c0 = 32 * hw; c0 < p.n3; c0 += 64) {
-                uint4 bv[4] = {};
-                const bool bvec = bias_vec && c0 + 32 <= p.n3;
-                if (bvec) {
-                    const uint4* bp = reinterpret_cast<const uint4*>(p.bias3 + c0);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) bv[e] = __ldg(bp + e);
-                }
-                uint32_t v[32];
-                tmem_ld_32x32(lane_addr + kAcc3Col + c0, v);
+            for (int c0 = 64 * hw; c0 < p.n3; c0 += 128) {
+                uint32_t v[64];
+                tmem_ld_32x32(lane_addr + kAcc3Col + c0, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                if (c0 + 32 < p.n3) tmem_ld_32x32(lane_addr + kAcc3Col + c0 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
                 tmem_ld_wait();
-                if (!row_ok) continue;
-                if (bvec) {
-                    const uint32_t* bw = reinterpret_cast<const uint32_t*>(bv);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        v[2 * e] = __float_as_uint(__uint_as_float(v[2 * e]) + __uint_as_float(bw[e] << 16));
-                        v[2 * e + 1] = __float_as_uint(__uint_as_float(v[2 * e + 1]) + __uint_as_float(bw[e] & 0xFFFF0000u));
-                    }
-                } else if (p.bias3) {
-                    for (int e = 0; e < 32; ++e)
-                        if (c0 + e < p.n3) v[e] = __float_as_uint(__uint_as_float(v[e]) + __bfloat162float(p.bias3[c0 + e]));
+                if (p.bias3) {
+                    bias_add(&v[0], &bias_s[c0]);
+                    bias_add(&v[32], &bias_s[c0 + 32]);
                 }
-#pragma unroll
-                for (int g = 0; g < 2; ++g) {
-                    uint32_t o[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) o[e] = pack_bf16(__uint_as_float(v[16 * g + 2 * e]), __uint_as_float(v[16 * g + 2 * e + 1]));
-                    __nv_bfloat16* d = dst_row + c0 + g * 16;
-                    if (sectors && c0 + g * 16 + 16 <= p.n3) {       // one whole 32-byte sector per store
-                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                                     ::"l"(d), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
-                        continue;
-                    }
-                    if (c0 + g * 16 + 8 <= p.n3) *reinterpret_cast<uint4*>(d) = make_uint4(o[0], o[1], o[2], o[3]);
-                    if (c0 + g * 16 + 16 <= p.n3) *reinterpret_cast<uint4*>(d + 8) = make_uint4(o[4], o[5], o[6], o[7]);
-                }
+                put_row64(slab, v);
+                __syncwarp();
+                store_rows64(slab, p.out3 + pix0 * p.n3, pix, c0, p.n3);
+                __syncwarp();
             }
         }
     }
