@@ -51,12 +51,17 @@ struct ChainParams {
     int t_steps_lg;           // log2 of the MMA k-steps (16 columns) per atom
     const __nv_bfloat16* bias;
     int has_tsave;
+    __nv_bfloat16* t_rows;    // T in rows that TMA cannot address, or nullptr
+    int64_t ld_rows;
+    int t_cols, M;
     unsigned int* timeout_flag;
     // Phase 2 of block c walks over the 64-column k-blocks of T in the order kb_order[c] (4 bits per position); k-block
     // kb needs the slices kb_lo .. kb_hi (4 bits per k-block each).
     uint32_t kb_order[kMaxCluster], kb_lo, kb_hi;
 };
 
+// ROWS: T goes to rows that TMA cannot address (a variant of its own: every other launch would fetch that code too)
+template <bool ROWS>
 __global__ void __launch_bounds__(kThreads, 1)
 chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ CUtensorMap tmP,
              const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmOut,
@@ -333,6 +338,10 @@ chain_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ C
             }
             __syncwarp();
         }
+        if (ROWS && ok) {                                // (behind the copies to the peers, which the first chunk waits for)
+            const int first = 16 * (warp - 2), rows = min(16, p.M - m0 - first);
+            store_slice_rows(t_base, p.taw, c * p.RS, p.RS, first, rows, p.t_rows + (int64_t)(m0 + first) * p.ld_rows, p.ld_rows, p.t_cols);
+        }
         // Epilogue: each warp on its own.  32 columns of its 32 rows at a time go through a [32 rows x 64 B] slab of the warp
         // (64-byte swizzle) and leave by one TMA store each; a piece is a chain of latencies (tensor memory, conversion, fence,
         // the store's read of the slab), so eight warps share the chunk, and a chunk's bias is fetched while the chunk before it
@@ -437,8 +446,11 @@ int pick_bn2(int64_t N2, int C) {
 }
 
 bool set_attributes() {
-    return cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) == cudaSuccess &&
-           cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    for (const void* f : {(const void*)chain_kernel<false>, (const void*)chain_kernel<true>})
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess ||
+            cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            return false;
+    return true;
 }
 
 // Clusters of C blocks that can be resident at once (a cluster needs C free SMs inside one GPC).
@@ -459,7 +471,7 @@ int max_active_clusters(int C) {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (!set_attributes() || cudaOccupancyMaxActiveClusters(&n, chain_kernel, &cfg) != cudaSuccess || n < 1) {
+        if (!set_attributes() || cudaOccupancyMaxActiveClusters(&n, chain_kernel<false>, &cfg) != cudaSuccess || n < 1) {
             cudaGetLastError();
             n = C > 8 ? 0 : (kNumSms - 20) / C;         // no answer (no device yet): a cautious guess
         }
@@ -580,7 +592,8 @@ lrd_status_t chain_launch(const ChainArgs& a, cudaStream_t stream) {
     p.taw = pl.taw;
     p.t_steps_lg = p.taw == 64 ? 2 : (p.taw == 32 ? 1 : 0);
     p.bias = (const __nv_bfloat16*)a.bias;
-    p.has_tsave = a.T_save ? 1 : 0;
+    p.has_tsave = a.T_save && !a.T_rows ? 1 : 0;
+    p.t_rows = (__nv_bfloat16*)a.T_rows; p.ld_rows = a.ld_rows; p.t_cols = a.t_cols; p.M = (int)a.M;
     // A block sends its slice of T to the peers c + 1, c + 2, ... in turn, so slice j reaches block c as the
     // ((c - j) mod C)-th arrival (0 = its own); phase 2 takes the k-blocks in the order in which the last slice
     // they touch arrives.  The order depends on the launch shape only, so results stay reproducible.
@@ -624,7 +637,7 @@ lrd_status_t chain_launch(const ChainArgs& a, cudaStream_t stream) {
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, chain_kernel, tIn, tP, tQ, tOut, tT, p) != cudaSuccess) return LRD_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, a.T_rows ? chain_kernel<true> : chain_kernel<false>, tIn, tP, tQ, tOut, tT, p) != cudaSuccess) return LRD_ERR_CUDA;
     count_launch();
     return LRD_OK;
 }

@@ -28,6 +28,8 @@ struct ChainArgs {
     const void* bias;                  // [N2] or nullptr
     void* Out; int64_t ld_out;         // [M x N2]
     void* T_save; int64_t ldt;         // [M x r] or nullptr
+    void* T_rows = nullptr;            // the first t_cols columns of T in rows of any stride and alignment, instead of T_save
+    int64_t ld_rows = 0; int t_cols = 0;
     lrd_dtype_t dtype;
     int sm_share = 0;                  // SMs this launch can count on when it runs beside others (0: all of them)
 };

@@ -63,12 +63,17 @@ struct PairParams {
     int t_steps_lg;           // log2 of the MMA k-steps (16 columns) per atom
     const __nv_bfloat16* bias[kChainMaxLayers];
     int has_tsave[kChainMaxLayers];
+    __nv_bfloat16* t_rows;    // T of a single layer in rows that TMA cannot address, or nullptr
+    int64_t ld_rows;
+    int t_cols;
     unsigned int* timeout_flag;
     // Phase 2 of pair p walks over the 64-column k-blocks of T in the order kb_order[p] (4 bits per position)
     // and needs the slices in kb_slices[p] (a 4-bit mask per position) for the k-block at that position.
     uint32_t kb_order[kMaxS], kb_slices[kMaxS];
 };
 
+// ROWS: as in the single-block kernel
+template <bool ROWS>
 __global__ void __launch_bounds__(kThreads, 1)
 chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -363,6 +368,10 @@ chain_pair_kernel(const __grid_constant__ PairGroup grp, const PairParams p) {
             }
             __syncwarp();
         }
+        if (ROWS && ok) {
+            const int first = 16 * (warp - 2), rows = min(16, p.M - m0 - first);
+            store_slice_rows(t_base, p.taw, pr * p.RS, p.RS, first, rows, p.t_rows + (int64_t)(m0 + first) * p.ld_rows, p.ld_rows, p.t_cols);
+        }
         // Epilogue: as in the single-block kernel, eight warps, the bias of a chunk fetched while the one before it is stored.
         const uint32_t slab0 = staging_base + (uint32_t)(warp - 2) * kSlabBytes;
         const uint32_t row_off = (uint32_t)lane * 64u;
@@ -457,6 +466,12 @@ int pick_bn2(int64_t N2, int S) {
     return best;
 }
 
+bool set_attributes() {
+    for (const void* f : {(const void*)chain_pair_kernel<false>, (const void*)chain_pair_kernel<true>})
+        if (!cuda_ok(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit), "cudaFuncSetAttribute(pair chain)")) return false;
+    return true;
+}
+
 // Clusters of n blocks that can be resident at once (a cluster needs n free SMs inside one GPC).
 int max_active_clusters(int n) {
     static int cache_on[kMaxDevices][2 * kMaxS + 1] = {};
@@ -475,8 +490,8 @@ int max_active_clusters(int n) {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (cudaFuncSetAttribute(chain_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&cnt, chain_pair_kernel, &cfg) != cudaSuccess || cnt < 1) {
+        if (!set_attributes() ||
+            cudaOccupancyMaxActiveClusters(&cnt, chain_pair_kernel<false>, &cfg) != cudaSuccess || cnt < 1) {
             cudaGetLastError();
             cnt = (kNumSms - 20) / n;                   // no answer (no device yet): a cautious guess
         }
@@ -602,8 +617,9 @@ lrd_status_t chain_pair_launch(const ChainArgs* layers, int n, cudaStream_t stre
             L.t = L.out;
         if (!ok) { cuda_ok(cudaErrorUnknown, "tensor map encode (pair chain)"); return LRD_ERR_CUDA; }
         p.bias[i] = (const __nv_bfloat16*)c.bias;
-        p.has_tsave[i] = c.T_save ? 1 : 0;
+        p.has_tsave[i] = c.T_save && !c.T_rows ? 1 : 0;
     }
+    p.t_rows = n == 1 ? (__nv_bfloat16*)a.T_rows : nullptr; p.ld_rows = a.ld_rows; p.t_cols = a.t_cols;
     p.S = pl.S; p.RS = pl.RS; p.swb = pl.swb; p.BN2 = pl.BN2;
     p.n_chunks = (int)((a.N2 + pl.BN2 - 1) / pl.BN2);
     p.kb1 = (int)((a.K1 + 63) / 64);
@@ -643,8 +659,7 @@ lrd_status_t chain_pair_launch(const ChainArgs* layers, int n, cudaStream_t stre
     static bool configured_on[kMaxDevices] = {};
     bool& configured = configured_on[device_slot()];
     if (!configured) {
-        if (!cuda_ok(cudaFuncSetAttribute(chain_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit), "cudaFuncSetAttribute(pair chain)"))
-            return LRD_ERR_CUDA;
+        if (!set_attributes()) return LRD_ERR_CUDA;
         configured = true;
     }
     cudaLaunchConfig_t cfg = {};
@@ -661,7 +676,7 @@ lrd_status_t chain_pair_launch(const ChainArgs* layers, int n, cudaStream_t stre
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (!cuda_ok(cudaLaunchKernelEx(&cfg, chain_pair_kernel, grp, p), "cudaLaunchKernelEx(pair chain)")) return LRD_ERR_CUDA;
+    if (!cuda_ok(cudaLaunchKernelEx(&cfg, p.t_rows ? chain_pair_kernel<true> : chain_pair_kernel<false>, grp, p), "cudaLaunchKernelEx(pair chain)")) return LRD_ERR_CUDA;
     count_launch();
     return LRD_OK;
 }

@@ -48,6 +48,7 @@ struct GemmArgs {
     // some 1.5 us behind the last block's exit and another for the first loads: 768 -> 768 at r = 192, a pass over 128 tokens
     // 18.5 -> 17.7 us, over 4096 25.5 -> 25.3; six layers of 768 (4096 tokens) 171.2 -> 168.3.
     bool a_early = false, b_early = false;
+    bool any_rows = false;     // weight gradients: C of any stride and alignment (single-SM kernels)
     bool in_turn = false;      // weight gradients: started only when the launch before has ended (blocks that wait on an SM for
                                // that end keep it from work in other streams)
 };
@@ -84,7 +85,8 @@ struct Copy2d {
     int cols_src, cols_dst;
 };
 constexpr int kMaxCopies = 6;
-// All of them in one launch.  Sources must not overlap destinations.
-lrd_status_t copy2d_bf16(const Copy2d* c, int n, cudaStream_t s);
+// All of them in one launch.  Sources must not overlap destinations.  early: nothing of them is written by, or read by, the launch
+// before this one (see GemmArgs::a_early).
+lrd_status_t copy2d_bf16(const Copy2d* c, int n, cudaStream_t s, bool early = false);
 
 }  // namespace lrd

@@ -252,9 +252,10 @@ struct CopyBatch {
     Copy2d job[kMaxCopies];
     int64_t unit0[kMaxCopies + 1];       // first (row, 128-column piece) of each job
     int n;
+    int early;                           // as GemmArgs::a_early
 };
 __global__ void __launch_bounds__(256) copy2d_bf16_kernel(const __grid_constant__ CopyBatch b) {
-    ptx::griddep_wait();
+    if (!b.early) ptx::griddep_wait();
     ptx::griddep_launch_dependents();
     const int lane = threadIdx.x % 32;
     const int64_t warps = (int64_t)gridDim.x * 8;
@@ -275,12 +276,14 @@ __global__ void __launch_bounds__(256) copy2d_bf16_kernel(const __grid_constant_
         for (int e = 0; e < 4; ++e)
             if (col0 + 32 * e < c.cols_dst) dst[col0 + 32 * e] = v[e];
     }
+    if (b.early) ptx::griddep_wait();
 }
 }  // namespace
 
-lrd_status_t copy2d_bf16(const Copy2d* c, int n, cudaStream_t s) {
+lrd_status_t copy2d_bf16(const Copy2d* c, int n, cudaStream_t s, bool early) {
     CopyBatch b;
     b.n = 0;
+    b.early = early;
     b.unit0[0] = 0;
     for (int i = 0; i < n; ++i) {
         if (c[i].rows_dst <= 0 || c[i].cols_dst <= 0) continue;
@@ -533,10 +536,14 @@ size_t lrd_dense_workspace_bytes(const lrd_linear_desc_t* desc, int is_bwd) {
     return 256 + need;
 }
 
+// A saved Z whose rows TMA cannot address: where a chain forms it, it is stored in place (`stored`), else the padded copy holds it.
+// With the gradients below: 8192 tokens, 4096 -> 4096 at rank 250, V frozen, replayed 132.9 -> 127.4 us a pass, five launches for eight.
+struct PackedZ { void* Z; int64_t ld; int cols; bool stored; };
 // One layer's forward on stream s.  sm_share: SMs the launch can count on beside concurrent launches (0: all).
 static lrd_status_t linear_fwd_on(const lrd_linear_desc_t* desc, const void* X, const void* V, const void* U,
                                   const void* bias, void* Y, void* Z_save, lrd_freeze_t freeze, void* workspace,
-                                  size_t workspace_bytes, cudaStream_t s, int sm_share, bool check_only = false) {
+                                  size_t workspace_bytes, cudaStream_t s, int sm_share, bool check_only = false,
+                                  PackedZ* packed = nullptr) {
     Linear L;
     LRD_TRY(parse_linear(desc, &L, false));
     if (freeze != LRD_FREEZE_NONE && freeze != LRD_FREEZE_U && freeze != LRD_FREEZE_V) return LRD_ERR_INVALID_ARG;
@@ -557,9 +564,10 @@ static lrd_status_t linear_fwd_on(const lrd_linear_desc_t* desc, const void* X, 
         const int r = (int)L.r, rp = (int)q.r;
         const Copy2d in[2] = {{w + o.Vp, rp, V, L.ldv, L.K, L.K, r, rp}, {w + o.Up, rp, U, L.ldu, L.N, L.N, r, rp}};
         LRD_TRY(copy2d_bf16(in, 2, s));
-        LRD_TRY(linear_fwd_on(&q, X, w + o.Vp, w + o.Up, bias, Y, Z_save ? w + o.Zp : nullptr, freeze, w, inner, s, sm_share));
+        PackedZ z{Z_save, L.ldz, r, false};
+        LRD_TRY(linear_fwd_on(&q, X, w + o.Vp, w + o.Up, bias, Y, Z_save ? w + o.Zp : nullptr, freeze, w, inner, s, sm_share, false, &z));
         const Copy2d out = {Z_save, L.ldz, w + o.Zp, rp, L.M, L.M, r, r};
-        return Z_save ? copy2d_bf16(&out, 1, s) : LRD_OK;
+        return Z_save && !z.stored ? copy2d_bf16(&out, 1, s) : LRD_OK;
     }
 
     const int path = g_path.load();
@@ -568,7 +576,9 @@ static lrd_status_t linear_fwd_on(const lrd_linear_desc_t* desc, const void* X, 
     // then the form to run: few tiles, most of the GPU is left to the others), and nowhere else
     const bool as_alone = sm_share > 0 && Z_save && alone_splits_t(c, path), whole = sm_share > 0 && Z_save && !as_alone;
     if (as_alone) c.sm_share = 0;
+    if (packed && Z_save) { c.T_rows = packed->Z; c.ld_rows = packed->ld; c.t_cols = packed->cols; }
     const lrd_status_t st = launch_chain(&c, 1, path, s, false, whole);
+    if (packed) packed->stored = st == LRD_OK;
     if (st != LRD_ERR_UNSUPPORTED) return st;
     void* Z = Z_save ? Z_save : workspace;
     const int64_t ldz = Z_save ? L.ldz : L.r;
@@ -597,6 +607,9 @@ static int linear_wgrads(const Linear& L, uint32_t plan, const void* dY, const v
     return n;
 }
 
+// The same of a backward pass's gradients.
+// (`z`: the copy of Z that only the gradients need, made beside the data pass)
+struct PackedGrads { void *dU, *dV; int64_t ldu, ldv, cols; bool stored; Copy2d z; };
 // One layer's backward on stream s.  With a side stream, the dU (+ db) product, which needs nothing the data
 // chain produces, runs there beside the chain; the caller has made `side` wait for s's earlier work and makes s
 // wait for `side` afterwards.  dV follows the chain (it reads the dZ the chain spills) and, when dU is computed too,
@@ -605,7 +618,7 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
                                   const void* U, const void* Z_save, void* dX, void* dU, void* dV, void* dbias,
                                   lrd_freeze_t freeze, void* workspace, size_t workspace_bytes, cudaStream_t s,
                                   cudaStream_t side, cudaEvent_t side_done, int sm_share, bool check_only = false,
-                                  int parts = 3, bool accumulate = false) {
+                                  int parts = 3, bool accumulate = false, PackedGrads* packed = nullptr) {
     // parts: 1 = the data half (dZ, dX), 2 = the weight-gradient half (it reads the dZ the data half left in the
     // workspace when V is unfrozen), 3 = both
     const bool do_data = (parts & 1) != 0, do_w = (parts & 2) != 0;
@@ -650,10 +663,12 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
         const int r = (int)L.r, rp = (int)q.r;
         const Copy2d in[3] = {{w + o.Vp, rp, V, L.ldv, L.K, do_data ? L.K : 0, r, rp}, {w + o.Up, rp, U, L.ldu, L.N, do_data ? L.N : 0, r, rp},
                               {w + o.Zp, rp, Z_save, L.ldz, L.M, du ? L.M : 0, r, rp}};
-        LRD_TRY(copy2d_bf16(in, 3, s));
+        LRD_TRY(copy2d_bf16(in, 2, s));
+        PackedGrads pg{dU, dV, L.ldu, L.ldv, r, false, in[2]};
         // the frozen factor's buffers were zero-filled above; the padded call gets none for them
-        LRD_TRY(linear_bwd_on(&q, dY, X, w + o.Vp, w + o.Up, w + o.Zp, dX, w + o.dUp, w + o.dVp, du ? dbias : nullptr, freeze, w, inner, s,
-                              nullptr, nullptr, sm_share, false, parts));
+        LRD_TRY(linear_bwd_on(&q, dY, X, w + o.Vp, w + o.Up, w + o.Zp, dX, du ? w + o.dUp : nullptr, dv ? w + o.dVp : nullptr, du ? dbias : nullptr,
+                              freeze, w, inner, s, nullptr, nullptr, sm_share, false, parts, false, &pg));
+        if (pg.stored) return LRD_OK;
         const Copy2d out[2] = {{dU, L.ldu, w + o.dUp, rp, L.N, du ? L.N : 0, r, r}, {dV, L.ldv, w + o.dVp, rp, L.K, dv ? L.K : 0, r, r}};
         return copy2d_bf16(out, 2, s);
     }
@@ -684,12 +699,25 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
     GemmArgs gw[2];
     const int n = linear_wgrads(L, plan, dY, X, Z_save, dZ, dU, dV, dbias, wsplit, gw);
     for (int i = 0; i < n; ++i) gw[i].add = accumulate;
-    // behind a launch of this call the gradients' operands that the data half does not write need not wait for it
-    if (!side && do_data && (dX || need_dz_in_memory))
-        for (int i = 0; i < n; ++i) {
-            gw[i].a_early = true;
-            gw[i].b_early = gw[i].B != dZ;
+    // behind a launch of this call what the data half does not write need not be waited for
+    const bool behind = !side && do_data && (dX || need_dz_in_memory);
+    if (packed) LRD_TRY(copy2d_bf16(&packed->z, 1, s, behind));
+    if (packed && !side && path == LRD_PATH_AUTO && n > 0) {
+        bool tc = true;
+        for (int i = 0; i < n; ++i) tc = tc && tc_gemm_eligible(gw[i]);
+        packed->stored = tc && tc_wgrads_any_rows(gw, n);
+        for (int i = 0; i < n && packed->stored; ++i) {
+            const bool is_dU = gw[i].C == dU;
+            gw[i].C = is_dU ? packed->dU : packed->dV;
+            gw[i].ldc = is_dU ? packed->ldu : packed->ldv;
+            gw[i].N = packed->cols;
+            gw[i].any_rows = true;
         }
+    }
+    for (int i = 0; i < n; ++i) {
+        gw[i].a_early = behind;
+        gw[i].b_early = behind && gw[i].B != dZ && !packed;
+    }
     if (side && n == 2) {
         LRD_TRY(run_gemm(gw[0], true, partials, partial_bytes, side));
         if (cudaEventRecord(side_done, side) != cudaSuccess || cudaStreamWaitEvent(s, side_done, 0) != cudaSuccess) return LRD_ERR_CUDA;

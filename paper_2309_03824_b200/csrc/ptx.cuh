@@ -353,6 +353,38 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// A warp's `n` (<= 8) rows of at most 64 bf16 columns out of shared memory -- lane l's two of row i at src(i) -- to rows of any
+// alignment, `to` = this lane's place in the first; `left`: columns from there on that exist.  All loads stand before all stores.
+template <typename Src> __device__ __forceinline__ void store_any_rows8(const Src& src, int n, __nv_bfloat16* to, int64_t ld, int left) {
+    uint32_t v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v[i]) : "r"(src(i)));
+    if (left <= 0) return;
+    if (left > 1 && (((uintptr_t)to | (uintptr_t)(2 * ld)) & 3u) == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i, to += ld)
+            if (i < n) *reinterpret_cast<uint32_t*>(to) = v[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i, to += ld) {
+            if (i >= n) continue;
+            to[0] = __ushort_as_bfloat16((unsigned short)v[i]);
+            if (left > 1) to[1] = __ushort_as_bfloat16((unsigned short)(v[i] >> 16));
+        }
+    }
+}
+// A slice of a chain's T buffer (columns [col0, col0 + n), atoms of [128 rows x taw columns], swizzled) to `rows` rows of a matrix
+// that TMA cannot address, from buffer row `row0` (a multiple of 8) on, whole groups of eight rows readable.
+__device__ __forceinline__ void store_slice_rows(uint32_t t_base, int taw, int col0, int n, int row0, int rows, __nv_bfloat16* dst, int64_t ld, int cols) {
+    const uint32_t t_sw = 2u * (uint32_t)taw;
+    for (int c = 2 * (int)(threadIdx.x & 31); c < n; c += 64) {
+        const uint32_t gc = (uint32_t)(col0 + c), in = gc & ((uint32_t)taw - 1u), at = t_base + (gc / (uint32_t)taw) * 128u * t_sw + (in & 7u) * 2u;
+        for (int r = 0; r < rows; r += 8)
+            store_any_rows8([&](int i) { const uint32_t row = (uint32_t)(row0 + r + i); return at + row * t_sw + (((in / 8u) ^ ((row * t_sw >> 7) & (t_sw / 16u - 1u))) << 4); },
+                            rows - r, dst + (int64_t)r * ld + gc, ld, cols - (int)gc);
+    }
+}
+
 // One warp's 32 rows x 64 columns of bf16 out of shared memory (rows of 128 bytes, 16-byte groups swizzled by the row) to rows of
 // `dst` (ld = cols of them, a multiple of 8): lane r's `row` is where row r goes, -1: nowhere.  Eight lanes share a row, so that an
 // instruction writes four whole lines; stored straight from the registers, a lane a row, it touches 32.

@@ -31,6 +31,7 @@ WgradForm& tc_wgrad_form();
 void tc_data_split_form(int columns, int split);
 double tc_wgrad_pair_estimate(const GemmArgs* g, int n);
 lrd_status_t tc_wgrad_pair(const GemmArgs* g, int n, cudaStream_t stream);       // (in the form of the test hook where that asks for pairs)
+bool tc_wgrads_any_rows(const GemmArgs* g, int n);             // whether these are as well stored to rows of any alignment
 lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const size_t* partial_bytes, cudaStream_t stream);
 // allow_split: a weight gradient (both operands MN-major), whose reduction may be split over blocks; else a data product (A
 // K-major, no column sums).

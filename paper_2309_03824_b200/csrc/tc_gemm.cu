@@ -95,11 +95,13 @@ __device__ __forceinline__ int conv_col(const TcParams& p, int col) {
     return blk < p.cv_nblk && c < p.cv_ci ? (blk / p.cv_nkc) * p.cv_ci + c : -1;
 }
 
-// ADD: C += the product rounded to bf16 (fp32 sum, one more rounding) instead of C = it; column sums too.  A variant of its own:
+// kAdd: C += the product rounded to bf16 (fp32 sum, one more rounding) instead of C = it; column sums too.  A variant of its own:
 // as a flag that every launch tests, its code stands between the stores of all of them, and a launch behind another kernel
 // fetches it cold.  Backward passes in a graph, flag / variant: 768 -> 768 at rank 192, 4096 tokens, V frozen 18.05 / 17.33 us;
 // 1024 -> 4096 at 512, 1021 tokens 23.7 / 22.7; 768 -> 3072 at 384, 600 tokens 18.95 / 18.10.
-template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1, bool ADD = false>
+// kRows: C's rows have any stride and alignment.
+constexpr int kStore = 0, kAdd = 1, kRows = 2;
+template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1, int OUT = kStore>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     int prod = 0;
@@ -113,7 +115,8 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         return;
     }
     static_assert(!ONES || (A_MN && B_MN && BN <= 192), "the ones block rides on an MN-major B of at most 192 columns");
-    static_assert(!ADD || !CONV, "only weight gradients add");
+    constexpr bool ADD = OUT == kAdd, ROWS = OUT == kRows;
+    static_assert(OUT == kStore || !CONV, "only weight gradients");
     static_assert(!CONV || (A_MN && B_MN && !ONES && BN <= 192), "the filter gradient: both operands MN-major, split over a cluster or not at all");
     using C = Cfg<BN, ONES>;
     constexpr int STAGES = C::STAGES, G = C::G;
@@ -384,7 +387,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                 sum8(c4, w0, a0);
                 const bool second = c4 + 8 < cs;
                 if (second) sum8(c4 + 8, w1, a1);
-                if (ADD) {
+                if (ADD || ROWS) {
                     st_shared_v4(slab + c4 * 2u, w0[0], w0[1], w0[2], w0[3]);
                     if (second) st_shared_v4(slab + c4 * 2u + 16u, w1[0], w1[1], w1[2], w1[3]);
                     continue;
@@ -400,6 +403,14 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
                     store8(c4, w0, a0);
                     if (second) store8(c4 + 8, w1, a1);
                 }
+            }
+            if (ROWS) {
+                __syncwarp();
+                const uint32_t rows0 = recv_base + self * chunk_bytes + quarter * 32u * cs * 2u;
+                for (uint32_t c = 2u * lane; c < cs; c += 64u)
+                    for (int r = 0; r < 32; r += 8)
+                        store_any_rows8([&](int i) { return rows0 + (uint32_t)(r + i) * cs * 2u + c * 2u; }, (int)(p.M - (m0 + quarter * 32 + r) < 8 ? p.M - (m0 + quarter * 32 + r) : 8),
+                                        (__nv_bfloat16*)p.C + (int64_t)(m0 + quarter * 32 + r) * p.ldc + gcol0 + c, p.ldc, (int)(p.N - gcol0 - c));
             }
             if (ADD) {
                 fence_proxy_async_smem();
@@ -492,6 +503,14 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
 #pragma unroll
                     for (int g = 0; g < 8; ++g)
                         st_shared_v4(slab + row_off + (((uint32_t)g ^ row_xor) << 4), w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+                    if (ROWS) {              // rows that TMA cannot address: a row at a time, a lane two columns
+                        __syncwarp();
+                        for (int r = 0; r < 32; r += 8)
+                            store_any_rows8([&](int i) { return slab + (uint32_t)(r + i) * 128u + ((((uint32_t)lane >> 2) ^ (uint32_t)i) << 4) + ((uint32_t)lane & 3u) * 4u; },
+                                            (int)(p.M - (m0 + quarter * 32 + r) < 8 ? p.M - (m0 + quarter * 32 + r) : 8),
+                                            (__nv_bfloat16*)p.C + (int64_t)(m0 + quarter * 32 + r) * p.ldc + col0 + 2 * lane, p.ldc, (int)(p.N - col0 - 2 * lane));
+                        continue;
+                    }
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (elect_one()) {
@@ -565,9 +584,9 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
         }
 }
 
-template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1, bool ADD = false>
+template <int BN, bool A_MN, bool B_MN, bool ONES = false, bool CONV = false, int NP = 1, int OUT = kStore>
 lrd_status_t launch(const TcLaunch<NP>& L, dim3 grid, cudaStream_t stream, bool wait_ahead = true) {
-    auto kern = tc_gemm_kernel<BN, A_MN, B_MN, ONES, CONV, NP, ADD>;
+    auto kern = tc_gemm_kernel<BN, A_MN, B_MN, ONES, CONV, NP, OUT>;
     const TcParams& p = L.p[0];
     static bool configured_on[kMaxDevices] = {};     // per instantiation; the attribute is sticky per function
     bool& configured = configured_on[device_slot()];
@@ -595,16 +614,20 @@ lrd_status_t launch(const TcLaunch<NP>& L, dim3 grid, cudaStream_t stream, bool 
     return LRD_OK;
 }
 
+int out_mode(const GemmArgs& g, bool scratch) { return scratch ? kStore : g.add ? kAdd : g.any_rows ? kRows : kStore; }
+
 template <int BN, bool ONES, int NP = 1>
-lrd_status_t launch_wgrad(bool add, const TcLaunch<NP>& L, dim3 grid, cudaStream_t s, bool wait_ahead = true) {
-    return add ? launch<BN, true, true, ONES, false, NP, true>(L, grid, s, wait_ahead) : launch<BN, true, true, ONES, false, NP>(L, grid, s, wait_ahead);
+lrd_status_t launch_wgrad(int out, const TcLaunch<NP>& L, dim3 grid, cudaStream_t s, bool wait_ahead = true) {
+    return out == kAdd    ? launch<BN, true, true, ONES, false, NP, kAdd>(L, grid, s, wait_ahead)
+           : out == kRows ? launch<BN, true, true, ONES, false, NP, kRows>(L, grid, s, wait_ahead)
+                          : launch<BN, true, true, ONES, false, NP>(L, grid, s, wait_ahead);
 }
 
 inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Tensor map of the result where it leaves by TMA, and the early operands.
 bool result_map(const GemmArgs& g, bool add, int bn, int cluster, bool partial, CUtensorMap* t, TcParams* p) {
-    p->has_c_map = !partial && (cluster <= 1 || add);
+    p->has_c_map = !partial && !g.any_rows && (cluster <= 1 || add);
     p->a_early = g.a_early; p->b_early = g.b_early;
     return !p->has_c_map || make_tmap_2d_bf16(t, g.C, (uint64_t)g.M, (uint64_t)g.N, (uint64_t)g.ldc, 32, cluster > 1 ? (uint32_t)(bn / cluster) : 64u, cluster <= 1);
 }
@@ -623,8 +646,8 @@ static_assert(Cfg<192>::G == 1 && Cfg<192, true>::G == 1 && Cfg<256>::G == 1, "s
 bool tc_gemm_eligible(const GemmArgs& g) {
     if (g.dtype != LRD_BF16 || g.M < 1 || g.N < 1 || g.K < 1) return false;
     if (g.M > (int64_t)65535 * BM || g.K > (int64_t)1 << 30 || g.N > (int64_t)1 << 30) return false;
-    if (!aligned16(g.A) || !aligned16(g.B) || !aligned16(g.C)) return false;
-    if (g.lda % 8 || g.ldb % 8 || g.ldc % 8) return false;
+    if (!aligned16(g.A) || !aligned16(g.B) || (!aligned16(g.C) && !g.any_rows)) return false;
+    if (g.lda % 8 || g.ldb % 8 || (g.ldc % 8 && !g.any_rows)) return false;
     return true;
 }
 
@@ -807,7 +830,8 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
         if (!g.a_mn_major || !g.b_mn_major) return LRD_ERR_UNSUPPORTED;
         double us;
         const WgradForm& form = tc_wgrad_form();
-        const SplitPlan sp = form.blocks ? SplitPlan{form.columns, form.split, 1} : pick_split(g.M, g.N, g.K, ones, g.max_cluster_split, &us);
+        const int64_t n = g.any_rows ? (g.N + 15) / 16 * 16 : g.N;          // (scratch was asked for at the padded rank)
+        const SplitPlan sp = form.blocks ? SplitPlan{form.columns, form.split, 1} : pick_split(g.M, n, g.K, ones, g.max_cluster_split, &us);
         // pairs where the tiles leave no room for a cluster per tile
         if (form.blocks ? form.blocks == 2 : tc_wgrad_pair_estimate(&g, 1) < 0.95 * us) return tc_wgrad_pair(&g, 1, stream);
         bn = sp.bn; cluster = sp.cluster; splits = sp.global;
@@ -848,19 +872,19 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     p.colsum_out = (ones && splits == 1) ? (__nv_bfloat16*)g.a_colsum : nullptr;
     dim3 grid((unsigned)((g.N + bn - 1) / bn), (unsigned)((g.M + BM - 1) / BM), (unsigned)zdim);
     lrd_status_t st;
-    const bool add = g.add && splits == 1;                 // (shares through scratch memory: the second kernel adds)
+    const int out = out_mode(g, splits > 1);               // (shares through scratch memory: the second kernel adds)
     if (ones) {
         switch (bn) {
-            case 192: st = launch_wgrad<192, true>(add, L, grid, stream, !g.in_turn); break;
-            case 128: st = launch_wgrad<128, true>(add, L, grid, stream, !g.in_turn); break;
-            default:  st = launch_wgrad<64, true>(add, L, grid, stream, !g.in_turn); break;
+            case 192: st = launch_wgrad<192, true>(out, L, grid, stream, !g.in_turn); break;
+            case 128: st = launch_wgrad<128, true>(out, L, grid, stream, !g.in_turn); break;
+            default:  st = launch_wgrad<64, true>(out, L, grid, stream, !g.in_turn); break;
         }
     } else if (allow_split) {
         switch (bn) {
-            case 256: st = launch_wgrad<256, false>(add, L, grid, stream, !g.in_turn); break;
-            case 192: st = launch_wgrad<192, false>(add, L, grid, stream, !g.in_turn); break;
-            case 128: st = launch_wgrad<128, false>(add, L, grid, stream, !g.in_turn); break;
-            default:  st = launch_wgrad<64, false>(add, L, grid, stream, !g.in_turn); break;
+            case 256: st = launch_wgrad<256, false>(out, L, grid, stream, !g.in_turn); break;
+            case 192: st = launch_wgrad<192, false>(out, L, grid, stream, !g.in_turn); break;
+            case 128: st = launch_wgrad<128, false>(out, L, grid, stream, !g.in_turn); break;
+            default:  st = launch_wgrad<64, false>(out, L, grid, stream, !g.in_turn); break;
         }
     } else if (bn == 128) {
         st = g.b_mn_major ? launch<128, false, true>(L, grid, stream) : launch<128, false, false>(L, grid, stream);
@@ -888,6 +912,21 @@ static double group_estimate(const GemmArgs* g, int n, int bn, int S) {
     return S > 1 && tiles > max_active_clusters(S) ? 1e300 : split_us(bn, S, tiles, deepest, kblocks);
 }
 
+// Gradients whose rows TMA cannot address run on single SMs only: worth it where pairs would not save more than the launch that
+// copies a padded result, some 3 us.
+bool tc_wgrads_any_rows(const GemmArgs* g, int n) {
+    if (tc_wgrad_form().blocks) return false;
+    double single = 0.0, pairs = 0.0;
+    for (int i = 0; i < n; ++i) {
+        double us;
+        pick_split(g[i].M, g[i].N, g[i].K, g[i].a_colsum != nullptr, g[i].max_cluster_split, &us);
+        single += us;
+        pairs += std::min(us, tc_wgrad_pair_estimate(&g[i], 1));
+    }
+    if (n > 1) pairs = std::min(pairs, tc_wgrad_pair_estimate(g, n));
+    return single <= pairs + 3.0;
+}
+
 template <int BN, bool ONES>
 static lrd_status_t launch_group(const GemmArgs* g, int n, int S, cudaStream_t stream) {
     TcLaunch<kMaxWgrads> L{};
@@ -911,7 +950,7 @@ static lrd_status_t launch_group(const GemmArgs* g, int n, int S, cudaStream_t s
         nx = std::max(nx, (unsigned)((g[i].N + BN - 1) / BN));
         ny += (unsigned)((g[i].M + BM - 1) / BM);
     }
-    return launch_wgrad<BN, ONES>(g[0].add, L, dim3(nx, ny, (unsigned)S), stream, !g[0].in_turn);
+    return launch_wgrad<BN, ONES>(out_mode(g[0], false), L, dim3(nx, ny, (unsigned)S), stream, !g[0].in_turn);
 }
 
 // The weight gradients of one backward pass.  Each alone has few output tiles and one pays for its launch, its first loads and
@@ -927,7 +966,7 @@ lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const s
     double separate = 2.0 * (n - 1);           // a launch behind another one drains and fills the SMs anew
     for (int i = 0; i < n && together; ++i) {
         together = tc_gemm_eligible(g[i]) && g[i].a_mn_major && g[i].b_mn_major && !g[i].bias && g[i].max_cluster_split == g[0].max_cluster_split &&
-                   g[i].add == g[0].add;
+                   g[i].add == g[0].add && g[i].any_rows == g[0].any_rows;
         if (!together) break;
         ones = ones || g[i].a_colsum;
         rows += (g[i].M + BM - 1) / BM;

@@ -414,7 +414,7 @@ double tc_wgrad_pair_estimate(const GemmArgs* g, int n) {
     int64_t rows = 0;
     if (n > kMaxWgrads) return 1e300;
     for (int i = 0; i < n; ++i) {
-        if (!tc_gemm_eligible(g[i]) || !g[i].a_mn_major || !g[i].b_mn_major || g[i].bias || g[i].N > (int64_t)65535 * 128) return 1e300;
+        if (g[i].any_rows || !tc_gemm_eligible(g[i]) || !g[i].a_mn_major || !g[i].b_mn_major || g[i].bias || g[i].N > (int64_t)65535 * 128) return 1e300;
         rows += (g[i].M + 255) / 256;
     }
     return rows > 65535 ? 1e300 : make_plan(g, n).us;

@@ -265,3 +265,41 @@ def test_gradients_that_start_beside_their_data_pass(shape, freeze, path):
     for a, c in zip(chain_of_calls(False), chain_of_calls(True)):
         assert torch.equal(a, c)
     assert b.lrd_check_device_status() == b.LRD_OK
+
+
+@pytest.mark.parametrize("freeze", [b.LRD_FREEZE_V, b.LRD_FREEZE_U, b.LRD_FREEZE_NONE])
+@pytest.mark.parametrize("shape", [(4096, 768, 768, 190), (4096, 768, 1024, 379), (300, 520, 264, 129), (1000, 136, 520, 121), (130, 264, 264, 33),
+                                   (1, 200, 136, 77), (5000, 1024, 1024, 250)])
+@pytest.mark.parametrize("pads", [(0, 0, 0), (3, 1, 5), (2, 4, 6)])
+def test_packed_ranks_store_their_rows_alone(shape, freeze, pads):
+    """Z and the gradients in rows of any stride: right, and nothing written between and behind them."""
+    M, K, N, r = shape
+    case = wl.random_factor_case(M, K, N, r, "bf16", 1010 + r)
+    ldz, ldu, ldv = (r + p for p in pads)
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16, ldv=ldv, ldu=ldu, ldz=ldz)
+
+    def rows(n, ld, fill, data=None):
+        flat = torch.full((n * ld + 40,), fill, dtype=torch.bfloat16, device="cuda")
+        view = flat[:n * ld].view(n, ld)
+        if data is not None:
+            view[:, :r] = data
+        return flat, view
+
+    X, dY, bias = (dev(case[k], "bf16") for k in ("X", "dY", "b"))
+    Vf, V = rows(K, ldv, 7.0, dev(case["V"], "bf16"))
+    Uf, U = rows(N, ldu, 7.0, dev(case["U"], "bf16"))
+    Zf, Z = rows(M, ldz, 7.0)
+    dUf, dU = rows(N, ldu, 7.0)
+    dVf, dV = rows(K, ldv, 7.0)
+    Y, dX, db = torch.empty_like(dY), torch.empty_like(X), torch.empty_like(bias)
+    ws = workspace(max(b.lrd_linear_workspace_bytes(desc, freeze, i) for i in (0, 1)))
+    b.lrd_linear_fwd(desc, X, Vf, Uf, bias, Y, None if freeze == b.LRD_FREEZE_U else Zf, freeze, ws)
+    b.lrd_linear_bwd(desc, dY, X, Vf, Uf, None if freeze == b.LRD_FREEZE_U else Zf, dX, dUf, dVf, db, freeze, ws)
+    assert b.lrd_check_device_status() == b.LRD_OK
+    Zr, Yr = o.linear_fwd(case["X"], case["V"], case["U"], case["b"])
+    g = o.linear_bwd(case["dY"], case["X"], case["V"], case["U"], Zr, freeze)
+    saved = freeze != b.LRD_FREEZE_U
+    for got, ref in [(Y, Yr), (dX, g["dX"]), (dU[:, :r], g["dU"]), (dV[:, :r], g["dV"])] + ([(Z[:, :r], Zr), (db, g["db"])] if saved else []):
+        assert rel_err(got, ref) <= 2e-2
+    for flat, view in ((Zf, Z), (dUf, dU), (dVf, dV)):
+        assert bool((flat[view.numel():] == 7).all()) and bool((view[:, r:] == 7).all())
