@@ -34,10 +34,12 @@ namespace {
 using namespace ptx;
 
 constexpr int kThreads = 320;
-constexpr int kSlots = 4;
+constexpr int kMaxSlots = 5;                         // as many as shared memory holds beside T1 and T2, four at least (five at rank
+                                                     // 96, and taps without rows past the rank: 64 x 14 x 14 34.2 -> 33.7 us replayed)
 constexpr uint32_t kTile = 128 * 128;                // 128 rows x 64 channels of bf16
 constexpr uint32_t kSlotBytes = 2 * kTile;           // a stage of any phase fits 32 KB
 constexpr uint32_t kZ2Bytes = 2 * kTile;             // T2: up to 128 channels
+constexpr uint32_t kSmemMost = 226 * 1024;           // dynamic; the barriers and the bias take the rest
 constexpr uint32_t kAcc2Col = 128, kAcc3Col = 256;   // tensor-memory columns of the three accumulators: 0, 128, 256
 
 struct FusedParams {
@@ -45,6 +47,7 @@ struct FusedParams {
     int c_in, nA, nB, n3;         // channels: input, after the first 1x1, after the core, output
     int g_ci;                     // row length of G per tap (r1)
     int swb;                      // swizzle span of the P1 boxes (bytes); a box is 64 rows x swb / 2 columns
+    int slots;                    // stages of the ring
     int z1_slots;                 // pixel slots of the T1 buffer (a slab is z1_slots * 16 bytes)
     __nv_bfloat16* save1;         // [B H W][nA] or nullptr
     __nv_bfloat16* save2;         // [B H W][nB] or nullptr
@@ -70,7 +73,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ CUtensorMap tmP1,
                     const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmP3, const FusedParams p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[kSlots], empty_bar[kSlots], acc_bar[3], ready_bar[2];
+    __shared__ __align__(8) uint64_t full_bar[kMaxSlots], empty_bar[kMaxSlots], acc_bar[3], ready_bar[2];
     __shared__ __align__(16) uint16_t bias_s[256];           // (bf16)
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
@@ -97,7 +100,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         prefetch_tmap(&tmP1);
         prefetch_tmap(&tmG);
         prefetch_tmap(&tmP3);
-        for (int s = 0; s < kSlots; ++s) {
+        for (int s = 0; s < p.slots; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 1);
             mbar_init(smem_u32(&empty_bar[s]), 1);
         }
@@ -142,8 +145,8 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
                         for (int cb = 0; cb < ncbB; ++cb)
                             for (int nb = 0; nb < nnb; ++nb)
                                 tma_load_2d(dst + (uint32_t)cb * kTile + (uint32_t)nb * 8192u, &tmG, fb, tap * p.g_ci + nb * 64, cb * 64);
-                    } else {           // B[n = o][k = i] = G[o][tap][i]: K-major, 128 o-rows x 64 i-columns per box
-                        mbar_expect_tx(fb, (uint32_t)ncbB * kTile);
+                    } else {           // B[n = o][k = i] = G[o][tap][i]: K-major, the nB o-rows x 64 i-columns per box
+                        mbar_expect_tx(fb, (uint32_t)(ncbB * p.nB) * 128u);
                         for (int cb = 0; cb < ncbB; ++cb) tma_load_2d(dst + (uint32_t)cb * kTile, &tmG, fb, tap * p.g_ci + cb * 64, 0);
                     }
                 } else {                                     // 64 columns of P3 (256 rows)
@@ -152,7 +155,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
                 }
             }
             __syncwarp();
-            if (++s == kSlots) { s = 0; ph ^= 1; }
+            if (++s == p.slots) { s = 0; ph ^= 1; }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
@@ -161,7 +164,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
         bool ok = true;
         uint32_t ready = mbar_test_wait(smem_u32(&full_bar[0]), 0);
         auto advance = [&] {                                 // to the next stage, with a first look at its barrier
-            if (++s == kSlots) { s = 0; ph ^= 1; }
+            if (++s == p.slots) { s = 0; ph ^= 1; }
             ready = mbar_test_wait(smem_u32(&full_bar[s]), ph);
         };
         // phase A: T1 = In_halo P1
@@ -341,7 +344,7 @@ tucker_fused_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_const
     }
 }
 
-struct FusedGeo { int bh, tiles_per_img, PW, z1_slots; uint32_t smem_bytes; };
+struct FusedGeo { int bh, tiles_per_img, PW, z1_slots, slots; uint32_t smem_bytes; };
 
 inline bool a16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
@@ -358,8 +361,9 @@ bool fused_geometry(int64_t B, int64_t H, int64_t W, int64_t c_in, int64_t nA, i
     g->tiles_per_img = (int)((H + bh - 1) / bh);
     g->z1_slots = (130 + 2 * PW + 7) / 8 * 8;            // the last of 128 rows at the largest shift still reads inside the buffer
     const uint32_t z1_bytes = ((uint32_t)(nA / 8) * (uint32_t)g->z1_slots * 16u + 1023u) & ~1023u;
-    g->smem_bytes = 1024u + z1_bytes + kZ2Bytes + kSlots * kSlotBytes;
-    return g->tiles_per_img <= 65535 && g->smem_bytes <= 226u * 1024u;
+    g->slots = 1024u + z1_bytes + kZ2Bytes + kMaxSlots * kSlotBytes <= kSmemMost ? kMaxSlots : kMaxSlots - 1;
+    g->smem_bytes = 1024u + z1_bytes + kZ2Bytes + (uint32_t)g->slots * kSlotBytes;
+    return g->tiles_per_img <= 65535 && g->smem_bytes <= kSmemMost;
 }
 
 }  // namespace
@@ -382,20 +386,20 @@ lrd_status_t tucker_fused(bool dgrad, const void* in, const void* P1, const void
     CUtensorMap tIn, tP1, tG, tP3;
     bool ok = make_tmap_nhwc_bf16(&tIn, in, (uint64_t)B, (uint64_t)H, (uint64_t)W, (uint64_t)c_in, (uint32_t)(g.bh + 2), (uint32_t)W, 64);
     ok = ok && make_tmap_2d_bf16(&tP1, P1, (uint64_t)c_in, (uint64_t)nA, (uint64_t)nA, 64, (uint32_t)swb / 2);
-    ok = ok && make_tmap_2d_bf16(&tG, G, (uint64_t)r2, (uint64_t)(9 * r1), (uint64_t)(9 * r1), dgrad ? 64 : 128, 64);
+    ok = ok && make_tmap_2d_bf16(&tG, G, (uint64_t)r2, (uint64_t)(9 * r1), (uint64_t)(9 * r1), dgrad ? 64u : (uint32_t)nB, 64);
     ok = ok && make_tmap_2d_bf16(&tP3, P3, (uint64_t)n3, (uint64_t)nB, (uint64_t)nB, 256, 64);
     if (!ok) return LRD_ERR_CUDA;
     FusedParams p;
     p.H = (int)H; p.W = (int)W; p.PW = g.PW; p.bh = g.bh;
     p.c_in = (int)c_in; p.nA = (int)nA; p.nB = (int)nB; p.n3 = (int)n3;
-    p.g_ci = (int)r1; p.swb = swb; p.z1_slots = g.z1_slots;
+    p.g_ci = (int)r1; p.swb = swb; p.z1_slots = g.z1_slots; p.slots = g.slots;
     p.save1 = (__nv_bfloat16*)save1; p.save2 = (__nv_bfloat16*)save2; p.out3 = (__nv_bfloat16*)out3;
     p.bias3 = (const __nv_bfloat16*)bias3;
     p.timeout_flag = device_timeout_flag();
     static bool configured_on[kMaxDevices] = {};
     bool& configured = configured_on[device_slot()];
     if (!configured) {
-        const int lim = 226 * 1024;
+        const int lim = (int)kSmemMost;
         if (cudaFuncSetAttribute(tucker_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) != cudaSuccess ||
             cudaFuncSetAttribute(tucker_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) != cudaSuccess)
             return LRD_ERR_CUDA;
