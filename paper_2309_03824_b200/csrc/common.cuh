@@ -41,12 +41,13 @@ struct GemmArgs {
     bool add = false;          // weight gradients on the tensor-core kernels: C (and a_colsum) += the product, rounded to the storage
                                // type before the fp32 sum and after it
     bool whole = false;        // data products: the reduction is not split over a cluster
-    // Weight gradients on the single-SM kernels: this operand is loaded without waiting for the launch before this one, which is of
-    // the same call and does not write it.  Everything else the call reads is complete by then, because every kernel here that a
-    // call can put in front of a gradient lets the next launch start only behind its own griddepcontrol.wait; and because the
-    // gradient launch waits for the one before it before it ends, whoever waits for it has waited for both.  A launch boundary costs
-    // some 1.5 us behind the last block's exit and another for the first loads: 768 -> 768 at r = 192, a pass over 128 tokens
-    // 18.5 -> 17.7 us, over 4096 25.5 -> 25.3; six layers of 768 (4096 tokens) 171.2 -> 168.3.
+    // Weight gradients on the single-SM kernels, and B of data products on the persistent one: this operand is loaded without waiting
+    // for the launch before this one, which is of the same call and does not write it.  Everything else the call reads is complete
+    // by then, because every kernel here that a call can put in front of such a product lets the next launch start only behind its
+    // own griddepcontrol.wait; and because the launch waits for the one before it before it ends, whoever waits for it has
+    // waited for both.  A launch boundary costs some 1.5 us behind the last block's exit and another for the first loads.
+    // Gradients: 768 -> 768 at r = 192, a pass over 128 tokens 18.5 -> 17.7 us, over 4096 26.3 -> 25.7; six layers of 768 (4096
+    // tokens) replayed 170.8 -> 168.6.  B of the second product: 768 -> 3072 at 384, 64 tokens, forward 8.7 -> 8.5.
     bool a_early = false, b_early = false;
     bool any_rows = false;     // weight gradients: C of any stride and alignment (single-SM kernels)
     bool in_turn = false;      // weight gradients: started only when the launch before has ended (blocks that wait on an SM for

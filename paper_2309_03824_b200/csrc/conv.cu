@@ -113,7 +113,7 @@ size_t tucker2_workspace_bytes(const lrd_tucker2_desc_t* d, lrd_tucker_freeze_t 
 
 lrd_status_t tucker2_fwd(const lrd_tucker2_desc_t* d, const void* X, const void* A, const void* G, const void* Bm,
                          const void* bias, void* Y, void* Z1_save, void* Z2_save, lrd_tucker_freeze_t freeze,
-                         void* ws, size_t ws_bytes, int path, cudaStream_t s) {
+                         void* ws, size_t ws_bytes, int path, cudaStream_t s, bool* z_before_last) {
     (void)ws_bytes;
     const Tk t = parse(d);
     if (t.P == 0) return LRD_OK;
@@ -125,10 +125,11 @@ lrd_status_t tucker2_fwd(const lrd_tucker2_desc_t* d, const void* X, const void*
         const int r1 = (int)t.r1, r2 = (int)t.r2, p1 = (int)q.r1, p2 = (int)q.r2;
         const Copy2d in[3] = {{w + o.A, p1, A, r1, t.C, t.C, r1, p1}, {w + o.G, p1, G, r1, r2 * t.taps, p2 * t.taps, r1, p1}, {w + o.Bm, p2, Bm, r2, t.S, t.S, r2, p2}};
         LRD_TRY(copy2d_bf16(in, 3, s));
+        bool beside = false;           // Z1 and Z2 stand before the last launch: their copies need not wait for it
         LRD_TRY(tucker2_fwd(&q, X, w + o.A, w + o.G, w + o.Bm, bias, Y, Z1_save ? w + o.Z1 : nullptr, Z2_save ? w + o.Z2 : nullptr, freeze,
-                            w, inner, path, s));
+                            w, inner, path, s, &beside));
         const Copy2d out[2] = {{Z1_save, r1, w + o.Z1, p1, t.P, Z1_save ? t.P : 0, r1, r1}, {Z2_save, r2, w + o.Z2, p2, t.Po, Z2_save ? t.Po : 0, r2, r2}};
-        return copy2d_bf16(out, 2, s);
+        return copy2d_bf16(out, 2, s, beside);
     }
     // the whole forward in one launch where the shape allows: Z1 and Z2 stay on chip unless the caller saves them
     if (t.plain && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) && (!bias || ((uintptr_t)bias % 2) == 0) &&
@@ -142,7 +143,10 @@ lrd_status_t tucker2_fwd(const lrd_tucker2_desc_t* d, const void* X, const void*
         tc_conv_chain_eligible(false, t.B, t.g, t.r1, t.r2, t.S, t.dt, Z1, G, Bm, Y, Z2_save) && (!bias || ((uintptr_t)bias % 2) == 0))
         return tc_conv_chain(false, Z1, G, Bm, bias, Y, Z2_save, t.B, t.g, t.r1, t.r2, t.S, s);
     LRD_TRY(conv_fwd(Z1, G, Z2, t.B, t.g, t.r1, t.r2, t.dt, path, s));
-    return run_gemm(make_gemm(t.Po, t.S, t.r2, Z2, t.r2, false, Bm, t.r2, false, Y, t.S, bias, t.dt), path, false, nullptr, 0, s);
+    GemmArgs last = make_gemm(t.Po, t.S, t.r2, Z2, t.r2, false, Bm, t.r2, false, Y, t.S, bias, t.dt);
+    last.b_early = true;
+    if (z_before_last) *z_before_last = true;
+    return run_gemm(last, path, false, nullptr, 0, s);
 }
 
 lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void* X, const void* A, const void* G,
@@ -230,7 +234,11 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     if (one_launch) {
     } else if (fuse_dx) keep(tc_conv_chain(true, dZ2, G, A, nullptr, dX, factors ? dZ1 : nullptr, t.B, t.g, t.r1, t.r2, t.C, s));
     else if (dX || factors) keep(conv_bwd_data(dZ2, G, dZ1, t.B, t.g, t.r1, t.r2, t.dt, path, s));
-    if (dX && !fuse_dx && !one_launch) keep(run_gemm(make_gemm(t.P, t.C, t.r1, dZ1, t.r1, false, A, t.r1, false, dX, t.C, nullptr, t.dt), path, false, nullptr, 0, s));
+    if (dX && !fuse_dx && !one_launch) {
+        GemmArgs last = make_gemm(t.P, t.C, t.r1, dZ1, t.r1, false, A, t.r1, false, dX, t.C, nullptr, t.dt);
+        last.b_early = true;
+        keep(run_gemm(last, path, false, nullptr, 0, s));
+    }
     if (factors) {
         GemmArgs gw[2] = {make_gemm(t.C, t.r1, t.P, X, t.C, true, dZ1, t.r1, true, dA, t.r1, nullptr, t.dt), dB_product};
         // the data path stands before them on this stream, and writes dZ1 alone of their operands

@@ -8,7 +8,7 @@ lrd_status_t tucker2_check(const lrd_tucker2_desc_t* d, lrd_tucker_freeze_t free
 size_t tucker2_workspace_bytes(const lrd_tucker2_desc_t* d, lrd_tucker_freeze_t freeze, int is_bwd);
 lrd_status_t tucker2_fwd(const lrd_tucker2_desc_t* d, const void* X, const void* A, const void* G, const void* Bm,
                          const void* bias, void* Y, void* Z1_save, void* Z2_save, lrd_tucker_freeze_t freeze,
-                         void* ws, size_t ws_bytes, int path, cudaStream_t s);
+                         void* ws, size_t ws_bytes, int path, cudaStream_t s, bool* z_before_last = nullptr);
 lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void* X, const void* A, const void* G,
                          const void* Bm, const void* Z1_save, const void* Z2_save, void* dX, void* dA, void* dG,
                          void* dB, void* dbias, lrd_tucker_freeze_t freeze, void* ws, size_t ws_bytes, int path,

@@ -585,7 +585,9 @@ static lrd_status_t linear_fwd_on(const lrd_linear_desc_t* desc, const void* X, 
     GemmArgs first = gemm(L.M, L.r, L.K, X, L.ldx, false, V, L.ldv, true, Z, ldz, nullptr, L.dt);
     first.whole = whole;
     LRD_TRY(run_gemm(first, false, nullptr, 0, s));
-    return run_gemm(gemm(L.M, L.N, L.r, Z, ldz, false, U, L.ldu, false, Y, L.ldy, bias, L.dt), false, nullptr, 0, s);
+    GemmArgs second = gemm(L.M, L.N, L.r, Z, ldz, false, U, L.ldu, false, Y, L.ldy, bias, L.dt);
+    second.b_early = true;
+    return run_gemm(second, false, nullptr, 0, s);
 }
 
 static lrd_status_t lrd_linear_fwd_impl(const lrd_linear_desc_t* desc, const void* X, const void* V, const void* U,
@@ -692,8 +694,11 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
     if (!chained) {
         if (dX || need_dz_in_memory)
             LRD_TRY(run_gemm(gemm(L.M, L.r, L.N, dY, L.ldy, false, U, L.ldu, true, dZ, L.r, nullptr, L.dt), false, nullptr, 0, s));
-        if (dX)
-            LRD_TRY(run_gemm(gemm(L.M, L.K, L.r, dZ, L.r, false, V, L.ldv, false, dX, L.ldx, nullptr, L.dt), false, nullptr, 0, s));
+        if (dX) {
+            GemmArgs second = gemm(L.M, L.K, L.r, dZ, L.r, false, V, L.ldv, false, dX, L.ldx, nullptr, L.dt);
+            second.b_early = true;
+            LRD_TRY(run_gemm(second, false, nullptr, 0, s));
+        }
     }
     if (!do_w) return LRD_OK;
     GemmArgs gw[2];

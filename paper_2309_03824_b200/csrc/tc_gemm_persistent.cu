@@ -57,6 +57,7 @@ __device__ __forceinline__ void load2d(uint32_t dst, const CUtensorMap* m, uint3
 struct PParams {
     int64_t M, N;
     int kb_total, m_tiles, n_tiles;
+    int b_early;              // the first stages' B is loaded before this launch's turn
     const __nv_bfloat16* bias;
     unsigned int* timeout_flag;
 };
@@ -119,6 +120,30 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only this block's own shared and tensor memory: it may overlap the tail of the
     // previous kernel in the stream; global memory is first touched below this line
+    // B of the first tile, as much as the ring holds, may be fetched even before the launch in front has ended (see
+    // GemmArgs::b_early): what follows the wait is then the load of A alone.
+    auto load_b = [&](int s, int kb, int n0, uint32_t fb) {
+        const uint32_t b_dst = ring_base + s * C::STAGE_BYTES + G * kATile;
+        if (B_MN) {
+#pragma unroll
+            for (int j = 0; j < BNH / 64; ++j) load2d<CG>(b_dst + j * (8192 * G), &tmB, fb, n0 + 64 * j, kb * BK);
+        } else {
+#pragma unroll
+            for (int g = 0; g < G; ++g) load2d<CG>(b_dst + g * C::B_TILE, &tmB, fb, (kb + g) * BK, n0);
+        }
+    };
+    int early = 0;                                           // stages whose B is on its way
+    if (p.b_early && warp == 0) {
+        early = min(STAGES, (p.kb_total + G - 1) / G);
+        if (unit >= n_tiles_total) early = 0;
+        if (elect_one())
+            for (int s = 0; s < early; ++s) {
+                const uint32_t fb_local = smem_u32(&full_bar[s]), fb = CG == 2 ? map_to_cta(fb_local, 0) : fb_local;
+                if (h == 0) mbar_expect_tx(fb_local, CG * C::STAGE_BYTES);
+                load_b(s, s * G, (unit / p.m_tiles) * BN + h * BNH, fb);
+            }
+        __syncwarp();
+    }
     griddep_wait();
     griddep_launch_dependents();       // (in this order: see GemmArgs::a_early)
 
@@ -135,20 +160,14 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
                 // a pair's loads all complete on the even block's barrier, which its MMA warp waits on
                 const uint32_t fb_local = smem_u32(&full_bar[s]);
                 const uint32_t fb = CG == 2 ? map_to_cta(fb_local, 0) : fb_local;
-                const uint32_t a_dst = ring_base + s * C::STAGE_BYTES, b_dst = a_dst + G * kATile;
-                const int k0 = kb * BK;
+                const uint32_t a_dst = ring_base + s * C::STAGE_BYTES;
                 if (elect_one()) {
-                    if (h == 0) mbar_expect_tx(fb_local, CG * C::STAGE_BYTES);
+                    if (h == 0 && early <= 0) mbar_expect_tx(fb_local, CG * C::STAGE_BYTES);
 #pragma unroll
-                    for (int g = 0; g < G; ++g) load2d<CG>(a_dst + g * kATile, &tmA, fb, k0 + g * BK, m0);
-                    if (B_MN) {
-#pragma unroll
-                        for (int j = 0; j < BNH / 64; ++j) load2d<CG>(b_dst + j * (8192 * G), &tmB, fb, n0 + 64 * j, k0);
-                    } else {
-#pragma unroll
-                        for (int g = 0; g < G; ++g) load2d<CG>(b_dst + g * C::B_TILE, &tmB, fb, k0 + g * BK, n0);
-                    }
+                    for (int g = 0; g < G; ++g) load2d<CG>(a_dst + g * kATile, &tmA, fb, (kb + g) * BK, m0);
+                    if (early <= 0) load_b(s, kb, n0, fb);
                 }
+                --early;
                 __syncwarp();
                 if (++s == STAGES) { s = 0; ph ^= 1; }
             }
@@ -386,6 +405,7 @@ lrd_status_t tc_gemm_persistent(const GemmArgs& g, cudaStream_t stream) {
     p.m_tiles = (int)((g.M + BM * cg - 1) / (BM * cg));
     p.n_tiles = (int)((g.N + bn - 1) / bn);
     p.bias = (const __nv_bfloat16*)g.bias;
+    p.b_early = g.b_early;
     p.timeout_flag = device_timeout_flag();
     const int64_t tiles = (int64_t)p.m_tiles * p.n_tiles, units_max = kNumSms / cg;
     // every unit (block or pair) gets the same number of tiles (+-1): units = tiles / ceil(tiles / units_max), rounded up
