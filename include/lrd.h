@@ -203,11 +203,12 @@ lrd_status_t lrd_gemm_tuning(int blocks_per_mma);
 lrd_status_t lrd_wgrad_tuning(int blocks_per_mma, int columns, int split);
 lrd_status_t lrd_data_split_tuning(int columns, int split);
 
-/* With the core unfrozen, lrd_tucker2_bwd enqueues its independent launches side by side (the dB + dbias product from the
+/* With nothing frozen (or, on the general kernels, the factors), lrd_tucker2_bwd enqueues its independent launches side by side (the dB + dbias product from the
  * start, the core's filter gradient once dZ2 exists, both on streams the library owns; the data path and dA on the
  * caller's stream, which waits for the others before the call returns) when `on` is non-zero - the default -
  * and one after the other on the caller's stream when it is zero.  Same bits either way.  With the core frozen everything
- * runs on the caller's stream, dA and dB in one launch, and the switch has no effect.  With the default,
+ * runs on the caller's stream, dA and dB in one launch, and the switch has no effect; with the factors frozen the filter
+ * gradient follows the data path there, and the switch only decides whether it may start before that path has ended.  With the default,
  * make a host thread's first backward call on a device outside any stream capture (it creates that thread's
  * streams).  The switch is process-wide; no counterpart in the paper. */
 lrd_status_t lrd_tucker2_overlap(int on);

@@ -197,7 +197,12 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     // gradient, and dB and dA in one launch behind the data path need no second stream: 64 x 14 x 14, 256 -> 256 at rank 96
     // 40.4 -> 38.5 us per step, 16 x 28 x 28, 128 -> 128 at 64 43.4 -> 41.8; with nothing frozen dB beside the data path
     // remains the faster way (64 x 7 x 7, 512 -> 512 at 309 92.5 against 96.0).
-    SideStreams* ss = g_tucker_overlap && core ? side_streams() : nullptr;
+    // With the factors frozen the filter gradient is the only one: on the tensor-core kernel it follows the data path and loads
+    // ahead what that path's last launch does not write, which spares the stream a fork and a join (64 x 28 x 28, stride 2, 256 -> 256
+    // at rank 96 59.4 -> 56.8 us, replayed the same 54.5).  With nothing frozen the streams remain (64 x 7 x 7 at rank 309, replayed:
+    // 81.4 against 83.2), and on the general kernels, which fill few SMs each (fp32, 10 x 14 x 14 at rank 128 223 against 259).
+    const bool filter_follows = core && !factors && path != LRD_PATH_GENERAL && tc_conv_eligible(t.B, t.g, t.r1, t.r2, t.dt, dZ2, Z1_save, dG);
+    SideStreams* ss = g_tucker_overlap && core && !filter_follows ? side_streams() : nullptr;
     cudaStream_t sB = ss && factors ? ss->aux[0] : s, sF = ss ? ss->aux[1] : s;
     lrd_status_t st = LRD_OK;
     auto keep = [&st](lrd_status_t x) { if (st == LRD_OK) st = x; };
@@ -209,8 +214,8 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     // (by itself with the switch off too: one launch with dA would share the pixels out differently, and the switch changes no bits)
     if (factors && core) keep(run_gemm(dB_product, path, true, pB, reg.dB, sB));
 
-    auto launch_filter = [&](cudaStream_t st_f) {
-        keep(conv_bwd_filter(dZ2, Z1_save, dG, t.B, t.g, t.r1, t.r2, t.dt, path, st_f));
+    auto launch_filter = [&](cudaStream_t st_f, bool a_early, bool b_early) {
+        keep(conv_bwd_filter(dZ2, Z1_save, dG, t.B, t.g, t.r1, t.r2, t.dt, path, a_early, b_early, st_f));
     };
     // the whole data path (dZ2 = dY Bm, transposed core, dX = dZ1 A^T) in one launch where the shape allows; dZ2 is
     // written only for the filter gradient, dZ1 only for dA.  (Giving the filter gradient a dZ2 product of its own
@@ -226,7 +231,7 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
         keep(run_gemm(make_gemm(t.Po, t.r2, t.S, dY, t.S, false, Bm, t.r2, true, dZ2, t.r2, nullptr, t.dt), path, false, nullptr, 0, s));
     if (core && sF != s) {
         if (!stream_after(sF, s, ss->mid)) keep(LRD_ERR_CUDA);
-        else launch_filter(sF);
+        else launch_filter(sF, false, false);
     }
     // transposed core + first 1x1 (dX = dZ1 A^T) in one launch where the shape allows; dZ1 is written only for dA
     const bool fuse_dx = !one_launch && dX && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
@@ -247,7 +252,8 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
         const size_t scratch_bytes[2] = {reg.dA, reg.dB};
         keep(run_wgrads(gw, core ? 1 : 2, path, scratch, scratch_bytes, s));
     }
-    if (core && sF == s) launch_filter(s);
+    // (behind the data path on its stream: Z1_save is none of its results, dZ2 one of its last launch only where that is its first)
+    if (core && sF == s) launch_filter(s, filter_follows && g_tucker_overlap && dX && !one_launch, filter_follows && g_tucker_overlap);
     // join even after a failed launch, so that a capture in progress is left whole
     if (sB != s && !stream_after(s, sB, ss->aux_done[0])) keep(LRD_ERR_CUDA);
     if (sF != s && !stream_after(s, sF, ss->aux_done[1])) keep(LRD_ERR_CUDA);
@@ -268,8 +274,8 @@ lrd_status_t conv_bwd_data(const void* dout, const void* G, void* din, int64_t B
     return simt_conv_bwd_data(dout, G, din, B, g, ci, co, dt, s);
 }
 lrd_status_t conv_bwd_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt,
-                             int path, cudaStream_t s) {
-    if (path != LRD_PATH_GENERAL && tc_conv_eligible(B, g, ci, co, dt, dout, in, dG)) return tc_conv_filter(dout, in, dG, B, g, ci, co, s);
+                             int path, bool a_early, bool b_early, cudaStream_t s) {
+    if (path != LRD_PATH_GENERAL && tc_conv_eligible(B, g, ci, co, dt, dout, in, dG)) return tc_conv_filter(dout, in, dG, B, g, ci, co, a_early, b_early, s);
     return simt_conv_bwd_filter(dout, in, dG, B, g, ci, co, dt, s);
 }
 

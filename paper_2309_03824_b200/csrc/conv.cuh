@@ -50,7 +50,8 @@ bool tc_conv_chain_eligible(bool dgrad, int64_t B, const ConvGeom& g, int64_t ci
 lrd_status_t tc_conv_chain(bool dgrad, const void* img, const void* G, const void* Q, const void* bias2, void* out2, void* core_out,
                            int64_t B, const ConvGeom& g, int64_t ci, int64_t co, int64_t n2, cudaStream_t s);
 // Filter gradient, one launch, no scratch.
-lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, cudaStream_t s);
+lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, bool a_early,
+                            bool b_early, cudaStream_t s);
 
 // A whole data pass of the layer in one launch (3 x 3 core, stride 1; ranks <= 128 and multiples of 16, at most 256 output
 // channels, images at most 40 pixels wide): forward (dgrad = false) out3 = conv(in P1, G) P3^T + bias3 with P1 = A [C x r1],
@@ -70,6 +71,6 @@ lrd_status_t conv_fwd(const void* in, const void* G, void* out, int64_t B, const
 lrd_status_t conv_bwd_data(const void* dout, const void* G, void* din, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt,
                            int path, cudaStream_t s);
 lrd_status_t conv_bwd_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt,
-                             int path, cudaStream_t s);
+                             int path, bool a_early, bool b_early, cudaStream_t s);       // early: see GemmArgs::a_early
 
 }  // namespace lrd

@@ -999,7 +999,7 @@ static lrd_status_t lrd_conv3x3_bwd_impl(int64_t B, int64_t H, int64_t W, int64_
     if (B == 0) return zero_fill(dW, S, 9 * C, 9 * C, (lrd_dtype_t)dtype, s);
     const ConvGeom g = conv_geom(H, W, 3, 1);
     if (dX) LRD_TRY(conv_bwd_data(dY, Wk, dX, B, g, C, S, (lrd_dtype_t)dtype, g_path.load(), s));
-    return conv_bwd_filter(dY, X, dW, B, g, C, S, (lrd_dtype_t)dtype, g_path.load(), s);
+    return conv_bwd_filter(dY, X, dW, B, g, C, S, (lrd_dtype_t)dtype, g_path.load(), false, false, s);
 }
 
 size_t lrd_tucker2_workspace_bytes(const lrd_tucker2_desc_t* desc, lrd_tucker_freeze_t freeze, int is_bwd) {

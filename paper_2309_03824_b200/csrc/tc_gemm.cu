@@ -1002,7 +1002,7 @@ lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const s
 
 // Filter gradient (see CONV above): M = co, N = taps x 64-column blocks, K = output pixels.
 lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t B, const ConvGeom& g, int64_t ci, int64_t co,
-                            cudaStream_t stream) {
+                            bool a_early, bool b_early, cudaStream_t stream) {
     if (!tc_conv_eligible(B, g, ci, co, LRD_BF16, dout, in, dG)) return LRD_ERR_UNSUPPORTED;
     const int64_t P = B * g.Ho * g.Wo, taps = (int64_t)g.k * g.k, nkc = (ci + 63) / 64, N = taps * nkc * 64;
     SplitPlan sp = pick_split(co, N, P, true);             // (tiles of at most 192 columns)
@@ -1021,6 +1021,7 @@ lrd_status_t tc_conv_filter(const void* dout, const void* in, void* dG, int64_t 
     p.cluster_splits = sp.cluster;
     p.timeout_flag = device_timeout_flag();
     p.C = dG; p.ldc = taps * ci;
+    p.a_early = a_early; p.b_early = b_early;
     p.cv_ci = (int)ci; p.cv_nkc = (int)nkc; p.cv_nblk = (int)(taps * nkc); p.cv_k = g.k;
     p.cv_Ho = g.Ho; p.cv_Wo = g.Wo; p.cv_stride = g.stride; p.cv_pad = g.pad;
     dim3 grid((unsigned)((N + sp.bn - 1) / sp.bn), (unsigned)((co + BM - 1) / BM), (unsigned)sp.cluster);
