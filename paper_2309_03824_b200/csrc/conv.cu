@@ -246,8 +246,9 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     }
     if (factors) {
         GemmArgs gw[2] = {make_gemm(t.C, t.r1, t.P, X, t.C, true, dZ1, t.r1, true, dA, t.r1, nullptr, t.dt), dB_product};
-        // the data path stands before them on this stream, and writes dZ1 alone of their operands
-        gw[0].a_early = gw[1].a_early = gw[1].b_early = true;
+        // the data path stands before them on this stream, and writes dZ1 alone of their operands (with the core unfrozen the side
+        // streams' gradients want the SMs that dA would wait on: 64 x 7 x 7 at rank 309 89.2 us loading ahead, 87.9 not)
+        gw[0].a_early = gw[1].a_early = gw[1].b_early = !core;
         float* const scratch[2] = {pA, pB};
         const size_t scratch_bytes[2] = {reg.dA, reg.dB};
         keep(run_wgrads(gw, core ? 1 : 2, path, scratch, scratch_bytes, s));

@@ -772,7 +772,7 @@ static lrd_status_t lrd_linear_bwd_accumulate_impl(const lrd_linear_desc_t* desc
     LRD_TRY(check_ws(workspace, workspace_bytes, lrd_linear_workspace_bytes(desc, freeze, 2)));
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // where the tensor-core kernels can write the caller's buffers, they add this step's gradients to them: 1024 -> 4096 at rank
-    // 512, 1021 tokens 44.3 us, with two launches that add from scratch 53.2
+    // 512, 1021 tokens 38.7 us (44.3 reading the old values in the epilogue, 53.2 with two launches that add from scratch)
     if (L.M > 0 && du_dv_addable(L, plan, dY, X, Z_save, dU, dV, workspace) && !needs_repack(L) && g_path.load() != LRD_PATH_GENERAL) {
         for (const void* p : {(const void*)dU, (const void*)dV, (const void*)dbias})
             if (p && !elem_aligned(p, L.dt)) return LRD_ERR_ALIGNMENT;
