@@ -168,7 +168,10 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only this block's own shared and tensor memory: it may overlap the tail of the
-    // previous kernel in the stream; global memory is first touched below this line, by the producers and then by the epilogue
+    // previous kernel in the stream; global memory is first touched below this line, by the producers and then by the epilogue.
+    // Unless both operands are early, every wait with a limit starts behind griddepcontrol.wait: the limit is for what this launch
+    // does, and the launch in front, which may be the caller's, takes what time it likes.
+    const bool all_early = A_MN && p.a_early && p.b_early;
     if (!A_MN) griddep_wait();         // (in this order: see GemmArgs::a_early)
     griddep_launch_dependents();
 
@@ -179,6 +182,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         for (int kb = kb_begin; kb < kb_end; kb += G, ++it) {          // (a k-block past this block's share is loaded, not multiplied)
             const int s = it % STAGES;
             const uint32_t ph = (it / STAGES) & 1;
+            if (A_MN && it == STAGES && !all_early) griddep_wait();        // (the ring is full and nothing multiplied before that)
             if (!mbar_wait_uniform(smem_u32(&empty_bar[s]), ph ^ 1, ab)) break;
             const uint32_t fb = smem_u32(&full_bar[s]);
             const uint32_t a_dst = smem_base + s * C::STAGE_BYTES;
@@ -204,6 +208,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         for (int kb = kb_begin; kb < kb_end; kb += G, ++it) {
             const int s = it % STAGES;
             const uint32_t ph = (it / STAGES) & 1;
+            if (A_MN && it == STAGES && !all_early) griddep_wait();        // (the ring is full and nothing multiplied before that)
             if (!mbar_wait_uniform(smem_u32(&empty_bar[s]), ph ^ 1, ab)) break;
             const uint32_t fb = smem_u32(&full_bar[s]);
             const uint32_t b_dst = smem_base + s * C::STAGE_BYTES + A_STAGE_BYTES;
@@ -237,6 +242,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         const uint32_t idesc = idesc_bf16(BN + (with_colsum ? 16 : 0), A_MN, B_MN);
         const uint64_t a_desc0 = A_MN ? smem_desc_sw128(smem_base, kBox, 1024) : smem_desc_sw128(smem_base, 0, 1024);
         const uint64_t b_desc0 = B_MN ? smem_desc_sw128(smem_base + A_STAGE_BYTES, kBox, 1024) : smem_desc_sw128(smem_base + A_STAGE_BYTES, 0, 1024);
+        if (A_MN && !all_early) griddep_wait();
         int s = 0;
         uint32_t ph = 0, ready = kb_begin < kb_end ? mbar_test_wait(smem_u32(&full_bar[0]), 0) : 0u;
         bool ok = true;
@@ -273,7 +279,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         const uint32_t chunk_bytes = 128u * cs * 4u, ngrp = cs / 4u;
         const uint32_t stage_base = smem_base, recv_base = smem_base + 128u * BN * 4u;
         const uint32_t cs_stage = recv_base + 128u * BN * 4u, cs_recv = cs_stage + 512u;
-        if (ADD) griddep_wait();
+        if (A_MN && (ADD || !all_early)) griddep_wait();
         bool ok = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         // barrier 1: this block's pipeline ring is dead (all its MMAs have completed).  Progress only: what the peers
@@ -436,7 +442,7 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         }
     } else {
         const int quarter = warp % 4;                      // lanes [32 q, 32 q + 32) of tensor memory
-        if (ADD) griddep_wait();
+        if (A_MN && (ADD || !all_early)) griddep_wait();
         const bool ready = mbar_wait_warp(smem_u32(&acc_bar), 0, ab);
         tc_fence_after();
         if (ready) {
