@@ -549,10 +549,9 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     }
 }
 
-// out[m][n] = sum_z partial[z][m][n] (+ bias[n]), z ascending; 4 columns per thread.
+// out[m][n] = sum_z partial[z][m][n], z ascending; 4 columns per thread.
 __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restrict__ partial, int splits, int64_t M,
                                                             int64_t N, int64_t ldp,
-                                                            const __nv_bfloat16* __restrict__ bias,
                                                             __nv_bfloat16* __restrict__ C, int64_t ldc,
                                                             const float* __restrict__ colsum_partial,
                                                             __nv_bfloat16* __restrict__ colsum_out, int add) {
@@ -583,10 +582,8 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
     }
     for (int e = 0; e < 4; ++e)
         if (n + e < N) {
-            float v = acc[e];
-            if (bias) v += __bfloat162float(bias[n + e]);
-            if (add) add_into_bf16(C + m * ldc + n + e, v);
-            else C[m * ldc + n + e] = __float2bfloat16_rn(v);
+            if (add) add_into_bf16(C + m * ldc + n + e, acc[e]);
+            else C[m * ldc + n + e] = __float2bfloat16_rn(acc[e]);
         }
 }
 
@@ -833,7 +830,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     const bool ones = g.a_colsum != nullptr;
     int splits = 1, cluster, bn;
     if (allow_split) {                                     // weight gradients
-        if (!g.a_mn_major || !g.b_mn_major) return LRD_ERR_UNSUPPORTED;
+        if (!g.a_mn_major || !g.b_mn_major || g.bias) return LRD_ERR_UNSUPPORTED;        // (only data products add a bias)
         double us;
         const WgradForm& form = tc_wgrad_form();
         const int64_t n = g.any_rows ? (g.N + 15) / 16 * 16 : g.N;          // (scratch was asked for at the padded rank)
@@ -873,7 +870,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     p.timeout_flag = device_timeout_flag();
     p.C = splits > 1 ? (void*)partials : g.C;
     p.ldc = g.ldc;
-    p.bias = splits > 1 ? nullptr : (const __nv_bfloat16*)g.bias;
+    p.bias = (const __nv_bfloat16*)g.bias;
     p.colsum_partial = (ones && splits > 1) ? (float*)((uint8_t*)partials + tile_bytes) : nullptr;
     p.colsum_out = (ones && splits == 1) ? (__nv_bfloat16*)g.a_colsum : nullptr;
     dim3 grid((unsigned)((g.N + bn - 1) / bn), (unsigned)((g.M + BM - 1) / BM), (unsigned)zdim);
@@ -900,7 +897,7 @@ lrd_status_t tc_gemm(const GemmArgs& g, bool allow_split, float* partials, size_
     if (st != LRD_OK || splits == 1) return st;
     const int64_t work = g.M * ((g.N + 3) / 4) + (ones ? g.M : 0);
     splitk_reduce_kernel<<<(unsigned)((work + 255) / 256), 256, 0, stream>>>(
-        partials, splits, g.M, g.N, ldp, (const __nv_bfloat16*)g.bias, (__nv_bfloat16*)g.C, g.ldc, p.colsum_partial,
+        partials, splits, g.M, g.N, ldp, (__nv_bfloat16*)g.C, g.ldc, p.colsum_partial,
         ones ? (__nv_bfloat16*)g.a_colsum : nullptr, g.add);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? LRD_OK : LRD_ERR_CUDA;
