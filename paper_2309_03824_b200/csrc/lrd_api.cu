@@ -609,8 +609,7 @@ static int linear_wgrads(const Linear& L, uint32_t plan, const void* dY, const v
 }
 
 // The same of a backward pass's gradients.
-// (`z`: the copy of Z that only the gradients need, made beside the data pass)
-struct PackedGrads { void *dU, *dV; int64_t ldu, ldv, cols; bool stored; Copy2d z; };
+struct PackedGrads { void *dU, *dV; int64_t ldu, ldv, cols; bool stored; };
 // One layer's backward on stream s.  With a side stream, the dU (+ db) product, which needs nothing the data
 // chain produces, runs there beside the chain; the caller has made `side` wait for s's earlier work and makes s
 // wait for `side` afterwards.  dV follows the chain (it reads the dZ the chain spills) and, when dU is computed too,
@@ -664,8 +663,11 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
         const int r = (int)L.r, rp = (int)q.r;
         const Copy2d in[3] = {{w + o.Vp, rp, V, L.ldv, L.K, do_data ? L.K : 0, r, rp}, {w + o.Up, rp, U, L.ldu, L.N, do_data ? L.N : 0, r, rp},
                               {w + o.Zp, rp, Z_save, L.ldz, L.M, du ? L.M : 0, r, rp}};
-        LRD_TRY(copy2d_bf16(in, 2, s));
-        PackedGrads pg{dU, dV, L.ldu, L.ldv, r, false, in[2]};
+        // (Z, which only the gradients need, goes with the factors: a launch of its own beside the data pass cost more than it hid, and
+        // kept dU from loading Z ahead.  156 backward passes of packed layers: V frozen 5.1 % faster on average, nothing frozen 2.9;
+        // 8192 tokens, 4096 -> 4096 at rank 250 77.6 -> 74.5 and 95.7 -> 93.2 us)
+        LRD_TRY(copy2d_bf16(in, 3, s));
+        PackedGrads pg{dU, dV, L.ldu, L.ldv, r, false};
         // the frozen factor's buffers were zero-filled above; the padded call gets none for them
         LRD_TRY(linear_bwd_on(&q, dY, X, w + o.Vp, w + o.Up, w + o.Zp, dX, du ? w + o.dUp : nullptr, dv ? w + o.dVp : nullptr, du ? dbias : nullptr,
                               freeze, w, inner, s, nullptr, nullptr, sm_share, false, parts, false, &pg));
@@ -705,7 +707,6 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
     for (int i = 0; i < n; ++i) gw[i].add = accumulate;
     // behind a launch of this call what the data half does not write need not be waited for
     const bool behind = !side && do_data && (dX || need_dz_in_memory);
-    if (packed) LRD_TRY(copy2d_bf16(&packed->z, 1, s, behind));
     if (packed && !side && path == LRD_PATH_AUTO && n > 0) {
         bool tc = true;
         for (int i = 0; i < n; ++i) tc = tc && tc_gemm_eligible(gw[i]);
@@ -720,7 +721,7 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
     }
     for (int i = 0; i < n; ++i) {
         gw[i].a_early = behind;
-        gw[i].b_early = behind && gw[i].B != dZ && !packed;
+        gw[i].b_early = behind && gw[i].B != dZ;
     }
     if (side && n == 2) {
         LRD_TRY(run_gemm(gw[0], true, partials, partial_bytes, side));

@@ -303,3 +303,18 @@ def test_packed_ranks_store_their_rows_alone(shape, freeze, pads):
         assert rel_err(got, ref) <= 2e-2
     for flat, view in ((Zf, Z), (dUf, dU), (dVf, dV)):
         assert bool((flat[view.numel():] == 7).all()) and bool((view[:, r:] == 7).all())
+
+
+@pytest.mark.parametrize("freeze", [b.LRD_FREEZE_V, b.LRD_FREEZE_U, b.LRD_FREEZE_NONE])
+def test_a_packed_backward_pass_is_three_launches(freeze):
+    """The factors and Z padded together, the data pass, the gradients to the caller's rows."""
+    case = wl.random_factor_case(4096, 768, 768, 190, "bf16", 1050)
+    X, V, U, dY = (dev(case[k], "bf16") for k in ("X", "V", "U", "dY"))
+    Z = (X.float() @ V.float()).to(torch.bfloat16)
+    desc = b.linear_desc(4096, 768, 768, 190, b.LRD_BF16)
+    dU, dV, dX = torch.empty_like(U), torch.empty_like(V), torch.empty_like(X)
+    ws = workspace(b.lrd_linear_workspace_bytes(desc, freeze, 1))
+    n0 = b.lrd_launch_count()
+    b.lrd_linear_bwd(desc, dY, X, V, U, Z, dX, dU if freeze != b.LRD_FREEZE_U else None, dV if freeze != b.LRD_FREEZE_V else None, None, freeze, ws)
+    assert b.lrd_launch_count() - n0 == 3
+    assert b.lrd_check_device_status() == b.LRD_OK
