@@ -253,10 +253,12 @@ struct CopyBatch {
     int64_t unit0[kMaxCopies + 1];       // first (row, 128-column piece) of each job
     int n;
 };
-// EARLY: as GemmArgs::a_early (a variant: with the test at run time each of the four launches around 64 x 7 x 7 at rank 309 took 0.4 us more)
+// EARLY: as GemmArgs::a_early (a variant: with the test at run time each of the four launches around 64 x 7 x 7 at rank 309 took 0.4 us more).
+// Either lets the next launch start at once, which then sets itself up beside the copy (768 -> 768 at rank 95, 64 tokens, forward
+// with U frozen 8.7 us behind the wait, 8.1 so): it is never the launch that an early one relies on, see GemmArgs.
 template <bool EARLY> __global__ void __launch_bounds__(256) copy2d_bf16_kernel(const __grid_constant__ CopyBatch b) {
-    if (!EARLY) ptx::griddep_wait();
     ptx::griddep_launch_dependents();
+    if (!EARLY) ptx::griddep_wait();
     const int lane = threadIdx.x % 32;
     const int64_t warps = (int64_t)gridDim.x * 8;
     int j = 0;
@@ -664,7 +666,7 @@ static lrd_status_t linear_bwd_on(const lrd_linear_desc_t* desc, const void* dY,
         const Copy2d in[3] = {{w + o.Vp, rp, V, L.ldv, L.K, do_data ? L.K : 0, r, rp}, {w + o.Up, rp, U, L.ldu, L.N, do_data ? L.N : 0, r, rp},
                               {w + o.Zp, rp, Z_save, L.ldz, L.M, du ? L.M : 0, r, rp}};
         // (Z, which only the gradients need, goes with the factors: a launch of its own beside the data pass cost more than it hid, and
-        // kept dU from loading Z ahead.  156 backward passes of packed layers: V frozen 5.1 % faster on average, nothing frozen 2.9;
+        // kept dU from loading Z ahead.  Backward passes of 120 packed layers: V frozen 5.1 % faster on average, nothing frozen 2.9;
         // 8192 tokens, 4096 -> 4096 at rank 250 77.6 -> 74.5 and 95.7 -> 93.2 us)
         LRD_TRY(copy2d_bf16(in, 3, s));
         PackedGrads pg{dU, dV, L.ldu, L.ldv, r, false};
