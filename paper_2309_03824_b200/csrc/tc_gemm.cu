@@ -169,8 +169,8 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only this block's own shared and tensor memory: it may overlap the tail of the
     // previous kernel in the stream; global memory is first touched below this line, by the producers and then by the epilogue.
-    // Unless both operands are early, every wait with a limit starts behind griddepcontrol.wait: the limit is for what this launch
-    // does, and the launch in front, which may be the caller's, takes what time it likes.
+    // Every wait with a limit starts behind griddepcontrol.wait, as the launch in front, which may be the caller's, takes what time
+    // it likes; with early operands it is a data pass of the same call, and the waits that need nothing of it start at once.
     const bool all_early = A_MN && p.a_early && p.b_early;
     if (!A_MN) griddep_wait();         // (in this order: see GemmArgs::a_early)
     griddep_launch_dependents();
@@ -182,7 +182,6 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         for (int kb = kb_begin; kb < kb_end; kb += G, ++it) {          // (a k-block past this block's share is loaded, not multiplied)
             const int s = it % STAGES;
             const uint32_t ph = (it / STAGES) & 1;
-            if (A_MN && it == STAGES && !all_early) griddep_wait();        // (the ring is full and nothing multiplied before that)
             if (!mbar_wait_uniform(smem_u32(&empty_bar[s]), ph ^ 1, ab)) break;
             const uint32_t fb = smem_u32(&full_bar[s]);
             const uint32_t a_dst = smem_base + s * C::STAGE_BYTES;
@@ -208,7 +207,6 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
         for (int kb = kb_begin; kb < kb_end; kb += G, ++it) {
             const int s = it % STAGES;
             const uint32_t ph = (it / STAGES) & 1;
-            if (A_MN && it == STAGES && !all_early) griddep_wait();        // (the ring is full and nothing multiplied before that)
             if (!mbar_wait_uniform(smem_u32(&empty_bar[s]), ph ^ 1, ab)) break;
             const uint32_t fb = smem_u32(&full_bar[s]);
             const uint32_t b_dst = smem_base + s * C::STAGE_BYTES + A_STAGE_BYTES;
