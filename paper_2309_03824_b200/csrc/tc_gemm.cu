@@ -913,18 +913,39 @@ static double group_estimate(const GemmArgs* g, int n, int bn, int S) {
     return S > 1 && tiles > max_active_clusters(S) ? 1e300 : split_us(bn, S, tiles, deepest, kblocks);
 }
 
+// The fastest of them by that estimate.
+static double best_group(const GemmArgs* g, int n, int* bn, int* S) {
+    const int top = g[0].max_cluster_split >= 2 && g[0].max_cluster_split < kMaxClusterSplits ? g[0].max_cluster_split : kMaxClusterSplits;
+    double us = 1e300;
+    for (int b : {192, 128, 64})
+        for (int c = top; c >= 1; --c) {
+            if (b % (8 * c)) continue;
+            const double t = group_estimate(g, n, b, c);
+            if (t < us) { us = t; *bn = b; *S = c; }
+        }
+    return us;
+}
+
+constexpr double kNextLaunch = 2.0;            // a launch behind another one drains and fills the SMs anew
+
 // Gradients whose rows TMA cannot address run on single SMs only: worth it where pairs would not save more than the launch that
-// copies a padded result, some 3 us.
+// copies a padded result, some 3 us.  Over 360 backward passes of packed layers (64 to 8192 tokens, ranks 61 to 1001, each mask) the
+// choice costs 0.3 % on average against the fastest measurement (always in place 0.5 %, always copied 7.0): 2048 tokens, 1024 -> 4096 at
+// rank 250, nothing frozen, in place / copied 30.1 / 32.7 us; 4096 tokens, 4096 -> 4096 at rank 499 84.3 / 80.7.
 bool tc_wgrads_any_rows(const GemmArgs* g, int n) {
     if (tc_wgrad_form().blocks) return false;
-    double single = 0.0, pairs = 0.0;
+    double single = kNextLaunch * (n - 1), pairs = single;
     for (int i = 0; i < n; ++i) {
         double us;
         pick_split(g[i].M, g[i].N, g[i].K, g[i].a_colsum != nullptr, g[i].max_cluster_split, &us);
         single += us;
         pairs += std::min(us, tc_wgrad_pair_estimate(&g[i], 1));
     }
-    if (n > 1) pairs = std::min(pairs, tc_wgrad_pair_estimate(g, n));
+    if (n > 1) {
+        int bn, S;
+        single = std::min(single, best_group(g, n, &bn, &S));
+        pairs = std::min(pairs, tc_wgrad_pair_estimate(g, n));
+    }
     return single <= pairs + 3.0;
 }
 
@@ -964,7 +985,7 @@ lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const s
     const WgradForm& form = tc_wgrad_form();
     bool ones = false, together = n > 1 && n <= kMaxWgrads;
     int64_t rows = 0;
-    double separate = 2.0 * (n - 1);           // a launch behind another one drains and fills the SMs anew
+    double separate = kNextLaunch * (n - 1);
     for (int i = 0; i < n && together; ++i) {
         together = tc_gemm_eligible(g[i]) && g[i].a_mn_major && g[i].b_mn_major && !g[i].bias && g[i].max_cluster_split == g[0].max_cluster_split &&
                    g[i].add == g[0].add && g[i].any_rows == g[0].any_rows;
@@ -976,15 +997,9 @@ lrd_status_t tc_wgrads(const GemmArgs* g, int n, float* const* partials, const s
         separate += std::min(us, tc_wgrad_pair_estimate(&g[i], 1));
     }
     if (together && rows <= 65535) {
-        const int top = g[0].max_cluster_split >= 2 && g[0].max_cluster_split < kMaxClusterSplits ? g[0].max_cluster_split : kMaxClusterSplits;
         int bn = 0, S = 1;
-        double us = separate;
-        for (int b : {192, 128, 64})
-            for (int c = top; c >= 1; --c) {
-                if (b % (8 * c)) continue;
-                const double t = group_estimate(g, n, b, c);
-                if (t < us) { us = t; bn = b; S = c; }
-            }
+        double us = best_group(g, n, &bn, &S);
+        if (!(us < separate)) { us = separate; bn = 0; }
         if (form.blocks) { bn = form.columns; S = form.split; }
         if (form.blocks ? form.blocks == 2 : tc_wgrad_pair_estimate(g, n) < us) return tc_wgrad_pair(g, n, stream);
         switch (bn) {

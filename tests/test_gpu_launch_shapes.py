@@ -306,12 +306,14 @@ def test_packed_ranks_store_their_rows_alone(shape, freeze, pads):
 
 
 @pytest.mark.parametrize("freeze", [b.LRD_FREEZE_V, b.LRD_FREEZE_U, b.LRD_FREEZE_NONE])
-def test_a_packed_backward_pass_is_three_launches(freeze):
-    """The factors and Z padded together, the data pass, the gradients to the caller's rows."""
-    case = wl.random_factor_case(4096, 768, 768, 190, "bf16", 1050)
+@pytest.mark.parametrize("shape", [(4096, 768, 768, 190), (4096, 768, 3072, 190)])
+def test_a_packed_backward_pass_is_three_launches(shape, freeze):
+    """The factors and Z padded together, the data pass, the gradients (two of them too) to the caller's rows."""
+    M, K, N, r = shape
+    case = wl.random_factor_case(M, K, N, r, "bf16", 1050)
     X, V, U, dY = (dev(case[k], "bf16") for k in ("X", "V", "U", "dY"))
     Z = (X.float() @ V.float()).to(torch.bfloat16)
-    desc = b.linear_desc(4096, 768, 768, 190, b.LRD_BF16)
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16)
     dU, dV, dX = torch.empty_like(U), torch.empty_like(V), torch.empty_like(X)
     ws = workspace(b.lrd_linear_workspace_bytes(desc, freeze, 1))
     n0 = b.lrd_launch_count()
