@@ -47,7 +47,7 @@ struct GemmArgs {
     // own griddepcontrol.wait; and because the launch waits for the one before it before it ends, whoever waits for it has
     // waited for both.  A launch boundary costs some 1.5 us behind the last block's exit and another for the first loads.
     // Gradients: 768 -> 768 at r = 192, a pass over 128 tokens 18.5 -> 17.7 us, over 4096 26.3 -> 25.7; six layers of 768 (4096
-    // tokens) replayed 170.8 -> 168.6.  B of the second product: 768 -> 3072 at 384, 64 tokens, forward 8.7 -> 8.5.
+    // tokens) replayed 170.8 -> 168.6.
     bool a_early = false, b_early = false;
     bool any_rows = false;     // weight gradients: C of any stride and alignment (single-SM kernels)
     bool in_turn = false;      // weight gradients: started only when the launch before has ended (blocks that wait on an SM for

@@ -118,10 +118,12 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     }
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
-    // set-up above touched only this block's own shared and tensor memory: it may overlap the tail of the
-    // previous kernel in the stream; global memory is first touched below this line
-    // B of the first tile, as much as the ring holds, may be fetched even before the launch in front has ended (see
-    // GemmArgs::b_early): what follows the wait is then the load of A alone.
+    // A pair's loads all complete on the even block's barrier, which its MMA warp waits on.
+    auto full = [&](int s) { return CG == 2 ? map_to_cta(smem_u32(&full_bar[s]), 0) : smem_u32(&full_bar[s]); };
+    auto load_a = [&](int s, int kb, int m0, uint32_t fb) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) load2d<CG>(ring_base + s * C::STAGE_BYTES + g * kATile, &tmA, fb, (kb + g) * BK, m0);
+    };
     auto load_b = [&](int s, int kb, int n0, uint32_t fb) {
         const uint32_t b_dst = ring_base + s * C::STAGE_BYTES + G * kATile;
         if (B_MN) {
@@ -132,15 +134,18 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
             for (int g = 0; g < G; ++g) load2d<CG>(b_dst + g * C::B_TILE, &tmB, fb, (kb + g) * BK, n0);
         }
     };
+    // set-up above touched only this block's own shared and tensor memory: it may overlap the tail of the
+    // previous kernel in the stream.  So may, where the call says so, the load of B for the first tile, as much as the ring holds
+    // (see GemmArgs::b_early): what follows the wait is then the load of A alone.  Everything else that touches global memory stands
+    // behind the wait.  Forward passes as two products, 72 shapes of 64 to 8192 tokens: 1.3 % on average, 1024 -> 4096 at rank 512,
+    // 64 tokens 8.9 -> 8.6 us, 768 -> 3072 at 384, 512 tokens 9.5 -> 9.2; the one that loses is 1024 -> 4096 at 512 tokens, 10.65 -> 10.85.
     int early = 0;                                           // stages whose B is on its way
-    if (p.b_early && warp == 0) {
+    if (p.b_early && warp == 0 && unit < n_tiles_total) {
         early = min(STAGES, (p.kb_total + G - 1) / G);
-        if (unit >= n_tiles_total) early = 0;
         if (elect_one())
             for (int s = 0; s < early; ++s) {
-                const uint32_t fb_local = smem_u32(&full_bar[s]), fb = CG == 2 ? map_to_cta(fb_local, 0) : fb_local;
-                if (h == 0) mbar_expect_tx(fb_local, CG * C::STAGE_BYTES);
-                load_b(s, s * G, (unit / p.m_tiles) * BN + h * BNH, fb);
+                if (h == 0) mbar_expect_tx(smem_u32(&full_bar[s]), CG * C::STAGE_BYTES);
+                load_b(s, s * G, (unit / p.m_tiles) * BN + h * BNH, full(s));
             }
         __syncwarp();
     }
@@ -149,28 +154,31 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        int s = 0;
+        int s = 0, kb0 = 0;
         uint32_t ph = 1;
         bool ok = true;
+        if (early) {             // (apart from the loop below: tests in it took 3072 -> 768 at 384, 4096 tokens, from 20.5 to 20.9 us)
+            if (elect_one())
+                for (int i = 0; i < early; ++i) load_a(i, i * G, (unit % p.m_tiles) * (BM * CG) + h * BM, full(i));
+            __syncwarp();
+            kb0 = early * G;
+            if (early < STAGES) s = early; else ph = 0;
+        }
         for (int t = unit; t < n_tiles_total && ok; t += n_units) {
             const int m0 = (t % p.m_tiles) * (BM * CG) + h * BM, n0 = (t / p.m_tiles) * BN + h * BNH;
-            for (int kb = 0; kb < p.kb_total; kb += G) {         // k-blocks past the last read as zeros
+            for (int kb = kb0; kb < p.kb_total; kb += G) {       // k-blocks past the last read as zeros
                 ok = mbar_wait_uniform(smem_u32(&empty_bar[s]), ph, ab);
                 if (!ok) break;
-                // a pair's loads all complete on the even block's barrier, which its MMA warp waits on
-                const uint32_t fb_local = smem_u32(&full_bar[s]);
-                const uint32_t fb = CG == 2 ? map_to_cta(fb_local, 0) : fb_local;
-                const uint32_t a_dst = ring_base + s * C::STAGE_BYTES;
+                const uint32_t fb = full(s);
                 if (elect_one()) {
-                    if (h == 0 && early <= 0) mbar_expect_tx(fb_local, CG * C::STAGE_BYTES);
-#pragma unroll
-                    for (int g = 0; g < G; ++g) load2d<CG>(a_dst + g * kATile, &tmA, fb, (kb + g) * BK, m0);
-                    if (early <= 0) load_b(s, kb, n0, fb);
+                    if (h == 0) mbar_expect_tx(smem_u32(&full_bar[s]), CG * C::STAGE_BYTES);
+                    load_a(s, kb, m0, fb);
+                    load_b(s, kb, n0, fb);
                 }
-                --early;
                 __syncwarp();
                 if (++s == STAGES) { s = 0; ph ^= 1; }
             }
+            kb0 = 0;
         }
     } else if (warp == 1 && h == 0) {
         // ------------------------------------------------------------------ MMA issuer (the even block of a pair)

@@ -6,7 +6,7 @@ import torch
 from paper_2309_03824_b200 import binding as b
 from paper_2309_03824_b200 import workloads as wl
 
-from helpers import dev, workspace
+from helpers import TOL, dev, workspace
 
 pytestmark = pytest.mark.gpu
 
@@ -65,3 +65,55 @@ def test_a_long_launch_in_front_of_gradients():
     nchw = lambda t: t.double().permute(0, 3, 1, 2)
     ref = torch.nn.grad.conv2d_weight(nchw(Xc), (S, C, 3, 3), nchw(dYc), padding=1).permute(0, 2, 3, 1)
     assert float((dW.double() - ref).abs().max() / ref.abs().max()) <= 2 ** -8
+
+
+def fresh_operands(bases, call, reference, ws, rounds=4):
+    """Calls one after the other, each on operands that other kernels wrote right before it, in a workspace of NaN, and that are
+    overwritten right behind it: what every call left is what the fp64 reference gives for its operands as they stood."""
+    live = {k: torch.empty_like(v) for k, v in bases.items()}
+    got = []
+    for i in range(rounds):
+        ws.view(torch.bfloat16).fill_(float("nan"))
+        for j, (k, v) in enumerate(bases.items()):
+            torch.mul(v, [1.0, -2.0, 0.5, 3.0][(i + j) % 4], out=live[k])
+        got.append(call(live))
+        for t in live.values():
+            t.fill_(7.0 + i)
+    torch.cuda.synchronize()
+    assert b.lrd_check_device_status() == b.LRD_OK
+    for i, out in enumerate(got):
+        ref = reference({k: (v.float() * [1.0, -2.0, 0.5, 3.0][(i + j) % 4]).double() for j, (k, v) in enumerate(bases.items())})
+        for k, t in out.items():
+            if t is not None:
+                assert float((t.double() - ref[k]).abs().max() / ref[k].abs().max()) <= TOL["bf16"], (i, k)
+
+
+def linear_operands(M, K, N, r, seed, Z=False):
+    case = wl.random_factor_case(M, K, N, r, "bf16", seed)
+    t = {k: dev(case[k], "bf16") for k in ("X", "V", "dY", "b", "U")}
+    return dict(t, Z=(t["X"].float() @ t["V"].float()).to(torch.bfloat16)) if Z else t
+
+
+# tokens, K, N, r of the second product (its reduction): one k-block, a ring that is not filled, one that is, and is reused; several
+# tiles a block; ranks whose rows are padded
+@pytest.mark.parametrize("shape", [(200, 264, 520, 40), (300, 264, 520, 256), (700, 720, 776, 640), (2500, 264, 1032, 136), (9000, 136, 1032, 72), (64, 1096, 2056, 1024), (1021, 264, 520, 129)],
+                         ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("blocks", [1, 2])
+@pytest.mark.parametrize("freeze", [b.LRD_FREEZE_U, b.LRD_FREEZE_V])
+def test_the_second_factor_of_two_products(shape, blocks, freeze):
+    M, K, N, r = shape
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16)
+    ws = workspace(b.lrd_linear_workspace_bytes(desc, freeze, 0))
+
+    def call(t):
+        out = {"Y": torch.empty_like(t["dY"]), "Z": None if freeze == b.LRD_FREEZE_U else torch.empty(M, r, dtype=torch.bfloat16, device="cuda")}
+        b.lrd_linear_fwd(desc, t["X"], t["V"], t["U"], t["b"], out["Y"], out["Z"], freeze, ws)
+        return out
+
+    b.lrd_set_path(b.LRD_PATH_UNFUSED)
+    b.lrd_gemm_tuning(blocks)
+    try:
+        fresh_operands(linear_operands(*shape, 1200 + M), call, lambda t: {"Z": t["X"] @ t["V"], "Y": (t["X"] @ t["V"]) @ t["U"].T + t["b"]}, ws)
+    finally:
+        b.lrd_set_path(b.LRD_PATH_AUTO)
+        b.lrd_gemm_tuning(0)
