@@ -140,7 +140,7 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     // behind the wait.  Forward passes as two products, 72 shapes of 64 to 8192 tokens: 1.3 % on average, 1024 -> 4096 at rank 512,
     // 64 tokens 8.9 -> 8.6 us, 768 -> 3072 at 384, 512 tokens 9.5 -> 9.2; the one that loses is 1024 -> 4096 at 512 tokens, 10.65 -> 10.85.
     int early = 0;                                           // stages whose B is on its way
-    if (p.b_early && warp == 0 && unit < n_tiles_total) {
+    if (!B_MN && p.b_early && warp == 0 && unit < n_tiles_total) {
         early = min(STAGES, (p.kb_total + G - 1) / G);
         if (elect_one())
             for (int s = 0; s < early; ++s) {
