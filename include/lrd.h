@@ -208,7 +208,8 @@ lrd_status_t lrd_data_split_tuning(int columns, int split);
  * caller's stream, which waits for the others before the call returns) when `on` is non-zero - the default -
  * and one after the other on the caller's stream when it is zero.  Same bits either way.  With the core frozen everything
  * runs on the caller's stream, dA and dB in one launch, and the switch has no effect; with the factors frozen the filter
- * gradient follows the data path there, and the switch only decides whether it may start before that path has ended.  With the default,
+ * gradient follows the data path there, and the switch decides whether it may start before that path has ended, or, in a
+ * stream capture, run beside it where SMs are left (if the thread's streams exist; else it follows).  With the default,
  * make a host thread's first backward call on a device outside any stream capture (it creates that thread's
  * streams).  The switch is process-wide; no counterpart in the paper. */
 lrd_status_t lrd_tucker2_overlap(int on);

@@ -54,6 +54,13 @@ size_t split_bytes(const Tk& t) {
 
 bool g_tucker_overlap = true;
 
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st == cudaStreamCaptureStatusActive;
+    cudaGetLastError();
+    return false;
+}
+
 // Ranks that are not multiples of 8 (rows of A, Bm, G, Z1, Z2 then start off 16-byte boundaries): as for the linear
 // layer, the factors -- small -- are copied into the workspace with the ranks rounded up to multiples of 16 (or 8) and
 // zeros in the padding, the layer runs on the tensor-core kernels at the padded ranks, and Z1 / Z2 / dA / dG / dB
@@ -199,9 +206,22 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     // remains the faster way (64 x 7 x 7, 512 -> 512 at 309 92.5 against 96.0).
     // With the factors frozen the filter gradient is the only one: on the tensor-core kernel it follows the data path and loads
     // ahead what that path's last launch does not write, which spares the stream a fork and a join (64 x 28 x 28, stride 2, 256 -> 256
-    // at rank 96 59.4 -> 56.8 us, replayed the same 54.5).  With nothing frozen the streams remain (64 x 7 x 7 at rank 309, replayed:
-    // 81.4 against 83.2), and on the general kernels, which fill few SMs each (fp32, 10 x 14 x 14 at rank 128 223 against 259).
-    const bool filter_follows = core && !factors && path != LRD_PATH_GENERAL && tc_conv_eligible(t.B, t.g, t.r1, t.r2, t.dt, dZ2, Z1_save, dG);
+    // at rank 96 59.4 -> 56.8 us).  A graph's replay has the fork for nothing: there it follows only where the core leaves it no
+    // SMs or the whole path, dZ2 included, is one launch.  Backward replayed, beside / behind: a core of 75 blocks (64 x 7 x 7 at rank
+    // 309) 37.5 / 42.9 us, 100 (64 x 14 x 14, 512 -> 512 at 256, stride 2) 30.1 / 32.5, 147 (32 x 14 x 14 at 320) 49.8 / 47.9, 294 (64
+    // images) 82.3 / 72.9, one launch (64 x 14 x 14 at 96) 25.1 / 23.1; on a stream 47.2 / 45.1, 35.3 / 33.9, 52.7 / 49.9, 81.0 / 75.4 and
+    // 28.6 / 23.4.  With nothing frozen the streams remain (64 x 7 x 7 at rank 309, replayed: 81.4 against 83.2), and on the general
+    // kernels, which fill few SMs each (fp32, 10 x 14 x 14 at rank 128 223 against 259).
+    const bool one_launch = dX && t.plain && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
+                            tucker_fused_eligible(t.B, t.H, t.W, t.S, t.r2, t.r1, t.C, t.dt, dY, Bm, G, A, dX, core ? dZ2 : nullptr,
+                                                  factors ? dZ1 : nullptr);
+    const bool fuse_dx = !one_launch && dX && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
+                         tc_conv_chain_eligible(true, t.B, t.g, t.r1, t.r2, t.C, t.dt, dZ2, G, A, dX, factors ? dZ1 : nullptr);
+    bool filter_follows = core && !factors && path != LRD_PATH_GENERAL && tc_conv_eligible(t.B, t.g, t.r1, t.r2, t.dt, dZ2, Z1_save, dG);
+    if (filter_follows && g_tucker_overlap && dX && !one_launch && 6 * tc_conv_blocks(true, fuse_dx, t.B, t.g, t.r1, t.r2) <= 5 * kNumSms) {
+        const bool captured = capturing(s);                  // (streams for a later capture are made outside of one)
+        filter_follows = !(side_streams(!captured) && captured);
+    }
     SideStreams* ss = g_tucker_overlap && core && !filter_follows ? side_streams() : nullptr;
     cudaStream_t sB = ss && factors ? ss->aux[0] : s, sF = ss ? ss->aux[1] : s;
     lrd_status_t st = LRD_OK;
@@ -221,9 +241,6 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
     // written only for the filter gradient, dZ1 only for dA.  (Giving the filter gradient a dZ2 product of its own
     // beside the pass, so that it need not wait for it, was slower: 44.5 against 41.2 us per step with the core
     // unfrozen -- the extra launch takes SMs from the pass.)
-    const bool one_launch = dX && t.plain && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
-                            tucker_fused_eligible(t.B, t.H, t.W, t.S, t.r2, t.r1, t.C, t.dt, dY, Bm, G, A, dX, core ? dZ2 : nullptr,
-                                                  factors ? dZ1 : nullptr);
     if (one_launch)
         keep(tucker_fused(true, dY, Bm, G, A, nullptr, dX, core ? dZ2 : nullptr, factors ? dZ1 : nullptr, t.B, t.H, t.W, t.S, t.r2,
                           t.r1, t.C, s));
@@ -234,8 +251,6 @@ lrd_status_t tucker2_bwd(const lrd_tucker2_desc_t* d, const void* dY, const void
         else launch_filter(sF, false, false);
     }
     // transposed core + first 1x1 (dX = dZ1 A^T) in one launch where the shape allows; dZ1 is written only for dA
-    const bool fuse_dx = !one_launch && dX && (path == LRD_PATH_AUTO || path == LRD_PATH_FUSED) &&
-                         tc_conv_chain_eligible(true, t.B, t.g, t.r1, t.r2, t.C, t.dt, dZ2, G, A, dX, factors ? dZ1 : nullptr);
     if (one_launch) {
     } else if (fuse_dx) keep(tc_conv_chain(true, dZ2, G, A, nullptr, dX, factors ? dZ1 : nullptr, t.B, t.g, t.r1, t.r2, t.C, s));
     else if (dX || factors) keep(conv_bwd_data(dZ2, G, dZ1, t.B, t.g, t.r1, t.r2, t.dt, path, s));

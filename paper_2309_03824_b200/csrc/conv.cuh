@@ -42,6 +42,8 @@ lrd_status_t simt_conv_bwd_filter(const void* dout, const void* in, void* dG, in
 // Tensor-core k x k core (bf16, channel counts multiples of 8, 16-byte aligned bases; any geometry above).
 bool tc_conv_eligible(int64_t B, const ConvGeom& g, int64_t ci, int64_t co, lrd_dtype_t dt, const void* p0, const void* p1, const void* p2);
 lrd_status_t tc_conv(bool dgrad, const void* img, const void* G, void* out, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, cudaStream_t s);
+// Blocks of that launch (fused: of the one below), up to a few of a strided data gradient.
+int64_t tc_conv_blocks(bool dgrad, bool fused, int64_t B, const ConvGeom& g, int64_t ci, int64_t co);
 // The core followed by the 1x1 product that consumes it, in one launch (the core's result stays on chip unless
 // core_out asks for it): forward (dgrad = false) out2 = conv(img, G) Q^T + bias2 with Q = Bm [S x r2]; backward
 // (dgrad = true) out2 = conv^T(img, G) Q^T with Q = A [C x r1].  n2 = rows of Q = columns of out2 (<= 256).

@@ -427,6 +427,13 @@ lrd_status_t tc_conv(bool dgrad, const void* img, const void* G, void* out, int6
     return dgrad ? launch_conv<true, false>(maps, p, 0, s) : launch_conv<false, false>(maps, p, 0, s);
 }
 
+int64_t tc_conv_blocks(bool dgrad, bool fused, int64_t B, const ConvGeom& g, int64_t ci, int64_t co) {
+    const int64_t tiles = (B * (dgrad ? (int64_t)g.H * g.W : (int64_t)g.Ho * g.Wo) + 127) / 128, n = dgrad ? ci : co, ka = dgrad ? co : ci;
+    if (fused) return tiles;
+    const int bn = pick_bn(tiles, n, (ka + 63) / 64 * g.k * g.k / (dgrad ? g.stride * g.stride : 1));
+    return tiles * ((n + bn - 1) / bn);
+}
+
 bool tc_conv_chain_eligible(bool dgrad, int64_t B, const ConvGeom& g, int64_t ci, int64_t co, int64_t n2, lrd_dtype_t dt,
                             const void* img, const void* G, const void* Q, const void* out2, const void* core_out) {
     const int64_t n1 = dgrad ? ci : co;                  // channels of the core's result = reduction of the 1x1 product

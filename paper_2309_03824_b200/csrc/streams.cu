@@ -7,12 +7,12 @@ thread_local SideStreams g_sides[kMaxDevices];
 thread_local int g_n_sides = 0;
 }  // namespace
 
-SideStreams* side_streams() {
+SideStreams* side_streams(bool make) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     for (int i = 0; i < g_n_sides; ++i)
         if (g_sides[i].device == dev) return &g_sides[i];
-    if (g_n_sides == kMaxDevices) return nullptr;
+    if (!make || g_n_sides == kMaxDevices) return nullptr;
     SideStreams* ss = &g_sides[g_n_sides];
     bool ok = cudaEventCreateWithFlags(&ss->fork, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&ss->mid, cudaEventDisableTiming) == cudaSuccess;

@@ -16,8 +16,8 @@ struct SideStreams {
     cudaEvent_t fork, mid, join[kSideStreams], aux_done[kSideStreams];
 };
 
-// The calling device's set, or nullptr if it could not be made.
-SideStreams* side_streams();
+// The calling device's set, or nullptr if it could not be made (or, make = false, has not been).
+SideStreams* side_streams(bool make = true);
 
 // waiter's next work follows what `done` holds so far
 inline bool stream_after(cudaStream_t waiter, cudaStream_t done, cudaEvent_t ev) {

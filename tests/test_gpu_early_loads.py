@@ -1,5 +1,8 @@
 """Launches that start, or load, before the launch in front of them has ended: what they read is what their call's operands hold, and
 the limit of their device-side waits does not count the time of the launch in front."""
+import ctypes
+import threading
+
 import pytest
 import torch
 
@@ -117,3 +120,68 @@ def test_the_second_factor_of_two_products(shape, blocks, freeze):
     finally:
         b.lrd_set_path(b.LRD_PATH_AUTO)
         b.lrd_gemm_tuning(0)
+
+
+def conv_layer(t, stride):
+    nchw = lambda x: x.permute(0, 3, 1, 2)
+    Z1 = t["X"] @ t["A"]
+    Z2 = torch.nn.functional.conv2d(nchw(Z1), t["G"].permute(0, 3, 1, 2), stride=stride, padding=t["G"].shape[1] // 2).permute(0, 2, 3, 1)
+    return Z1, Z2, Z2 @ t["Bm"].T + t["b"]
+
+
+def conv_operands(geom, seed):
+    B, H, W, C, S, r1, r2, k, stride = geom
+    case = wl.random_tucker_case(B, H, W, C, S, r1, r2, k, "bf16", seed, stride=stride)
+    return {n: dev(case[n], "bf16") for n in ("X", "A", "G", "Bm", "b", "dY")}
+
+
+class Edge(ctypes.Structure):
+    _fields_ = [("from_port", ctypes.c_ubyte), ("to_port", ctypes.c_ubyte), ("type", ctypes.c_ubyte), ("reserved", ctypes.c_ubyte * 5)]
+
+
+def branches(graph):
+    """Launches of a captured graph that more than one other follows."""
+    cu, count = ctypes.CDLL("libcuda.so.1"), ctypes.c_size_t(64)
+    ends, edges = [(ctypes.c_void_p * 64)() for _ in range(2)], (Edge * 64)()
+    assert cu.cuGraphGetEdges_v2(ctypes.c_void_p(graph.raw_cuda_graph()), ends[0], ends[1], edges, ctypes.byref(count)) == 0
+    froms = ends[0][:count.value]
+    return sum(froms.count(n) > 1 for n in set(froms))
+
+
+# the core's data gradient on few blocks; on as many as there are SMs; the whole data path in one launch
+@pytest.mark.parametrize("geom,beside", [((16, 7, 7, 264, 272, 136, 144, 3, 1), True), ((8, 14, 14, 72, 136, 48, 48, 3, 2), True), ((64, 14, 14, 264, 272, 320, 256, 3, 1), False),
+                                         ((16, 14, 14, 64, 72, 32, 48, 3, 1), False)], ids=lambda g: str(g))
+def test_a_captured_filter_gradient_runs_beside_a_data_path_that_leaves_it_room(geom, beside):
+    """With the factors frozen: beside the data path in a graph, behind it elsewhere and where a thread's first call is captured (it has no
+    streams then); the same bits each way."""
+    B, H, W, C, S, r1, r2, k, stride = geom
+    r1, r2 = min(r1, C), min(r2, S)
+    freeze = b.LRD_TK_FREEZE_FACTORS
+    desc = b.tucker2_desc(B, H, W, C, S, r1, r2, b.LRD_BF16, k=k, stride=stride, pad=(k - 1) // 2)
+    t = conv_operands((B, H, W, C, S, r1, r2, k, stride), 1600 + B)
+    Z1 = (t["X"].float() @ t["A"].float()).to(torch.bfloat16)
+    ws = workspace(b.lrd_tucker2_workspace_bytes(desc, freeze, 1))
+    dX, dG = torch.empty_like(t["X"]), torch.empty_like(t["G"])
+    call = lambda: b.lrd_tucker2_bwd(desc, t["dY"], None, t["A"], t["G"], t["Bm"], Z1, None, dX, None, dG, None, None, freeze, ws)
+    call()
+    torch.cuda.synchronize()
+    want = dX.clone(), dG.clone()
+    found = []
+
+    def capture():
+        side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side, capture_error_mode="thread_local"):
+            call()
+        dX.zero_()
+        dG.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        found.append((branches(graph), torch.equal(dX, want[0]), torch.equal(dG, want[1])))
+
+    capture()
+    other = threading.Thread(target=capture)
+    other.start()
+    other.join()
+    assert found == [(1 if beside else 0, True, True), (0, True, True)]
+    assert b.lrd_check_device_status() == b.LRD_OK
