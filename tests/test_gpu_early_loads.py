@@ -122,6 +122,47 @@ def test_the_second_factor_of_two_products(shape, blocks, freeze):
         b.lrd_gemm_tuning(0)
 
 
+def linear_gradients(t, add=0.0):
+    dZ = t["dY"] @ t["U"]
+    return {"dX": dZ @ t["V"].T, "dU": t["dY"].T @ t["Z"] + add, "dV": t["X"].T @ dZ + add, "db": t["dY"].sum(0) + add}
+
+
+@pytest.mark.parametrize("freeze", [b.LRD_FREEZE_V, b.LRD_FREEZE_U, b.LRD_FREEZE_NONE])
+@pytest.mark.parametrize("shape", [(4096, 768, 768, 192), (128, 768, 768, 192), (1021, 1024, 1024, 512), (300, 520, 520, 250), (2000, 264, 264, 64), (2048, 1024, 2056, 250)],
+                         ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("path", [b.LRD_PATH_AUTO, b.LRD_PATH_UNFUSED])
+@pytest.mark.parametrize("adding", [False, True])
+def test_the_gradients_of_a_layer(shape, freeze, path, adding):
+    """What dU, dV and the second factor of the data pass load ahead; adding, to what an earlier launch left in the caller's buffers."""
+    M, K, N, r = shape
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16)
+    ws = workspace(b.lrd_linear_workspace_bytes(desc, freeze, 2 if adding else 1))
+    backward = b.lrd_linear_bwd_accumulate if adding else b.lrd_linear_bwd
+
+    def call(t):
+        out = {k: torch.full(s, 2.0 if adding else float("nan"), dtype=torch.bfloat16, device="cuda") for k, s in (("dU", (N, r)), ("dV", (K, r)), ("db", (N,)))}
+        if freeze == b.LRD_FREEZE_U:
+            out.update(dU=None, db=None)
+        if freeze == b.LRD_FREEZE_V:
+            out.update(dV=None)
+        out["dX"] = torch.empty_like(t["X"])
+        backward(desc, t["dY"], t["X"], t["V"], t["U"], t["Z"], out["dX"], out["dU"], out["dV"], out["db"], freeze, ws)
+        return out
+
+    b.lrd_set_path(path)
+    try:
+        fresh_operands(linear_operands(*shape, 1300 + M, Z=True), call, lambda t: linear_gradients(t, 2.0 if adding else 0.0), ws)
+    finally:
+        b.lrd_set_path(b.LRD_PATH_AUTO)
+
+
+MASKS = [b.LRD_TK_FREEZE_NONE, b.LRD_TK_FREEZE_FACTORS, b.LRD_TK_FREEZE_CORE]
+# whole pass in one launch; 1x1 products apart from the core, then (S > 256) the last one too; the same at ranks whose rows are padded;
+# stride 2 with the core and one product in a launch, then apart, then padded
+CONVS = [(16, 14, 14, 64, 72, 32, 48, 3, 1), (8, 9, 11, 136, 128, 96, 104, 3, 1), (16, 7, 7, 264, 272, 136, 144, 3, 1), (16, 7, 7, 264, 272, 135, 141, 3, 1),
+         (8, 14, 14, 72, 136, 48, 48, 3, 2), (16, 13, 14, 264, 272, 136, 152, 3, 2), (16, 14, 13, 264, 272, 130, 150, 3, 2), (8, 9, 9, 40, 264, 24, 40, 5, 1)]
+
+
 def conv_layer(t, stride):
     nchw = lambda x: x.permute(0, 3, 1, 2)
     Z1 = t["X"] @ t["A"]
@@ -133,6 +174,61 @@ def conv_operands(geom, seed):
     B, H, W, C, S, r1, r2, k, stride = geom
     case = wl.random_tucker_case(B, H, W, C, S, r1, r2, k, "bf16", seed, stride=stride)
     return {n: dev(case[n], "bf16") for n in ("X", "A", "G", "Bm", "b", "dY")}
+
+
+@pytest.mark.parametrize("geom", CONVS, ids=lambda g: "x".join(map(str, g)))
+@pytest.mark.parametrize("freeze", MASKS)
+def test_the_second_factor_and_the_copies_of_a_convolution(geom, freeze):
+    """The forward pass: the last product's factor, and Z1 and Z2 copied to the caller's rows beside it."""
+    B, H, W, C, S, r1, r2, k, stride = geom
+    desc = b.tucker2_desc(B, H, W, C, S, r1, r2, b.LRD_BF16, k=k, stride=stride, pad=(k - 1) // 2)
+    ws = workspace(b.lrd_tucker2_workspace_bytes(desc, freeze, 0))
+    Ho, Wo = (H - 1) // stride + 1, (W - 1) // stride + 1
+
+    def call(t):
+        new = lambda *s: torch.empty(*s, dtype=torch.bfloat16, device="cuda")
+        out = {"Y": new(B, Ho, Wo, S), "Z1": None if freeze == b.LRD_TK_FREEZE_CORE else new(B, H, W, r1), "Z2": None if freeze == b.LRD_TK_FREEZE_FACTORS else new(B, Ho, Wo, r2)}
+        b.lrd_tucker2_fwd(desc, t["X"], t["A"], t["G"], t["Bm"], t["b"], out["Y"], out["Z1"], out["Z2"], freeze, ws)
+        return out
+
+    fresh_operands(conv_operands(geom, 1400 + C), call, lambda t: dict(zip(("Z1", "Z2", "Y"), conv_layer(t, stride))), ws)
+
+
+@pytest.mark.parametrize("geom", CONVS, ids=lambda g: "x".join(map(str, g)))
+@pytest.mark.parametrize("freeze", MASKS)
+@pytest.mark.parametrize("overlap", [True, False])
+def test_the_gradients_of_a_convolution(geom, freeze, overlap):
+    """dA and dB with the core frozen, the filter gradient that follows the data path or runs beside it, the last product's factor."""
+    B, H, W, C, S, r1, r2, k, stride = geom
+    desc = b.tucker2_desc(B, H, W, C, S, r1, r2, b.LRD_BF16, k=k, stride=stride, pad=(k - 1) // 2)
+    ws = workspace(b.lrd_tucker2_workspace_bytes(desc, freeze, 1))
+    bases = conv_operands(geom, 1500 + C)
+    with torch.no_grad():
+        Z1, Z2, _ = conv_layer({n: v.double() for n, v in bases.items()}, stride)
+    bases.update(Z1=Z1.to(torch.bfloat16).contiguous(), Z2=Z2.to(torch.bfloat16).contiguous())
+    factors, core = freeze != b.LRD_TK_FREEZE_FACTORS, freeze != b.LRD_TK_FREEZE_CORE
+
+    def call(t):
+        out = {"dX": torch.empty_like(t["X"]), "dA": torch.empty_like(t["A"]) if factors else None, "dB": torch.empty_like(t["Bm"]) if factors else None,
+               "db": torch.empty_like(t["b"]) if factors else None, "dG": torch.empty_like(t["G"]) if core else None}
+        b.lrd_tucker2_bwd(desc, t["dY"], t["X"] if factors else None, t["A"], t["G"], t["Bm"], t["Z1"] if core else None, t["Z2"] if factors else None, out["dX"],
+                          out["dA"], out["dG"], out["dB"], out["db"], freeze, ws)
+        return out
+
+    def reference(t):
+        nchw = lambda x: x.permute(0, 3, 1, 2)
+        G, pad = nchw(t["G"]), k // 2
+        dZ2 = t["dY"] @ t["Bm"]
+        dZ1 = torch.nn.grad.conv2d_input((B, r1, H, W), G, nchw(dZ2), stride=stride, padding=pad).permute(0, 2, 3, 1)
+        dG = torch.nn.grad.conv2d_weight(nchw(t["Z1"]), G.shape, nchw(dZ2), stride=stride, padding=pad).permute(0, 2, 3, 1)
+        flat = lambda x: x.reshape(-1, x.shape[-1])
+        return {"dX": dZ1 @ t["A"].T, "dA": flat(t["X"]).T @ flat(dZ1), "dB": flat(t["dY"]).T @ flat(t["Z2"]), "db": flat(t["dY"]).sum(0), "dG": dG}
+
+    b.lrd_tucker2_overlap(overlap)
+    try:
+        fresh_operands(bases, call, reference, ws)
+    finally:
+        b.lrd_tucker2_overlap(True)
 
 
 class Edge(ctypes.Structure):

@@ -137,3 +137,29 @@ def test_adding_leaves_the_rest_alone(form, shape, forms):
     assert float((dU[:, :r].double() - ref - 3).abs().max() / (ref.abs().max() + 3)) <= 2 ** -7
     assert float((db.double() - dY.double().sum(0) - 1).abs().max() / dY.double().sum(0).abs().max()) <= 2 ** -7
     assert bool((dU[:, r:] == 3).all())
+
+
+SPECIAL = [0x0000, 0x8000, 0x0001, 0x807f, 0x0040, 0x0080, 0x80ff, 0x3f80, 0xbf80, 0x3f81, 0x7b80, 0x7f00, 0x7f7f, 0xff7f, 0x7f80, 0xff80, 0x7fc0]
+
+
+@gpu
+@pytest.mark.parametrize("form", [f for f in SINGLE if f[2] in (1, 3, 8)] + PAIRS[::3], ids=lambda f: "x".join(map(str, f)))
+def test_adding_special_values(form, forms):
+    """Infinities and their opposites, NaN, sums that overflow, subnormals: the fp32 sum of what stood there and the product, rounded once."""
+    M, K, N, r = 64, 136, 264, 64
+    S = torch.tensor(SPECIAL, dtype=torch.int32).to(torch.int16).view(torch.bfloat16).cuda()
+    dY, Z = torch.zeros(M, N, dtype=torch.bfloat16, device="cuda"), torch.zeros(M, r, dtype=torch.bfloat16, device="cuda")
+    dY[0], Z[0] = S.repeat(N // len(S) + 1)[:N], 1                     # dU[n][c] = dY[0][n], whatever c
+    V, U = torch.zeros(K, r, dtype=torch.bfloat16, device="cuda"), torch.zeros(N, r, dtype=torch.bfloat16, device="cuda")
+    before = S.repeat(r // len(S) + 1)[:r].repeat(N, 1)
+    dU, alone = before.clone(), torch.empty(N, r, dtype=torch.bfloat16, device="cuda")
+    dX, db = torch.empty(M, K, dtype=torch.bfloat16, device="cuda"), torch.zeros(N, dtype=torch.bfloat16, device="cuda")
+    desc = b.linear_desc(M, K, N, r, b.LRD_BF16)
+    ws = torch.empty(b.lrd_linear_workspace_bytes(desc, b.LRD_FREEZE_V, 2), dtype=torch.uint8, device="cuda")
+    b.lrd_wgrad_tuning(*form)
+    b.lrd_linear_bwd_accumulate(desc, dY, None, V, U, Z, dX, dU, None, db, b.LRD_FREEZE_V, ws)
+    b.lrd_linear_bwd(desc, dY, None, V, U, Z, dX, alone, None, db, b.LRD_FREEZE_V, ws)
+    assert b.lrd_check_device_status() == b.LRD_OK
+    want = (alone.float() + before.float()).to(torch.bfloat16)
+    assert bool(((dU.view(torch.int16) == want.view(torch.int16)) | (dU.isnan() & want.isnan())).all())
+    assert bool(alone[:17].isinf().any()) and bool(want.isnan().any())

@@ -251,14 +251,18 @@ def test_gradients_that_start_beside_their_data_pass(shape, freeze, path):
                 dY.copy_(dX)                                            # (K = N)
             torch.mul(Z0, 1.0 + i, out=Z)
             torch.mul(X, 1.0 - i, out=Xc)
-            g = [torch.empty(s, dtype=torch.bfloat16, device="cuda") for s in ((N, r), (K, r), (N,))]
             for _ in range(2):                                          # the second call's data pass behind the first one's gradients
-                b.lrd_linear_bwd(desc, dY, Xc, V, U, Z, dX, g[0], g[1], g[2], freeze, ws)
+                g = [torch.empty(s, dtype=torch.bfloat16, device="cuda") for s in ((N, r), (K, r), (N,))] + [torch.empty_like(X)]
+                b.lrd_linear_bwd(desc, dY, Xc, V, U, Z, g[3], g[0], g[1], g[2], freeze, ws)
                 if wait:
                     torch.cuda.synchronize()
+                out += g
+                dX.copy_(g[3])
+                for t in (dY, Z, Xc):                                   # other operands, and nothing of this call in the workspace
+                    t.mul_(-0.5)
+                ws.view(torch.bfloat16).fill_(float("nan"))
             for t in (dY, Z, Xc):
                 t.zero_()
-            out += g + [dX.clone()]
         torch.cuda.synchronize()
         return out
 
