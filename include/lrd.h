@@ -226,7 +226,7 @@ lrd_status_t lrd_check_device_status(void);
 
 /* Self-test of the bounded device-side wait (no counterpart in the paper): enqueues one small block that waits,
  * through the same routine and with the same limit as every pipeline wait of the library's kernels, on a barrier
- * nothing ever arrives at.  The wait runs out after a second or so, raises the timeout flag and the block
+ * nothing ever arrives at.  The wait runs out after some 17 seconds, raises the timeout flag and the block
  * returns in order (nothing is in flight, no tensor memory is held).  The next lrd_check_device_status() returns
  * LRD_ERR_TIMEOUT once, the one after LRD_OK, and every other entry point keeps working.  Returns
  * LRD_ERR_ARCH / LRD_ERR_CUDA as the other entry points do. */

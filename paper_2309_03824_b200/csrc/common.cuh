@@ -42,10 +42,13 @@ struct GemmArgs {
                                // type before the fp32 sum and after it
     bool whole = false;        // data products: the reduction is not split over a cluster
     // Weight gradients on the single-SM kernels, and B of data products on the persistent one: this operand is loaded without waiting
-    // for the launch before this one, which is of the same call and does not write it.  Everything else the call reads is complete
-    // by then, because every kernel here that a call can put in front of such a product lets the next launch start only behind its
-    // own griddepcontrol.wait; and because the launch waits for the one before it before it ends, whoever waits for it has
-    // waited for both.  A launch boundary costs some 1.5 us behind the last block's exit and another for the first loads.
+    // for the launch before this one (griddepcontrol.wait).  Two things have to hold.  Between the start of the call and this
+    // launch stands one that lets the next launch start only behind its own wait: all data passes (both chains, the data products,
+    // convolutions, the one-launch pass, the general products) do, weight gradients (both kernels) and repacking copies let it start
+    // before, and are nothing to rely on.  What the call found in memory is complete by then.  And neither that launch nor a later
+    // one of the call writes the operand.  Every launch waits for the one before it before it ends, early ones too, so that whoever
+    // waits for the last has waited for all.  A launch boundary costs some 1.5 us behind the last block's exit and another for the
+    // first loads.
     // Gradients: 768 -> 768 at r = 192, a pass over 128 tokens 18.5 -> 17.7 us, over 4096 26.3 -> 25.7; six layers of 768 (4096
     // tokens) replayed 170.8 -> 168.6.
     bool a_early = false, b_early = false;

@@ -211,7 +211,7 @@ conv_kernel(const __grid_constant__ ConvMaps maps, const ConvParams p) {
             }
         }
     } else {
-        const int q = warp % 4, hw = (warp - 2) / 4;             // two warps share a quarter of the rows: alternate 32-column pieces
+        const int q = warp % 4, hw = (warp - 2) / 4;             // two warps share a quarter of the rows: alternate 64-column blocks
         const int m = m0 + q * 32 + lane;
         int pix = m < cl.pixels ? m : -1;                        // this lane's pixel of the output image(s); -1: none
         if (p.step > 1 && pix >= 0) {

@@ -299,7 +299,7 @@ lrd_status_t copy2d_bf16(const Copy2d* c, int n, cudaStream_t s, bool early) {
     cfg.blockDim = dim3(256, 1, 1);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) before it touches global memory
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) before it copies, EARLY before it ends
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;

@@ -255,8 +255,8 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int n, bool a_mn_major, bool b
 // ---- programmatic dependent launch ----------------------------------------------------------------
 // A kernel launched with the programmatic-serialization attribute may start while its predecessor in
 // the stream is still running.  launch_dependents: this block no longer holds the next kernel back.
-// wait: returns once the predecessor has completed and its memory operations are visible; nothing
-// before it may touch global memory.  Both are no-ops in a kernel launched without the attribute.
+// wait: returns once the predecessor has completed and its memory operations are visible; before it global memory
+// may only be touched by the rule at GemmArgs::a_early.  Both are no-ops in a kernel launched without the attribute.
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

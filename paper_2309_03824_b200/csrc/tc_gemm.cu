@@ -168,7 +168,8 @@ tc_gemm_kernel(const __grid_constant__ TcLaunch<NP> L) {
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only this block's own shared and tensor memory: it may overlap the tail of the
-    // previous kernel in the stream; global memory is first touched below this line, by the producers and then by the epilogue.
+    // previous kernel in the stream, and so may the loads of early operands (GemmArgs::a_early); everything else that touches global
+    // memory stands behind the wait.
     // Every wait with a limit starts behind griddepcontrol.wait, as the launch in front, which may be the caller's, takes what time
     // it likes; with early operands it is a data pass of the same call, and the waits that need nothing of it start at once.
     const bool all_early = A_MN && p.a_early && p.b_early;
@@ -606,7 +607,7 @@ lrd_status_t launch(const TcLaunch<NP>& L, dim3 grid, cudaStream_t stream, bool 
     attr[0].val.clusterDim.x = 1;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = p.cluster_splits > 1 ? (unsigned)p.cluster_splits : 1u;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) before it touches global memory
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) for all but early operands
     attr[1].val.programmaticStreamSerializationAllowed = wait_ahead ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 2;

@@ -332,7 +332,7 @@ lrd_status_t launch_p(const CUtensorMap& tA, const CUtensorMap& tB, const CUtens
     cfg.dynamicSmemBytes = PCfg<BN, CG>::SMEM_BYTES;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) before it touches global memory
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits (griddepcontrol.wait) for all but an early B
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = CG;

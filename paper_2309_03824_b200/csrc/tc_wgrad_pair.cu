@@ -156,7 +156,7 @@ wgrad_pair_kernel(const __grid_constant__ WgradLaunch<NP> L) {
     const uint32_t tmem_base = tmem_base_slot;
     // set-up above touched only shared and tensor memory: it may overlap the tail of the previous kernel in the stream;
     // global memory is first touched below this line
-    griddep_launch_dependents();
+    griddep_launch_dependents();       // (before the wait: nothing for an early launch to rely on, see GemmArgs::a_early)
     griddep_wait();
 
     if (warp == 0) {
