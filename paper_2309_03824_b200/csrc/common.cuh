@@ -44,8 +44,8 @@ struct GemmArgs {
     // Weight gradients on the single-SM kernels, and B of data products on the persistent one: this operand is loaded without waiting
     // for the launch before this one (griddepcontrol.wait).  Two things have to hold.  Between the start of the call and this
     // launch stands one that lets the next launch start only behind its own wait: all data passes (both chains, the data products,
-    // convolutions, the one-launch pass, the general products) do, weight gradients (both kernels) and repacking copies let it start
-    // before, and are nothing to rely on.  What the call found in memory is complete by then.  And neither that launch nor a later
+    // convolutions, the one-launch pass, the general products) do, weight gradients (both kernels) and copies that are early
+    // themselves let it start before, and are nothing to rely on.  What the call found in memory is complete by then.  And neither that launch nor a later
     // one of the call writes the operand.  Every launch waits for the one before it before it ends, early ones too, so that whoever
     // waits for the last has waited for all.  A launch boundary costs some 1.5 us behind the last block's exit and another for the
     // first loads.

@@ -254,11 +254,12 @@ struct CopyBatch {
     int n;
 };
 // EARLY: as GemmArgs::a_early (a variant: with the test at run time each of the four launches around 64 x 7 x 7 at rank 309 took 0.4 us more).
-// Either lets the next launch start at once, which then sets itself up beside the copy (768 -> 768 at rank 95, 64 tokens, forward
-// with U frozen 8.7 us behind the wait, 8.1 so): it is never the launch that an early one relies on, see GemmArgs.
+// The others wait before they let the next launch start: the other way round two of them in a row (a pass's last and the next one's
+// first) hold the launch behind them back, 1 x 28 x 28 at rank 49 as training steps 28.3 -> 31.1 us, 46 cases 1.6 % on average, for
+// 3 % of a forward pass alone.
 template <bool EARLY> __global__ void __launch_bounds__(256) copy2d_bf16_kernel(const __grid_constant__ CopyBatch b) {
-    ptx::griddep_launch_dependents();
     if (!EARLY) ptx::griddep_wait();
+    ptx::griddep_launch_dependents();
     const int lane = threadIdx.x % 32;
     const int64_t warps = (int64_t)gridDim.x * 8;
     int j = 0;
