@@ -931,8 +931,8 @@ constexpr double kNextLaunch = 2.0;            // a launch behind another one dr
 
 // Gradients whose rows TMA cannot address run on single SMs only: worth it where pairs would not save more than the launch that
 // copies a padded result, some 3 us.  Over 360 backward passes of packed layers (64 to 8192 tokens, ranks 61 to 1001, each mask) the
-// choice costs 0.3 % on average against the fastest measurement (always in place 0.5 %, always copied 7.0): 2048 tokens, 1024 -> 4096 at
-// rank 250, nothing frozen, in place / copied 30.1 / 32.7 us; 4096 tokens, 4096 -> 4096 at rank 499 84.3 / 80.7.
+// choice costs 0.3 % on average against the fastest measurement (always in place 0.5 %, always copied 7.0): 2048 tokens, 4096 -> 4096 at
+// rank 250, nothing frozen, in place / copied 37.8 / 41.2 us; 4096 tokens, 4096 -> 4096 at rank 499 84.3 / 80.7.
 bool tc_wgrads_any_rows(const GemmArgs* g, int n) {
     if (tc_wgrad_form().blocks) return false;
     double single = kNextLaunch * (n - 1), pairs = single;
